@@ -22,6 +22,8 @@
 #include <type_traits>
 #include <cuda_runtime.h>
 
+#include "tables.cuh"
+
 namespace pa {
 
 // Element arithmetic of the transforms. Arith<float> / Arith<double> work on
@@ -158,87 +160,20 @@ __host__ __device__ constexpr double trig_frac(int a, int b, bool want_sin) {
 __host__ __device__ constexpr double cos_frac(int a, int b) { return trig_frac(a, b, false); }
 __host__ __device__ constexpr double sin_frac(int a, int b) { return trig_frac(a, b, true); }
 
-// x * w_N^J (forward root w_N = exp(-2 pi i / N); the inverse uses the conjugate),
-// with the half and quarter turns done exactly.
-template <typename T, int N, int J, bool INV>
-__device__ __forceinline__ cx<T> rot_const(cx<T> x) {
-    constexpr int j = J % N;
-    if constexpr (j == 0) {
-        return x;
-    } else if constexpr (2 * j == N) {
-        return Arith<T>::mk(-x.x, -x.y);
-    } else if constexpr (4 * j == N) {
-        return INV ? Arith<T>::mk(-x.y, x.x) : Arith<T>::mk(x.y, -x.x);
-    } else if constexpr (4 * j == 3 * N) {
-        return INV ? Arith<T>::mk(x.y, -x.x) : Arith<T>::mk(-x.y, x.x);
-    } else {
-        constexpr T c = (T)cos_frac(j, N);
-        constexpr T sn = (T)sin_frac(j, N);
-        constexpr T s = INV ? sn : -sn;
-        return Arith<T>::mk(x.x * c - x.y * s, x.x * s + x.y * c);
-    }
-}
-
-// a[n2 * RO + k1] *= w_{RO R0}^{n2 k1} for n2 >= N2, k1 >= K1 (compile-time indices).
-template <typename T, int RO, int R0, int N2, int K1, bool INV>
-__device__ __forceinline__ void comp_twiddle_row(cx<T> *a) {
-    if constexpr (K1 < RO) {
-        a[N2 * RO + K1] = rot_const<T, RO * R0, N2 * K1, INV>(a[N2 * RO + K1]);
-        comp_twiddle_row<T, RO, R0, N2, K1 + 1, INV>(a);
-    }
-}
-template <typename T, int RO, int R0, int N2, bool INV>
-__device__ __forceinline__ void comp_twiddles(cx<T> *a) {
-    if constexpr (N2 < R0) {
-        comp_twiddle_row<T, RO, R0, N2, 1, INV>(a);
-        comp_twiddles<T, RO, R0, N2 + 1, INV>(a);
-    }
-}
-
-template <typename T, int R, bool INV> __device__ __forceinline__ void dft(cx<T> *v);
-
-// In-register DFT of RC = RO * R0 values (RO in {3, 5, 9}, R0 a power of two),
-// natural order in and out, by one Cooley-Tukey step: with n = R0 n1 + n2 and
-// k = k1 + RO k2, X[k] = sum_n2 w_R0^{n2 k2} w_RC^{n2 k1} sum_n1 w_RO^{n1 k1} x[n].
-template <typename T, int RO, int R0, bool INV>
-__device__ __forceinline__ void dft_comp(cx<T> *x) {
-    if constexpr (R0 == 1) {
-        dft_odd<T, RO, INV>(x);
-    } else {
-        cx<T> a[RO * R0];  // a[n2 * RO + k1]
-#pragma unroll
-        for (int n2 = 0; n2 < R0; ++n2) {
-            cx<T> u[RO];
-#pragma unroll
-            for (int n1 = 0; n1 < RO; ++n1) u[n1] = x[R0 * n1 + n2];
-            dft_odd<T, RO, INV>(u);
-#pragma unroll
-            for (int k1 = 0; k1 < RO; ++k1) a[n2 * RO + k1] = u[k1];
-        }
-        comp_twiddles<T, RO, R0, 1, INV>(a);
-#pragma unroll
-        for (int k1 = 0; k1 < RO; ++k1) {
-            cx<T> w[R0];
-#pragma unroll
-            for (int n2 = 0; n2 < R0; ++n2) w[n2] = a[n2 * RO + k1];
-            dft<T, R0, INV>(w);
-#pragma unroll
-            for (int k2 = 0; k2 < R0; ++k2) x[k1 + RO * k2] = w[k2];
-        }
-    }
-}
-
-// Twiddle table pair for the length-L transform root w_L: w_L^e = hi[e >> B] * lo[e & (2^B-1)].
-// Complex roots are exp(-2*pi*i/L), computed in double precision on the host and rounded to T.
+// Twiddle tables of a length-L transform as the kernels take them (layout: tables.cuh).
+// Complex roots are exp(-2*pi*i/L), the inverse transform takes the conjugates; the exact
+// transform has tables of its own for the inverse passes.
+template <typename T> struct PassTw {
+    const cx<T> *a;  // a[tq * (S / COLS) + blk]
+    const cx<T> *c;  // c[tq * COLS + col]
+    const cx<T> *g;  // g[u]
+};
 template <typename T> struct TwTab {
     const cx<T> *hi;
     const cx<T> *lo;
-    uint32_t B;    // split position
-    uint32_t lgL;  // log2 L
-    // In-CTA stage twiddles: fine[j] = w_F^j, where F (a divisor of L) is a
-    // multiple of every pass length of the plan.
-    const cx<T> *fine;
-    uint32_t F;
+    uint32_t B;              // w_L^e = hi[e >> B] * lo[e & (2^B - 1)]
+    const cx<T> *st[3];      // stage tables: first pass, middle strided pass, innermost pass
+    PassTw<T> fw[2], iv[2];  // pass tables of the first and the middle strided pass
 };
 
 template <typename T> struct ComplexArith {
@@ -247,19 +182,16 @@ template <typename T> struct ComplexArith {
     static __device__ __forceinline__ E add(E a, E b) { return mk(a.x + b.x, a.y + b.y); }
     static __device__ __forceinline__ E sub(E a, E b) { return mk(a.x - b.x, a.y - b.y); }
     static __device__ __forceinline__ E mul(E a, E b) { return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
-    // x * w^j with w = exp(-2*pi*i/32) (forward) or its conjugate (inverse). j is a
-    // compile-time constant after unrolling, so the branches fold away.
-    template <bool INV> static __device__ __forceinline__ E rot32(E x, int j) {
-        if (j == 0) return x;
-        if (j == 8) return INV ? mk(-x.y, x.x) : mk(x.y, -x.x);
-        const T c = (T)cos32(j);
-        const T s = INV ? (T)sin32(j) : -(T)sin32(j);
-        return mk(x.x * c - x.y * s, x.x * s + x.y * c);
-    }
-    template <bool INV> static __device__ __forceinline__ E fine(const TwTab<T> &t, uint32_t e) {
-        E w = __ldg(t.fine + e);
-        if (INV) w.y = -w.y;
-        return w;
+    // k*a + c for a real k
+    static __device__ __forceinline__ E fmak(T k, E a, E c) { return mk(k * a.x + c.x, k * a.y + c.y); }
+    static __device__ __forceinline__ E mulk(T k, E a) { return mk(k * a.x, k * a.y); }
+    // (a, b) -> (a + w b, a - w b), w = c + i s: six fused multiply-adds, the difference
+    // as 2a - (a + w b).
+    static __device__ __forceinline__ void bfly(E &a, E &b, T c, T s) {
+        const E t = fmak(c, b, a);
+        const E p = mk(fma(-s, b.y, t.x), fma(s, b.x, t.y));
+        b = mk(fma((T)2, a.x, -p.x), fma((T)2, a.y, -p.y));
+        a = p;
     }
     template <bool INV> static __device__ __forceinline__ E omega(const TwTab<T> &t, uint32_t e) {
         E a = __ldg(t.hi + (e >> t.B));
@@ -293,6 +225,17 @@ __device__ __forceinline__ float2 f2_sub(float2 a, float2 b) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
 }
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
+    float2 d;
+    asm("{.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\t"
+        "mov.b64 rb, {%4, %5};\n\t"
+        "mul.rn.f32x2 rd, ra, rb;\n\t"
+        "mov.b64 {%0, %1}, rd;}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 // d = a * b + c on both lanes of an f32x2 pair (one packed instruction).
 __device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
     float2 d;
@@ -309,6 +252,14 @@ __device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
 template <> struct Arith<float> : ComplexArith<float> {
     static __device__ __forceinline__ E add(E a, E b) { return f2_add(a, b); }
     static __device__ __forceinline__ E sub(E a, E b) { return f2_sub(a, b); }
+    static __device__ __forceinline__ E fmak(float k, E a, E c) { return f2_fma(make_float2(k, k), a, c); }
+    static __device__ __forceinline__ E mulk(float k, E a) { return f2_mul(make_float2(k, k), a); }
+    static __device__ __forceinline__ void bfly(E &a, E &b, float c, float s) {
+        const E t = fmak(c, b, a);
+        const E p = mk(fmaf(-s, b.y, t.x), fmaf(s, b.x, t.y));
+        b = mk(fmaf(2.f, a.x, -p.x), fmaf(2.f, a.y, -p.y));
+        a = p;
+    }
 };
 template <> struct Arith<double> : ComplexArith<double> {};
 
@@ -318,75 +269,262 @@ template <> struct Arith<double> : ComplexArith<double> {};
 
 namespace pa {
 
-__host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
-__host__ __device__ constexpr int bitrev(int v, int bits) {
-    int r = 0;
-    for (int b = 0; b < bits; ++b) r |= ((v >> b) & 1) << (bits - 1 - b);
-    return r;
+// (a, b) -> (a + w b, a - w b) for w = w_32^J (forward root; the inverse uses the conjugate),
+// the whole and quarter turns without multiplications.
+template <typename T, int J, bool INV>
+__device__ __forceinline__ void bfly32(cx<T> &a, cx<T> &b) {
+    if constexpr (J == 0) {
+        const cx<T> p = Arith<T>::add(a, b);
+        b = Arith<T>::sub(a, b);
+        a = p;
+    } else if constexpr (J == 8) {  // w = -i (inverse: i)
+        const cx<T> r = INV ? Arith<T>::mk(-b.y, b.x) : Arith<T>::mk(b.y, -b.x);
+        b = Arith<T>::mk(a.x - r.x, a.y - r.y);
+        a = Arith<T>::mk(a.x + r.x, a.y + r.y);
+    } else {
+        Arith<T>::bfly(a, b, (T)cos32(J), INV ? (T)sin32(J) : (T)-sin32(J));
+    }
 }
 
-// In-register DFT of R = 2^s <= 32 values, natural order in and out:
-// radix-2 decimation in frequency followed by a register renaming.
+template <typename T, int R, bool INV, int LEVEL, int P>
+__device__ __forceinline__ void dft_const_sub(cx<T> *v) {
+    if constexpr (P < (1 << LEVEL)) {
+        constexpr int h = R >> (LEVEL + 1), base = bitrev(P, LEVEL) * (R >> LEVEL);
+#pragma unroll
+        for (int r = 0; r < h; ++r) bfly32<T, (P << (4 - LEVEL)), INV>(v[base + r], v[base + r + h]);
+        dft_const_sub<T, R, INV, LEVEL, P + 1>(v);
+    }
+}
+template <typename T, int R, bool INV, int LEVEL>
+__device__ __forceinline__ void dft_const(cx<T> *v) {
+    if constexpr ((1 << LEVEL) < R) {
+        dft_const_sub<T, R, INV, LEVEL, 0>(v);
+        dft_const<T, R, INV, LEVEL + 1>(v);
+    }
+}
+
+template <typename T, int R>
+__device__ __forceinline__ void bitrev_regs(cx<T> *v) {
+    cx<T> t[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) t[k] = v[bitrev(k, ilog2(R))];
+#pragma unroll
+    for (int k = 0; k < R; ++k) v[k] = t[k];
+}
+
+// In-register DFT of R = 2^s <= 32 values, natural order in and out. Complex: radix-2
+// decimation in time; level l combines the halves of the 2^l sub-transforms p (outputs
+// k = p mod 2^l) with the root w_{2^(l+1)}^p, which the butterfly's multiply-adds absorb.
+// Exact transform: decimation in frequency with the shift roots.
 template <typename T, int R, bool INV>
 __device__ __forceinline__ void dft(cx<T> *v) {
     static_assert(R >= 1 && R <= 32 && (R & (R - 1)) == 0, "radix must be a power of two <= 32");
     if constexpr (R > 1) {
+        if constexpr (std::is_same<T, Zp>::value) {
 #pragma unroll
-        for (int len = R; len >= 2; len >>= 1) {
+            for (int len = R; len >= 2; len >>= 1) {
 #pragma unroll
-            for (int b = 0; b < R; b += len) {
+                for (int b = 0; b < R; b += len) {
 #pragma unroll
-                for (int j = 0; j < len / 2; ++j) {
-                    cx<T> a = v[b + j], c = v[b + j + len / 2];
-                    v[b + j] = Arith<T>::add(a, c);
-                    v[b + j + len / 2] = Arith<T>::template rot32<INV>(Arith<T>::sub(a, c), j * (32 / len));
+                    for (int j = 0; j < len / 2; ++j) {
+                        cx<T> a = v[b + j], c = v[b + j + len / 2];
+                        v[b + j] = Arith<T>::add(a, c);
+                        v[b + j + len / 2] = Arith<T>::template rot32<INV>(Arith<T>::sub(a, c), j * (32 / len));
+                    }
                 }
             }
+        } else {
+            dft_const<T, R, INV, 0>(v);
         }
-        cx<T> t[R];
-#pragma unroll
-        for (int k = 0; k < R; ++k) t[k] = v[bitrev(k, ilog2(R))];
-#pragma unroll
-        for (int k = 0; k < R; ++k) v[k] = t[k];
+        bitrev_regs<T, R>(v);
     }
 }
 
-// v[r] *= w_L^{e0 + r*de} for r = 0..N-1: two table lookups, then a chain of
-// complex products (relative error grows by about one rounding per step).
-template <typename T, bool INV, int N>
-__device__ __forceinline__ void twiddle_chain(cx<T> *v, const TwTab<T> &tw, uint32_t e0, uint32_t de) {
-    const cx<T> g = Arith<T>::template omega<INV>(tw, de);
-    cx<T> w = (e0 == 0u) ? g : Arith<T>::template omega<INV>(tw, e0 + de);
-    if (e0 != 0u) v[0] = Arith<T>::mul(v[0], Arith<T>::template omega<INV>(tw, e0));
+// Two consecutive table entries (a row pair).
+__device__ __forceinline__ void load_pair(const float2 *p, float2 &a, float2 &b) {
+    const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+    a = make_float2(q.x, q.y);
+    b = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void load_pair(const double2 *p, double2 &a, double2 &b) {
+    a = __ldg(p);
+    b = __ldg(p + 1);
+}
+__device__ __forceinline__ void load_pair(const unsigned long long *p, unsigned long long &a, unsigned long long &b) {
+    const ulonglong2 q = __ldg(reinterpret_cast<const ulonglong2 *>(p));
+    a = q.x;
+    b = q.y;
+}
+// The ROWS multipliers of butterfly k of a stage of span P.
+template <typename T, int ROWS, int P>
+__device__ __forceinline__ void load_rows(const cx<T> *tab, uint32_t k, cx<T> *w) {
+    const cx<T> *t = tab + 2 * k;
 #pragma unroll
-    for (int r = 1; r < N; ++r) {
+    for (int r = 0; r < ROWS; r += 2) {
+        if (r + 1 < ROWS) {
+            load_pair(t + r * P, w[r], w[r + 1]);
+        } else {
+            w[r] = __ldg(t + r * P);
+        }
+    }
+}
+
+// DFT of v[r] * w^r, r < R, natural order in and out, with the multipliers of stage_list's
+// rows for this w: level l, sub-transform p needs (w w_R^p)^(R / 2^(l+1)), and the upper half
+// of the p are a quarter turn away from the lower half, so R/2 multipliers do. Every
+// butterfly absorbs its multiplier (bfly): a radix-16 stage takes 192 multiply-add slots,
+// where twiddling first (15 products, and 14 more to form the powers) took 284.
+template <typename T, int R, bool INV>
+__device__ __forceinline__ void dft_rows(cx<T> *v, const cx<T> *w) {
+    if constexpr (std::is_same<T, Zp>::value) {
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[r] = Arith<T>::mul(v[r], w[r - 1]);
+        dft<T, R, INV>(v);
+    } else {
+#pragma unroll
+        for (int l = 0; (1 << l) < R; ++l) {
+            const int h = R >> (l + 1);
+#pragma unroll
+            for (int p = 0; p < (1 << l); ++p) {
+                const int half = l ? (1 << (l - 1)) : 1;
+                const cx<T> m = w[l ? half + (p % half) : 0];
+                const bool turn = p >= half;  // a further factor -i (inverse: i)
+                const T c = turn ? m.y : m.x, s = turn ? -m.x : m.y;
+                const int base = bitrev(p, l) * (R >> l);
+#pragma unroll
+                for (int r = 0; r < h; ++r)
+                    Arith<T>::bfly(v[base + r], v[base + r + h], c, INV ? -s : s);
+            }
+        }
+        bitrev_regs<T, R>(v);
+    }
+}
+
+// (a, b) -> (a + w b, a - w b) for w = w_N^J (forward root; the inverse uses the conjugate).
+template <typename T, int N, int J, bool INV>
+__device__ __forceinline__ void bfly_const(cx<T> &a, cx<T> &b) {
+    constexpr int j = J % N;
+    if constexpr (j == 0) {
+        bfly32<T, 0, INV>(a, b);
+    } else if constexpr (4 * j == N) {
+        bfly32<T, 8, INV>(a, b);
+    } else {
+        constexpr T c = (T)cos_frac(j, N), s = (T)sin_frac(j, N);
+        Arith<T>::bfly(a, b, c, INV ? s : -s);
+    }
+}
+// DFT of u[n2] * w_{RO R0}^{K1 n2}, n2 < R0, output in bit-reversed slots: level l,
+// sub-transform p has the root w_RC^{K1 R0 / 2^(l+1)} w_{2^(l+1)}^p.
+template <typename T, int RO, int R0, int K1, bool INV, int LEVEL, int P>
+__device__ __forceinline__ void comp_sub(cx<T> *u) {
+    if constexpr ((1 << LEVEL) < R0) {
+        if constexpr (P < (1 << LEVEL)) {
+            constexpr int h = R0 >> (LEVEL + 1), base = bitrev(P, LEVEL) * (R0 >> LEVEL);
+#pragma unroll
+            for (int r = 0; r < h; ++r)
+                bfly_const<T, RO * R0, K1 * h + P * (RO * R0 >> (LEVEL + 1)), INV>(u[base + r], u[base + r + h]);
+            comp_sub<T, RO, R0, K1, INV, LEVEL, P + 1>(u);
+        } else {
+            comp_sub<T, RO, R0, K1, INV, LEVEL + 1, 0>(u);
+        }
+    }
+}
+// The radix-R0 step of column k1 = K1, ..., RO-1 of dft_comp.
+template <typename T, int RO, int R0, int K1, bool INV>
+__device__ __forceinline__ void comp_cols(const cx<T> *a, cx<T> *x) {
+    if constexpr (K1 < RO) {
+        cx<T> u[R0];
+#pragma unroll
+        for (int n2 = 0; n2 < R0; ++n2) u[n2] = a[n2 * RO + K1];
+        comp_sub<T, RO, R0, K1, INV, 0, 0>(u);
+#pragma unroll
+        for (int k2 = 0; k2 < R0; ++k2) x[K1 + RO * k2] = u[bitrev(k2, ilog2(R0))];
+        comp_cols<T, RO, R0, K1 + 1, INV>(a, x);
+    }
+}
+
+// In-register DFT of RC = RO * R0 values (RO in {3, 5, 9}, R0 a power of two),
+// natural order in and out, by one Cooley-Tukey step: with n = R0 n1 + n2 and
+// k = k1 + RO k2, X[k] = sum_n2 w_R0^{n2 k2} w_RC^{n2 k1} sum_n1 w_RO^{n1 k1} x[n].
+// The twiddle between the two steps goes into the butterflies of the second.
+template <typename T, int RO, int R0, bool INV>
+__device__ __forceinline__ void dft_comp(cx<T> *x) {
+    if constexpr (R0 == 1) {
+        dft_odd<T, RO, INV>(x);
+    } else {
+        cx<T> a[RO * R0];  // a[n2 * RO + k1]
+#pragma unroll
+        for (int n2 = 0; n2 < R0; ++n2) {
+            cx<T> u[RO];
+#pragma unroll
+            for (int n1 = 0; n1 < RO; ++n1) u[n1] = x[R0 * n1 + n2];
+            dft_odd<T, RO, INV>(u);
+#pragma unroll
+            for (int k1 = 0; k1 < RO; ++k1) a[n2 * RO + k1] = u[k1];
+        }
+        comp_cols<T, RO, R0, 0, INV>(a, x);
+    }
+}
+
+// dft_comp of x[n] * w^n (the inverse transform's last stage) with the multipliers of butterfly
+// k of the odd stage (odd_exponent): w^{R0 n1} before the odd step, then radix-R0 stages whose
+// multipliers carry w w_RC^{k1}.
+template <typename T, int RO, int R0, int P, bool INV>
+__device__ __forceinline__ void dft_comp_rows(cx<T> *x, const cx<T> *tab, uint32_t k) {
+    constexpr int ROWS = odd_rows(RO, R0);
+    cx<T> w[ROWS];
+    load_rows<T, ROWS, P>(tab, k, w);
+    if constexpr (INV) {
+#pragma unroll
+        for (int r = 0; r < RO - 1; ++r) w[r].y = -w[r].y;
+    }
+#pragma unroll
+    for (int n1 = 1; n1 < RO; ++n1) {
+#pragma unroll
+        for (int n2 = 0; n2 < R0; ++n2) x[R0 * n1 + n2] = Arith<T>::mul(x[R0 * n1 + n2], w[n1 - 1]);
+    }
+    if constexpr (R0 == 1) {
+        dft_odd<T, RO, INV>(x);
+    } else {
+        cx<T> a[RO * R0];
+#pragma unroll
+        for (int n2 = 0; n2 < R0; ++n2) {
+            cx<T> u[RO];
+#pragma unroll
+            for (int n1 = 0; n1 < RO; ++n1) u[n1] = x[R0 * n1 + n2];
+            dft_odd<T, RO, INV>(u);
+#pragma unroll
+            for (int k1 = 0; k1 < RO; ++k1) a[n2 * RO + k1] = u[k1];
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < RO; ++k1) {
+            cx<T> u[R0], m[R0 / 2];
+#pragma unroll
+            for (int n2 = 0; n2 < R0; ++n2) u[n2] = a[n2 * RO + k1];
+#pragma unroll
+            for (int r = 0; r < R0 / 2; ++r) m[r] = w[RO - 1 + r * RO + k1];
+            dft_rows<T, R0, INV>(u, m);
+#pragma unroll
+            for (int k2 = 0; k2 < R0; ++k2) x[k1 + RO * k2] = u[k2];
+        }
+    }
+}
+
+// The pass twiddles: v[s] *= w^{(tq + s*TC) u} for s = 0 .. N-1 and column u = blk*COLS + col
+// (nblk column blocks): one product for s = 0, then a chain of products with g = w^{TC u}.
+template <typename T, bool INV, int N, int COLS>
+__device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint32_t nblk, uint32_t tq, uint32_t blk,
+                                              uint32_t col) {
+    cx<T> w = Arith<T>::mul(__ldg(t.a + (uint64_t)tq * nblk + blk), __ldg(t.c + tq * COLS + col));
+    cx<T> g = __ldg(t.g + blk * COLS + col);
+    if constexpr (INV && !std::is_same<T, Zp>::value) {
+        w.y = -w.y;
+        g.y = -g.y;
+    }
+#pragma unroll
+    for (int r = 0; r < N; ++r) {
         v[r] = Arith<T>::mul(v[r], w);
         if (r + 1 < N) w = Arith<T>::mul(w, g);
-    }
-}
-
-// v[r] *= w_F^{r*step} for r = 1..N-1 (the stage twiddle w_{R p}^{r k} is
-// w_F^{r k F/(R p)}). CHAIN = true (used by every pass): one table load, then a
-// chain of products -- fewest loads and registers, measured faster than one
-// load per value in every pass but the last inverse one, where it is even.
-// CHAIN = false: one table load per value.
-template <typename T, bool INV, int N, bool CHAIN = true>
-__device__ __forceinline__ void stage_twiddles(cx<T> *v, const TwTab<T> &tw, uint32_t step) {
-    if constexpr (CHAIN) {
-        const cx<T> g = Arith<T>::template fine<INV>(tw, step);
-        cx<T> w = g;
-#pragma unroll
-        for (int r = 1; r < N; ++r) {
-            v[r] = Arith<T>::mul(v[r], w);
-            if (r + 1 < N) w = Arith<T>::mul(w, g);
-        }
-    } else {
-        uint32_t e = step;
-#pragma unroll
-        for (int r = 1; r < N; ++r) {
-            v[r] = Arith<T>::mul(v[r], Arith<T>::template fine<INV>(tw, e));
-            e += step;
-        }
     }
 }
 
@@ -400,37 +538,22 @@ __device__ __forceinline__ uint32_t sidx(uint32_t a, uint32_t col) {
 template <int LEN, int COLS>
 constexpr uint32_t smem_elems() { return (uint32_t)LEN * COLS + ((uint32_t)LEN * COLS >> 4) + 1; }
 
-// Stage plan of a Stockham FFT of length LEN with E values per thread:
-// q stages; the forward transform uses radices [R0, E, ..., E], the inverse
-// [E, ..., E, R0], so the forward's output distribution over threads equals
-// the inverse's input distribution and the two chain in registers.
-__host__ __device__ constexpr int odd_part(int v) { return (v & 1) ? v : odd_part(v >> 1); }
-constexpr int kMaxCompositeRadix = 24;
 __host__ __device__ constexpr int ipow(int b, int e) { return e == 0 ? 1 : b * ipow(b, e - 1); }
 
-// Stage plan of a Stockham FFT of length LEN = RO * 2^k2 (RO odd: 1, 3, 5 or 9)
-// with E values per thread (TC = LEN / E threads per column). Radices:
-//   forward  [RO], R0, E, ..., E        inverse  E, ..., E, R0, [RO]
-// so the forward's output distribution over threads equals the inverse's input
-// distribution (the two chain in registers). An odd stage exists only in
-// transforms that read their input from, and write their output to, memory
-// (the innermost pass), because its E / RO groups per thread do not divide.
+// The stage plan of tables.cuh at compile time.
 template <int LEN, int E> struct Plan {
-    static constexpr int RO = odd_part(LEN);
-    static constexpr int K2 = LEN / RO;
-    static constexpr int k = ilog2(K2), e = ilog2(E);
-    static constexpr int q = (k + e - 1) / e;  // power-of-two stages
-    static constexpr int r0 = 1 << (k - (q - 1) * e);
-    static constexpr int TC = LEN / E;  // threads per column
-    // The odd stage absorbs the radix-r0 stage when r0 < E and the composite radix
-    // RO * r0 stays within a register budget: stages [RO * r0], E, ..., E.
-    static constexpr bool FOLD = RO > 1 && r0 < E && RO * r0 <= kMaxCompositeRadix;
-    static constexpr int R0C = FOLD ? r0 : 1;  // power-of-two factor of the odd stage
-    static constexpr int RC = RO * R0C;        // radix of the odd stage
+    static constexpr StageShape sh = stage_shape(LEN, E);
+    static constexpr int RO = sh.RO, K2 = sh.K2, q = sh.q, r0 = sh.r0;
+    static constexpr int TC = sh.TC;  // threads per column
+    static constexpr bool FOLD = sh.fold;
+    static constexpr int R0C = sh.R0C;  // power-of-two factor of the odd stage
+    static constexpr int RC = sh.RC;    // radix of the odd stage
     static_assert(RO == 1 || RO == 3 || RO == 5 || RO == 9, "odd factor must be 1, 3, 5 or 9");
     static_assert(RO > 1 || q >= 2, "LEN must exceed E");
-    static_assert((1 << k) == K2 && (1 << e) == E && K2 >= E, "power-of-two part must be >= E");
+    static_assert(K2 >= E, "power-of-two part must be >= E");
 };
+template <typename T, int LEN, int E>
+constexpr StageList stages() { return stage_list(LEN, E, !std::is_same<T, Zp>::value); }
 
 // Index of the element that register slot s of thread tq holds at the start
 // (first-stage input) and at the end (last-stage output) of a transform.
@@ -511,21 +634,33 @@ constexpr int slot_period() {
     }
 }
 
+// Butterfly k of a radix-R stage of span P whose table rows start at OFF.
+template <typename T, int R, int P, int OFF, bool INV>
+__device__ __forceinline__ void stage_dft(cx<T> *v, const cx<T> *st, uint32_t k) {
+    if constexpr (P == 1) {
+        dft<T, R, INV>(v);
+    } else {
+        constexpr int ROWS = stage_rows(R, !std::is_same<T, Zp>::value);
+        cx<T> w[ROWS];
+        load_rows<T, ROWS, P>(st + OFF, k, w);
+        dft_rows<T, R, INV>(v, w);
+    }
+}
+
 // One Stockham stage of radix R at span P, from registers (already loaded
 // with this stage's inputs) to shared memory. Thread tq handles the E/R
 // butterfly groups i = tq + b*TC; group i reads elements i + r*LEN/R,
-// multiplies by w_{R P}^{r k} (k = i mod P; w_{R P}^{j} = w_F^{j F/(R P)}),
-// transforms, and writes element (i - k)*R + k + r*P.
-template <typename T, int LEN, int COLS, int E, int R, int P, bool INV>
-__device__ __forceinline__ void stage_to_smem(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw) {
+// multiplies by w_{R P}^{r k} (k = i mod P), transforms, and writes element
+// (i - k)*R + k + r*P.
+template <typename T, int LEN, int COLS, int E, int R, int P, int OFF, bool INV>
+__device__ __forceinline__ void stage_to_smem(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     constexpr int TC = LEN / E;
     constexpr int Q = slot_period<T, LEN, COLS, E, P * R>();
 #pragma unroll
     for (int b = 0; b < E / R; ++b) {
         const uint32_t i = tq + (uint32_t)b * TC;
         const uint32_t k = i % P;
-        if (P > 1) stage_twiddles<T, INV, R>(v + b * R, tw, k * (tw.F / (R * P)));
-        dft<T, R, INV>(v + b * R);
+        stage_dft<T, R, P, OFF, INV>(v + b * R, st, k);
         const uint32_t base = (i - k) * R + k;
         if constexpr (P % Q == 0 || (P == 1 && R % Q == 0)) {
             // offsets r*P are multiples of Q, or (P = 1, so k = 0) base = i*R is one
@@ -560,15 +695,14 @@ __device__ __forceinline__ void load_from_smem(const cx<T> *sm, cx<T> *v, uint32
 }
 
 // Last stage: twiddle + DFT in registers, results stay in registers.
-template <typename T, int LEN, int COLS, int E, int R, int P, bool INV>
-__device__ __forceinline__ void stage_in_regs(cx<T> *v, uint32_t tq, const TwTab<T> &tw) {
+template <typename T, int LEN, int COLS, int E, int R, int P, int OFF, bool INV>
+__device__ __forceinline__ void stage_in_regs(cx<T> *v, uint32_t tq, const cx<T> *st) {
     constexpr int TC = LEN / E;
 #pragma unroll
     for (int b = 0; b < E / R; ++b) {
         const uint32_t i = tq + (uint32_t)b * TC;
         const uint32_t k = i % P;
-        if (P > 1) stage_twiddles<T, INV, R>(v + b * R, tw, k * (tw.F / (R * P)));
-        dft<T, R, INV>(v + b * R);
+        stage_dft<T, R, P, OFF, INV>(v + b * R, st, k);
     }
 }
 
@@ -576,19 +710,21 @@ __device__ __forceinline__ void stage_in_regs(cx<T> *v, uint32_t tq, const TwTab
 // E), starting at span P0. Stage S's inputs are in registers when FROM_REGS,
 // else in shared memory. The last stage leaves its outputs in registers.
 template <typename T, int LEN, int COLS, int E, int S, int P0, bool FROM_REGS>
-__device__ __forceinline__ void fwd_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw) {
+__device__ __forceinline__ void fwd_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     using PL = Plan<LEN, E>;
-    constexpr int R = (S == 0) ? PL::r0 : E;
+    constexpr StageRow row = stages<T, LEN, E>().fwd[S];
+    constexpr int R = row.R;
+    static_assert(row.P == P0, "stage list and stage order agree");
     if constexpr (!FROM_REGS) {
         __syncthreads();
         load_from_smem<T, LEN, COLS, E, R, P0>(sm, v, tq, col);
     }
     if constexpr (S == PL::q - 1) {
-        stage_in_regs<T, LEN, COLS, E, R, P0, false>(v, tq, tw);
+        stage_in_regs<T, LEN, COLS, E, R, P0, row.off, false>(v, tq, st);
     } else {
         if constexpr (!FROM_REGS) __syncthreads();
-        stage_to_smem<T, LEN, COLS, E, R, P0, false>(sm, v, tq, col, tw);
-        fwd_pow2<T, LEN, COLS, E, S + 1, P0 * R, false>(sm, v, tq, col, tw);
+        stage_to_smem<T, LEN, COLS, E, R, P0, row.off, false>(sm, v, tq, col, st);
+        fwd_pow2<T, LEN, COLS, E, S + 1, P0 * R, false>(sm, v, tq, col, st);
     }
 }
 
@@ -599,19 +735,20 @@ __device__ __forceinline__ void fwd_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint3
 // LAST is the index of the last power-of-two stage to run (q - 1, or q - 2 when
 // the odd stage absorbs the radix-r0 stage).
 template <typename T, int LEN, int COLS, int E, int S, int P0, bool TO_SMEM, int LAST = Plan<LEN, E>::q - 1>
-__device__ __forceinline__ void inv_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw) {
-    using PL = Plan<LEN, E>;
-    constexpr int R = (S == PL::q - 1) ? PL::r0 : E;
+__device__ __forceinline__ void inv_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
+    constexpr StageRow row = stages<T, LEN, E>().inv[S];
+    constexpr int R = row.R;
+    static_assert(row.P == P0, "stage list and stage order agree");
     if constexpr (S > 0) {
         __syncthreads();
         load_from_smem<T, LEN, COLS, E, R, P0>(sm, v, tq, col);
     }
     if constexpr (S == LAST && !TO_SMEM) {
-        stage_in_regs<T, LEN, COLS, E, R, P0, true>(v, tq, tw);
+        stage_in_regs<T, LEN, COLS, E, R, P0, row.off, true>(v, tq, st);
     } else {
         if constexpr (S > 0) __syncthreads();
-        stage_to_smem<T, LEN, COLS, E, R, P0, true>(sm, v, tq, col, tw);
-        if constexpr (S < LAST) inv_pow2<T, LEN, COLS, E, S + 1, P0 * R, TO_SMEM, LAST>(sm, v, tq, col, tw);
+        stage_to_smem<T, LEN, COLS, E, R, P0, row.off, true>(sm, v, tq, col, st);
+        if constexpr (S < LAST) inv_pow2<T, LEN, COLS, E, S + 1, P0 * R, TO_SMEM, LAST>(sm, v, tq, col, st);
     }
 }
 
@@ -621,12 +758,12 @@ __device__ __forceinline__ void inv_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint3
 // idx_r0 layout). The caller must __syncthreads() before the call if shared
 // memory is still being read from a previous transform.
 template <typename T, int LEN, int COLS, int E, bool INV>
-__device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw) {
+__device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     static_assert(Plan<LEN, E>::RO == 1, "odd lengths use cta_fft_fwd_odd / cta_fft_inv_odd");
     if constexpr (!INV) {
-        fwd_pow2<T, LEN, COLS, E, 0, 1, true>(sm, v, tq, col, tw);
+        fwd_pow2<T, LEN, COLS, E, 0, 1, true>(sm, v, tq, col, st);
     } else {
-        inv_pow2<T, LEN, COLS, E, 0, 1, false>(sm, v, tq, col, tw);
+        inv_pow2<T, LEN, COLS, E, 0, 1, false>(sm, v, tq, col, st);
     }
 }
 
@@ -657,28 +794,28 @@ __device__ __forceinline__ void odd_first_stage(cx<T> *sm, uint32_t tq, Ld ld) {
 }
 
 template <typename T, int LEN, int E>
-__device__ __forceinline__ void fwd_odd_rest(cx<T> *sm, cx<T> *v, uint32_t tq, const TwTab<T> &tw) {
+__device__ __forceinline__ void fwd_odd_rest(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st) {
     using PL = Plan<LEN, E>;
-    fwd_pow2<T, LEN, 1, E, PL::FOLD ? 1 : 0, PL::RC, false>(sm, v, tq, 0, tw);
+    fwd_pow2<T, LEN, 1, E, PL::FOLD ? 1 : 0, PL::RC, false>(sm, v, tq, 0, st);
 }
 
 template <typename T, int LEN, int E, class Ld>
-__device__ __forceinline__ void cta_fft_fwd_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const TwTab<T> &tw, Ld ld) {
+__device__ __forceinline__ void cta_fft_fwd_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st, Ld ld) {
     odd_first_stage<T, LEN, E>(sm, tq, ld);
-    fwd_odd_rest<T, LEN, E>(sm, v, tq, tw);
+    fwd_odd_rest<T, LEN, E>(sm, v, tq, st);
 }
 
 // Inverse transform of a row (RO > 1): power-of-two stages from registers
 // (idx_e layout) into shared memory, then the odd (or composite) last stage at
 // span K = LEN / RC: group g = tq + j TC < K reads slots g + r K, takes the twiddles
-// w_LEN^{-r g}, transforms, and its output g + r K goes through st(j TC + r K, value)
+// w_LEN^{-r g}, transforms, and its output g + r K goes through put(j TC + r K, value)
 // (offset from element tq, as for ld above).
 template <typename T, int LEN, int E, class St>
-__device__ __forceinline__ void cta_fft_inv_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const TwTab<T> &tw, St st) {
+__device__ __forceinline__ void cta_fft_inv_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st, St put) {
     using PL = Plan<LEN, E>;
     constexpr int RC = PL::RC, K = LEN / RC, TC = PL::TC;
     constexpr int G = (K + TC - 1) / TC;
-    inv_pow2<T, LEN, 1, E, 0, 1, true, PL::FOLD ? PL::q - 2 : PL::q - 1>(sm, v, tq, 0, tw);
+    inv_pow2<T, LEN, 1, E, 0, 1, true, PL::FOLD ? PL::q - 2 : PL::q - 1>(sm, v, tq, 0, st);
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < G; ++j) {
@@ -693,10 +830,9 @@ __device__ __forceinline__ void cta_fft_inv_odd(cx<T> *sm, cx<T> *v, uint32_t tq
 #pragma unroll
                 for (int r = 0; r < RC; ++r) u[r] = sm[ridx<T, LEN, E, K>(g + (uint32_t)r * K)];
             }
-            stage_twiddles<T, true, RC>(u, tw, g * (tw.F / LEN));
-            dft_comp<T, PL::RO, PL::R0C, true>(u);
+            dft_comp_rows<T, PL::RO, PL::R0C, K, true>(u, st + stages<T, LEN, E>().odd.off, g);
 #pragma unroll
-            for (int r = 0; r < RC; ++r) st((uint32_t)(j * TC + r * K), u[r]);
+            for (int r = 0; r < RC; ++r) put((uint32_t)(j * TC + r * K), u[r]);
         }
     }
 }

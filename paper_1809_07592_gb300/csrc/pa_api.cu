@@ -64,8 +64,7 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 // per-bin seed tables, so a lone key costs half the transform work of a key pair.
 struct RealMode {
     Geometry geo;  // the length-N transform, N = geo.L
-    void *tw_hi = nullptr, *tw_lo = nullptr, *tw_fine = nullptr;
-    uint32_t twB = 0;
+    TwSet tw;      // its twiddle tables
     void *tabs = nullptr;  // 3N values: E_s, O_s, w_N^k O_s (times 1/N), digit-reversed bin order
     bool seeded = false;
 };
@@ -92,9 +91,7 @@ struct pa_plan {
     int device = 0;
     uint64_t L = 0;
     Geometry geo;  // pass split of L
-    uint32_t twB = 0;
-    void *tw_hi = nullptr, *tw_lo = nullptr;
-    void *tw_fine = nullptr;  // stage twiddles w_F^j, F = geo.F()
+    TwSet tw;      // its twiddle tables
     void *spec = nullptr;        // L complex values, seed spectrum in digit-reversed order, times 1/L
     void *work = nullptr;        // work_pairs * L complex values
     uint32_t work_pairs = 0;
@@ -177,134 +174,21 @@ size_t elem_bytes(pa_dtype_t d) {
     return d == PA_FP32_GUARD ? sizeof(float2) : d == PA_FP64 ? sizeof(double2) : sizeof(uint64_t);
 }
 
-// ---- modular helpers (host) for the NTT mode -------------------------------------------------
-uint64_t zp_mul_host(uint64_t a, uint64_t b) {
-    unsigned __int128 x = (unsigned __int128)a * b;
-    return zp_reduce((uint64_t)(x >> 64), (uint64_t)x);
-}
-uint64_t zp_pow_host(uint64_t a, uint64_t e) {
-    uint64_t r = 1;
-    while (e) {
-        if (e & 1) r = zp_mul_host(r, a);
-        a = zp_mul_host(a, a);
-        e >>= 1;
-    }
-    return r;
-}
-// Root of unity of order L (a power of two, 32 <= L <= 2^32) whose L/32-th power
-// is 2^6, the root the in-register DFTs use.
-uint64_t zp_root(uint64_t L) {
-    const uint64_t g = 7;  // generates the multiplicative group mod p
-    const uint64_t w = zp_pow_host(g, (kP - 1) / L);
-    const uint64_t w32 = zp_pow_host(w, L / 32);
-    for (uint64_t j = 1; j < 64; j += 2) {
-        if (zp_pow_host(w32, j) == 64ull) return zp_pow_host(w, j);
-    }
-    return 0;
-}
-
-template <typename T>
-int make_twiddles(uint64_t Lu, uint32_t F, void **dhi, void **dlo, uint32_t *Bout, void **dfine) {
-    int lgL = 0;
-    while ((1ull << lgL) < Lu) ++lgL;
-    const uint32_t B = (uint32_t)(lgL + 1) / 2;
-    const uint64_t nlo = 1ull << B, nhi = (Lu + nlo - 1) >> B;
-    std::vector<cx<T>> hi(nhi), lo(nlo), fine(F);
-    const double L = (double)Lu;
-    const double two_pi = 6.283185307179586476925286766559;
-    for (uint64_t h = 0; h < nhi; ++h) {
-        const double a = two_pi * (double)(h << B) / L;
-        hi[h].x = (T)std::cos(a);
-        hi[h].y = (T)-std::sin(a);
-    }
-    for (uint64_t l = 0; l < nlo; ++l) {
-        const double a = two_pi * (double)l / L;
-        lo[l].x = (T)std::cos(a);
-        lo[l].y = (T)-std::sin(a);
-    }
-    for (uint64_t j = 0; j < F; ++j) {
-        const double a = two_pi * (double)j / (double)F;
-        fine[j].x = (T)std::cos(a);
-        fine[j].y = (T)-std::sin(a);
-    }
-    PA_CUDA(cudaMalloc(dhi, nhi * sizeof(cx<T>)));
-    PA_CUDA(cudaMalloc(dlo, nlo * sizeof(cx<T>)));
-    PA_CUDA(cudaMalloc(dfine, (size_t)F * sizeof(cx<T>)));
-    PA_CUDA(cudaMemcpy(*dhi, hi.data(), nhi * sizeof(cx<T>), cudaMemcpyHostToDevice));
-    PA_CUDA(cudaMemcpy(*dlo, lo.data(), nlo * sizeof(cx<T>), cudaMemcpyHostToDevice));
-    PA_CUDA(cudaMemcpy(*dfine, fine.data(), (size_t)F * sizeof(cx<T>), cudaMemcpyHostToDevice));
-    *Bout = B;
-    return PA_OK;
-}
-
-template <>
-int make_twiddles<Zp>(uint64_t Lu, uint32_t F, void **dhi, void **dlo, uint32_t *Bout, void **dfine) {
-    if (Lu & (Lu - 1)) return PA_EUNSUPPORTED;  // the exact transform keeps power-of-two lengths
-    int lgL = 0;
-    while ((1ull << lgL) < Lu) ++lgL;
-    const uint32_t B = (uint32_t)(lgL + 1) / 2;
-    const uint64_t nhi = 1ull << (lgL - B), nlo = 1ull << B;
-    std::vector<uint64_t> hi(nhi), lo(nlo), fine(F);
-    const uint64_t w = zp_root(Lu);
-    if (w == 0 || Lu % F) return PA_EUNSUPPORTED;
-    const uint64_t wB = zp_pow_host(w, 1ull << B);
-    uint64_t x = 1;
-    for (uint64_t h = 0; h < nhi; ++h) { hi[h] = x; x = zp_mul_host(x, wB); }
-    x = 1;
-    for (uint64_t l = 0; l < nlo; ++l) { lo[l] = x; x = zp_mul_host(x, w); }
-    const uint64_t wF = zp_pow_host(w, Lu / F);  // w_F = w_L^(L/F): the same root system
-    x = 1;
-    for (uint64_t j = 0; j < F; ++j) { fine[j] = x; x = zp_mul_host(x, wF); }
-    PA_CUDA(cudaMalloc(dhi, nhi * sizeof(uint64_t)));
-    PA_CUDA(cudaMalloc(dlo, nlo * sizeof(uint64_t)));
-    PA_CUDA(cudaMalloc(dfine, (size_t)F * sizeof(uint64_t)));
-    PA_CUDA(cudaMemcpy(*dhi, hi.data(), nhi * sizeof(uint64_t), cudaMemcpyHostToDevice));
-    PA_CUDA(cudaMemcpy(*dlo, lo.data(), nlo * sizeof(uint64_t), cudaMemcpyHostToDevice));
-    PA_CUDA(cudaMemcpy(*dfine, fine.data(), (size_t)F * sizeof(uint64_t), cudaMemcpyHostToDevice));
-    *Bout = B;
-    return PA_OK;
-}
-
-template <typename T>
-int build_twiddles(pa_plan_t *p) {
-    return make_twiddles<T>(p->L, p->geo.F(), &p->tw_hi, &p->tw_lo, &p->twB, &p->tw_fine);
-}
-
-// 1/L as the element type's scaling factor.
-template <typename T> cx<T> inv_length(uint64_t L) {
+// 1/L (and the reciprocal of the keys' scale) as the element type's scaling factor.
+template <typename T> cx<T> spec_scale(uint64_t L) {
     cx<T> s;
-    s.x = (decltype(s.x))(1.0 / (double)L);
+    s.x = (decltype(s.x))(kSpecScale / (double)L);
     s.y = 0;
     return s;
 }
-template <> cx<Zp> inv_length<Zp>(uint64_t L) { return zp_pow_host(L, kP - 2); }
-template <typename T> cx<T> one() { return inv_length<T>(1); }
-
-template <typename T>
-TwTab<T> tw_of(const pa_plan_t *p) {
-    TwTab<T> t;
-    t.hi = static_cast<const cx<T> *>(p->tw_hi);
-    t.lo = static_cast<const cx<T> *>(p->tw_lo);
-    t.B = p->twB;
-    t.lgL = 0;
-    while ((1ull << t.lgL) < p->L) ++t.lgL;  // log2 L for the power-of-two lengths of the exact transform
-    t.fine = static_cast<const cx<T> *>(p->tw_fine);
-    t.F = p->geo.F();
-    return t;
+template <> cx<Zp> spec_scale<Zp>(uint64_t L) { return zp_pow_host(L, kP - 2); }
+template <typename T> cx<T> one() {
+    cx<T> s;
+    s.x = 1;
+    s.y = 0;
+    return s;
 }
-
-template <typename T>
-TwTab<T> tw_of_real(const RealMode *r) {
-    TwTab<T> t;
-    t.hi = static_cast<const cx<T> *>(r->tw_hi);
-    t.lo = static_cast<const cx<T> *>(r->tw_lo);
-    t.B = r->twB;
-    t.lgL = 0;
-    while ((1ull << t.lgL) < r->geo.L) ++t.lgL;
-    t.fine = static_cast<const cx<T> *>(r->tw_fine);
-    t.F = r->geo.F();
-    return t;
-}
+template <> cx<Zp> one<Zp>() { return 1; }
 
 int ensure_work(pa_plan_t *p, uint32_t pairs) {
     if (pairs <= p->work_pairs) return PA_OK;
@@ -375,7 +259,7 @@ cudaError_t round_stored(const pa_plan_t *p, cx<T> *slots, uint32_t pairs, cudaS
 
 template <typename T>
 int run_seed(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
-    const TwTab<T> tw = tw_of<T>(p);
+    const TwTab<T> tw = tw_tab<T>(p->tw.lay, p->tw.mem);
     cx<T> *W = static_cast<cx<T> *>(p->work);
     cx<T> *spec = static_cast<cx<T> *>(p->spec);
     const Geometry &g = p->geo;
@@ -384,7 +268,7 @@ int run_seed(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
         Timed t_(p, K_MID_FWD, st);
         PA_CUDA(launch_mid<T>(g.lgM, false, W, p->L, g.inner(), 1, tw, st));
     }
-    { Timed t_(p, K_MIDDLE_SPEC, st); PA_CUDA(launch_middle<T>(g.ro, g.lgI, 1, W, spec, p->L, 1, tw, inv_length<T>(p->L), st)); }
+    { Timed t_(p, K_MIDDLE_SPEC, st); PA_CUDA(launch_middle<T>(g.ro, g.lgI, 1, W, spec, p->L, 1, tw, spec_scale<T>(p->L), st)); }
     PA_CUDA(round_stored<T>(p, spec, 1, st));
     return PA_OK;
 }
@@ -393,14 +277,14 @@ int run_seed(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
 template <typename T>
 int run_seed_real(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
     RealMode *r = p->real;
-    const TwTab<T> tw = tw_of_real<T>(r);
+    const TwTab<T> tw = tw_tab<T>(r->tw.lay, r->tw.mem);
     cx<T> *W = static_cast<cx<T> *>(p->work);
     const Geometry &g = r->geo;
     const uint64_t N = g.L;
     PA_CUDA(launch_fwd_seed<T>(g.lg1, seed, p->n, p->m, W, N, tw, st, true));
     if (g.lgM) PA_CUDA(launch_mid<T>(g.lgM, false, W, N, g.inner(), 1, tw, st));
     PA_CUDA(launch_middle_real<T>(g.ro, g.lgI, 1, W, static_cast<cx<T> *>(r->tabs), N, (uint32_t)g.lg1,
-                                  (uint32_t)g.lgM, tw, (T)(1.0 / (double)N), 1, st));
+                                  (uint32_t)g.lgM, tw, (T)(kSpecScale / (double)N), 1, st));
     return PA_OK;
 }
 
@@ -410,7 +294,7 @@ template <typename T>
 int run_keys_real(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstride, uint64_t *out,
                   uint64_t ostride, uint32_t *popc, uint32_t *marg, cudaStream_t st) {
     RealMode *r = p->real;
-    const TwTab<T> tw = tw_of_real<T>(r);
+    const TwTab<T> tw = tw_tab<T>(r->tw.lay, r->tw.mem);
     cx<T> *W = static_cast<cx<T> *>(p->work);
     cx<T> *tabs = static_cast<cx<T> *>(r->tabs);
     const Geometry &g = r->geo;
@@ -457,7 +341,7 @@ int run_keys(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstrid
                                     ostride, popc + k, marg + k, st);
         }
     }
-    const TwTab<T> tw = tw_of<T>(p);
+    const TwTab<T> tw = tw_tab<T>(p->tw.lay, p->tw.mem);
     cx<T> *W = static_cast<cx<T> *>(p->work);
     cx<T> *spec = static_cast<cx<T> *>(p->spec);
     const Geometry &g = p->geo;
@@ -489,9 +373,7 @@ int run_keys(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstrid
 
 void free_real_mode(pa_plan_t *p) {
     if (!p->real) return;
-    cudaFree(p->real->tw_hi);
-    cudaFree(p->real->tw_lo);
-    cudaFree(p->real->tw_fine);
+    pa_internal_free_twiddles(&p->real->tw);
     cudaFree(p->real->tabs);
     delete p->real;
     p->real = nullptr;
@@ -500,9 +382,7 @@ void free_real_mode(pa_plan_t *p) {
 void free_plan(pa_plan_t *p) {
     if (!p) return;
     if (p->fallback) free_plan(p->fallback);
-    cudaFree(p->tw_hi);
-    cudaFree(p->tw_lo);
-    cudaFree(p->tw_fine);
+    pa_internal_free_twiddles(&p->tw);
     cudaFree(p->spec);
     cudaFree(p->work);
     cudaFree(p->popc);
@@ -540,19 +420,6 @@ void split_lengths(const Geometry &g, uint32_t *L1, uint32_t *L2, uint32_t *L3) 
     *L1 = 1u << g.lg1;
     *L2 = g.lgM ? (1u << g.lgM) : g.inner();
     *L3 = g.lgM ? g.inner() : 1u;
-}
-
-int build_plan_twiddles(pa_plan_t *p) {
-    return (p->dtype == PA_FP32_GUARD) ? build_twiddles<float>(p)
-           : (p->dtype == PA_FP64)     ? build_twiddles<double>(p)
-                                       : build_twiddles<Zp>(p);
-}
-
-void free_plan_twiddles(pa_plan_t *p) {
-    cudaFree(p->tw_hi);
-    cudaFree(p->tw_lo);
-    cudaFree(p->tw_fine);
-    p->tw_hi = p->tw_lo = p->tw_fine = nullptr;
 }
 
 // ---- split autotuner ---------------------------------------------------------------------------
@@ -635,12 +502,12 @@ int tune_split(pa_plan_t *p, const std::vector<Geometry> &cand) {
     if ((rc = ensure_work(p, pairs)) != PA_OK || (rc = ensure_keys(p, nkeys)) != PA_OK) return fail(rc);
     for (size_t i = 0; i < cand.size(); ++i) {
         p->geo = cand[i];
-        if ((rc = build_plan_twiddles(p)) != PA_OK) return fail(rc);
+        if ((rc = pa_internal_twiddles(p->geo, p->dtype, &p->tw)) != PA_OK) return fail(rc);
         float ms = 0.f;
         rc = (p->dtype == PA_FP32_GUARD) ? time_split<float>(p, nkeys, keys, kw, out, ow, st, a, b, &ms)
              : (p->dtype == PA_FP64)     ? time_split<double>(p, nkeys, keys, kw, out, ow, st, a, b, &ms)
                                          : time_split<Zp>(p, nkeys, keys, kw, out, ow, st, a, b, &ms);
-        free_plan_twiddles(p);
+        pa_internal_free_twiddles(&p->tw);
         if (rc != PA_OK) return fail(rc);
         if (i == 0 || ms < best) {
             best = ms;
@@ -725,15 +592,12 @@ int tune_real(pa_plan_t *p, RealMode *r) {
     Geometry bestg = r->geo;
     for (size_t i = 0; i < cand.size(); ++i) {
         r->geo = cand[i];
-        rc = pa_internal_twiddles(r->geo.L, r->geo.F(), (int)p->dtype, &r->tw_hi, &r->tw_lo, &r->twB, &r->tw_fine);
+        rc = pa_internal_twiddles(r->geo, p->dtype, &r->tw);
         float ms = 0.f;
         if (rc == PA_OK)
             rc = (p->dtype == PA_FP32_GUARD) ? time_real<float>(p, key, kw, out, ow, st, a, b, &ms)
                                              : time_real<double>(p, key, kw, out, ow, st, a, b, &ms);
-        cudaFree(r->tw_hi);
-        cudaFree(r->tw_lo);
-        cudaFree(r->tw_fine);
-        r->tw_hi = r->tw_lo = r->tw_fine = nullptr;
+        pa_internal_free_twiddles(&r->tw);
         if (rc != PA_OK) return done(rc);
         if (i == 0 || ms < best) {
             best = ms;
@@ -763,7 +627,7 @@ int build_real_mode(pa_plan_t *p) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(real tables)");
     int rc = tune_real(p, r);
     if (rc != PA_OK) return rc;
-    return pa_internal_twiddles(r->geo.L, r->geo.F(), (int)p->dtype, &r->tw_hi, &r->tw_lo, &r->twB, &r->tw_fine);
+    return pa_internal_twiddles(r->geo, p->dtype, &r->tw);
 }
 
 // pa_plan (or pa_plan_modified), with the split forced when `force` is given. For the
@@ -809,7 +673,7 @@ int plan_create(uint64_t n, uint64_t m, pa_dtype_t dtype, const Geometry *force,
         const std::vector<Geometry> cand = geometry_candidates(p->L, dtype, false);
         if (cand.size() > 1) rc = tune_split(p, cand);
     }
-    if (rc == PA_OK) rc = build_plan_twiddles(p);
+    if (rc == PA_OK) rc = pa_internal_twiddles(p->geo, p->dtype, &p->tw);
     if (rc == PA_OK && dtype != PA_NTT64 && build_real_mode(p) != PA_OK) {
         // The half-length form is an optimisation: without memory for its tables a lone
         // key takes the pair form instead.
@@ -910,12 +774,6 @@ int ensure_staging(pa_plan_t *p, size_t key_words, size_t out_words) {
 }
 
 }  // namespace
-
-int pa_internal_twiddles(uint64_t L, uint32_t F, int dtype, void **hi, void **lo, uint32_t *B, void **fine) {
-    return dtype == PA_FP32_GUARD ? make_twiddles<float>(L, F, hi, lo, B, fine)
-           : dtype == PA_FP64     ? make_twiddles<double>(L, F, hi, lo, B, fine)
-                                  : make_twiddles<Zp>(L, F, hi, lo, B, fine);
-}
 
 extern "C" {
 

@@ -23,9 +23,7 @@ struct ClassRun {
     void *Wf = nullptr;    // complex: nb slots of L values; NTT: one slot
     void *Wi = nullptr;    // complex: ceil(nb/2) slots
     void *spec = nullptr;  // NTT: one seed-spectrum slot
-    const void *tw_hi = nullptr, *tw_lo = nullptr;
-    uint32_t B = 0;
-    const void *tw_fine = nullptr;  // stage twiddles, length geo.F()
+    TwSet tw;              // twiddle tables of geo (not owned)
 };
 
 // Transform length of a block of an uneven batch / the serving loop.

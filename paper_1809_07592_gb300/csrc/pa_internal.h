@@ -6,12 +6,10 @@
 
 #include <cuda_runtime.h>
 
+#include "tables.cuh"
+
 // Records "what: cuda error string" as the calling thread's last CUDA error and returns PA_ECUDA.
 int pa_internal_cuda_fail(cudaError_t e, const char *what);
-
-// Device twiddle tables of the length-L transform for a pa_dtype_t (cudaMalloc'd; caller frees):
-// the two-level table hi/lo split at B, and the stage table fine of length F (F divides L).
-int pa_internal_twiddles(uint64_t L, uint32_t F, int dtype, void **hi, void **lo, uint32_t *B, void **fine);
 
 #include "pa.h"
 
@@ -42,4 +40,21 @@ Geometry default_geometry(uint64_t L, pa_dtype_t dtype, bool split);
 // (ro = 1 only for the exact transform), together with its default split.
 Geometry choose_geometry(uint64_t need, pa_dtype_t dtype, bool split);
 
+// Twiddle tables of a transform: where they sit in one block of memory, and filling that
+// block on `st` (cudaErrorInvalidValue if the arithmetic has no root of order L).
+TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype);
+cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t st);
+
+// The tables of one transform in device memory of their own.
+struct TwSet {
+    TwLayout lay;
+    void *mem = nullptr;
+};
+
+uint64_t zp_pow_host(uint64_t a, uint64_t e);  // a^e mod p (the exact transform's prime)
+
 }  // namespace pa
+
+// Allocate and fill the tables (waits for the fill) / release them.
+int pa_internal_twiddles(const pa::Geometry &g, pa_dtype_t dtype, pa::TwSet *out);
+void pa_internal_free_twiddles(pa::TwSet *t);

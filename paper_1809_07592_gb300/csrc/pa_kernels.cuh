@@ -58,13 +58,19 @@ __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes =
 // 1.5 * 2^(mantissa bits): exact for |x| < 2^22 (float) / 2^51 (double); the
 // integer's parity is the lowest bit of the sum's encoding.
 template <typename T> struct Magic;
-template <> struct Magic<float> { static constexpr float v = 12582912.0f, limit = 2097152.0f; };
-template <> struct Magic<double> { static constexpr double v = 6755399441055744.0, limit = 1125899906842624.0; };
+template <> struct Magic<float> {
+    static constexpr float v = 12582912.0f, limit = 2097152.0f;
+    static __device__ __forceinline__ float from_high(uint32_t hi) { return __uint_as_float(hi); }
+};
+template <> struct Magic<double> {
+    static constexpr double v = 6755399441055744.0, limit = 1125899906842624.0;
+    static __device__ __forceinline__ double from_high(uint32_t hi) { return __hiloint2double((int)hi, 0); }
+};
 __device__ __forceinline__ uint32_t low_bit(float x) { return __float_as_uint(x) & 1u; }
 __device__ __forceinline__ uint32_t low_bit(double x) { return (uint32_t)__double_as_longlong(x) & 1u; }
 
 // Encoding of inputs and decoding of outputs per arithmetic.
-// Complex: key bits 0/1 in the real (key 2p) and imaginary (key 2p+1) parts,
+// Complex: key bits in the real (key 2p) and imaginary (key 2p+1) parts,
 // seed as +-1; the decoded value is w = ((P mod 4) - r)/2 (see above).
 // Zp: key 2p + 2^32 * key 2p+1 packed in one residue, seed as 0/1; the
 // convolution counts c_a, c_b < 2^32 come out exactly as the low and high
@@ -72,8 +78,21 @@ __device__ __forceinline__ uint32_t low_bit(double x) { return (uint32_t)__doubl
 template <typename T> struct Enc {
     using E = cx<T>;
     using M = T;  // margin accumulator
-    static __device__ __forceinline__ E key_pair(uint32_t ba, uint32_t bb) {
-        return Arith<T>::mk(ba ? (T)1 : (T)0, bb ? (T)1 : (T)0);
+    // Bit 30 alone is the encoding of 2.0f (and of the high
+    // word of 2.0), so a shift and a mask make the value 0 or 2. The spectra carry the factor's
+    // reciprocal (kSpecScale; with key and seed in one transform, its square): a power of
+    // two, so no rounding changes.
+    static __device__ __forceinline__ T two_if(uint32_t x, int bit) {
+        return Magic<T>::from_high((bit <= 30 ? x << (30 - bit) : x >> 1) & 0x40000000u);
+    }
+    // bit j of x: key a, bit 16 + j: key b
+    static __device__ __forceinline__ E key_pair(uint32_t x, int j) {
+        return Arith<T>::mk(two_if(x, j), two_if(x, 16 + j));
+    }
+    // bit j of x: key, bit 16 + j: seed; bit j of in: the seed position is inside the seed
+    static __device__ __forceinline__ E key_seed(uint32_t x, uint32_t in, int j) {
+        const uint32_t sign = (x << (15 - j)) & 0x80000000u;
+        return Arith<T>::mk(two_if(x, j), Magic<T>::from_high(((in << (30 - j)) & 0x40000000u) | sign));
     }
     static __device__ __forceinline__ E seed(bool in_range, uint32_t bit) {
         return Arith<T>::mk(in_range ? (bit ? (T)-1 : (T)1) : (T)0, (T)0);
@@ -100,7 +119,9 @@ template <typename T> struct Enc {
 template <> struct Enc<Zp> {
     using E = cx<Zp>;
     using M = float;
-    static __device__ __forceinline__ E key_pair(uint32_t ba, uint32_t bb) { return (E)ba | ((E)bb << 32); }
+    static __device__ __forceinline__ E key_pair(uint32_t x, int j) {
+        return (E)((x >> j) & 1u) | ((E)((x >> (16 + j)) & 1u) << 32);
+    }
     static __device__ __forceinline__ E seed(bool in_range, uint32_t bit) { return (in_range && bit) ? 1ull : 0ull; }
     // (the exact transform has no half-length packing of one key: its values are not complex)
     static __device__ __forceinline__ E seed_pair(bool, uint32_t, bool, uint32_t) { return 0ull; }
@@ -117,40 +138,64 @@ template <> struct Enc<Zp> {
 };
 
 // ---------------------------------------------------------------------------
-// Bit staging for the level-1 forward passes: per row, the CTA's COLS input bits
-// (low 16 bits: key or key a; high 16 bits: key b or seed) after the transform's
-// shared memory.
-template <typename T, int LEN, int COLS>
-__device__ __forceinline__ uint32_t *key_stage(unsigned char *smem_raw) {
-    return reinterpret_cast<uint32_t *>(smem_raw + smem_elems<LEN, COLS>() * sizeof(cx<T>));
+// Input bits of the level-1 forward passes. Thread (tq, col) transforms the E rows
+// tq + j*TC, j < E, of column col, but a row's bits lie together in memory: lane j of a
+// group of E lanes loads the row's bits, one word for two bit vectors (low and high half),
+// and log2 E exchange steps transpose the E x E bit matrices across the group. Column c's
+// word ends in lane c, which is the thread that transforms it (E = COLS: one row group of
+// E threads; E = 2*COLS: the group's rows are those of two neighbouring tq, the second's
+// bits above the first's). No shared memory, no barrier, and every element is two
+// shift-and-mask instructions at constant positions: on rows of 256 the first pass went
+// from 859 to about 690 instructions per thread with this and the tables of tables.cuh.
+template <int E>
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x) {
+    static_assert(E == 8 || E == 16, "groups of 8 or 16 lanes");
+    const uint32_t lane = threadIdx.x & 31;
+#pragma unroll
+    for (int d = E / 2; d >= 1; d >>= 1) {
+        // bit positions whose index has bit d clear, in both halves
+        const uint32_t m = d == 8 ? 0x00FF00FFu : d == 4 ? 0x0F0F0F0Fu : d == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
+        x = (lane & d) ? ((x & ~m) | ((y >> d) & m)) : ((x & m) | ((y & m) << d));
+    }
+    return x;
 }
-template <typename T, int LEN, int COLS>
-constexpr size_t stage_bytes() { return (size_t)LEN * sizeof(uint32_t); }
+// Rows (and their bit offset in the group word) that this lane loads: row(0), and row(1) when E = 2*COLS.
+template <int LEN, int COLS, int E>
+__device__ __forceinline__ uint32_t lane_row(int h) {
+    static_assert(E == COLS || E == 2 * COLS, "one or two rows per lane");
+    const uint32_t unit = threadIdx.x / E, j = threadIdx.x % E;
+    return (E == COLS ? unit : 2 * unit + (uint32_t)h) + j * (uint32_t)(LEN / E);
+}
+// Position j of the row of register slot s (first-stage layout idx_r0): row = tq + j*TC.
+template <int LEN, int E>
+constexpr int slot_pos(int s) {
+    return s / Plan<LEN, E>::r0 + (s % Plan<LEN, E>::r0) * (E / Plan<LEN, E>::r0);
+}
 
-// Two per-thread counters reduced over the CTA (sum, or max when MAX): warp reductions,
-// then warp 0 over the warps' partial results (kept in scratch, 64 words of shared
-// memory). The totals are valid in thread 0. Every thread of the CTA must call it (it
-// holds a barrier). The per-key counters of a batch (key popcounts, rounding margins)
-// are accumulated with one atomic per key and CTA this way: one atomic per warp on the
-// same few words from thousands of CTAs at once queues up in the memory system and
-// measurably slows the whole pass.
+// Two per-thread counters reduced over the CTA (sum, or max when MAX): warp reductions into
+// scratch (64 words of shared memory; cta_reduce_put), a barrier of the caller's, then warp 0
+// over the warps' partial results (cta_reduce_get: the totals are valid in thread 0). The
+// per-key counters of a batch (key popcounts, rounding margins) are accumulated with one
+// atomic per key and CTA this way: one atomic per warp on the same few words from thousands
+// of CTAs at once queues up in the memory system and measurably slows the whole pass.
 template <bool MAX>
-__device__ __forceinline__ void cta_reduce2(uint32_t &a, uint32_t &b, uint32_t *scratch) {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void cta_reduce_put(uint32_t a, uint32_t b, uint32_t *scratch) {
     a = MAX ? __reduce_max_sync(0xffffffffu, a) : __reduce_add_sync(0xffffffffu, a);
     b = MAX ? __reduce_max_sync(0xffffffffu, b) : __reduce_add_sync(0xffffffffu, b);
-    if (lane == 0) {
-        scratch[warp] = a;
-        scratch[32 + warp] = b;
+    if ((threadIdx.x & 31) == 0) {
+        scratch[threadIdx.x >> 5] = a;
+        scratch[32 + (threadIdx.x >> 5)] = b;
     }
-    __syncthreads();
-    if (warp == 0) {
-        const uint32_t nw = blockDim.x >> 5;
-        a = lane < nw ? scratch[lane] : 0u;
-        b = lane < nw ? scratch[32 + lane] : 0u;
-        a = MAX ? __reduce_max_sync(0xffffffffu, a) : __reduce_add_sync(0xffffffffu, a);
-        b = MAX ? __reduce_max_sync(0xffffffffu, b) : __reduce_add_sync(0xffffffffu, b);
-    }
+}
+template <bool MAX>
+__device__ __forceinline__ void cta_reduce_get(uint32_t &a, uint32_t &b, const uint32_t *scratch) {
+    if (threadIdx.x >= 32) return;
+    const uint32_t lane = threadIdx.x, nw = blockDim.x >> 5;
+    a = lane < nw ? scratch[lane] : 0u;
+    b = lane < nw ? scratch[32 + lane] : 0u;
+    a = MAX ? __reduce_max_sync(0xffffffffu, a) : __reduce_add_sync(0xffffffffu, a);
+    b = MAX ? __reduce_max_sync(0xffffffffu, b) : __reduce_add_sync(0xffffffffu, b);
 }
 
 // Single keys in half-length transforms: transform element t carries key bits 2t
@@ -211,36 +256,40 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint64_t u = (uint64_t)blockIdx.x * COLS + col;
     const uint32_t pair = blockIdx.y;
     const bool has_b = 2 * pair + 1 < nkeys;
-    // Stage the CTA's COLS bits of every row of both keys in shared memory first:
-    // one word load per row instead of one per element, all in flight together.
-    uint32_t *stage = key_stage<T, LEN, COLS>(smem_raw);
     const uint64_t u0 = (uint64_t)blockIdx.x * COLS;
-    uint32_t ca = 0, cb = 0;  // the CTA's share of each key's popcount P (the CTAs tile every bit once)
     // The transform's input element t is key bit koff + t (koff = 0, or m for the modified
     // Toeplitz hash, whose Toeplitz block multiplies key bits m .. n-1).
     const uint64_t nk = n + koff;
     const bool aligned = (koff % COLS) == 0;
     const uint64_t *xa = keys + (uint64_t)(PACK ? pair : 2 * pair) * kstride, *xb = xa + kstride;
-    for (uint32_t a = threadIdx.x; a < LEN; a += blockDim.x) {
-        const uint64_t t0 = (uint64_t)a * S + u0 + koff;  // S % 64 == 0: aligned COLS bits sit in one word
+    uint32_t xa_bits = 0u, xb_bits = 0u;  // this lane's share of the two bit matrices
+#pragma unroll
+    for (int h = 0; h < E / COLS; ++h) {
+        const uint64_t r0 = (uint64_t)lane_row<LEN, COLS, E>(h) * S + u0;  // S % 64 == 0: aligned COLS bits sit in one word
         uint32_t wa, wb = 0u;
         if constexpr (PACK) {  // 2*COLS key bits from 2*(a*S + u0): the even ones real, the odd ones imaginary
-            const uint32_t c = bits_at(xa, nk, 2 * ((uint64_t)a * S + u0) + koff, 2 * COLS);
+            const uint32_t c = bits_at(xa, nk, 2 * r0 + koff, 2 * COLS);
             wa = even_bits(c);
             wb = even_bits(c >> 1);
         } else if (aligned) {
-            wa = aligned_bits<COLS>(xa, nk, t0);
-            if (has_b) wb = aligned_bits<COLS>(xb, nk, t0);
+            wa = aligned_bits<COLS>(xa, nk, r0 + koff);
+            if (has_b) wb = aligned_bits<COLS>(xb, nk, r0 + koff);
         } else {
-            wa = bits_at(xa, nk, t0, COLS);
-            if (has_b) wb = bits_at(xb, nk, t0, COLS);
+            wa = bits_at(xa, nk, r0 + koff, COLS);
+            if (has_b) wb = bits_at(xb, nk, r0 + koff, COLS);
         }
-        stage[a] = wa | (wb << 16);
-        ca += __popc(wa);
-        cb += __popc(wb);
+        xa_bits |= wa << (h * COLS);
+        xb_bits |= wb << (h * COLS);
     }
     __shared__ uint32_t red[64];
-    cta_reduce2<false>(ca, cb, red);  // also publishes the staged rows
+    uint32_t ca = __popc(xa_bits), cb = __popc(xb_bits);  // the CTA's share of each key's popcount P (the CTAs tile every bit once)
+    cta_reduce_put<false>(ca, cb, red);
+    const uint32_t x = transpose_bits<E>(xa_bits | (xb_bits << 16));
+    cx<T> v[E];
+#pragma unroll
+    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_pair(x, slot_pos<LEN, E>(s));
+    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+    cta_reduce_get<false>(ca, cb, red);  // behind the transform's barriers
     if (threadIdx.x == 0 && (ca | cb)) {
         if (PACK) {
             atomicAdd(popc + pair, ca + cb);
@@ -249,16 +298,8 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
             if (cb) atomicAdd(popc + 2 * pair + 1, cb);
         }
     }
-    cx<T> v[E];
-#pragma unroll
-    for (int s = 0; s < E; ++s) {
-        const uint32_t w2 = stage[idx_r0<LEN, E>(tq, s)];
-        v[s] = Enc<T>::key_pair((w2 >> col) & 1u, (w2 >> (16 + col)) & 1u);
-    }
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw);
     cx<T> *w = W + (uint64_t)pair * L;
-    // k = tq + s*TC: w_L^{k u} = w_L^{tq u} * (w_L^{TC u})^s
-    twiddle_chain<T, false, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
 #pragma unroll
     for (int s = 0; s < E; ++s) w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
 }
@@ -300,18 +341,18 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
             v[s] = Enc<T>::seed(in_range, bit);
         }
     }
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw);
-    twiddle_chain<T, false, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
+    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
 #pragma unroll
     for (int s = 0; s < E; ++s) W[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
 }
 
 // Middle-level strided pass (three-level plans only), forward or inverse.
-// S is the innermost length (the stride of this pass); blocks of LEN*S elements;
-// w_{LEN*S}^e = w_L^{e * mult} with mult = L / (LEN*S). Grid (S/COLS, blocks * pairs).
+// S is the innermost length (the stride of this pass); blocks of LEN*S elements.
+// Grid (S/COLS, blocks * pairs).
 template <typename T, int LEN, int COLS, int E, bool INV>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
-    k_mid(cx<T> *__restrict__ W, uint64_t L, uint32_t S, uint32_t mult, TwTab<T> tw) {
+    k_mid(cx<T> *__restrict__ W, uint64_t L, uint32_t S, TwTab<T> tw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
@@ -326,9 +367,9 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         const uint32_t a = INV ? idx_e<LEN, E>(tq, s) : idx_r0<LEN, E>(tq, s);
         v[s] = w[(uint64_t)a * S + u];
     }
-    if (INV) twiddle_chain<T, true, E>(v, tw, (tq * u) * mult, ((LEN / E) * u) * mult);
-    cta_fft<T, LEN, COLS, E, INV>(sm, v, tq, col, tw);
-    if (!INV) twiddle_chain<T, false, E>(v, tw, (tq * u) * mult, ((LEN / E) * u) * mult);
+    if (INV) pass_twiddles<T, true, E, COLS>(v, tw.iv[1], gridDim.x, tq, blockIdx.x, col);
+    cta_fft<T, LEN, COLS, E, INV>(sm, v, tq, col, tw.st[1]);
+    if (!INV) pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, tq, blockIdx.x, col);
 #pragma unroll
     for (int s = 0; s < E; ++s) {
         const uint32_t a = INV ? idx_r0<LEN, E>(tq, s) : idx_e<LEN, E>(tq, s);
@@ -353,9 +394,9 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
     if constexpr (Plan<LEN, E>::RO == 1) {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
-        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw);
+        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw, [&](uint32_t o) { return wt[o]; });
+        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
     }
     if constexpr (MODE == 1) {
 #pragma unroll
@@ -365,11 +406,11 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
         for (int s = 0; s < E; ++s) v[s] = Arith<T>::mul(v[s], spt[idx_e<LEN, E>(0, s)]);
         __syncthreads();  // the forward transform's last shared-memory reads are done
         if constexpr (Plan<LEN, E>::RO == 1) {
-            cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw);
+            cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw.st[2]);
 #pragma unroll
             for (int s = 0; s < E; ++s) wt[idx_r0<LEN, E>(0, s)] = v[s];
         } else {
-            cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw, [&](uint32_t o, cx<T> x) { wt[o] = x; });
+            cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o, cx<T> x) { wt[o] = x; });
         }
     }
 }
@@ -462,7 +503,9 @@ __device__ __forceinline__ void pack_pair_bits(const cx<T> *v, uint32_t tq, uint
     }
     uint32_t fa = __float_as_uint(margin_to_float(ma)), fb = __float_as_uint(margin_to_float(mb));
     __shared__ uint32_t red[64];
-    cta_reduce2<true>(fa, fb, red);
+    cta_reduce_put<true>(fa, fb, red);
+    __syncthreads();
+    cta_reduce_get<true>(fa, fb, red);
     if (threadIdx.x == 0) {
         atomicMax(margin_bits + ka, fa);
         if (has_b) atomicMax(margin_bits + kb, fb);
@@ -496,8 +539,8 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     cx<T> v[E];
 #pragma unroll
     for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u];
-    twiddle_chain<T, true, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
-    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw);
+    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, tq, blockIdx.x, col);
+    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
 
     const uint32_t popa = popc[ka];
     const uint32_t popb = PACK ? popa : (has_b ? popc[kb] : 0u);
@@ -555,7 +598,9 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         }
         uint32_t f = __float_as_uint(margin_to_float(ma > mb ? ma : mb)), unused = 0u;
         __shared__ uint32_t red[64];
-        cta_reduce2<true>(f, unused, red);
+        cta_reduce_put<true>(f, unused, red);
+        __syncthreads();
+        cta_reduce_get<true>(f, unused, red);
         if (threadIdx.x == 0) atomicMax(margin_bits + ka, f);
         return;
     }
@@ -645,11 +690,11 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
             next_tile = nt;  // read by every thread after pack_pair_bits' barrier
         }
         const uint32_t pair = t / ncolt;
-        const uint64_t u0 = (uint64_t)(t % ncolt) * COLS, u = u0 + col;
+        const uint64_t u0 = (uint64_t)(t % ncolt) * COLS;
         const uint32_t ka = 2 * pair, kb = ka + 1;
         const bool has_b = kb < nkeys;
-        twiddle_chain<T, true, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
-        cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw);
+        pass_twiddles<T, true, E, COLS>(v, tw.iv[0], ncolt, tq, t % ncolt, col);
+        cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
         const uint32_t popa = popc[ka], popb = has_b ? popc[kb] : 0u;
         word_t *oa = reinterpret_cast<word_t *>(out + (uint64_t)ka * ostride);
         word_t *ob = reinterpret_cast<word_t *>(out + (uint64_t)kb * ostride);
@@ -697,17 +742,16 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint64_t u = (uint64_t)blockIdx.x * COLS + col;
     const BlockDev bd = blocks[blockIdx.y];
     const uint64_t n = bd.n, sbits = bd.n + bd.m - 1;
-    // stage per row: the CTA's COLS key bits (aligned), COLS seed bits at the rotated
+    // per row: the CTA's COLS key bits (aligned), COLS seed bits at the rotated
     // position j = a*S + u0 + n - 1 (mod L; the window may wrap past L) and the mask
     // of window positions inside the seed (past it the value is 0, not +-1)
-    uint64_t *stage = reinterpret_cast<uint64_t *>(key_stage<T, LEN, COLS>(smem_raw));
     const uint64_t u0 = (uint64_t)blockIdx.x * COLS;
     const uint32_t full = (1u << COLS) - 1u;
-    uint32_t ck = 0;  // the CTA's share of the key's popcount P (the CTAs tile every bit once)
-    for (uint32_t a = threadIdx.x; a < LEN; a += blockDim.x) {
-        const uint64_t t0 = (uint64_t)a * S + u0;
+    uint32_t kbits = 0u, sbit = 0u, inbits = 0u;
+#pragma unroll
+    for (int h = 0; h < E / COLS; ++h) {
+        const uint64_t t0 = (uint64_t)lane_row<LEN, COLS, E>(h) * S + u0;
         const uint32_t wk = aligned_bits<COLS>(bd.key, n, t0);
-        ck += __popc(wk);
         uint64_t j0 = t0 + n - 1;
         if (j0 >= L) j0 -= L;
         uint32_t ws, inr;
@@ -721,23 +765,22 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
             const uint32_t nw = sbits >= COLS - c1 ? COLS - c1 : (uint32_t)sbits;  // wrapped positions inside the seed
             inr = lo | (((1u << nw) - 1u) << c1);
         }
-        stage[a] = (uint64_t)wk | ((uint64_t)ws << 16) | ((uint64_t)inr << 32);
+        kbits |= wk << (h * COLS);
+        sbit |= ws << (h * COLS);
+        inbits |= inr << (h * COLS);
     }
-    uint32_t unused = 0u;
+    uint32_t ck = __popc(kbits), unused = 0u;  // the CTA's share of the key's popcount P (the CTAs tile every bit once)
     __shared__ uint32_t red[64];
-    cta_reduce2<false>(ck, unused, red);  // also publishes the staged rows
-    if (threadIdx.x == 0 && ck) atomicAdd(popc + bd.id, ck);
+    cta_reduce_put<false>(ck, unused, red);
+    const uint32_t x = transpose_bits<E>(kbits | (sbit << 16)), in = transpose_bits<E>(inbits);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) {
-        const uint64_t w3 = stage[idx_r0<LEN, E>(tq, s)];
-        const uint32_t bx = (uint32_t)(w3 >> col) & 1u, bs = (uint32_t)(w3 >> (16 + col)) & 1u;
-        const uint32_t inr = (uint32_t)(w3 >> (32 + col)) & 1u;
-        v[s] = Arith<T>::mk(bx ? (T)1 : (T)0, inr ? (bs ? (T)-1 : (T)1) : (T)0);
-    }
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw);
+    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, in, slot_pos<LEN, E>(s));
+    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+    cta_reduce_get<false>(ck, unused, red);  // behind the transform's barriers
+    if (threadIdx.x == 0 && ck) atomicAdd(popc + bd.id, ck);
     cx<T> *w = W + (uint64_t)blockIdx.y * L;
-    twiddle_chain<T, false, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
 #pragma unroll
     for (int s = 0; s < E; ++s) w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
 }
@@ -781,9 +824,9 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
         if constexpr (Plan<LEN, E>::RO == 1) {
 #pragma unroll
             for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
-            cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw);
+            cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
         } else {
-            cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw, [&](uint32_t o) { return wt[o]; });
+            cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
         }
         __syncthreads();
 #pragma unroll
@@ -813,12 +856,12 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     cx<T> *wot = Wi + (uint64_t)blockIdx.y * L + (uint64_t)row * LEN + tq;
     const bool store = !(self_paired && g == 1);  // a self-paired row is written once
     if constexpr (Plan<LEN, E>::RO == 1) {
-        cta_fft<T, LEN, 1, E, true>(sm, y, tq, 0, tw);
+        cta_fft<T, LEN, 1, E, true>(sm, y, tq, 0, tw.st[2]);
         if (!store) return;
 #pragma unroll
         for (int s = 0; s < E; ++s) wot[idx_r0<LEN, E>(0, s)] = y[s];
     } else {
-        cta_fft_inv_odd<T, LEN, E>(sm, y, tq, tw, [&](uint32_t o, cx<T> x) {
+        cta_fft_inv_odd<T, LEN, E>(sm, y, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
             if (store) wot[o] = x;
         });
     }
@@ -857,9 +900,9 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     if constexpr (Plan<LEN, E>::RO == 1) {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
-        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw);
+        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw, [&](uint32_t o) { return wt[o]; });
+        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
     }
     __syncthreads();
 #pragma unroll
@@ -897,12 +940,12 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
         __syncthreads();  // the mirror reads of both groups are done
         const bool store = !(self_paired && g == 1);  // a self-paired row is written once
         if constexpr (Plan<LEN, E>::RO == 1) {
-            cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw);
+            cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw.st[2]);
             if (!store) return;
 #pragma unroll
             for (int s = 0; s < E; ++s) wt[idx_r0<LEN, E>(0, s)] = v[s];
         } else {
-            cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw, [&](uint32_t o, cx<T> x) {
+            cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
                 if (store) wt[o] = x;
             });
         }
@@ -930,8 +973,8 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     cx<T> v[E];
 #pragma unroll
     for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u];
-    twiddle_chain<T, true, E>(v, tw, (uint32_t)(tq * u), (uint32_t)((LEN / E) * u));
-    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw);
+    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, tq, blockIdx.x, col);
+    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
     const uint32_t popa = popc[ba_.id];
     const uint32_t popb = has_b ? popc[bb_.id] : 0u;
     word_t *oa = reinterpret_cast<word_t *>(ba_.out);

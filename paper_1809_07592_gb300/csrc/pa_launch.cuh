@@ -47,7 +47,7 @@ cudaError_t fwd_keys_at(const uint64_t *keys, uint32_t nkeys, uint64_t kstride, 
                         uint32_t pairs, TwTab<T> tw, uint32_t *popc, cudaStream_t st, uint64_t koff) {
     constexpr int E = Shape<T>::E, COLS = strided_cols<T, LEN>();
     auto kern = k_fwd_keys<T, LEN, COLS, E, PACK>;
-    constexpr size_t sb = smem_bytes<T, LEN, COLS>() + stage_bytes<T, LEN, COLS>();
+    constexpr size_t sb = smem_bytes<T, LEN, COLS>();
     cudaError_t e = set_smem(kern, sb);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((L / LEN) / COLS), pairs);
@@ -106,18 +106,17 @@ cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S
         constexpr int COLS = strided_cols<T, LEN>();
         constexpr size_t sb = smem_bytes<T, LEN, COLS>();
         const uint64_t nblk = L / ((uint64_t)LEN * S);
-        const uint32_t mult = (uint32_t)(L / ((uint64_t)LEN * S));
         dim3 grid((unsigned)(S / COLS), (unsigned)(nblk * pairs));
         if (inverse) {
             auto kern = k_mid<T, LEN, COLS, E, true>;
             cudaError_t e = set_smem(kern, sb);
             if (e != cudaSuccess) return e;
-            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, mult, tw);
+            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, tw);
         } else {
             auto kern = k_mid<T, LEN, COLS, E, false>;
             cudaError_t e = set_smem(kern, sb);
             if (e != cudaSuccess) return e;
-            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, mult, tw);
+            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, tw);
         }
         return cudaGetLastError();
     });
@@ -300,7 +299,7 @@ cudaError_t launch_fwd_keyseed(int lgLEN, const BlockDev *blocks, uint32_t nbloc
         constexpr int LEN = decltype(c)::value;
         constexpr int COLS = strided_cols<T, LEN>();
         auto kern = k_fwd_keyseed<T, LEN, COLS, E>;
-        constexpr size_t sb = smem_bytes<T, LEN, COLS>() + 2 * stage_bytes<T, LEN, COLS>();  // 64-bit stage
+        constexpr size_t sb = smem_bytes<T, LEN, COLS>();
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
         dim3 grid((unsigned)((L / LEN) / COLS), nblocks);
@@ -319,7 +318,8 @@ cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, u
     if (e != cudaSuccess) return e;
     const uint32_t R = (uint32_t)(L / LEN);
     dim3 grid(R / 2 + 1, (nblocks + 1) / 2);
-    kern<<<grid, 2 * (LEN / E), sb, st>>>(Wf, Wi, L, nblocks, lgL1, lgM, tw, (T)(1.0 / (double)L));
+    kern<<<grid, 2 * (LEN / E), sb, st>>>(Wf, Wi, L, nblocks, lgL1, lgM, tw,
+                                         (T)(kSpecScale * kSpecScale / (double)L));
     return cudaGetLastError();
 }
 

@@ -25,10 +25,31 @@ template <> struct Shape<double> { static constexpr int E = 8, COLS = 8; };
 template <> struct Shape<Zp> { static constexpr int E = 8, COLS = 8; };
 // Columns per CTA of a strided pass of length LEN: single precision takes 8 instead of 16 at
 // LEN = 1024 (512 threads, two CTAs per SM instead of one).
+constexpr int strided_cols_of(bool single, int len) { return single ? (len >= 1024 ? 8 : Shape<float>::COLS) : 8; }
 template <typename T, int LEN>
 constexpr int strided_cols() {
-    return (std::is_same<T, float>::value && LEN >= 1024) ? 8 : Shape<T>::COLS;
+    static_assert(Shape<double>::COLS == 8 && Shape<Zp>::COLS == 8, "one width for the 64-bit types");
+    return strided_cols_of(std::is_same<T, float>::value, LEN);
 }
+
+// The kernels' view of a transform's tables at mem (layout y).
+template <typename T>
+TwTab<T> tw_tab(const TwLayout &y, const void *mem) {
+    const cx<T> *m = static_cast<const cx<T> *>(mem);
+    TwTab<T> t;
+    t.hi = m + y.hi;
+    t.lo = m + y.lo;
+    t.B = y.B;
+    for (int p = 0; p < 3; ++p) t.st[p] = m + y.st[p];
+    for (int p = 0; p < 2; ++p) {
+        t.fw[p] = PassTw<T>{m + y.pass[p].a, m + y.pass[p].c, m + y.pass[p].g};
+        t.iv[p] = PassTw<T>{m + y.pass[p].ai, m + y.pass[p].ci, m + y.pass[p].gi};
+    }
+    return t;
+}
+
+// The complex passes take key bits as 0 / 2 (Enc in pa_kernels.cuh); spectra are scaled back by this.
+constexpr double kSpecScale = 0.5;
 
 // Supported pass lengths (log2).
 constexpr int kMinLgStrided = 6, kMaxLgStrided = 10;

@@ -60,11 +60,6 @@ struct Slot {  // one stream and its in-flight micro-batch
     int launch_rc = PA_OK;
 };
 
-struct Twiddles {
-    void *hi = nullptr, *lo = nullptr, *fine = nullptr;
-    uint32_t B = 0;
-};
-
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
@@ -87,22 +82,22 @@ struct pa_server {
     std::vector<Slot> slots;
     size_t next_slot = 0;
     cudaMemPool_t pool = nullptr;
-    std::map<std::pair<uint64_t, uint32_t>, Twiddles> tw;  // by (L, F)
+    std::map<std::vector<uint64_t>, TwSet> tw;  // by length and split
     std::map<std::pair<uint64_t, uint64_t>, pa_plan_t *> esc;
     cudaStream_t esc_stream = nullptr;
 };
 
 namespace {
 
-int twiddles_for(pa_server_t *s, const Geometry &g, Twiddles *out) {
-    const auto key = std::make_pair(g.L, g.F());
+int twiddles_for(pa_server_t *s, const Geometry &g, TwSet *out) {
+    const std::vector<uint64_t> key{g.L, (uint64_t)g.lg1, (uint64_t)g.lgM};
     auto it = s->tw.find(key);
     if (it != s->tw.end()) {
         *out = it->second;
         return PA_OK;
     }
-    Twiddles t;
-    int rc = pa_internal_twiddles(g.L, g.F(), (int)s->cfg.dtype, &t.hi, &t.lo, &t.B, &t.fine);
+    TwSet t;
+    int rc = pa_internal_twiddles(g, s->cfg.dtype, &t);
     if (rc != PA_OK) return rc;
     s->tw[key] = t;
     *out = t;
@@ -153,17 +148,12 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         if (rc != PA_OK) break;
         ClassRun c;
         if (!pa::blocks::cached_split(kv.first, s->cfg.dtype, &c.geo)) c.geo = pa::blocks::default_split(kv.first, s->cfg.dtype);
-        Twiddles t;
-        rc = twiddles_for(s, c.geo, &t);
+        rc = twiddles_for(s, c.geo, &c.tw);
         if (rc != PA_OK) break;
         c.d_blocks = d_desc + class_first[ci];
         c.nb = (uint32_t)kv.second.size();
         c.Wf = mem + work_off[ci].first;
         c.Wi = mem + work_off[ci].second;
-        c.tw_hi = t.hi;
-        c.tw_lo = t.lo;
-        c.B = t.B;
-        c.tw_fine = t.fine;
         rc = pa::blocks::run_complex(s->cfg.dtype, c, popc, marg, sl.st);
         ++ci;
     }
@@ -311,11 +301,7 @@ void free_server(pa_server_t *s) {
         if (sl.h_desc) cudaFreeHost(sl.h_desc);
         if (sl.h_marg) cudaFreeHost(sl.h_marg);
     }
-    for (auto &kv : s->tw) {
-        cudaFree(kv.second.hi);
-        cudaFree(kv.second.lo);
-        cudaFree(kv.second.fine);
-    }
+    for (auto &kv : s->tw) pa_internal_free_twiddles(&kv.second);
     for (auto &kv : s->esc) pa_plan_destroy(kv.second);
     if (s->esc_stream) cudaStreamDestroy(s->esc_stream);
     if (s->pool) cudaMemPoolDestroy(s->pool);

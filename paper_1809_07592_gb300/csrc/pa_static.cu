@@ -22,6 +22,7 @@
 #include <cuda.h>  // driver types of the context-id query (resolved at run time, no link to libcuda)
 
 #include "pa.h"
+#include "pa_internal.h"
 #include "pa_launch.h"
 
 using namespace pa;
@@ -33,6 +34,7 @@ namespace {
 // plus twiddle tables and per-key counters.
 constexpr int kMaxLgL = 21;
 constexpr size_t kSlotBytes = ((size_t)1 << kMaxLgL) * 16;        // 32 MiB
+constexpr size_t kTableBytes = (size_t)960 << 10;                     // twiddle tables (at most 720 KiB are used)
 constexpr size_t kScratchBytes = 2 * kSlotBytes + ((size_t)1 << 20);  // + 1 MiB tables and counters
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -104,72 +106,10 @@ float static_guard() {
     return (end && end != s) ? v : 0.25f;
 }
 
-// Twiddles of the complex transforms, exp(-2 pi i e / L) in double precision:
-// the two-level table (hi, lo) and the stage table fine[j] = w_F^j, F = 2^lgF.
-template <typename T>
-__global__ void k_twiddles_complex(cx<T> *hi, cx<T> *lo, uint32_t B, uint32_t lgL, cx<T> *fine, uint32_t lgF) {
-    const uint32_t nhi = 1u << (lgL - B), nlo = 1u << B, nf = 1u << lgF;
-    const double inv = 1.0 / (double)(1ull << lgL);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nhi + nlo + nf; i += gridDim.x * blockDim.x) {
-        double s, c;
-        if (i < nhi + nlo) {
-            const uint64_t e = i < nhi ? ((uint64_t)i << B) : (uint64_t)(i - nhi);
-            sincospi(2.0 * (double)e * inv, &s, &c);
-        } else {
-            sincospi(2.0 * (double)(i - nhi - nlo) / (double)nf, &s, &c);
-        }
-        cx<T> w;
-        w.x = (T)c;
-        w.y = (T)-s;
-        if (i < nhi) hi[i] = w; else if (i < nhi + nlo) lo[i - nhi] = w; else fine[i - nhi - nlo] = w;
-    }
-}
-
-// w_L^e modulo p for the exact transform, by square-and-multiply from the root w;
-// the stage table holds w_F^j = w_L^(j L/F).
-__global__ void k_twiddles_zp(uint64_t *hi, uint64_t *lo, uint32_t B, uint32_t lgL, uint64_t w, uint64_t *fine,
-                              uint32_t lgF) {
-    const uint32_t nhi = 1u << (lgL - B), nlo = 1u << B, nf = 1u << lgF;
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nhi + nlo + nf; i += gridDim.x * blockDim.x) {
-        uint64_t e = i < nhi ? ((uint64_t)i << B)
-                     : i < nhi + nlo ? (uint64_t)(i - nhi)
-                                     : ((uint64_t)(i - nhi - nlo) << (lgL - lgF));
-        uint64_t r = 1, b = w;
-        while (e) {
-            if (e & 1) r = zp_mul(r, b);
-            b = zp_mul(b, b);
-            e >>= 1;
-        }
-        if (i < nhi) hi[i] = r; else if (i < nhi + nlo) lo[i - nhi] = r; else fine[i - nhi - nlo] = r;
-    }
-}
-
-uint64_t mulmod_host(uint64_t a, uint64_t b) {
-    unsigned __int128 x = (unsigned __int128)a * b;
-    return zp_reduce((uint64_t)(x >> 64), (uint64_t)x);
-}
-uint64_t powmod_host(uint64_t a, uint64_t e) {
-    uint64_t r = 1;
-    while (e) {
-        if (e & 1) r = mulmod_host(r, a);
-        a = mulmod_host(a, a);
-        e >>= 1;
-    }
-    return r;
-}
-// Root of order L whose L/32-th power is 2^6 (the in-register root), as in the plans.
-uint64_t root_of_order(uint64_t L) {
-    const uint64_t w = powmod_host(7, (kP - 1) / L);
-    const uint64_t w32 = powmod_host(w, L / 32);
-    for (uint64_t j = 1; j < 64; j += 2)
-        if (powmod_host(w32, j) == 64ull) return powmod_host(w, j);
-    return 0;
-}
-
 template <typename T> cx<T> scale_of(uint64_t L);
-template <> cx<float> scale_of<float>(uint64_t L) { return make_float2((float)(1.0 / (double)L), 0.f); }
-template <> cx<double> scale_of<double>(uint64_t L) { return make_double2(1.0 / (double)L, 0.0); }
-template <> cx<Zp> scale_of<Zp>(uint64_t L) { return powmod_host(L, kP - 2); }
+template <> cx<float> scale_of<float>(uint64_t L) { return make_float2((float)(kSpecScale / (double)L), 0.f); }
+template <> cx<double> scale_of<double>(uint64_t L) { return make_double2(kSpecScale / (double)L, 0.0); }
+template <> cx<Zp> scale_of<Zp>(uint64_t L) { return zp_pow_host(L, kP - 2); }
 template <typename T> cx<T> unit();
 template <> cx<float> unit<float>() { return make_float2(1.f, 0.f); }
 template <> cx<double> unit<double>() { return make_double2(1.0, 0.0); }
@@ -188,33 +128,23 @@ int run_static(unsigned char *base, int lgL, uint64_t n, uint64_t m, const uint6
     cx<T> *W = reinterpret_cast<cx<T> *>(base);
     cx<T> *spec = reinterpret_cast<cx<T> *>(base + kSlotBytes);
     unsigned char *tail = base + 2 * kSlotBytes;
-    const uint32_t B = (uint32_t)(lgL + 1) / 2;
-    cx<T> *hi = reinterpret_cast<cx<T> *>(tail);
-    cx<T> *lo = hi + (1u << (lgL - B));
     int lg1 = lgL - 12;
     if (lg1 < kMinLgStrided) lg1 = kMinLgStrided;
     if (lg1 > kMaxLgStrided) lg1 = kMaxLgStrided;
     const int lg2 = lgL - lg1;  // <= 12 for lgL <= 21: always a two-level split
-    const uint32_t lgF = (uint32_t)(lg1 > lg2 ? lg1 : lg2);  // stage table: lcm of the pass lengths
-    cx<T> *fine = reinterpret_cast<cx<T> *>(tail + (64u << 10));  // after hi/lo (<= 48 KiB); <= 64 KiB
-    uint32_t *popc = reinterpret_cast<uint32_t *>(tail + (512u << 10));
+    uint32_t *popc = reinterpret_cast<uint32_t *>(tail + kTableBytes);
     uint32_t *marg = popc + 2;
-    if constexpr (std::is_same<T, Zp>::value) {
-        const uint64_t w = root_of_order(L);
-        if (!w) return PA_EUNSUPPORTED;
-        k_twiddles_zp<<<64, 256, 0, st>>>(reinterpret_cast<uint64_t *>(hi), reinterpret_cast<uint64_t *>(lo), B,
-                                          (uint32_t)lgL, w, reinterpret_cast<uint64_t *>(fine), lgF);
-    } else {
-        k_twiddles_complex<T><<<64, 256, 0, st>>>(hi, lo, B, (uint32_t)lgL, fine, lgF);
-    }
-    STATIC_CUDA(cudaGetLastError());
-    TwTab<T> tw;
-    tw.hi = hi;
-    tw.lo = lo;
-    tw.B = B;
-    tw.lgL = (uint32_t)lgL;
-    tw.fine = fine;
-    tw.F = 1u << lgF;
+    const pa_dtype_t dtype = std::is_same<T, float>::value    ? PA_FP32_GUARD
+                             : std::is_same<T, double>::value ? PA_FP64
+                                                              : PA_NTT64;
+    Geometry geo;
+    geo.L = L;
+    geo.lg1 = lg1;
+    geo.lgI = lg2;
+    const TwLayout lay = tw_layout(geo, dtype);
+    if (lay.total * sizeof(cx<T>) > kTableBytes) return PA_EUNSUPPORTED;
+    STATIC_CUDA(tw_fill(lay, dtype, tail, st));
+    const TwTab<T> tw = tw_tab<T>(lay, tail);
     STATIC_CUDA(launch_fwd_seed<T>(lg1, seed, n, m, W, L, tw, st));
     STATIC_CUDA(launch_middle<T>(1, lg2, 1, W, spec, L, 1, tw, scale_of<T>(L), st));
     STATIC_CUDA(launch_zero_keys(nkeys, popc, marg, st));  // the forward pass accumulates the popcounts
@@ -245,7 +175,7 @@ extern "C" int pa_hash_static(uint64_t n, uint64_t m, pa_dtype_t dtype, const ui
     int rc = scratch_address(&base);
     if (rc != PA_OK) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    uint32_t *marg = reinterpret_cast<uint32_t *>(base + 2 * kSlotBytes + (512u << 10)) + 2;
+    uint32_t *marg = reinterpret_cast<uint32_t *>(base + 2 * kSlotBytes + kTableBytes) + 2;
 
     if (dtype == PA_NTT64) {
         rc = run_static<Zp>(base, lgL, n, m, seed_dev, keys_dev, nkeys, key_stride_words, out_dev,

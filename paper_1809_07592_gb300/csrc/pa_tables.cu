@@ -1,0 +1,192 @@
+// pa_tables.cu -- layout and filling of the twiddle tables (tables.cuh) of a transform.
+#include "pa.h"
+#include "pa_internal.h"
+#include "pa_launch.h"
+
+using namespace pa;
+
+namespace {
+
+constexpr uint64_t kAlignElems = 32;  // every table starts on a 256-byte boundary (8-byte elements)
+uint64_t take(uint64_t *total, uint64_t n) {
+    const uint64_t at = *total;
+    *total += (n + kAlignElems - 1) / kAlignElems * kAlignElems;
+    return at;
+}
+
+// Exponent (of w_L, not reduced) of element i of the block; inverse tables of the exact
+// transform come back with *neg set. Padding elements read as w^0.
+__device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, bool complex_, bool *neg) {
+    *neg = false;
+    if (i >= y.hi && i < y.hi + y.nhi) return (i - y.hi) << y.B;
+    if (i >= y.lo && i < y.lo + y.nlo) return i - y.lo;
+    for (int p = 0; p < 3; ++p) {
+        if (y.len[p] == 0) continue;
+        const StageList l = stage_list(y.len[p], y.E, complex_);
+        if (i < y.st[p] || i >= y.st[p] + (uint64_t)l.total) continue;
+        const int o = (int)(i - y.st[p]);
+        const StageShape s = stage_shape(y.len[p], y.E);
+        for (int j = 0; j <= 2 * kMaxStages; ++j) {
+            const bool odd = j == 2 * kMaxStages;
+            const StageRow r = odd ? l.odd : j < kMaxStages ? l.fwd[j] : l.inv[j - kMaxStages];
+            const int n = (r.rows + 1) / 2 * 2 * r.P;
+            if (r.rows == 0 || o < r.off || o >= r.off + n) continue;
+            const int q = (o - r.off) / 2;
+            const int row = 2 * (q / r.P) + ((o - r.off) & 1);
+            const uint32_t k = (uint32_t)(q % r.P);
+            if (row >= r.rows) return 0;
+            *neg = !complex_ && j >= kMaxStages;
+            return odd ? odd_exponent(r, s.RO, s.R0C, row, k, y.L) : stage_exponent(r, row, k, y.L, complex_);
+        }
+        return 0;
+    }
+    for (int p = 0; p < 2; ++p) {
+        const PassShape &t = y.pass[p];
+        if (t.stride == 0) continue;
+        const uint64_t mult = p == 0 ? 1 : (uint64_t)y.len[0], nblk = t.stride / t.cols;
+        for (int inv = 0; inv < (complex_ ? 1 : 2); ++inv) {
+            const uint64_t a = inv ? t.ai : t.a, c = inv ? t.ci : t.c, g = inv ? t.gi : t.g;
+            *neg = inv != 0;
+            if (i >= a && i < a + t.tc * nblk) return (i - a) / nblk * ((i - a) % nblk) * t.cols * mult;
+            if (i >= c && i < c + (uint64_t)t.tc * t.cols) return (i - c) / t.cols * ((i - c) % t.cols) * mult;
+            if (i >= g && i < g + t.stride) return t.tc * (i - g) * mult;
+        }
+    }
+    *neg = false;
+    return 0;
+}
+
+// exp(-2 pi i e / L), each part rounded once from double precision.
+template <typename T>
+__device__ cx<T> root_power(uint64_t e, uint64_t L, uint64_t) {
+    double s, c;
+    sincospi(2.0 * ((double)e / (double)L), &s, &c);
+    cx<T> w;
+    w.x = (T)c;
+    w.y = (T)-s;
+    return w;
+}
+template <>
+__device__ cx<Zp> root_power<Zp>(uint64_t e, uint64_t, uint64_t w) {
+    uint64_t r = 1;
+    for (uint64_t b = w; e; e >>= 1) {
+        if (e & 1) r = zp_mul(r, b);
+        b = zp_mul(b, b);
+    }
+    return r;
+}
+
+template <typename T>
+__global__ void k_fill_tables(cx<T> *mem, TwLayout y, uint64_t root) {
+    constexpr bool kComplex = !std::is_same<T, Zp>::value;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < y.total; i += (uint64_t)gridDim.x * blockDim.x) {
+        bool neg;
+        uint64_t e = exponent_at(y, i, kComplex, &neg) % y.L;
+        if (neg && e) e = y.L - e;
+        mem[i] = root_power<T>(e, y.L, root);
+    }
+}
+
+uint64_t zp_mul_host(uint64_t a, uint64_t b) {
+    unsigned __int128 x = (unsigned __int128)a * b;
+    return zp_reduce((uint64_t)(x >> 64), (uint64_t)x);
+}
+
+// Root of unity of order L (a power of two, 32 <= L <= 2^32) whose L/32-th power
+// is 2^6, the root the in-register DFTs use.
+uint64_t zp_root(uint64_t L) {
+    const uint64_t w = zp_pow_host(7, (kP - 1) / L);  // 7 generates the multiplicative group mod p
+    const uint64_t w32 = zp_pow_host(w, L / 32);
+    for (uint64_t j = 1; j < 64; j += 2) {
+        if (zp_pow_host(w32, j) == 64ull) return zp_pow_host(w, j);
+    }
+    return 0;
+}
+
+}  // namespace
+
+namespace pa {
+
+uint64_t zp_pow_host(uint64_t a, uint64_t e) {
+    uint64_t r = 1;
+    for (; e; e >>= 1) {
+        if (e & 1) r = zp_mul_host(r, a);
+        a = zp_mul_host(a, a);
+    }
+    return r;
+}
+
+TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
+    const bool complex_ = dtype != PA_NTT64;
+    TwLayout y;
+    y.L = g.L;
+    int lgL = 0;
+    while ((1ull << lgL) < g.L) ++lgL;
+    y.B = (uint32_t)(lgL + 1) / 2;
+    y.nlo = 1ull << y.B;
+    y.nhi = (g.L + y.nlo - 1) >> y.B;
+    y.E = dtype == PA_FP32_GUARD ? Shape<float>::E : dtype == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
+    y.len[0] = 1 << g.lg1;
+    y.len[1] = g.lgM ? 1 << g.lgM : 0;
+    y.len[2] = (int)g.inner();
+    y.hi = take(&y.total, y.nhi);
+    y.lo = take(&y.total, y.nlo);
+    for (int p = 0; p < 3; ++p)
+        if (y.len[p]) y.st[p] = take(&y.total, (uint64_t)stage_list(y.len[p], y.E, complex_).total);
+    for (int p = 0; p < 2; ++p) {
+        if (!y.len[p]) continue;
+        PassShape &t = y.pass[p];
+        t.tc = (uint32_t)(y.len[p] / y.E);
+        t.cols = (uint32_t)strided_cols_of(dtype == PA_FP32_GUARD, y.len[p]);
+        t.stride = p == 0 ? g.L >> g.lg1 : (uint64_t)g.inner();
+        t.a = t.ai = take(&y.total, t.tc * (t.stride / t.cols));
+        t.c = t.ci = take(&y.total, (uint64_t)t.tc * t.cols);
+        t.g = t.gi = take(&y.total, t.stride);
+        if (!complex_) {  // residues have no conjugate: the inverse passes read tables of their own
+            t.ai = take(&y.total, t.tc * (t.stride / t.cols));
+            t.ci = take(&y.total, (uint64_t)t.tc * t.cols);
+            t.gi = take(&y.total, t.stride);
+        }
+    }
+    return y;
+}
+
+cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t st) {
+    const uint64_t want = (y.total + 255) / 256;
+    const unsigned grid = (unsigned)(want < 1216 ? want : 1216);
+    if (dtype == PA_FP32_GUARD) {
+        k_fill_tables<float><<<grid, 256, 0, st>>>(static_cast<float2 *>(mem), y, 0);
+    } else if (dtype == PA_FP64) {
+        k_fill_tables<double><<<grid, 256, 0, st>>>(static_cast<double2 *>(mem), y, 0);
+    } else {
+        const uint64_t w = (y.L & (y.L - 1)) ? 0 : zp_root(y.L);  // the exact transform keeps power-of-two lengths
+        if (!w) return cudaErrorInvalidValue;
+        k_fill_tables<Zp><<<grid, 256, 0, st>>>(static_cast<unsigned long long *>(mem), y, w);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace pa
+
+int pa_internal_twiddles(const Geometry &g, pa_dtype_t dtype, TwSet *out) {
+    out->lay = tw_layout(g, dtype);
+    const size_t esz = dtype == PA_FP32_GUARD ? sizeof(float2) : dtype == PA_FP64 ? sizeof(double2) : sizeof(uint64_t);
+    cudaError_t e = cudaMalloc(&out->mem, out->lay.total * esz);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        out->mem = nullptr;
+        return PA_ENOMEM;
+    }
+    if (e == cudaSuccess) e = tw_fill(out->lay, dtype, out->mem, nullptr);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // filled before any stream of the caller reads them
+    if (e != cudaSuccess) {
+        pa_internal_free_twiddles(out);
+        return pa_internal_cuda_fail(e, "twiddle tables");
+    }
+    return PA_OK;
+}
+
+void pa_internal_free_twiddles(TwSet *t) {
+    cudaFree(t->mem);
+    t->mem = nullptr;
+}

@@ -40,10 +40,7 @@ struct UClass {
     BlockDev *d_blocks = nullptr;    // device descriptors
     void *Wf = nullptr, *Wi = nullptr;  // forward slots (one per block), inverse slots (one per pair)
     void *spec = nullptr;            // NTT mode: one seed-spectrum slot, blocks run one after another
-    void *tw_hi = nullptr, *tw_lo = nullptr;
-    uint32_t B = 0;
-    void *tw_fine = nullptr;         // stage twiddles, length geo.F() (rebuilt when the split changes F)
-    uint32_t fineF = 0;
+    TwSet tw;                        // twiddle tables of geo
     cudaStream_t st = nullptr;
     cudaEvent_t done = nullptr;
     ClassRun run(const Geometry &g) const {
@@ -54,10 +51,7 @@ struct UClass {
         r.Wf = Wf;
         r.Wi = Wi;
         r.spec = spec;
-        r.tw_hi = tw_hi;
-        r.tw_lo = tw_lo;
-        r.B = B;
-        r.tw_fine = tw_fine;
+        r.tw = tw;
         return r;
     }
 };
@@ -104,25 +98,12 @@ struct pa_uneven {
 
 namespace {
 
-template <typename T>
-TwTab<T> tw_of(const ClassRun &c) {
-    TwTab<T> t;
-    t.hi = static_cast<const cx<T> *>(c.tw_hi);
-    t.lo = static_cast<const cx<T> *>(c.tw_lo);
-    t.B = c.B;
-    t.lgL = 0;
-    while ((1ull << t.lgL) < c.geo.L) ++t.lgL;
-    t.fine = static_cast<const cx<T> *>(c.tw_fine);
-    t.F = c.geo.F();
-    return t;
-}
-
 // Middle strided pass over `slots` consecutive slots, chunked to the grid's y limit.
 template <typename T>
 int mid_chunks(const ClassRun &c, bool inverse, cx<T> *W, uint32_t slots, cudaStream_t st) {
     const uint32_t nblk = 1u << c.geo.lg1;
     const uint32_t per = 65535u / nblk;
-    const TwTab<T> tw = tw_of<T>(c);
+    const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
     for (uint32_t s0 = 0; s0 < slots; s0 += per) {
         const uint32_t k = (slots - s0 < per) ? slots - s0 : per;
         U_CUDA(launch_mid<T>(c.geo.lgM, inverse, W + (uint64_t)s0 * c.geo.L, c.geo.L, c.geo.inner(), k, tw, st));
@@ -135,7 +116,7 @@ template <typename T>
 int run_class_complex(const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStream_t st) {
     const Geometry &g = c.geo;
     const uint32_t nb = c.nb;
-    const TwTab<T> tw = tw_of<T>(c);
+    const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
     cx<T> *Wf = static_cast<cx<T> *>(c.Wf), *Wi = static_cast<cx<T> *>(c.Wi);
     U_CUDA(launch_zero_blocks(c.d_blocks, nb, popc, marg, st));
     U_CUDA(launch_fwd_keyseed<T>(g.lg1, c.d_blocks, nb, Wf, g.L, tw, popc, st));
@@ -155,11 +136,11 @@ int run_class_complex(const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStr
 // NTT mode: per block, seed transform into the class's spectrum slot, then the key.
 int run_class_ntt(const ClassRun &c, const pa_block_desc_t *hb, const uint32_t *ids, uint32_t *popc,
                   uint32_t *marg, cudaStream_t st) {
-    const TwTab<Zp> tw = tw_of<Zp>(c);
+    const TwTab<Zp> tw = tw_tab<Zp>(c.tw.lay, c.tw.mem);
     cx<Zp> *W = static_cast<cx<Zp> *>(c.Wf), *spec = static_cast<cx<Zp> *>(c.spec);
     const Geometry &g = c.geo;
     const uint64_t L = g.L;
-    const cx<Zp> invL = zp_pow2(192 - (int)tw.lgL);  // L^-1 mod p = 2^(192 - log2 L)
+    const cx<Zp> invL = zp_pow_host(L, kP - 2);
     for (uint32_t i = 0; i < c.nb; ++i) {
         const pa_block_desc_t &b = hb[ids[i]];
         const uint64_t kw = (b.n + 63) / 64;
@@ -182,20 +163,11 @@ int run_class(pa_uneven_t *u, const UClass &c, cudaStream_t st) {
     return pa::blocks::run_complex(u->dtype, c.run(c.geo), u->popc, u->marg, st);
 }
 
-// (Re)build the stage-twiddle table of a class for the F of its current split.
-int class_fine(pa_uneven_t *u, UClass &c) {
-    const uint32_t F = c.geo.F();
-    if (c.tw_fine && c.fineF == F) return PA_OK;
-    if (c.tw_fine) cudaFree(c.tw_fine);
-    c.tw_fine = nullptr;
-    void *hi = nullptr, *lo = nullptr;
-    uint32_t B = 0;
-    int rc = pa_internal_twiddles(c.geo.L, F, (int)u->dtype, &hi, &lo, &B, &c.tw_fine);
-    if (rc != PA_OK) return rc;
-    cudaFree(hi);
-    cudaFree(lo);
-    c.fineF = F;
-    return PA_OK;
+// Give a class the split g: its twiddle tables are built anew.
+int set_split(pa_uneven_t *u, UClass &c, const Geometry &g) {
+    pa_internal_free_twiddles(&c.tw);
+    c.geo = g;
+    return pa_internal_twiddles(g, u->dtype, &c.tw);
 }
 
 // Choose a class's split: cached, else time every candidate on the class's own data.
@@ -203,11 +175,12 @@ int tune_class(pa_uneven_t *u, UClass &c) {
     const uint64_t L = c.geo.L;
     std::vector<Geometry> cand = pa::blocks::candidates(L, u->dtype);
     if (cand.empty()) return PA_EUNSUPPORTED;
-    if (pa::blocks::cached_split(L, u->dtype, &c.geo)) return class_fine(u, c);
+    Geometry known;
+    if (pa::blocks::cached_split(L, u->dtype, &known)) return set_split(u, c, known);
     if (cand.size() == 1 || u->dtype == PA_NTT64) {
-        c.geo = pa::blocks::default_split(L, u->dtype);
-        pa::blocks::store_split(c.geo, u->dtype);
-        return class_fine(u, c);
+        known = pa::blocks::default_split(L, u->dtype);
+        pa::blocks::store_split(known, u->dtype);
+        return set_split(u, c, known);
     }
     cudaEvent_t a, b;
     U_CUDA(cudaEventCreate(&a));
@@ -215,8 +188,7 @@ int tune_class(pa_uneven_t *u, UClass &c) {
     float best = 1e30f;
     Geometry bestg = cand[0];
     for (const Geometry &g : cand) {
-        c.geo = g;
-        int rc = class_fine(u, c);
+        int rc = set_split(u, c, g);
         if (rc != PA_OK) return rc;
         float total = 0.f;
         for (int rep = 0; rep < 3; ++rep) {
@@ -236,9 +208,8 @@ int tune_class(pa_uneven_t *u, UClass &c) {
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);
-    c.geo = bestg;
-    pa::blocks::store_split(c.geo, u->dtype);
-    return class_fine(u, c);
+    pa::blocks::store_split(bestg, u->dtype);
+    return set_split(u, c, bestg);
 }
 
 void free_uneven(pa_uneven_t *u) {
@@ -250,9 +221,7 @@ void free_uneven(pa_uneven_t *u) {
         cudaFree(c.Wf);
         cudaFree(c.Wi);
         cudaFree(c.spec);
-        cudaFree(c.tw_hi);
-        cudaFree(c.tw_lo);
-        cudaFree(c.tw_fine);
+        pa_internal_free_twiddles(&c.tw);
         if (c.st) cudaStreamDestroy(c.st);
         if (c.done) cudaEventDestroy(c.done);
     }
@@ -428,9 +397,6 @@ int pa_uneven_create(const pa_block_desc_t *blocks, uint32_t nblocks, pa_dtype_t
             U_TRY(cudaMalloc(&c.Wf, (size_t)nb * L * esz));
             U_TRY(cudaMalloc(&c.Wi, (size_t)((nb + 1) / 2) * L * esz));
         }
-        rc = pa_internal_twiddles(L, c.geo.F(), (int)dtype, &c.tw_hi, &c.tw_lo, &c.B, &c.tw_fine);
-        if (rc != PA_OK) return fail(rc);
-        c.fineF = c.geo.F();
         rc = tune_class(u, c);
         if (rc != PA_OK) return fail(rc);
     }
