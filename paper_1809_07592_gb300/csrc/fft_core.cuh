@@ -11,9 +11,9 @@
 // of Algorithm 2's observation that the spectrum's order is irrelevant to PA,
 // without Algorithm 2's permutation of the final key.
 //
-// Inside a CTA a short transform of length LEN runs as a Stockham autosort FFT:
-// every thread holds E complex values in registers, does radix-R butterflies
-// (R <= E) in registers, and exchanges through shared memory between stages.
+// Inside a CTA every thread of a short transform of length LEN holds E complex values in
+// registers, does radix-R butterflies (R <= E) on them, and exchanges through shared memory
+// between stages, in place.
 // A CTA works on COLS transforms at once, interleaved column-wise in shared
 // memory, so that a warp's global accesses touch COLS consecutive elements.
 #pragma once
@@ -528,311 +528,237 @@ __device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint
     }
 }
 
-// Shared-memory slot of element a of column col (COLS columns interleaved),
-// skewed by one slot every 16 to keep Stockham's strided writes conflict-free.
-template <int COLS>
-__device__ __forceinline__ uint32_t sidx(uint32_t a, uint32_t col) {
-    uint32_t i = a * COLS + col;
-    return i + (i >> 4);
+// ---- in-CTA transforms ---------------------------------------------------------------------
+// A transform of LEN values per column lives in the CTA's registers, E per thread, and passes
+// through shared memory between stages (stage_plan in tables.cuh). Every stage works in place:
+// a thread writes the slots it has read, so an exchange needs one barrier, between the writes of
+// one stage and the reads of the next, and the stage after it none. Stage i's exchange with stage
+// i+1 stays inside blocks of N[i] elements, which N[i] / E neighbouring threads hold: with the last
+// two stages of radix E that is half a warp (E = 16) or less, and the exchange needs no CTA
+// barrier at all. A row of 20*16*16 values has two CTA barriers in the fused innermost pass,
+// where a self-sorting (Stockham) order of the same stages had seven: the in-CTA transforms alone,
+// with no global access, took 143 of that pass's 177 us there.
+//
+// In-place stages leave the spectrum in digit-reversed order. A column's frequency digits are put
+// right where it leaves the CTA (freq_of); rows keep the order, since nothing but the pointwise
+// product, stored in the same order, sees it.
+// Twiddles sit on a stage's inputs in both directions: forward stage i multiplies element r of block b
+// by w_{R P}^{r f} with f the frequency digits found so far (block_freq), inverse stage i by
+// w_N^{-r j} at offset j.
+
+// Shared-memory slot of element a of column col (COLS columns interleaved; one: a row), skewed by
+// one slot every 128 bytes. A stage's r-th element sits at base + r*s with s a multiple of the skew's
+// period, or (s = 1) base a multiple of E: slot(base + r*s) = slot(base) + slot(r*s).
+template <typename T, int COLS>
+constexpr int slot_lg() { return COLS == 1 && sizeof(cx<T>) == 16 ? 3 : 4; }
+template <typename T, int COLS>
+__host__ __device__ constexpr uint32_t slot_of(uint32_t a, uint32_t col) {
+    const uint32_t i = a * COLS + col;
+    return i + (i >> slot_lg<T, COLS>());
 }
-template <int LEN, int COLS>
-constexpr uint32_t smem_elems() { return (uint32_t)LEN * COLS + ((uint32_t)LEN * COLS >> 4) + 1; }
+template <typename T, int LEN, int COLS>
+constexpr uint32_t smem_elems() { return (uint32_t)LEN * COLS + ((uint32_t)LEN * COLS >> slot_lg<T, COLS>()) + 1; }
 
-__host__ __device__ constexpr int ipow(int b, int e) { return e == 0 ? 1 : b * ipow(b, e - 1); }
-
-// The stage plan of tables.cuh at compile time.
-template <int LEN, int E> struct Plan {
-    static constexpr StageShape sh = stage_shape(LEN, E);
-    static constexpr int RO = sh.RO, K2 = sh.K2, q = sh.q, r0 = sh.r0;
-    static constexpr int TC = sh.TC;  // threads per column
-    static constexpr bool FOLD = sh.fold;
-    static constexpr int R0C = sh.R0C;  // power-of-two factor of the odd stage
-    static constexpr int RC = sh.RC;    // radix of the odd stage
+// The stage plan at compile time.
+template <typename T, int LEN, int E> struct Plan {
+    static constexpr StagePlan p = stage_plan(LEN, E, !std::is_same<T, Zp>::value);
+    static constexpr int RO = p.RO, TC = p.TC, r0 = p.r0, n = p.n;
     static_assert(RO == 1 || RO == 3 || RO == 5 || RO == 9, "odd factor must be 1, 3, 5 or 9");
-    static_assert(RO > 1 || q >= 2, "LEN must exceed E");
-    static_assert(K2 >= E, "power-of-two part must be >= E");
+    static_assert(n >= 2 && p.R[n - 1] == E, "at least two stages, the last of radix E");
 };
+
+// block_freq and freq_block (tables.cuh) of stage I with every radix a compile-time constant.
+template <typename T, int LEN, int E, int I>
+__device__ __forceinline__ uint32_t block_to_freq(uint32_t b) {
+    if constexpr (I == 0) {
+        return 0u;
+    } else {
+        constexpr uint32_t R = (uint32_t)Plan<T, LEN, E>::p.R[I - 1], P = (uint32_t)Plan<T, LEN, E>::p.P[I - 1];
+        return b % R * P + block_to_freq<T, LEN, E, I - 1>(b / R);
+    }
+}
+template <typename T, int LEN, int E, int I>
+__device__ __forceinline__ uint32_t freq_to_block(uint32_t f, uint32_t b = 0u) {
+    if constexpr (I == Plan<T, LEN, E>::n - 1) {
+        return b;
+    } else {
+        constexpr uint32_t R = (uint32_t)Plan<T, LEN, E>::p.R[I];
+        return freq_to_block<T, LEN, E, I + 1>(f / R, b * R + f % R);
+    }
+}
+// Frequency (mod TC) of the values that thread tq holds at the end of a forward transform and at
+// the start of an inverse one: register slot s is frequency freq_of(tq) + s*TC. thread_of is the inverse.
 template <typename T, int LEN, int E>
-constexpr StageList stages() { return stage_list(LEN, E, !std::is_same<T, Zp>::value); }
-
-// Index of the element that register slot s of thread tq holds at the start
-// (first-stage input) and at the end (last-stage output) of a transform.
-//   forward start / inverse end:  slot b*R0 + r  ->  tq + b*TC + r*(LEN/R0)   (RO == 1)
-//   forward end / inverse start:  slot r         ->  tq + r*TC
-template <int LEN, int E>
-__device__ __forceinline__ uint32_t idx_r0(uint32_t tq, int s) {
-    using P = Plan<LEN, E>;
-    return tq + (uint32_t)(s / P::r0) * P::TC + (uint32_t)(s % P::r0) * (LEN / P::r0);
+__device__ __forceinline__ uint32_t freq_of(uint32_t tq) {
+    return block_to_freq<T, LEN, E, Plan<T, LEN, E>::n - 1>(tq);
 }
-template <int LEN, int E>
-__device__ __forceinline__ uint32_t idx_e(uint32_t tq, int s) {
-    return tq + (uint32_t)s * (LEN / E);
+template <typename T, int LEN, int E>
+__device__ __forceinline__ uint32_t thread_of(uint32_t f) {
+    return freq_to_block<T, LEN, E, 0>(f);
+}
+// Index of the element in register slot s of thread tq at the start of a forward transform and at
+// the end of an inverse one (no odd stage): stage 0's butterfly s / r0, element s % r0.
+template <typename T, int LEN, int E>
+__device__ __forceinline__ uint32_t elem_of(uint32_t tq, int s) {
+    constexpr int r0 = Plan<T, LEN, E>::r0;
+    return tq + (uint32_t)(s / r0) * (LEN / E) + (uint32_t)(s % r0) * (LEN / r0);
 }
 
-__host__ __device__ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
-
-// Shared-memory slot of element a of a contiguous row (one column) at a stage
-// boundary of span SPAN (the reading stage's span: the writing stage has P * R = SPAN).
-// Power-of-two spans (every boundary of a power-of-two row, and the inverse
-// transform's) use the skew of sidx. A row with an odd stage of radix RC writes
-// with strides RC and R * RC in the forward transform, which that skew leaves
-// 2-4-way bank conflicted; those boundaries (spans divisible by RC) pad one slot
-// every lcm(RC, W) elements instead (W = elements per 128 bytes), and the first one
-// keeps the plain index when RC is odd (an odd stride is conflict-free as it is).
-template <typename T, int LEN, int E, int SPAN>
-__device__ __forceinline__ uint32_t ridx(uint32_t a) {
-    constexpr int RC = Plan<LEN, E>::RC;
-    if constexpr (RC > 1 && SPAN % RC == 0) {
-        if constexpr (RC % 2 == 1) {
-            if constexpr (SPAN == RC) {
-                return a;
-            } else {
-                return a + (a >> 4);
-            }
-        } else {
-            constexpr int W = 128 / (int)sizeof(cx<T>);
-            constexpr uint32_t D = (uint32_t)(RC / gcd_c(RC, W) * W);  // lcm(RC, W) >= 16: fits smem_elems
-            return a + a / D;
-        }
+// Barrier of an exchange inside blocks of N elements.
+template <int N, int E>
+__device__ __forceinline__ void exchange_barrier() {
+    constexpr int scope = N / E;  // threads per block
+    if constexpr (scope <= 32 && 32 % scope == 0) {
+        __syncwarp();
     } else {
-        return a + (a >> 4);
-    }
-}
-// Slot at a stage boundary: ridx for rows, sidx for interleaved columns.
-template <typename T, int LEN, int COLS, int E, int SPAN>
-__device__ __forceinline__ uint32_t bslot(uint32_t a, uint32_t col) {
-    if constexpr (COLS == 1) {
-        return ridx<T, LEN, E, SPAN>(a);
-    } else {
-        return sidx<COLS>(a, col);
+        __syncthreads();
     }
 }
 
-// Period of a boundary's slot map: every map above satisfies
-//     slot(x + Q) = slot(x) + slot(Q)   for all x
-// (Q = 16 / COLS for interleaved columns, 16 for a skewed row, D for a padded row,
-// 1 for the plain index), and hence slot(x + c, col) = slot(x, col) + slot(c, 0)
-// whenever x or c is a multiple of Q. Stage loops use that to compute one slot per
-// butterfly group and reach the others by compile-time offsets.
-template <typename T, int LEN, int COLS, int E, int SPAN>
-constexpr int slot_period() {
-    static_assert(COLS == 1 || 16 % COLS == 0, "interleaved columns must divide 16");
-    if constexpr (COLS > 1) {
-        return 16 / COLS;
-    } else {
-        constexpr int RC = Plan<LEN, E>::RC;
-        if constexpr (RC > 1 && SPAN % RC == 0) {
-            if constexpr (RC % 2 == 1) {
-                return SPAN == RC ? 1 : 16;
-            } else {
-                constexpr int W = 128 / (int)sizeof(cx<T>);
-                return RC / gcd_c(RC, W) * W;
-            }
+// Butterfly g < E / R[I] of thread tq in stage I: block tq / T, offset j = tq % T + g*T, where the
+// T = N[I] / E threads of a block share its butterflies (so that the next exchange stays among them).
+template <typename T, int LEN, int E, int I> struct StageMap {
+    static constexpr StagePlan p = Plan<T, LEN, E>::p;
+    static constexpr int R = p.R[I], N = p.N[I], s = p.s[I], threads = N / E, groups = E / R;
+    static_assert(threads * E == N, "a block is a whole number of threads");
+    static __device__ __forceinline__ uint32_t block(uint32_t tq) { return tq / (uint32_t)threads; }
+    static __device__ __forceinline__ uint32_t offset(uint32_t tq, int g) {
+        return tq % (uint32_t)threads + (uint32_t)(g * threads);
+    }
+    template <int COLS> static __device__ __forceinline__ uint32_t slot(uint32_t tq, int g, uint32_t col) {
+        return slot_of<T, COLS>(block(tq) * (uint32_t)N + offset(tq, g), col);
+    }
+};
+template <typename T, int LEN, int COLS, int E, int I>
+__device__ __forceinline__ void load_stage(const cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col) {
+    using M = StageMap<T, LEN, E, I>;
+#pragma unroll
+    for (int g = 0; g < M::groups; ++g) {
+        const uint32_t s0 = M::template slot<COLS>(tq, g, col);
+#pragma unroll
+        for (int r = 0; r < M::R; ++r) v[g * M::R + r] = sm[s0 + slot_of<T, COLS>((uint32_t)(r * M::s), 0)];
+    }
+}
+template <typename T, int LEN, int COLS, int E, int I>
+__device__ __forceinline__ void store_stage(cx<T> *sm, const cx<T> *v, uint32_t tq, uint32_t col) {
+    using M = StageMap<T, LEN, E, I>;
+#pragma unroll
+    for (int g = 0; g < M::groups; ++g) {
+        const uint32_t s0 = M::template slot<COLS>(tq, g, col);
+#pragma unroll
+        for (int r = 0; r < M::R; ++r) sm[s0 + slot_of<T, COLS>((uint32_t)(r * M::s), 0)] = v[g * M::R + r];
+    }
+}
+// The butterflies of stage I on the thread's registers.
+template <typename T, int LEN, int E, int I, bool INV>
+__device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *st) {
+    using M = StageMap<T, LEN, E, I>;
+    constexpr StagePlan p = Plan<T, LEN, E>::p;
+    constexpr int COUNT = INV ? p.s[I] : p.P[I];
+    constexpr StageRow row = INV ? p.inv[I] : p.fwd[I];
+#pragma unroll
+    for (int g = 0; g < M::groups; ++g) {
+        if constexpr (row.rows == 0) {
+            dft<T, M::R, INV>(v + g * M::R);
         } else {
-            return 16;
+            cx<T> w[row.rows];
+            load_rows<T, row.rows, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
+            dft_rows<T, M::R, INV>(v + g * M::R, w);
         }
     }
 }
 
-// Butterfly k of a radix-R stage of span P whose table rows start at OFF.
-template <typename T, int R, int P, int OFF, bool INV>
-__device__ __forceinline__ void stage_dft(cx<T> *v, const cx<T> *st, uint32_t k) {
-    if constexpr (P == 1) {
-        dft<T, R, INV>(v);
-    } else {
-        constexpr int ROWS = stage_rows(R, !std::is_same<T, Zp>::value);
-        cx<T> w[ROWS];
-        load_rows<T, ROWS, P>(st + OFF, k, w);
-        dft_rows<T, R, INV>(v, w);
-    }
-}
-
-// One Stockham stage of radix R at span P, from registers (already loaded
-// with this stage's inputs) to shared memory. Thread tq handles the E/R
-// butterfly groups i = tq + b*TC; group i reads elements i + r*LEN/R,
-// multiplies by w_{R P}^{r k} (k = i mod P), transforms, and writes element
-// (i - k)*R + k + r*P.
-template <typename T, int LEN, int COLS, int E, int R, int P, int OFF, bool INV>
-__device__ __forceinline__ void stage_to_smem(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
-    constexpr int TC = LEN / E;
-    constexpr int Q = slot_period<T, LEN, COLS, E, P * R>();
-#pragma unroll
-    for (int b = 0; b < E / R; ++b) {
-        const uint32_t i = tq + (uint32_t)b * TC;
-        const uint32_t k = i % P;
-        stage_dft<T, R, P, OFF, INV>(v + b * R, st, k);
-        const uint32_t base = (i - k) * R + k;
-        if constexpr (P % Q == 0 || (P == 1 && R % Q == 0)) {
-            // offsets r*P are multiples of Q, or (P = 1, so k = 0) base = i*R is one
-            const uint32_t s0 = bslot<T, LEN, COLS, E, P * R>(base, col);
-#pragma unroll
-            for (int r = 0; r < R; ++r) sm[s0 + bslot<T, LEN, COLS, E, P * R>((uint32_t)(r * P), 0)] = v[b * R + r];
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) sm[bslot<T, LEN, COLS, E, P * R>(base + (uint32_t)r * P, col)] = v[b * R + r];
-        }
-    }
-}
-
-// Load a stage's inputs from shared memory: group i = tq + b*TC, elements i + r*LEN/R
-// (boundary of span SPAN, the reading stage's span).
-template <typename T, int LEN, int COLS, int E, int R, int SPAN>
-__device__ __forceinline__ void load_from_smem(const cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col) {
-    constexpr int TC = LEN / E;
-    constexpr int Q = slot_period<T, LEN, COLS, E, SPAN>();
-#pragma unroll
-    for (int b = 0; b < E / R; ++b) {
-        const uint32_t i = tq + (uint32_t)b * TC;
-        if constexpr ((LEN / R) % Q == 0) {  // offsets r*LEN/R are multiples of Q
-            const uint32_t s0 = bslot<T, LEN, COLS, E, SPAN>(i, col);
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b * R + r] = sm[s0 + bslot<T, LEN, COLS, E, SPAN>((uint32_t)(r * (LEN / R)), 0)];
-        } else {
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b * R + r] = sm[bslot<T, LEN, COLS, E, SPAN>(i + (uint32_t)r * (LEN / R), col)];
-        }
-    }
-}
-
-// Last stage: twiddle + DFT in registers, results stay in registers.
-template <typename T, int LEN, int COLS, int E, int R, int P, int OFF, bool INV>
-__device__ __forceinline__ void stage_in_regs(cx<T> *v, uint32_t tq, const cx<T> *st) {
-    constexpr int TC = LEN / E;
-#pragma unroll
-    for (int b = 0; b < E / R; ++b) {
-        const uint32_t i = tq + (uint32_t)b * TC;
-        const uint32_t k = i % P;
-        stage_dft<T, R, P, OFF, INV>(v + b * R, st, k);
-    }
-}
-
-// Power-of-two stages S .. q-1 of the forward transform (radix R0 first, then
-// E), starting at span P0. Stage S's inputs are in registers when FROM_REGS,
-// else in shared memory. The last stage leaves its outputs in registers.
-template <typename T, int LEN, int COLS, int E, int S, int P0, bool FROM_REGS>
-__device__ __forceinline__ void fwd_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
-    using PL = Plan<LEN, E>;
-    constexpr StageRow row = stages<T, LEN, E>().fwd[S];
-    constexpr int R = row.R;
-    static_assert(row.P == P0, "stage list and stage order agree");
+// Forward stages I .. n-1, stage I's inputs in shared memory (a barrier away) unless FROM_REGS;
+// the outputs end in registers (frequencies freq_of(tq) + s*TC).
+template <typename T, int LEN, int COLS, int E, int I, bool FROM_REGS>
+__device__ __forceinline__ void fwd_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
+    using PL = Plan<T, LEN, E>;
     if constexpr (!FROM_REGS) {
-        __syncthreads();
-        load_from_smem<T, LEN, COLS, E, R, P0>(sm, v, tq, col);
+        exchange_barrier<COLS * PL::p.N[I - 1], E>();
+        load_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
     }
-    if constexpr (S == PL::q - 1) {
-        stage_in_regs<T, LEN, COLS, E, R, P0, row.off, false>(v, tq, st);
-    } else {
-        if constexpr (!FROM_REGS) __syncthreads();
-        stage_to_smem<T, LEN, COLS, E, R, P0, row.off, false>(sm, v, tq, col, st);
-        fwd_pow2<T, LEN, COLS, E, S + 1, P0 * R, false>(sm, v, tq, col, st);
+    stage_regs<T, LEN, E, I, false>(v, tq, st);
+    if constexpr (I < PL::n - 1) {
+        store_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
+        fwd_stages<T, LEN, COLS, E, I + 1, false>(sm, v, tq, col, st);
+    }
+}
+// Inverse stages I .. LAST (counting down), stage I's inputs in registers; the outputs of stage LAST
+// end in registers, or, with TO_SMEM, in shared memory.
+template <typename T, int LEN, int COLS, int E, int I, int LAST, bool TO_SMEM>
+__device__ __forceinline__ void inv_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
+    using PL = Plan<T, LEN, E>;
+    stage_regs<T, LEN, E, I, true>(v, tq, st);
+    if constexpr (I > LAST || TO_SMEM) store_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
+    if constexpr (I > LAST) {
+        exchange_barrier<COLS * PL::p.N[I - 1], E>();
+        load_stage<T, LEN, COLS, E, I - 1>(sm, v, tq, col);
+        inv_stages<T, LEN, COLS, E, I - 1, LAST, TO_SMEM>(sm, v, tq, col, st);
     }
 }
 
-// Power-of-two stages of the inverse transform: E, ..., E, R0 (stage S counts
-// from the first). The first stage's inputs are in registers. With TO_SMEM the
-// last stage writes its outputs to shared memory (an odd stage follows),
-// otherwise they stay in registers.
-// LAST is the index of the last power-of-two stage to run (q - 1, or q - 2 when
-// the odd stage absorbs the radix-r0 stage).
-template <typename T, int LEN, int COLS, int E, int S, int P0, bool TO_SMEM, int LAST = Plan<LEN, E>::q - 1>
-__device__ __forceinline__ void inv_pow2(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
-    constexpr StageRow row = stages<T, LEN, E>().inv[S];
-    constexpr int R = row.R;
-    static_assert(row.P == P0, "stage list and stage order agree");
-    if constexpr (S > 0) {
-        __syncthreads();
-        load_from_smem<T, LEN, COLS, E, R, P0>(sm, v, tq, col);
-    }
-    if constexpr (S == LAST && !TO_SMEM) {
-        stage_in_regs<T, LEN, COLS, E, R, P0, row.off, true>(v, tq, st);
-    } else {
-        if constexpr (S > 0) __syncthreads();
-        stage_to_smem<T, LEN, COLS, E, R, P0, row.off, true>(sm, v, tq, col, st);
-        if constexpr (S < LAST) inv_pow2<T, LEN, COLS, E, S + 1, P0 * R, TO_SMEM, LAST>(sm, v, tq, col, st);
-    }
-}
-
-// Full power-of-two transform of length LEN on COLS interleaved columns. On
-// entry v holds the first-stage inputs (forward: idx_r0 layout; inverse:
-// idx_e layout); on exit v holds the outputs (forward: idx_e layout; inverse:
-// idx_r0 layout). The caller must __syncthreads() before the call if shared
-// memory is still being read from a previous transform.
+// Full power-of-two transform of length LEN on COLS interleaved columns. Forward: v holds
+// elements elem_of(tq, s) on entry and frequencies freq_of(tq) + s*TC on exit; inverse the
+// other way round. A forward transform writes shared memory that other threads may still be
+// reading (from an earlier one): the caller puts a barrier before it. An inverse transform
+// first writes the slots the same thread read last in the forward one.
 template <typename T, int LEN, int COLS, int E, bool INV>
 __device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
-    static_assert(Plan<LEN, E>::RO == 1, "odd lengths use cta_fft_fwd_odd / cta_fft_inv_odd");
+    using PL = Plan<T, LEN, E>;
+    static_assert(PL::RO == 1, "odd lengths use cta_fft_fwd_odd / cta_fft_inv_odd");
     if constexpr (!INV) {
-        fwd_pow2<T, LEN, COLS, E, 0, 1, true>(sm, v, tq, col, st);
+        fwd_stages<T, LEN, COLS, E, 0, true>(sm, v, tq, col, st);
     } else {
-        inv_pow2<T, LEN, COLS, E, 0, 1, false>(sm, v, tq, col, st);
+        inv_stages<T, LEN, COLS, E, PL::n - 1, 0, false>(sm, v, tq, col, st);
     }
 }
 
 // Forward transform of a contiguous row of LEN = RO * 2^k elements (RO > 1).
-// The first stage has the odd (or composite) radix RC = Plan::RC at span 1: group
-// g = tq + j TC < LEN / RC reads elements g + r LEN / RC through ld(offset), the offset
-// j TC + r LEN / RC counted from element tq (a compile-time constant, so the caller's
-// base pointer for thread tq takes immediate offsets), transforms, and writes
-// shared-memory slots g RC + r (odd_first_stage). The power-of-two stages follow
-// (fwd_odd_rest); outputs end in registers (idx_e).
-template <typename T, int LEN, int E, class Ld>
-__device__ __forceinline__ void odd_first_stage(cx<T> *sm, uint32_t tq, Ld ld) {
-    using PL = Plan<LEN, E>;
-    constexpr int RC = PL::RC, K = LEN / RC, TC = PL::TC;
-    constexpr int G = (K + TC - 1) / TC;  // groups per thread (the last may be partial)
-#pragma unroll
-    for (int j = 0; j < G; ++j) {
-        const uint32_t g = tq + (uint32_t)j * TC;
-        if (g < (uint32_t)K) {
-            cx<T> u[RC];
-#pragma unroll
-            for (int r = 0; r < RC; ++r) u[r] = ld((uint32_t)(j * TC + r * K));
-            dft_comp<T, PL::RO, PL::R0C, false>(u);
-#pragma unroll
-            for (int r = 0; r < RC; ++r) sm[ridx<T, LEN, E, RC>(g * RC + (uint32_t)r)] = u[r];
-        }
-    }
-}
-
-template <typename T, int LEN, int E>
-__device__ __forceinline__ void fwd_odd_rest(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st) {
-    using PL = Plan<LEN, E>;
-    fwd_pow2<T, LEN, 1, E, PL::FOLD ? 1 : 0, PL::RC, false>(sm, v, tq, 0, st);
-}
-
+// Stage 0 has the odd (or composite) radix RC: group b = tq + g TC < K = LEN / RC reads elements
+// b + r K through ld(offset), the offset g TC + r K counted from element tq (a compile-time
+// constant, so the caller's base pointer for thread tq takes immediate offsets).
 template <typename T, int LEN, int E, class Ld>
 __device__ __forceinline__ void cta_fft_fwd_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st, Ld ld) {
-    odd_first_stage<T, LEN, E>(sm, tq, ld);
-    fwd_odd_rest<T, LEN, E>(sm, v, tq, st);
+    constexpr StagePlan p = Plan<T, LEN, E>::p;
+    constexpr int RC = p.RC, K = LEN / RC, TC = p.TC;
+    constexpr int G = (K + TC - 1) / TC;  // groups per thread (the last may be partial)
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const uint32_t b = tq + (uint32_t)g * TC;
+        if (b < (uint32_t)K) {
+            cx<T> u[RC];
+#pragma unroll
+            for (int r = 0; r < RC; ++r) u[r] = ld((uint32_t)(g * TC + r * K));
+            dft_comp<T, p.RO, p.R0C, false>(u);
+            const uint32_t s0 = slot_of<T, 1>(b, 0);
+#pragma unroll
+            for (int r = 0; r < RC; ++r) sm[s0 + slot_of<T, 1>((uint32_t)(r * K), 0)] = u[r];
+        }
+    }
+    fwd_stages<T, LEN, 1, E, 1, false>(sm, v, tq, 0, st);
 }
 
-// Inverse transform of a row (RO > 1): power-of-two stages from registers
-// (idx_e layout) into shared memory, then the odd (or composite) last stage at
-// span K = LEN / RC: group g = tq + j TC < K reads slots g + r K, takes the twiddles
-// w_LEN^{-r g}, transforms, and its output g + r K goes through put(j TC + r K, value)
-// (offset from element tq, as for ld above).
+// Inverse transform of a row (RO > 1): the power-of-two stages from registers into shared memory,
+// then stage 0: group b reads slots b + r K, and its output b + r K goes through
+// put(g TC + r K, value) (offset from element tq, as for ld above).
 template <typename T, int LEN, int E, class St>
 __device__ __forceinline__ void cta_fft_inv_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st, St put) {
-    using PL = Plan<LEN, E>;
-    constexpr int RC = PL::RC, K = LEN / RC, TC = PL::TC;
+    constexpr StagePlan p = Plan<T, LEN, E>::p;
+    constexpr int RC = p.RC, K = LEN / RC, TC = p.TC;
     constexpr int G = (K + TC - 1) / TC;
-    inv_pow2<T, LEN, 1, E, 0, 1, true, PL::FOLD ? PL::q - 2 : PL::q - 1>(sm, v, tq, 0, st);
-    __syncthreads();
+    inv_stages<T, LEN, 1, E, p.n - 1, 1, true>(sm, v, tq, 0, st);
+    exchange_barrier<LEN, E>();
 #pragma unroll
-    for (int j = 0; j < G; ++j) {
-        const uint32_t g = tq + (uint32_t)j * TC;
-        if (g < (uint32_t)K) {
+    for (int g = 0; g < G; ++g) {
+        const uint32_t b = tq + (uint32_t)g * TC;
+        if (b < (uint32_t)K) {
             cx<T> u[RC];
-            if constexpr (K % slot_period<T, LEN, 1, E, K>() == 0) {  // offsets r*K are multiples of the period
-                const uint32_t s0 = ridx<T, LEN, E, K>(g);
+            const uint32_t s0 = slot_of<T, 1>(b, 0);
 #pragma unroll
-                for (int r = 0; r < RC; ++r) u[r] = sm[s0 + ridx<T, LEN, E, K>((uint32_t)(r * K))];
-            } else {
+            for (int r = 0; r < RC; ++r) u[r] = sm[s0 + slot_of<T, 1>((uint32_t)(r * K), 0)];
+            dft_comp_rows<T, p.RO, p.R0C, K, true>(u, st + p.inv[0].off, b);
 #pragma unroll
-                for (int r = 0; r < RC; ++r) u[r] = sm[ridx<T, LEN, E, K>(g + (uint32_t)r * K)];
-            }
-            dft_comp_rows<T, PL::RO, PL::R0C, K, true>(u, st + stages<T, LEN, E>().odd.off, g);
-#pragma unroll
-            for (int r = 0; r < RC; ++r) put((uint32_t)(j * TC + r * K), u[r]);
+            for (int r = 0; r < RC; ++r) put((uint32_t)(g * TC + r * K), u[r]);
         }
     }
 }

@@ -167,10 +167,11 @@ __device__ __forceinline__ uint32_t lane_row(int h) {
     const uint32_t unit = threadIdx.x / E, j = threadIdx.x % E;
     return (E == COLS ? unit : 2 * unit + (uint32_t)h) + j * (uint32_t)(LEN / E);
 }
-// Position j of the row of register slot s (first-stage layout idx_r0): row = tq + j*TC.
-template <int LEN, int E>
+// Position j of the row of register slot s (elem_of): row = tq + j*TC.
+template <typename T, int LEN, int E>
 constexpr int slot_pos(int s) {
-    return s / Plan<LEN, E>::r0 + (s % Plan<LEN, E>::r0) * (E / Plan<LEN, E>::r0);
+    constexpr int r0 = Plan<T, LEN, E>::r0;
+    return s / r0 + (s % r0) * (E / r0);
 }
 
 // Two per-thread counters reduced over the CTA (sum, or max when MAX): warp reductions into
@@ -287,7 +288,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t x = transpose_bits<E>(xa_bits | (xb_bits << 16));
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_pair(x, slot_pos<LEN, E>(s));
+    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_pair(x, slot_pos<T, LEN, E>(s));
     cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
     cta_reduce_get<false>(ca, cb, red);  // behind the transform's barriers
     if (threadIdx.x == 0 && (ca | cb)) {
@@ -299,9 +300,10 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         }
     }
     cx<T> *w = W + (uint64_t)pair * L;
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
+    const uint32_t f = freq_of<T, LEN, E>(tq);
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
 #pragma unroll
-    for (int s = 0; s < E; ++s) w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
+    for (int s = 0; s < E; ++s) w[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
 }
 
 // Level-1 forward pass of the rotated, +-1 encoded seed (real input). PACK: the
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     cx<T> v[E];
 #pragma unroll
     for (int s = 0; s < E; ++s) {
-        const uint64_t pos = (uint64_t)idx_r0<LEN, E>(tq, s) * S + u;
+        const uint64_t pos = (uint64_t)elem_of<T, LEN, E>(tq, s) * S + u;
         if constexpr (PACK) {
             const uint64_t L2 = 2 * L;
             uint32_t bit[2];
@@ -342,9 +344,10 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         }
     }
     cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
+    const uint32_t f = freq_of<T, LEN, E>(tq);
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
 #pragma unroll
-    for (int s = 0; s < E; ++s) W[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
+    for (int s = 0; s < E; ++s) W[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
 }
 
 // Middle-level strided pass (three-level plans only), forward or inverse.
@@ -360,21 +363,19 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint64_t nblk = L / blk_len;
     const uint64_t pair = blockIdx.y / nblk, blk = blockIdx.y % nblk;
     const uint32_t u = blockIdx.x * COLS + col;
-    cx<T> *w = W + pair * L + blk * blk_len;
+    cx<T> *w = W + pair * L + blk * blk_len + u;
+    const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) {
-        const uint32_t a = INV ? idx_e<LEN, E>(tq, s) : idx_r0<LEN, E>(tq, s);
-        v[s] = w[(uint64_t)a * S + u];
-    }
-    if (INV) pass_twiddles<T, true, E, COLS>(v, tw.iv[1], gridDim.x, tq, blockIdx.x, col);
+    for (int s = 0; s < E; ++s) v[s] = w[(INV ? f + s * (LEN / E) : elem_of<T, LEN, E>(tq, s)) * S];
+    if (INV) pass_twiddles<T, true, E, COLS>(v, tw.iv[1], gridDim.x, f, blockIdx.x, col);
     cta_fft<T, LEN, COLS, E, INV>(sm, v, tq, col, tw.st[1]);
-    if (!INV) pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, tq, blockIdx.x, col);
+    if (!INV) pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
+    // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
+    // addresses in registers through the transform (80 bytes of spills)
+    asm volatile("" : "+r"(S));
 #pragma unroll
-    for (int s = 0; s < E; ++s) {
-        const uint32_t a = INV ? idx_r0<LEN, E>(tq, s) : idx_e<LEN, E>(tq, s);
-        w[(uint64_t)a * S + u] = v[s];
-    }
+    for (int s = 0; s < E; ++s) w[(INV ? elem_of<T, LEN, E>(tq, s) : f + s * (LEN / E)) * S] = v[s];
 }
 
 // Innermost level: contiguous rows of LEN elements. MODE 0: forward, times
@@ -391,24 +392,23 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
     cx<T> *wt = W + pair * L + row * LEN + tq;
     cx<T> *spt = spec + row * LEN + tq;
     cx<T> v[E];
-    if constexpr (Plan<LEN, E>::RO == 1) {
+    if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
+        for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
         cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
         cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
     }
     if constexpr (MODE == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) spt[idx_e<LEN, E>(0, s)] = Arith<T>::mul(v[s], scale);
+        for (int s = 0; s < E; ++s) spt[s * (LEN / E)] = Arith<T>::mul(v[s], scale);
     } else {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = Arith<T>::mul(v[s], spt[idx_e<LEN, E>(0, s)]);
-        __syncthreads();  // the forward transform's last shared-memory reads are done
-        if constexpr (Plan<LEN, E>::RO == 1) {
+        for (int s = 0; s < E; ++s) v[s] = Arith<T>::mul(v[s], spt[s * (LEN / E)]);
+        if constexpr (Plan<T, LEN, E>::RO == 1) {
             cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw.st[2]);
 #pragma unroll
-            for (int s = 0; s < E; ++s) wt[idx_r0<LEN, E>(0, s)] = v[s];
+            for (int s = 0; s < E; ++s) wt[elem_of<T, LEN, E>(0, s)] = v[s];
         } else {
             cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o, cx<T> x) { wt[o] = x; });
         }
@@ -425,7 +425,7 @@ __device__ __forceinline__ float margin_to_float(float x) { return x; }
 __device__ __forceinline__ float margin_to_float(double x) { return __double2float_ru(x); }
 
 // Round, mod 2 and pack the outputs of the level-1 inverse transform of one column
-// (pair form): v holds rows t1 = idx_r0(tq, s) of column u = u0 + col, the real part
+// (pair form): v holds rows t1 = elem_of(tq, s) of column u = u0 + col, the real part
 // belonging to key ka with ma_bits outputs, the imaginary part to key kb (if has_b) with
 // mb_bits outputs (the uneven batch pairs blocks of different lengths; a plan's pairs
 // have ma_bits = mb_bits = m). Output bit i = t1*S + u of a key is element i of the
@@ -459,11 +459,11 @@ __device__ __forceinline__ void pack_pair_bits(const cx<T> *v, uint32_t tq, uint
     [[maybe_unused]] const float2 half_p = make_float2(0.5f * (float)(popa & 3u), 0.5f * (float)(popb & 3u));
 #pragma unroll
     for (int s = 0; s < E; ++s) {
-        const uint32_t t1 = idx_r0<LEN, E>(tq, s);
-        if constexpr (Plan<LEN, E>::r0 == E) {  // t1 = tq + s*TC: every later slot is past the bound too
-            if (idx_r0<LEN, E>(tq0, s) >= nrow) break;
+        const uint32_t t1 = elem_of<T, LEN, E>(tq, s);
+        if constexpr (Plan<T, LEN, E>::r0 == E) {  // t1 = tq + s*TC: every later slot is past the bound too
+            if (elem_of<T, LEN, E>(tq0, s) >= nrow) break;
         } else {
-            if (idx_r0<LEN, E>(tq0, s) >= nrow) continue;
+            if (elem_of<T, LEN, E>(tq0, s) >= nrow) continue;
         }
         const uint32_t row0 = t1 * S32 + u032;  // output bit of this row's first column
         const bool valid_a = row0 + col < ma32, valid_b = row0 + col < mb32;
@@ -536,10 +536,11 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t ka = PACK ? pair : 2 * pair, kb = 2 * pair + 1;
     const bool has_b = !PACK && kb < nkeys;
     const cx<T> *w = W + (uint64_t)pair * L;
+    const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u];
-    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, tq, blockIdx.x, col);
+    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)(f + s * (LEN / E)) * S + u];
+    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, f, blockIdx.x, col);
     cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
 
     const uint32_t popa = popc[ka];
@@ -561,11 +562,11 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         const uint32_t nrow = half > u032 ? (half - u032 + S32 - 1u) / S32 : 0u;
 #pragma unroll
         for (int s = 0; s < E; ++s) {
-            const uint32_t t1 = idx_r0<LEN, E>(tq, s);
-            if constexpr (Plan<LEN, E>::r0 == E) {
-                if (idx_r0<LEN, E>(tq0, s) >= nrow) break;
+            const uint32_t t1 = elem_of<T, LEN, E>(tq, s);
+            if constexpr (Plan<T, LEN, E>::r0 == E) {
+                if (elem_of<T, LEN, E>(tq0, s) >= nrow) break;
             } else {
-                if (idx_r0<LEN, E>(tq0, s) >= nrow) continue;
+                if (elem_of<T, LEN, E>(tq0, s) >= nrow) continue;
             }
             const uint32_t row0 = t1 * S32 + u032;
             const uint32_t t = row0 + col;
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
         }
         cx<T> v[E];
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = stg[idx_e<LEN, E>(tq, s) * COLS + col];
+        for (int s = 0; s < E; ++s) v[s] = stg[(freq_of<T, LEN, E>(tq) + s * (LEN / E)) * COLS + col];
         __syncthreads();  // the staged tile has been read: refill it with the next tile
         if (threadIdx.x == 0) {
             const uint32_t nt = atomicAdd(ctl + 1, 1u);
@@ -693,7 +694,7 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
         const uint64_t u0 = (uint64_t)(t % ncolt) * COLS;
         const uint32_t ka = 2 * pair, kb = ka + 1;
         const bool has_b = kb < nkeys;
-        pass_twiddles<T, true, E, COLS>(v, tw.iv[0], ncolt, tq, t % ncolt, col);
+        pass_twiddles<T, true, E, COLS>(v, tw.iv[0], ncolt, freq_of<T, LEN, E>(tq), t % ncolt, col);
         cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
         const uint32_t popa = popc[ka], popb = has_b ? popc[kb] : 0u;
         word_t *oa = reinterpret_cast<word_t *>(out + (uint64_t)ka * ostride);
@@ -775,14 +776,15 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t x = transpose_bits<E>(kbits | (sbit << 16)), in = transpose_bits<E>(inbits);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, in, slot_pos<LEN, E>(s));
+    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, in, slot_pos<T, LEN, E>(s));
     cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
     cta_reduce_get<false>(ck, unused, red);  // behind the transform's barriers
     if (threadIdx.x == 0 && ck) atomicAdd(popc + bd.id, ck);
     cx<T> *w = W + (uint64_t)blockIdx.y * L;
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, tq, blockIdx.x, col);
+    const uint32_t f = freq_of<T, LEN, E>(tq);
+    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
 #pragma unroll
-    for (int s = 0; s < E; ++s) w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u] = v[s];
+    for (int s = 0; s < E; ++s) w[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
 }
 
 // Storage row of the frequency low part rho (lgM = log2 of the middle strided
@@ -790,6 +792,26 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 __device__ __forceinline__ uint32_t split_row(uint32_t rho, uint32_t lgL1, uint32_t lgM) {
     return ((rho & ((1u << lgL1) - 1u)) << lgM) + (rho >> lgL1);
 }
+
+// The mirror bins of a thread's spectrum values (frequency p = f + s*TC of its row) in the
+// mirror row's spectrum in shared memory: frequency LEN-1-p, or in the row of the zero
+// frequency low part -p mod LEN. LEN-1-p complements every digit of p, so thread TC-1-tq holds
+// it, in register slot E-1-s.
+template <typename T, int LEN, int E> struct Mirror {
+    const cx<T> *base;
+    uint32_t shift;  // -p mod LEN for f = 0: the thread's own block, one register slot further
+    __device__ __forceinline__ Mirror(const cx<T> *spectrum, uint32_t tq, bool zero_row) : shift(0) {
+        constexpr uint32_t TC = LEN / E;
+        uint32_t t = TC - 1u - tq;
+        if (zero_row) {
+            const uint32_t f = freq_of<T, LEN, E>(tq);
+            t = f ? thread_of<T, LEN, E>(TC - f) : 0u;
+            shift = f ? 0u : 1u;
+        }
+        base = spectrum + slot_of<T, 1>(t * E, 0);
+    }
+    __device__ __forceinline__ cx<T> at(int s) const { return base[((uint32_t)(E - 1 - s) + shift) % E]; }
+};
 
 // Fused innermost pass of the uneven batch. CTA (rho, pair): rows rho and
 // -rho of blocks 2*pair and 2*pair+1 (if present), one thread group per row.
@@ -802,7 +824,7 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
-    constexpr uint32_t SE = smem_elems<LEN, 1>();
+    constexpr uint32_t SE = smem_elems<T, LEN, 1>();
     const uint32_t g = threadIdx.x / TC, tq = threadIdx.x % TC;
     const uint32_t R = (uint32_t)(L / LEN);  // rows per block
     const uint32_t rho = blockIdx.x;          // 0 .. R/2
@@ -814,6 +836,7 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     const cx<T> *sm_other = smem + (self_paired ? g : 1u - g) * SE;  // where the mirror row's spectrum sits
     const uint32_t b1 = 2 * blockIdx.y, b2 = b1 + 1;
     const bool has2 = b2 < nblocks;
+    const Mirror<T, LEN, E> mir(sm_other, tq, my_rho == 0);
     cx<T> y[E];
 #pragma unroll
     for (int s = 0; s < E; ++s) y[s] = Arith<T>::mk((T)0, (T)0);
@@ -821,23 +844,18 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
         const cx<T> *wt = Wf + (uint64_t)(which ? b2 : b1) * L + (uint64_t)row * LEN + tq;
         cx<T> v[E];
         __syncthreads();  // previous use of the scratch is finished
-        if constexpr (Plan<LEN, E>::RO == 1) {
+        if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-            for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
+            for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
             cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
         } else {
             cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
         }
-        __syncthreads();
-#pragma unroll
-        for (int s = 0; s < E; ++s) sm[sidx<1>(idx_e<LEN, E>(tq, s), 0)] = v[s];
+        store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
         __syncthreads();
 #pragma unroll
         for (int s = 0; s < E; ++s) {
-            const uint32_t p = idx_e<LEN, E>(tq, s);
-            // mirror of position p: -p mod LEN in the row of the zero frequency low part, else LEN-1-p
-            const uint32_t pm = (my_rho == 0) ? (p == 0 ? 0u : (uint32_t)LEN - p) : ((uint32_t)LEN - 1u - p);
-            const cx<T> z = v[s], zm = sm_other[sidx<1>(pm, 0)];
+            const cx<T> z = v[s], zm = mir.at(s);
             // Eq. 7-10: X = (Z(k) + conj Z(-k)) / 2, V = (Z(k) - conj Z(-k)) / (2i)
             const cx<T> X = Arith<T>::mk((z.x + zm.x) * (T)0.5, (z.y - zm.y) * (T)0.5);
             const cx<T> V = Arith<T>::mk((z.y + zm.y) * (T)0.5, (zm.x - z.x) * (T)0.5);
@@ -855,11 +873,11 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     __syncthreads();
     cx<T> *wot = Wi + (uint64_t)blockIdx.y * L + (uint64_t)row * LEN + tq;
     const bool store = !(self_paired && g == 1);  // a self-paired row is written once
-    if constexpr (Plan<LEN, E>::RO == 1) {
+    if constexpr (Plan<T, LEN, E>::RO == 1) {
         cta_fft<T, LEN, 1, E, true>(sm, y, tq, 0, tw.st[2]);
         if (!store) return;
 #pragma unroll
-        for (int s = 0; s < E; ++s) wot[idx_r0<LEN, E>(0, s)] = y[s];
+        for (int s = 0; s < E; ++s) wot[elem_of<T, LEN, E>(0, s)] = y[s];
     } else {
         cta_fft_inv_odd<T, LEN, E>(sm, y, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
             if (store) wot[o] = x;
@@ -885,7 +903,7 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
-    constexpr uint32_t SE = smem_elems<LEN, 1>();
+    constexpr uint32_t SE = smem_elems<T, LEN, 1>();
     const uint32_t g = threadIdx.x / TC, tq = threadIdx.x % TC;
     const uint32_t R = (uint32_t)(N / LEN);  // rows
     const uint32_t rho = blockIdx.x;          // 0 .. R/2
@@ -897,34 +915,31 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     const cx<T> *sm_other = smem + (self_paired ? g : 1u - g) * SE;
     cx<T> *wt = W + (uint64_t)blockIdx.y * N + (uint64_t)row * LEN + tq;
     cx<T> v[E];
-    if constexpr (Plan<LEN, E>::RO == 1) {
+    if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = wt[idx_r0<LEN, E>(0, s)];
+        for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
         cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
         cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
     }
+    store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
     __syncthreads();
-#pragma unroll
-    for (int s = 0; s < E; ++s) sm[sidx<1>(idx_e<LEN, E>(tq, s), 0)] = v[s];
-    __syncthreads();
+    const Mirror<T, LEN, E> mir(sm_other, tq, my_rho == 0);
+    [[maybe_unused]] const uint32_t f = freq_of<T, LEN, E>(tq);
     const cx<T> *Es = tabs, *Os = tabs + N, *Bp = tabs + 2 * N;
     const bool write_tab = !(self_paired && g == 1);
 #pragma unroll
     for (int s = 0; s < E; ++s) {
-        const uint32_t p = idx_e<LEN, E>(tq, s);
-        // mirror of position p: -p mod LEN in the row of the zero frequency low part, else LEN-1-p
-        const uint32_t pm = (my_rho == 0) ? (p == 0 ? 0u : (uint32_t)LEN - p) : ((uint32_t)LEN - 1u - p);
-        const cx<T> z = v[s], zm = sm_other[sidx<1>(pm, 0)];
+        const cx<T> z = v[s], zm = mir.at(s);
         const cx<T> ex = Arith<T>::mk((z.x + zm.x) * (T)0.5, (z.y - zm.y) * (T)0.5);
         const cx<T> ox = Arith<T>::mk((z.y + zm.y) * (T)0.5, (zm.x - z.x) * (T)0.5);
-        const uint64_t e = (uint64_t)row * LEN + p;
+        const uint64_t e = (uint64_t)row * LEN + tq + s * TC;  // the tables keep the registers' order
         if constexpr (MODE == 1) {
             if (write_tab) {
                 const cx<T> es = Arith<T>::mk(ex.x * scale, ex.y * scale);
                 const cx<T> os = Arith<T>::mk(ox.x * scale, ox.y * scale);
-                // frequency of this bin: low part from the strided passes, high part p
-                const uint32_t k = my_rho + R * p;
+                // frequency of this bin: low part from the strided passes, high part from the row
+                const uint32_t k = my_rho + R * (f + s * TC);
                 tabs[e] = es;
                 tabs[N + e] = os;
                 tabs[2 * N + e] = Arith<T>::mul(Arith<T>::template omega<false>(tw, k), os);
@@ -939,11 +954,11 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     if constexpr (MODE == 0) {
         __syncthreads();  // the mirror reads of both groups are done
         const bool store = !(self_paired && g == 1);  // a self-paired row is written once
-        if constexpr (Plan<LEN, E>::RO == 1) {
+        if constexpr (Plan<T, LEN, E>::RO == 1) {
             cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw.st[2]);
             if (!store) return;
 #pragma unroll
-            for (int s = 0; s < E; ++s) wt[idx_r0<LEN, E>(0, s)] = v[s];
+            for (int s = 0; s < E; ++s) wt[elem_of<T, LEN, E>(0, s)] = v[s];
         } else {
             cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
                 if (store) wt[o] = x;
@@ -970,10 +985,11 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const BlockDev ba_ = blocks[ia];
     const BlockDev bb_ = blocks[has_b ? ib : ia];
     const cx<T> *w = W + (uint64_t)blockIdx.y * L;
+    const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)idx_e<LEN, E>(tq, s) * S + u];
-    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, tq, blockIdx.x, col);
+    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)(f + s * (LEN / E)) * S + u];
+    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, f, blockIdx.x, col);
     cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
     const uint32_t popa = popc[ba_.id];
     const uint32_t popb = has_b ? popc[bb_.id] : 0u;

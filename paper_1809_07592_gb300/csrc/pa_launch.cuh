@@ -28,7 +28,7 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
 
 template <typename T, int LEN, int COLS>
 constexpr size_t smem_bytes() {
-    return (size_t)smem_elems<LEN, COLS>() * sizeof(cx<T>);
+    return (size_t)smem_elems<T, LEN, COLS>() * sizeof(cx<T>);
 }
 
 // Calls f(std::integral_constant<int, LEN>) for LEN = 2^lg in [2^LO, 2^HI].

@@ -22,21 +22,21 @@ __device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, bool complex_, bo
     if (i >= y.lo && i < y.lo + y.nlo) return i - y.lo;
     for (int p = 0; p < 3; ++p) {
         if (y.len[p] == 0) continue;
-        const StageList l = stage_list(y.len[p], y.E, complex_);
+        const StagePlan l = stage_plan(y.len[p], y.E, complex_);
         if (i < y.st[p] || i >= y.st[p] + (uint64_t)l.total) continue;
         const int o = (int)(i - y.st[p]);
-        const StageShape s = stage_shape(y.len[p], y.E);
-        for (int j = 0; j <= 2 * kMaxStages; ++j) {
-            const bool odd = j == 2 * kMaxStages;
-            const StageRow r = odd ? l.odd : j < kMaxStages ? l.fwd[j] : l.inv[j - kMaxStages];
-            const int n = (r.rows + 1) / 2 * 2 * r.P;
-            if (r.rows == 0 || o < r.off || o >= r.off + n) continue;
-            const int q = (o - r.off) / 2;
-            const int row = 2 * (q / r.P) + ((o - r.off) & 1);
-            const uint32_t k = (uint32_t)(q % r.P);
+        for (int j = 0; j < 2 * l.n; ++j) {
+            const int stage = j % l.n;
+            const bool inv = j >= l.n;
+            const StageRow r = inv ? l.inv[stage] : l.fwd[stage];
+            const int count = inv ? l.s[stage] : l.P[stage];
+            if (r.rows == 0 || o < r.off || o >= r.off + (r.rows + 1) / 2 * 2 * count) continue;
+            const int q = (o - r.off) / 2, row = 2 * (q / count) + ((o - r.off) & 1);
+            const uint32_t x = (uint32_t)(q % count);
             if (row >= r.rows) return 0;
-            *neg = !complex_ && j >= kMaxStages;
-            return odd ? odd_exponent(r, s.RO, s.R0C, row, k, y.L) : stage_exponent(r, row, k, y.L, complex_);
+            *neg = !complex_ && inv;
+            if (inv && stage == 0 && l.RO > 1) return odd_exponent(l.RO, l.R0C, count, row, x, y.L);
+            return stage_exponent(l.R[stage], count, row, inv ? x : block_freq(l, stage, x), y.L, complex_);
         }
         return 0;
     }
@@ -132,7 +132,7 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
     y.hi = take(&y.total, y.nhi);
     y.lo = take(&y.total, y.nlo);
     for (int p = 0; p < 3; ++p)
-        if (y.len[p]) y.st[p] = take(&y.total, (uint64_t)stage_list(y.len[p], y.E, complex_).total);
+        if (y.len[p]) y.st[p] = take(&y.total, (uint64_t)stage_plan(y.len[p], y.E, complex_).total);
     for (int p = 0; p < 2; ++p) {
         if (!y.len[p]) continue;
         PassShape &t = y.pass[p];

@@ -8,7 +8,7 @@
 // warp of the first pass needs.) Three kinds:
 //   hi, lo       w_L^e = hi[e >> B] * lo[e mod 2^B], for single powers at any e;
 //   stage tables (one per pass length): the multipliers of every in-CTA butterfly stage
-//                (stage_list gives the stages, stage_exponent what each row holds);
+//                (stage_plan gives the stages, stage_exponent what each row holds);
 //   pass tables  (one set per strided pass): w^{k u} for output k = tq + s*TC of column
 //                u = blk*COLS + col as a[tq][blk] * c[tq][col] * g[u]^s.
 #pragma once
@@ -27,101 +27,94 @@ __host__ __device__ constexpr int bitrev(int v, int bits) {
 __host__ __device__ constexpr int odd_part(int v) { return (v & 1) ? v : odd_part(v >> 1); }
 constexpr int kMaxCompositeRadix = 24;
 
-// Stage plan of a Stockham FFT of length LEN = RO * 2^k2 (RO odd: 1, 3, 5 or 9)
-// with E values per thread (TC = LEN / E threads per column). Radices:
-//   forward  [RC], R0, E, ..., E        inverse  E, ..., E, R0, [RC]
-// so the forward's output distribution over threads equals the inverse's input
-// distribution (the two chain in registers). An odd stage exists only in
-// transforms that read their input from, and write their output to, memory
-// (the innermost pass), because its E / RO groups per thread do not divide. It
-// absorbs the radix-r0 stage when r0 < E and the composite radix RC = RO * r0
-// stays within a register budget.
-struct StageShape {
-    int RO, K2, q, r0, TC, R0C, RC;
-    bool fold;
-};
-__host__ __device__ constexpr StageShape stage_shape(int len, int E) {
-    StageShape s{};
-    s.RO = odd_part(len);
-    s.K2 = len / s.RO;
-    const int k = ilog2(s.K2), e = ilog2(E);
-    s.q = (k + e - 1) / e;  // power-of-two stages
-    s.r0 = 1 << (k - (s.q - 1) * e);
-    s.TC = len / E;
-    s.fold = s.RO > 1 && s.r0 < E && s.RO * s.r0 <= kMaxCompositeRadix;
-    s.R0C = s.fold ? s.r0 : 1;
-    s.RC = s.RO * s.R0C;
-    return s;
-}
-
-// The twiddled stages of one pass length: radix R at span P reads `rows` multipliers per
-// butterfly k < P. Rows are stored in pairs, entry (row, k) at off + 2*((row/2)*P + k) + row%2,
-// so that one 16-byte load of single-precision values brings two multipliers.
-struct StageRow {
-    int R, P, rows, off;
-};
+// Stage plan of an in-CTA transform of length LEN = RO * 2^k2 (RO odd: 1, 3, 5 or 9) with E
+// values per thread (TC = LEN / E threads per column). The forward transform runs stages
+// 0 .. n-1 of radix R[i], the inverse n-1 .. 0; stage i combines, within blocks of N[i]
+// elements (block P[i] of them), the R[i] elements s[i] = N[i] / R[i] apart, in place. Radices:
+// [RC], r0, E, ..., E with r0 * E^(q-1) = 2^k2. The odd radix RC exists only in transforms that
+// read their input from, and write their output to, memory (the innermost pass), because its
+// groups do not divide a thread's E values; it absorbs the radix-r0 stage when r0 < E and
+// RC = RO * r0 stays within a register budget.
 constexpr int kMaxStages = 6;
-struct StageList {
-    StageRow fwd[kMaxStages];  // power-of-two stage S of the forward transform (span 1 stages have no rows)
-    StageRow inv[kMaxStages];  // power-of-two stage S of the inverse transform
-    StageRow odd;              // the inverse transform's odd stage
-    int total;                 // entries
+struct StageRow {
+    int rows, off;  // twiddle rows of a stage and where they start
+};
+struct StagePlan {
+    int n, RO, R0C, RC, TC, r0;
+    int R[kMaxStages], N[kMaxStages], s[kMaxStages], P[kMaxStages];
+    // Twiddle tables: butterfly (block b, offset j) of forward stage i reads rows at index b < P[i],
+    // of inverse stage i at index j < s[i]. Rows are stored in pairs, entry (row, x) at
+    // off + 2*((row/2)*count + x) + row%2, so that one 16-byte load of single-precision values
+    // brings two multipliers. rows = 0: no twiddles (forward stage 0, inverse stage n-1).
+    StageRow fwd[kMaxStages], inv[kMaxStages];
+    int total;  // entries
 };
 
 // Rows of a radix-R power-of-two stage. Complex arithmetic: the distinct multipliers of the
-// log2 R butterfly levels (dft_tw in fft_core.cuh); the exact transform: w^r, r = 1 .. R-1.
+// log2 R butterfly levels (dft_rows in fft_core.cuh); the exact transform: w^r, r = 1 .. R-1.
 __host__ __device__ constexpr int stage_rows(int R, bool complex_) { return complex_ ? R / 2 : R - 1; }
 // Rows of the odd stage of radix RO * R0: w^{R0 n1}, then the levels of a radix-R0 stage per k1 < RO.
 __host__ __device__ constexpr int odd_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
 
-__host__ __device__ constexpr StageList stage_list(int len, int E, bool complex_) {
-    StageList l{};
-    const StageShape s = stage_shape(len, E);
-    int off = 0;
-    int P = s.RO > 1 ? s.RC : 1;
-    for (int S = s.fold ? 1 : 0; S < s.q; ++S) {
-        const int R = S == 0 ? s.r0 : E;
-        const int rows = P > 1 ? stage_rows(R, complex_) : 0;
-        l.fwd[S] = StageRow{R, P, rows, off};
+__host__ __device__ constexpr StagePlan stage_plan(int len, int E, bool complex_) {
+    StagePlan l{};
+    l.RO = odd_part(len);
+    const int k = ilog2(len / l.RO), e = ilog2(E);
+    const int q = (k + e - 1) / e;  // power-of-two stages
+    l.r0 = 1 << (k - (q - 1) * e);
+    const bool fold = l.RO > 1 && l.r0 < E && l.RO * l.r0 <= kMaxCompositeRadix;
+    l.R0C = fold ? l.r0 : 1;
+    l.RC = l.RO * l.R0C;
+    l.TC = len / E;
+    if (l.RO > 1) l.R[l.n++] = l.RC;
+    for (int S = fold ? 1 : 0; S < q; ++S) l.R[l.n++] = S == 0 ? l.r0 : E;
+    int P = 1, off = 0;
+    for (int i = 0; i < l.n; ++i) {
+        l.P[i] = P;
+        l.N[i] = len / P;
+        l.s[i] = l.N[i] / l.R[i];
+        const int rows = i == 0 ? 0 : stage_rows(l.R[i], complex_);
+        l.fwd[i] = StageRow{rows, off};
         off += (rows + 1) / 2 * 2 * P;
-        P *= R;
+        P *= l.R[i];
     }
-    P = 1;
-    for (int S = 0; S < (s.fold ? s.q - 1 : s.q); ++S) {
-        const int R = S == s.q - 1 ? s.r0 : E;
-        const int rows = P > 1 ? stage_rows(R, complex_) : 0;
-        l.inv[S] = StageRow{R, P, rows, off};
-        off += (rows + 1) / 2 * 2 * P;
-        P *= R;
-    }
-    if (s.RO > 1) {
-        const int K = len / s.RC, rows = odd_rows(s.RO, s.R0C);
-        l.odd = StageRow{s.RC, K, rows, off};
-        off += (rows + 1) / 2 * 2 * K;
+    for (int i = 0; i < l.n; ++i) {
+        const int rows = i == l.n - 1 ? 0 : i == 0 && l.RO > 1 ? odd_rows(l.RO, l.R0C) : stage_rows(l.R[i], complex_);
+        l.inv[i] = StageRow{rows, off};
+        off += (rows + 1) / 2 * 2 * l.s[i];
     }
     l.total = off;
     return l;
 }
 
+// Frequency of block b of stage i: b's digits, outermost first, are the output digits k_0, ...,
+// k_{i-1} of the earlier stages, and the frequency is k_0 + R[0] (k_1 + R[1] (...)).
+__host__ __device__ constexpr uint32_t block_freq(const StagePlan &l, int i, uint32_t b) {
+    uint32_t f = 0;
+    for (int t = i - 1; t >= 0; --t) {  // the last digit of b is k_{i-1}
+        f += (b % (uint32_t)l.R[t]) * (uint32_t)l.P[t];
+        b /= (uint32_t)l.R[t];
+    }
+    return f;
+}
 // Level and position of row `row` of a complex radix-R stage: level l >= 0 has rows
 // (l == 0: row 0; else rows 2^(l-1) .. 2^l - 1, p = row - 2^(l-1)).
 __host__ __device__ constexpr int row_level(int row) { return row == 0 ? 0 : ilog2(row) + 1; }
 __host__ __device__ constexpr int row_pos(int row) { return row == 0 ? 0 : row - (1 << ilog2(row)); }
 
-// Exponent e (of w_L) held by row `row` of butterfly k of the stage `s` (pass length len).
-__host__ __device__ inline uint64_t stage_exponent(const StageRow &s, int row, uint32_t k, uint64_t L, bool complex_) {
-    const uint64_t unit = L / ((uint64_t)s.R * s.P);  // w_{R P} = w_L^unit
+// Exponent e (of w_L) held by row `row` of a radix-R stage for the twiddle base w_{R P}^k.
+__host__ __device__ inline uint64_t stage_exponent(int R, uint64_t P, int row, uint64_t k, uint64_t L, bool complex_) {
+    const uint64_t unit = L / ((uint64_t)R * P);  // w_{R P} = w_L^unit
     if (!complex_) return (uint64_t)(row + 1) * k * unit;
     const int l = row_level(row);
-    return (uint64_t)(s.R >> (l + 1)) * k * unit + (uint64_t)row_pos(row) * (L >> (l + 1));
+    return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)row_pos(row) * (L >> (l + 1));
 }
-__host__ __device__ inline uint64_t odd_exponent(const StageRow &s, int RO, int R0, int row, uint32_t k, uint64_t L) {
-    const uint64_t unit = L / ((uint64_t)s.R * s.P);
+__host__ __device__ inline uint64_t odd_exponent(int RO, int R0, uint64_t P, int row, uint64_t k, uint64_t L) {
+    const uint64_t RC = (uint64_t)RO * R0, unit = L / (RC * P);
     if (row < RO - 1) return (uint64_t)R0 * (row + 1) * k * unit;
     const int t = row - (RO - 1), k1 = t % RO, r = t / RO;  // level row r of the radix-R0 stage of k1
     const int l = row_level(r);
-    return (uint64_t)(R0 >> (l + 1)) * ((uint64_t)k * unit + (uint64_t)k1 * (L / s.R)) +
-           (uint64_t)row_pos(r) * (L >> (l + 1));
+    return (uint64_t)(R0 >> (l + 1)) * (k * unit + (uint64_t)k1 * (L / RC)) + (uint64_t)row_pos(r) * (L >> (l + 1));
 }
 
 // Where every table of one transform sits in its block of memory (offsets in elements).
