@@ -93,7 +93,7 @@ struct pa_plan {
     Geometry geo;  // pass split of L
     TwSet tw;      // its twiddle tables
     void *spec = nullptr;        // L complex values, seed spectrum in digit-reversed order, times 1/L
-    void *work = nullptr;        // work_pairs * L complex values
+    void *work = nullptr;        // work_pairs * L complex values, then the bit scratch of as many elements
     uint32_t work_pairs = 0;
     uint32_t max_chunk_pairs = 1;
     uint32_t *popc = nullptr;    // per key
@@ -190,6 +190,24 @@ template <typename T> cx<T> one() {
 }
 template <> cx<Zp> one<Zp>() { return 1; }
 
+int elems_per_thread(pa_dtype_t d) {
+    return d == PA_FP32_GUARD ? Shape<float>::E : d == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
+}
+
+// Values of `pairs` slots; the transposed input bits and partial popcounts of the first pass follow them.
+size_t work_bytes(const pa_plan_t *p, uint32_t pairs) { return (size_t)pairs * p->L * elem_bytes(p->dtype); }
+
+// Slots of the half-length form that fit the work memory.
+uint64_t real_slots(const pa_plan_t *p, const RealMode *r) {
+    uint64_t cap = (uint64_t)p->work_pairs * p->L / r->geo.L;
+    return cap < 1 ? 1 : cap;
+}
+
+BitScratch bit_scratch(const pa_plan_t *p, uint64_t L, uint64_t slots) {
+    return bit_scratch_at(static_cast<unsigned char *>(p->work) + work_bytes(p, p->work_pairs), L,
+                          elems_per_thread(p->dtype), slots);
+}
+
 int ensure_work(pa_plan_t *p, uint32_t pairs) {
     if (pairs <= p->work_pairs) return PA_OK;
     if (p->work) {
@@ -198,7 +216,17 @@ int ensure_work(pa_plan_t *p, uint32_t pairs) {
         p->work_pairs = 0;
         if (e != cudaSuccess) return cuda_fail(e, "cudaFree(work)");
     }
-    cudaError_t e = cudaMalloc(&p->work, (size_t)pairs * p->L * elem_bytes(p->dtype));
+    const int E = elems_per_thread(p->dtype);
+    size_t scratch = bit_scratch_bytes(p->L, E, pairs);
+    if (p->real) {
+        uint64_t slots = (uint64_t)pairs * p->L / p->real->geo.L;
+        const uint64_t N = p->real->geo.L;
+        const size_t r = bit_scratch_bytes(N, E, slots < 1 ? 1 : slots);
+        const size_t seed = bit_scratch_bytes(p->L, E, 1) + (size_t)bits_words(N, E) * sizeof(uint32_t);  // both forms' bits
+        if (r > scratch) scratch = r;
+        if (seed > scratch) scratch = seed;
+    }
+    cudaError_t e = cudaMalloc(&p->work, work_bytes(p, pairs) + scratch);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         return PA_ENOMEM;
@@ -257,34 +285,37 @@ cudaError_t round_stored(const pa_plan_t *p, cx<T> *slots, uint32_t pairs, cudaS
     return cudaSuccess;
 }
 
+// The seed's spectrum and, with a half-length form, its seed tables.
 template <typename T>
 int run_seed(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
+    // the bits of both forms of the spectrum in one launch; the second's lie behind the first's
+    const BitForm full = bit_form<T>(p->geo.lg1, p->L);
+    BitForm half = full;
+    if (p->real) half = bit_form<T>(p->real->geo.lg1, p->real->geo.L);
+    uint32_t *bits = bit_scratch(p, p->L, 1).bits, *half_bits = bits + bits_words(p->L, full.E);
+    { Timed t_(p, K_PREP, st); PA_CUDA(launch_seed_bits(seed, p->n, p->m, full, bits, p->real ? &half : nullptr, half_bits, st)); }
     const TwTab<T> tw = tw_tab<T>(p->tw.lay, p->tw.mem);
     cx<T> *W = static_cast<cx<T> *>(p->work);
     cx<T> *spec = static_cast<cx<T> *>(p->spec);
     const Geometry &g = p->geo;
-    { Timed t_(p, K_FWD_SEED, st); PA_CUDA(launch_fwd_seed<T>(g.lg1, seed, p->n, p->m, W, p->L, tw, st)); }
+    { Timed t_(p, K_FWD_SEED, st); PA_CUDA(launch_fwd<T>(g.lg1, In::SEED, seed_args<T>(bits, p->n, p->m, false, p->L), 1, W, p->L, tw, st)); }
     if (g.lgM) {
         Timed t_(p, K_MID_FWD, st);
         PA_CUDA(launch_mid<T>(g.lgM, false, W, p->L, g.inner(), 1, tw, st));
     }
     { Timed t_(p, K_MIDDLE_SPEC, st); PA_CUDA(launch_middle<T>(g.ro, g.lgI, 1, W, spec, p->L, 1, tw, spec_scale<T>(p->L), st)); }
     PA_CUDA(round_stored<T>(p, spec, 1, st));
-    return PA_OK;
-}
-
-// Seed tables of the half-length form: packed seed transform, then the bin-pair split.
-template <typename T>
-int run_seed_real(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
-    RealMode *r = p->real;
-    const TwTab<T> tw = tw_tab<T>(r->tw.lay, r->tw.mem);
-    cx<T> *W = static_cast<cx<T> *>(p->work);
-    const Geometry &g = r->geo;
-    const uint64_t N = g.L;
-    PA_CUDA(launch_fwd_seed<T>(g.lg1, seed, p->n, p->m, W, N, tw, st, true));
-    if (g.lgM) PA_CUDA(launch_mid<T>(g.lgM, false, W, N, g.inner(), 1, tw, st));
-    PA_CUDA(launch_middle_real<T>(g.ro, g.lgI, 1, W, static_cast<cx<T> *>(r->tabs), N, (uint32_t)g.lg1,
-                                  (uint32_t)g.lgM, tw, (T)(kSpecScale / (double)N), 1, st));
+    if constexpr (!std::is_same<T, Zp>::value) {
+        if (RealMode *r = p->real) {  // seed tables: packed seed transform, then the bin-pair split
+            const TwTab<T> twr = tw_tab<T>(r->tw.lay, r->tw.mem);
+            const Geometry &h = r->geo;
+            const uint64_t N = h.L;
+            PA_CUDA(launch_fwd<T>(h.lg1, In::SEED, seed_args<T>(half_bits, p->n, p->m, true, N), 1, W, N, twr, st));
+            if (h.lgM) PA_CUDA(launch_mid<T>(h.lgM, false, W, N, h.inner(), 1, twr, st));
+            PA_CUDA(launch_middle_real<T>(h.ro, h.lgI, 1, W, static_cast<cx<T> *>(r->tabs), N, (uint32_t)h.lg1,
+                                          (uint32_t)h.lgM, twr, (T)(kSpecScale / (double)N), 1, st));
+        }
+    }
     return PA_OK;
 }
 
@@ -299,15 +330,16 @@ int run_keys_real(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t k
     cx<T> *tabs = static_cast<cx<T> *>(r->tabs);
     const Geometry &g = r->geo;
     const uint64_t N = g.L;
-    uint64_t cap = (uint64_t)p->work_pairs * p->L / N;  // slots that fit the work buffer
-    if (cap < 1) cap = 1;
+    uint64_t cap = real_slots(p, r);
     if (g.lgM && cap > 65535u >> g.lg1) cap = 65535u >> g.lg1;  // grid y of the middle strided pass
-    { Timed t_(p, K_PREP, st); PA_CUDA(launch_zero_keys(nkeys, popc, marg, st)); }
     for (uint32_t k0 = 0; k0 < nkeys; k0 += (uint32_t)cap) {
         const uint32_t ns = (nkeys - k0 < cap) ? nkeys - k0 : (uint32_t)cap;
         const uint64_t *kp = keys + (uint64_t)k0 * kstride;
         uint64_t *op = out + (uint64_t)k0 * ostride;
-        { Timed t_(p, K_FWD_KEYS, st); PA_CUDA(launch_fwd_keys<T>(g.lg1, kp, ns, kstride, p->n, W, N, ns, tw, popc + k0, st, p->koff, true)); }
+        const KeyBits kb{kp, ns, ns, kstride, p->n, p->koff, true};
+        FwdArgs in;
+        { Timed t_(p, K_PREP, st); PA_CUDA(prepare_keys<T>(g.lg1, kb, N, bit_scratch(p, N, ns), popc + k0, marg + k0, st, &in)); }
+        { Timed t_(p, K_FWD_KEYS, st); PA_CUDA(launch_fwd<T>(g.lg1, In::KEYS, in, ns, W, N, tw, st)); }
         if (g.lgM) { Timed t_(p, K_MID_FWD, st); PA_CUDA(launch_mid<T>(g.lgM, false, W, N, g.inner(), ns, tw, st)); }
         { Timed t_(p, K_MIDDLE_CONV, st); PA_CUDA(launch_middle_real<T>(g.ro, g.lgI, 0, W, tabs, N, (uint32_t)g.lg1, (uint32_t)g.lgM, tw, (T)1, ns, st)); }
         if (g.lgM) { Timed t_(p, K_MID_INV, st); PA_CUDA(launch_mid<T>(g.lgM, true, W, N, g.inner(), ns, tw, st)); }
@@ -345,7 +377,6 @@ int run_keys(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstrid
     cx<T> *W = static_cast<cx<T> *>(p->work);
     cx<T> *spec = static_cast<cx<T> *>(p->spec);
     const Geometry &g = p->geo;
-    { Timed t_(p, K_PREP, st); PA_CUDA(launch_zero_keys(nkeys, popc, marg, st)); }
     const uint32_t npairs = (nkeys + 1) / 2;
     for (uint32_t p0 = 0; p0 < npairs; p0 += p->work_pairs) {
         const uint32_t pairs = (npairs - p0 < p->work_pairs) ? npairs - p0 : p->work_pairs;
@@ -353,7 +384,10 @@ int run_keys(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstrid
         const uint32_t nk = (nkeys - k0 < 2 * pairs) ? nkeys - k0 : 2 * pairs;
         const uint64_t *kp = keys + (uint64_t)k0 * kstride;
         uint64_t *op = out + (uint64_t)k0 * ostride;
-        { Timed t_(p, K_FWD_KEYS, st); PA_CUDA(launch_fwd_keys<T>(g.lg1, kp, nk, kstride, p->n, W, p->L, pairs, tw, popc + k0, st, p->koff)); }
+        const KeyBits kb{kp, nk, pairs, kstride, p->n, p->koff, false};
+        FwdArgs in;
+        { Timed t_(p, K_PREP, st); PA_CUDA(prepare_keys<T>(g.lg1, kb, p->L, bit_scratch(p, p->L, pairs), popc + k0, marg + k0, st, &in)); }
+        { Timed t_(p, K_FWD_KEYS, st); PA_CUDA(launch_fwd<T>(g.lg1, In::KEYS, in, pairs, W, p->L, tw, st)); }
         PA_CUDA(round_stored<T>(p, W, pairs, st));
         if (g.lgM) {
             { Timed t_(p, K_MID_FWD, st); PA_CUDA(launch_mid<T>(g.lgM, false, W, p->L, g.inner(), pairs, tw, st)); }
@@ -940,17 +974,12 @@ int pa_set_seed(pa_plan_t *p, const uint64_t *seed_dev, uint64_t seed_bits, pa_s
     const size_t sw = (size_t)((seed_bits + 63) / 64);
     if (!p->seed_copy) PA_CUDA(cudaMalloc(&p->seed_copy, sw * sizeof(uint64_t)));
     PA_CUDA(cudaMemcpyAsync(p->seed_copy, seed_dev, sw * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
+    if (p->real) p->real->seeded = false;
     rc = (p->dtype == PA_FP32_GUARD) ? run_seed<float>(p, p->seed_copy, st)
          : (p->dtype == PA_FP64)     ? run_seed<double>(p, p->seed_copy, st)
                                      : run_seed<Zp>(p, p->seed_copy, st);
     if (rc != PA_OK) return rc;
-    if (p->real) {
-        p->real->seeded = false;
-        rc = (p->dtype == PA_FP32_GUARD) ? run_seed_real<float>(p, p->seed_copy, st)
-                                         : run_seed_real<double>(p, p->seed_copy, st);
-        if (rc != PA_OK) return rc;
-        p->real->seeded = true;
-    }
+    if (p->real) p->real->seeded = true;
     PA_CUDA(cudaEventRecord(p->done, st));
     p->seeded = true;
     if (p->fallback) p->fallback->seeded = false;  // re-seeded lazily on the next escalation

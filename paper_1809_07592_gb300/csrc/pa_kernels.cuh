@@ -29,6 +29,7 @@
 
 #include "bulk.cuh"
 #include "fft_core.cuh"
+#include "pa_launch.h"
 
 namespace pa {
 
@@ -78,27 +79,26 @@ __device__ __forceinline__ uint32_t low_bit(double x) { return (uint32_t)__doubl
 template <typename T> struct Enc {
     using E = cx<T>;
     using M = T;  // margin accumulator
-    // Bit 30 alone is the encoding of 2.0f (and of the high
-    // word of 2.0), so a shift and a mask make the value 0 or 2. The spectra carry the factor's
-    // reciprocal (kSpecScale; with key and seed in one transform, its square): a power of
-    // two, so no rounding changes.
-    static __device__ __forceinline__ T two_if(uint32_t x, int bit) {
-        return Magic<T>::from_high((bit <= 30 ? x << (30 - bit) : x >> 1) & 0x40000000u);
+    // Bit 30 alone is the encoding of 2.0f (and of the high word of 2.0), so a shift and a mask
+    // make a key bit the value 0 or 2, and one more of each a seed bit +-2. The spectra are
+    // scaled back by kSpecScale: powers of two, so no rounding changes.
+    static __device__ __forceinline__ uint32_t two_if(uint32_t x, int bit) {
+        return (bit <= 30 ? x << (30 - bit) : x >> 1) & 0x40000000u;
     }
-    // bit j of x: key a, bit 16 + j: key b
-    static __device__ __forceinline__ E key_pair(uint32_t x, int j) {
-        return Arith<T>::mk(two_if(x, j), two_if(x, 16 + j));
+    static __device__ __forceinline__ T pm_two(uint32_t x, int bit, uint32_t in, int j) {
+        return Magic<T>::from_high(two_if(in, j) | ((x << (31 - bit)) & 0x80000000u));
     }
-    // bit j of x: key, bit 16 + j: seed; bit j of in: the seed position is inside the seed
+    // bit j of x: real part, bit 16 + j: imaginary part (key a and key b, or a key's even and odd bits)
+    static __device__ __forceinline__ E keys(uint32_t x, int j) {
+        return Arith<T>::mk(Magic<T>::from_high(two_if(x, j)), Magic<T>::from_high(two_if(x, 16 + j)));
+    }
+    // bit j of x: key, bit 16 + j: seed; bit j of in: the position is inside the seed
     static __device__ __forceinline__ E key_seed(uint32_t x, uint32_t in, int j) {
-        const uint32_t sign = (x << (15 - j)) & 0x80000000u;
-        return Arith<T>::mk(two_if(x, j), Magic<T>::from_high(((in << (30 - j)) & 0x40000000u) | sign));
+        return Arith<T>::mk(Magic<T>::from_high(two_if(x, j)), pm_two(x, 16 + j, in, j));
     }
-    static __device__ __forceinline__ E seed(bool in_range, uint32_t bit) {
-        return Arith<T>::mk(in_range ? (bit ? (T)-1 : (T)1) : (T)0, (T)0);
-    }
-    static __device__ __forceinline__ E seed_pair(bool in0, uint32_t b0, bool in1, uint32_t b1) {
-        return Arith<T>::mk(in0 ? (b0 ? (T)-1 : (T)1) : (T)0, in1 ? (b1 ? (T)-1 : (T)1) : (T)0);
+    // seed bits in both parts
+    static __device__ __forceinline__ E seed(uint32_t x, uint32_t in_re, uint32_t in_im, int j) {
+        return Arith<T>::mk(pm_two(x, j, in_re, j), pm_two(x, 16 + j, in_im, j));
     }
     // bits and margins of the two values carried by v (valid_b: the imaginary part's own range)
     static __device__ __forceinline__ void decode(E v, uint32_t popa, uint32_t popb, bool valid, bool &bit_a,
@@ -119,12 +119,12 @@ template <typename T> struct Enc {
 template <> struct Enc<Zp> {
     using E = cx<Zp>;
     using M = float;
-    static __device__ __forceinline__ E key_pair(uint32_t x, int j) {
+    static __device__ __forceinline__ E keys(uint32_t x, int j) {
         return (E)((x >> j) & 1u) | ((E)((x >> (16 + j)) & 1u) << 32);
     }
-    static __device__ __forceinline__ E seed(bool in_range, uint32_t bit) { return (in_range && bit) ? 1ull : 0ull; }
-    // (the exact transform has no half-length packing of one key: its values are not complex)
-    static __device__ __forceinline__ E seed_pair(bool, uint32_t, bool, uint32_t) { return 0ull; }
+    // (the exact transform has no half-length packing and no key+seed form: its values are not complex)
+    static __device__ __forceinline__ E seed(uint32_t x, uint32_t, uint32_t, int j) { return (E)((x >> j) & 1u); }
+    static __device__ __forceinline__ E key_seed(uint32_t, uint32_t, int) { return 0ull; }
     static __device__ __forceinline__ void decode(E v, uint32_t, uint32_t, bool valid, bool &bit_a, bool &bit_b, M &,
                                                   M &) {
         bit_a = valid && (v & 1ull);
@@ -138,35 +138,13 @@ template <> struct Enc<Zp> {
 };
 
 // ---------------------------------------------------------------------------
-// Input bits of the level-1 forward passes. Thread (tq, col) transforms the E rows
-// tq + j*TC, j < E, of column col, but a row's bits lie together in memory: lane j of a
-// group of E lanes loads the row's bits, one word for two bit vectors (low and high half),
-// and log2 E exchange steps transpose the E x E bit matrices across the group. Column c's
-// word ends in lane c, which is the thread that transforms it (E = COLS: one row group of
-// E threads; E = 2*COLS: the group's rows are those of two neighbouring tq, the second's
-// bits above the first's). No shared memory, no barrier, and every element is two
-// shift-and-mask instructions at constant positions: on rows of 256 the first pass went
-// from 859 to about 690 instructions per thread with this and the tables of tables.cuh.
-template <int E>
-__device__ __forceinline__ uint32_t transpose_bits(uint32_t x) {
-    static_assert(E == 8 || E == 16, "groups of 8 or 16 lanes");
-    const uint32_t lane = threadIdx.x & 31;
-#pragma unroll
-    for (int d = E / 2; d >= 1; d >>= 1) {
-        // bit positions whose index has bit d clear, in both halves
-        const uint32_t m = d == 8 ? 0x00FF00FFu : d == 4 ? 0x0F0F0F0Fu : d == 2 ? 0x33333333u : 0x55555555u;
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
-        x = (lane & d) ? ((x & ~m) | ((y >> d) & m)) : ((x & m) | ((y & m) << d));
-    }
-    return x;
-}
-// Rows (and their bit offset in the group word) that this lane loads: row(0), and row(1) when E = 2*COLS.
-template <int LEN, int COLS, int E>
-__device__ __forceinline__ uint32_t lane_row(int h) {
-    static_assert(E == COLS || E == 2 * COLS, "one or two rows per lane");
-    const uint32_t unit = threadIdx.x / E, j = threadIdx.x % E;
-    return (E == COLS ? unit : 2 * unit + (uint32_t)h) + j * (uint32_t)(LEN / E);
-}
+// Input bits of the level-1 forward passes. Thread (tq, col) of column block blk transforms the
+// rows tq + j*TC, j < E, of column blk*COLS + col, whose bits lie E/32 of a row apart in memory:
+// a CTA would touch LEN lines for LEN words of 16 bits each (32 wavefronts per load and warp). The
+// bits are therefore transposed once, by k_key_bits and its kin (pa_prep.cu), into one 32-bit word per thread:
+// bit j: the real part's bit of row j, bit 16 + j: the imaginary part's, word (blk, tq, col) of a
+// slot in thread order, so a pass reads one coalesced word per thread and makes every element
+// with two shift-and-mask instructions at constant positions.
 // Position j of the row of register slot s (elem_of): row = tq + j*TC.
 template <typename T, int LEN, int E>
 constexpr int slot_pos(int s) {
@@ -200,15 +178,7 @@ __device__ __forceinline__ void cta_reduce_get(uint32_t &a, uint32_t &b, const u
 }
 
 // Single keys in half-length transforms: transform element t carries key bits 2t
-// (real part) and 2t+1 (imaginary part). even_bits gathers the even-position bits of
-// x into the low 16 bits; spread_bits is its inverse (low 16 bits to even positions).
-__device__ __forceinline__ uint32_t even_bits(uint32_t x) {
-    x &= 0x55555555u;
-    x = (x | (x >> 1)) & 0x33333333u;
-    x = (x | (x >> 2)) & 0x0F0F0F0Fu;
-    x = (x | (x >> 4)) & 0x00FF00FFu;
-    return (x | (x >> 8)) & 0x0000FFFFu;
-}
+// (real part) and 2t+1 (imaginary part). spread_bits moves the low 16 bits of x to the even positions.
 __device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
     x &= 0x0000FFFFu;
     x = (x | (x << 8)) & 0x00FF00FFu;
@@ -242,112 +212,60 @@ __device__ __forceinline__ uint32_t bits_at(const uint64_t *v, uint64_t nbits, u
 }
 
 // ---------------------------------------------------------------------------
-// Level-1 forward pass from packed key bits. Grid (S/COLS, pairs); pair p
-// carries key 2p in the real part and key 2p+1 (if any) in the imaginary part.
-// PACK: slot p carries one key, p, in a half-length transform: element t is key
-// bits 2t (real part) and 2t+1 (imaginary part).
-template <typename T, int LEN, int COLS, int E, bool PACK = false>
+// Level-1 forward pass from transposed bits. Grid (S/COLS, slots). KEYS: slot p holds keys 2p
+// and 2p+1 (or, one key per slot, its even and odd bits); SEED: the rotated, +-1 encoded seed in
+// the real part (or its even and odd positions); BLOCKS: block p's key and rotated seed.
+// The slot's first CTA also adds up the popcounts the transposition left per part: popc[p * ppk] (+1 for the
+// imaginary part's key; ppk = 1: both parts are one key's), or popc[block id].
+template <typename T, int LEN, int COLS, int E, In KIND>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
-    k_fwd_keys(const uint64_t *__restrict__ keys, uint32_t nkeys, uint64_t kstride, uint64_t n,
-               cx<T> *__restrict__ W, uint64_t L, TwTab<T> tw, uint32_t *__restrict__ popc, uint64_t koff) {
+    k_fwd(FwdArgs in, cx<T> *__restrict__ W, uint64_t L, TwTab<T> tw) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
-    const uint64_t S = L >> ilog2(LEN);
-    const uint64_t u = (uint64_t)blockIdx.x * COLS + col;
-    const uint32_t pair = blockIdx.y;
-    const bool has_b = 2 * pair + 1 < nkeys;
-    const uint64_t u0 = (uint64_t)blockIdx.x * COLS;
-    // The transform's input element t is key bit koff + t (koff = 0, or m for the modified
-    // Toeplitz hash, whose Toeplitz block multiplies key bits m .. n-1).
-    const uint64_t nk = n + koff;
-    const bool aligned = (koff % COLS) == 0;
-    const uint64_t *xa = keys + (uint64_t)(PACK ? pair : 2 * pair) * kstride, *xb = xa + kstride;
-    uint32_t xa_bits = 0u, xb_bits = 0u;  // this lane's share of the two bit matrices
-#pragma unroll
-    for (int h = 0; h < E / COLS; ++h) {
-        const uint64_t r0 = (uint64_t)lane_row<LEN, COLS, E>(h) * S + u0;  // S % 64 == 0: aligned COLS bits sit in one word
-        uint32_t wa, wb = 0u;
-        if constexpr (PACK) {  // 2*COLS key bits from 2*(a*S + u0): the even ones real, the odd ones imaginary
-            const uint32_t c = bits_at(xa, nk, 2 * r0 + koff, 2 * COLS);
-            wa = even_bits(c);
-            wb = even_bits(c >> 1);
-        } else if (aligned) {
-            wa = aligned_bits<COLS>(xa, nk, r0 + koff);
-            if (has_b) wb = aligned_bits<COLS>(xb, nk, r0 + koff);
-        } else {
-            wa = bits_at(xa, nk, r0 + koff, COLS);
-            if (has_b) wb = bits_at(xb, nk, r0 + koff, COLS);
-        }
-        xa_bits |= wa << (h * COLS);
-        xb_bits |= wb << (h * COLS);
-    }
-    __shared__ uint32_t red[64];
-    uint32_t ca = __popc(xa_bits), cb = __popc(xb_bits);  // the CTA's share of each key's popcount P (the CTAs tile every bit once)
-    cta_reduce_put<false>(ca, cb, red);
-    const uint32_t x = transpose_bits<E>(xa_bits | (xb_bits << 16));
+    const uint32_t S = (uint32_t)(L >> ilog2(LEN)), u = blockIdx.x * COLS + col;
+    const uint32_t x = __ldg(in.bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
     cx<T> v[E];
+    if constexpr (KIND == In::KEYS) {
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_pair(x, slot_pos<T, LEN, E>(s));
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
-    cta_reduce_get<false>(ca, cb, red);  // behind the transform's barriers
-    if (threadIdx.x == 0 && (ca | cb)) {
-        if (PACK) {
-            atomicAdd(popc + pair, ca + cb);
-        } else {
-            if (ca) atomicAdd(popc + 2 * pair, ca);
-            if (cb) atomicAdd(popc + 2 * pair + 1, cb);
-        }
+        for (int s = 0; s < E; ++s) v[s] = Enc<T>::keys(x, slot_pos<T, LEN, E>(s));
+    } else if constexpr (KIND == In::SEED) {
+        const uint32_t re = in.re.mask(tq * S + u), im = in.im.mask(tq * S + u);
+#pragma unroll
+        for (int s = 0; s < E; ++s) v[s] = Enc<T>::seed(x, re, im, slot_pos<T, LEN, E>(s));
+    } else {
+        const uint32_t inside = in.blocks[blockIdx.y].in.mask(tq * S + u);
+#pragma unroll
+        for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, inside, slot_pos<T, LEN, E>(s));
     }
-    cx<T> *w = W + (uint64_t)pair * L;
+    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
     const uint32_t f = freq_of<T, LEN, E>(tq);
     pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
+    cx<T> *w = W + (uint64_t)blockIdx.y * L + u;
 #pragma unroll
-    for (int s = 0; s < E; ++s) w[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
-}
-
-// Level-1 forward pass of the rotated, +-1 encoded seed (real input). PACK: the
-// seed of a length-2L convolution in a length-L transform, element t carrying
-// rotated positions 2t (real part) and 2t+1 (imaginary part).
-template <typename T, int LEN, int COLS, int E, bool PACK = false>
-__global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
-    k_fwd_seed(const uint64_t *__restrict__ seed, uint64_t n, uint64_t m, cx<T> *__restrict__ W, uint64_t L,
-               TwTab<T> tw) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
-    const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
-    const uint64_t S = L >> ilog2(LEN);
-    const uint64_t u = (uint64_t)blockIdx.x * COLS + col;
-    const uint64_t sbits = n + m - 1;
-    cx<T> v[E];
-#pragma unroll
-    for (int s = 0; s < E; ++s) {
-        const uint64_t pos = (uint64_t)elem_of<T, LEN, E>(tq, s) * S + u;
-        if constexpr (PACK) {
-            const uint64_t L2 = 2 * L;
-            uint32_t bit[2];
-            bool in_range[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                uint64_t j = 2 * pos + h + n - 1;  // seed index at rotated position 2*pos + h
-                if (j >= L2) j -= L2;
-                in_range[h] = j < sbits;
-                bit[h] = in_range[h] ? (uint32_t)(__ldg(seed + (j >> 6)) >> (j & 63)) & 1u : 0u;
+    for (int s = 0; s < E; ++s) w[(f + s * (LEN / E)) * S] = v[s];
+    if constexpr (KIND != In::SEED) {
+        if (blockIdx.x == 0 && threadIdx.x < 32) {
+            uint32_t ca = 0, cb = 0;
+            for (uint32_t i = threadIdx.x; i < in.nparts; i += 32) {
+                const uint2 c = in.parts[(uint64_t)blockIdx.y * in.nparts + i];
+                ca += c.x;
+                cb += c.y;
             }
-            v[s] = Enc<T>::seed_pair(in_range[0], bit[0], in_range[1], bit[1]);
-        } else {
-            uint64_t j = pos + n - 1;  // seed index whose value sits at rotated position pos
-            if (j >= L) j -= L;
-            const bool in_range = j < sbits;
-            const uint32_t bit = in_range ? (uint32_t)(__ldg(seed + (j >> 6)) >> (j & 63)) & 1u : 0u;
-            v[s] = Enc<T>::seed(in_range, bit);
+            ca = __reduce_add_sync(0xffffffffu, ca);
+            cb = __reduce_add_sync(0xffffffffu, cb);
+            if (threadIdx.x == 0) {
+                if constexpr (KIND == In::BLOCKS) {
+                    in.popc[in.blocks[blockIdx.y].id] = ca;
+                } else if (in.ppk == 1) {
+                    in.popc[blockIdx.y] = ca + cb;
+                } else {
+                    in.popc[2 * blockIdx.y] = ca;
+                    if (2 * blockIdx.y + 1 < in.nkeys) in.popc[2 * blockIdx.y + 1] = cb;
+                }
+            }
         }
     }
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
-    const uint32_t f = freq_of<T, LEN, E>(tq);
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
-#pragma unroll
-    for (int s = 0; s < E; ++s) W[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
 }
 
 // Middle-level strided pass (three-level plans only), forward or inverse.
@@ -720,72 +638,6 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
 // sends two blocks' products through one inverse transform as Y1 + i*Y2.
 // ===========================================================================
 namespace pa {
-
-// Device-side block descriptor.
-struct BlockDev {
-    uint64_t n, m;
-    const uint64_t *key;   // ceil(n/64) words
-    const uint64_t *seed;  // ceil((n+m-1)/64) words
-    uint64_t *out;         // ceil(m/64) words
-    uint32_t id;           // index of the block in the caller's list (popcount / margin slot)
-    uint32_t pad;
-};
-
-// Level-1 forward pass of z = x + i*sigma for every block of a class. Grid (S/COLS, blocks).
-template <typename T, int LEN, int COLS, int E>
-__global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
-    k_fwd_keyseed(const BlockDev *__restrict__ blocks, cx<T> *__restrict__ W, uint64_t L, TwTab<T> tw,
-                  uint32_t *__restrict__ popc) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
-    const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
-    const uint64_t S = L >> ilog2(LEN);
-    const uint64_t u = (uint64_t)blockIdx.x * COLS + col;
-    const BlockDev bd = blocks[blockIdx.y];
-    const uint64_t n = bd.n, sbits = bd.n + bd.m - 1;
-    // per row: the CTA's COLS key bits (aligned), COLS seed bits at the rotated
-    // position j = a*S + u0 + n - 1 (mod L; the window may wrap past L) and the mask
-    // of window positions inside the seed (past it the value is 0, not +-1)
-    const uint64_t u0 = (uint64_t)blockIdx.x * COLS;
-    const uint32_t full = (1u << COLS) - 1u;
-    uint32_t kbits = 0u, sbit = 0u, inbits = 0u;
-#pragma unroll
-    for (int h = 0; h < E / COLS; ++h) {
-        const uint64_t t0 = (uint64_t)lane_row<LEN, COLS, E>(h) * S + u0;
-        const uint32_t wk = aligned_bits<COLS>(bd.key, n, t0);
-        uint64_t j0 = t0 + n - 1;
-        if (j0 >= L) j0 -= L;
-        uint32_t ws, inr;
-        if (j0 + COLS <= L) {
-            ws = bits_at(bd.seed, sbits, j0, COLS);
-            inr = j0 >= sbits ? 0u : (sbits - j0 >= COLS ? full : (1u << (sbits - j0)) - 1u);
-        } else {  // positions j0 .. L-1, then 0 .. COLS-c1-1 (wrapped)
-            const uint32_t c1 = (uint32_t)(L - j0);
-            ws = bits_at(bd.seed, sbits, j0, c1) | (bits_at(bd.seed, sbits, 0, COLS - c1) << c1);
-            const uint32_t lo = j0 >= sbits ? 0u : (sbits - j0 >= c1 ? (1u << c1) - 1u : (1u << (sbits - j0)) - 1u);
-            const uint32_t nw = sbits >= COLS - c1 ? COLS - c1 : (uint32_t)sbits;  // wrapped positions inside the seed
-            inr = lo | (((1u << nw) - 1u) << c1);
-        }
-        kbits |= wk << (h * COLS);
-        sbit |= ws << (h * COLS);
-        inbits |= inr << (h * COLS);
-    }
-    uint32_t ck = __popc(kbits), unused = 0u;  // the CTA's share of the key's popcount P (the CTAs tile every bit once)
-    __shared__ uint32_t red[64];
-    cta_reduce_put<false>(ck, unused, red);
-    const uint32_t x = transpose_bits<E>(kbits | (sbit << 16)), in = transpose_bits<E>(inbits);
-    cx<T> v[E];
-#pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, in, slot_pos<T, LEN, E>(s));
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
-    cta_reduce_get<false>(ck, unused, red);  // behind the transform's barriers
-    if (threadIdx.x == 0 && ck) atomicAdd(popc + bd.id, ck);
-    cx<T> *w = W + (uint64_t)blockIdx.y * L;
-    const uint32_t f = freq_of<T, LEN, E>(tq);
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
-#pragma unroll
-    for (int s = 0; s < E; ++s) w[(uint64_t)(f + s * (LEN / E)) * S + u] = v[s];
-}
 
 // Storage row of the frequency low part rho (lgM = log2 of the middle strided
 // pass length, 0 for two-level plans): rho = k1 + L1*k2 sits at row k1*M + k2.

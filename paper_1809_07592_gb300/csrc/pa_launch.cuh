@@ -42,58 +42,30 @@ static cudaError_t by_len(int lg, F &&f) {
     }
 }
 
-template <typename T, int LEN, bool PACK>
-cudaError_t fwd_keys_at(const uint64_t *keys, uint32_t nkeys, uint64_t kstride, uint64_t n, cx<T> *W, uint64_t L,
-                        uint32_t pairs, TwTab<T> tw, uint32_t *popc, cudaStream_t st, uint64_t koff) {
+template <typename T, int LEN, In KIND>
+cudaError_t fwd_at(const FwdArgs &in, uint32_t slots, cx<T> *W, uint64_t L, TwTab<T> tw, cudaStream_t st) {
     constexpr int E = Shape<T>::E, COLS = strided_cols<T, LEN>();
-    auto kern = k_fwd_keys<T, LEN, COLS, E, PACK>;
+    auto kern = k_fwd<T, LEN, COLS, E, KIND>;
     constexpr size_t sb = smem_bytes<T, LEN, COLS>();
     cudaError_t e = set_smem(kern, sb);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((L / LEN) / COLS), pairs);
-    kern<<<grid, COLS * LEN / E, sb, st>>>(keys, nkeys, kstride, n, W, L, tw, popc, koff);
+    dim3 grid((unsigned)((L / LEN) / COLS), slots);
+    kern<<<grid, COLS * LEN / E, sb, st>>>(in, W, L, tw);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_fwd_keys(int lgLEN, const uint64_t *keys, uint32_t nkeys, uint64_t kstride, uint64_t n,
-                            cx<T> *W, uint64_t L, uint32_t pairs, TwTab<T> tw, uint32_t *popc, cudaStream_t st,
-                            uint64_t koff, bool pack) {
+cudaError_t launch_fwd(int lgLEN, In kind, const FwdArgs &in, uint32_t slots, cx<T> *W, uint64_t L, TwTab<T> tw,
+                       cudaStream_t st) {
     return by_len<kMinLgStrided, kMaxLgStrided>(lgLEN, [&](auto c) {
         constexpr int LEN = decltype(c)::value;
-        if constexpr (!std::is_same<T, Zp>::value) {
-            if (pack) return fwd_keys_at<T, LEN, true>(keys, nkeys, kstride, n, W, L, pairs, tw, popc, st, koff);
+        if (kind == In::KEYS) return fwd_at<T, LEN, In::KEYS>(in, slots, W, L, tw, st);
+        if (kind == In::SEED) return fwd_at<T, LEN, In::SEED>(in, slots, W, L, tw, st);
+        if constexpr (!std::is_same<T, Zp>::value) {  // residues have no key+seed form
+            return fwd_at<T, LEN, In::BLOCKS>(in, slots, W, L, tw, st);
         } else {
-            if (pack) return cudaErrorInvalidValue;  // the exact transform has no half-length packing
+            return cudaErrorInvalidValue;
         }
-        return fwd_keys_at<T, LEN, false>(keys, nkeys, kstride, n, W, L, pairs, tw, popc, st, koff);
-    });
-}
-
-template <typename T, int LEN, bool PACK>
-cudaError_t fwd_seed_at(const uint64_t *seed, uint64_t n, uint64_t m, cx<T> *W, uint64_t L, TwTab<T> tw,
-                        cudaStream_t st) {
-    constexpr int E = Shape<T>::E, COLS = strided_cols<T, LEN>();
-    auto kern = k_fwd_seed<T, LEN, COLS, E, PACK>;
-    constexpr size_t sb = smem_bytes<T, LEN, COLS>();
-    cudaError_t e = set_smem(kern, sb);
-    if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((L / LEN) / COLS), 1);
-    kern<<<grid, COLS * LEN / E, sb, st>>>(seed, n, m, W, L, tw);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_fwd_seed(int lgLEN, const uint64_t *seed, uint64_t n, uint64_t m, cx<T> *W, uint64_t L,
-                            TwTab<T> tw, cudaStream_t st, bool pack) {
-    return by_len<kMinLgStrided, kMaxLgStrided>(lgLEN, [&](auto c) {
-        constexpr int LEN = decltype(c)::value;
-        if constexpr (!std::is_same<T, Zp>::value) {
-            if (pack) return fwd_seed_at<T, LEN, true>(seed, n, m, W, L, tw, st);
-        } else {
-            if (pack) return cudaErrorInvalidValue;
-        }
-        return fwd_seed_at<T, LEN, false>(seed, n, m, W, L, tw, st);
     });
 }
 
@@ -278,11 +250,8 @@ cudaError_t launch_inv_bits(int lgLEN, const cx<T> *W, uint64_t L, uint64_t m, u
 }
 
 #define PA_INSTANTIATE_LAUNCHERS(T)                                                                              \
-    template cudaError_t launch_fwd_keys<T>(int, const uint64_t *, uint32_t, uint64_t, uint64_t, cx<T> *,        \
-                                            uint64_t, uint32_t, TwTab<T>, uint32_t *, cudaStream_t, uint64_t,    \
-                                            bool);                                                               \
-    template cudaError_t launch_fwd_seed<T>(int, const uint64_t *, uint64_t, uint64_t, cx<T> *, uint64_t,        \
-                                            TwTab<T>, cudaStream_t, bool);                                       \
+    template cudaError_t launch_fwd<T>(int, In, const FwdArgs &, uint32_t, cx<T> *, uint64_t, TwTab<T>,          \
+                                       cudaStream_t);                                                            \
     template cudaError_t launch_mid<T>(int, bool, cx<T> *, uint64_t, uint32_t, uint32_t, TwTab<T>,               \
                                        cudaStream_t);                                                           \
     template cudaError_t launch_middle<T>(int, int, int, cx<T> *, cx<T> *, uint64_t, uint32_t, TwTab<T>, cx<T>,  \
@@ -290,23 +259,6 @@ cudaError_t launch_inv_bits(int lgLEN, const cx<T> *W, uint64_t L, uint64_t m, u
     template cudaError_t launch_inv_bits<T>(int, const cx<T> *, uint64_t, uint64_t, uint32_t, const uint32_t *,  \
                                             uint32_t *, uint64_t *, uint64_t, uint32_t, TwTab<T>, cudaStream_t,  \
                                             const uint64_t *, uint64_t, bool, uint32_t *, uint32_t);
-
-template <typename T>
-cudaError_t launch_fwd_keyseed(int lgLEN, const BlockDev *blocks, uint32_t nblocks, cx<T> *W, uint64_t L,
-                               TwTab<T> tw, uint32_t *popc, cudaStream_t st) {
-    constexpr int E = Shape<T>::E;
-    return by_len<kMinLgStrided, kMaxLgStrided>(lgLEN, [&](auto c) {
-        constexpr int LEN = decltype(c)::value;
-        constexpr int COLS = strided_cols<T, LEN>();
-        auto kern = k_fwd_keyseed<T, LEN, COLS, E>;
-        constexpr size_t sb = smem_bytes<T, LEN, COLS>();
-        cudaError_t e = set_smem(kern, sb);
-        if (e != cudaSuccess) return e;
-        dim3 grid((unsigned)((L / LEN) / COLS), nblocks);
-        kern<<<grid, COLS * LEN / E, sb, st>>>(blocks, W, L, tw, popc);
-        return cudaGetLastError();
-    });
-}
 
 template <typename T, int LEN>
 cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1, uint32_t lgM,
@@ -319,7 +271,7 @@ cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, u
     const uint32_t R = (uint32_t)(L / LEN);
     dim3 grid(R / 2 + 1, (nblocks + 1) / 2);
     kern<<<grid, 2 * (LEN / E), sb, st>>>(Wf, Wi, L, nblocks, lgL1, lgM, tw,
-                                         (T)(kSpecScale * kSpecScale / (double)L));
+                                         (T)(kSpecScale / (double)L));
     return cudaGetLastError();
 }
 
@@ -378,8 +330,6 @@ cudaError_t launch_inv_bits_blocks(int lgLEN, const cx<T> *Wi, uint64_t L, const
 }
 
 #define PA_INSTANTIATE_UNEVEN(T)                                                                                 \
-    template cudaError_t launch_fwd_keyseed<T>(int, const BlockDev *, uint32_t, cx<T> *, uint64_t, TwTab<T>,     \
-                                               uint32_t *, cudaStream_t);                                       \
     template cudaError_t launch_middle_split<T>(int, int, const cx<T> *, cx<T> *, uint64_t, uint32_t, uint32_t,  \
                                                 uint32_t, TwTab<T>, cudaStream_t);                               \
     template cudaError_t launch_inv_bits_blocks<T>(int, const cx<T> *, uint64_t, const BlockDev *, uint32_t,     \

@@ -48,8 +48,8 @@ TwTab<T> tw_tab(const TwLayout &y, const void *mem) {
     return t;
 }
 
-// The complex passes take key bits as 0 / 2 (Enc in pa_kernels.cuh); spectra are scaled back by this.
-constexpr double kSpecScale = 0.5;
+// The complex passes take key bits as 0 / 2 and seed bits as +-2 (Enc in pa_kernels.cuh); products are scaled back by this.
+constexpr double kSpecScale = 0.25;
 
 // Supported pass lengths (log2).
 constexpr int kMinLgStrided = 6, kMaxLgStrided = 10;
@@ -59,25 +59,142 @@ template <> struct MaxLgMiddle<double> { static constexpr int v = 13; };
 template <> struct MaxLgMiddle<Zp> { static constexpr int v = 13; };
 constexpr int kMinLgMiddle = 6;
 
-// Zero the per-key popcounts and margins of a batch (the level-1 forward pass accumulates the popcounts).
-cudaError_t launch_zero_keys(uint32_t nkeys, uint32_t *popc, uint32_t *margin_bits, cudaStream_t st);
+// Which elements of a rotated seed are inside the seed: element t holds a seed value iff t < M or
+// t >= Z. For a thread's elements x + j*D (D = L / E, x < D), j < E, that is j < M/D + (x < M%D) or
+// j >= Z/D + (x < Z%D).
+struct SeedRange {
+    uint32_t mq, mr, zq, zr;
+    __host__ __device__ SeedRange() : mq(0), mr(0), zq(0), zr(0) {}
+    __host__ __device__ SeedRange(uint64_t M, uint64_t Z, uint64_t D)
+        : mq((uint32_t)(M / D)), mr((uint32_t)(M % D)), zq((uint32_t)(Z / D)), zr((uint32_t)(Z % D)) {}
+    __device__ __forceinline__ uint32_t mask(uint32_t x) const {
+        const uint32_t below = (1u << (mq + (x < mr))) - 1u, from = (1u << (zq + (x < zr))) - 1u;  // both counts <= 16
+        return below | ~from;
+    }
+};
+
+// Device-side block descriptor of the uneven batch.
+struct BlockDev {
+    uint64_t n, m;
+    const uint64_t *key;   // ceil(n/64) words
+    const uint64_t *seed;  // ceil((n+m-1)/64) words
+    uint64_t *out;         // ceil(m/64) words
+    uint32_t id;           // index of the block in the caller's list (popcount / margin slot)
+    uint32_t pad;
+    SeedRange in;          // seed window of the block in its class's transform
+};
+
+// Scratch of the level-1 forward passes: transposed input bits (bits_words per slot) and partial
+// popcounts (parts_count per slot).
+struct BitScratch {
+    uint32_t *bits = nullptr;
+    uint2 *parts = nullptr;
+};
+inline uint64_t bits_words(uint64_t L, int E) { return L / (uint64_t)E; }
+constexpr uint32_t kBitThreads = 128;  // threads of a transposition CTA, 16 columns of E rows each
+inline uint64_t parts_count(uint64_t L, int E) { return (L / 16 / (uint64_t)E + kBitThreads - 1) / kBitThreads; }
+// Bytes of scratch for `slots` slots, parts first.
+inline size_t bit_scratch_bytes(uint64_t L, int E, uint64_t slots) {
+    return (size_t)((parts_count(L, E) * slots * sizeof(uint2) + 255) / 256 * 256 + bits_words(L, E) * slots * sizeof(uint32_t));
+}
+inline BitScratch bit_scratch_at(void *mem, uint64_t L, int E, uint64_t slots) {
+    BitScratch b;
+    b.parts = static_cast<uint2 *>(mem);
+    b.bits = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(mem) +
+                                          (parts_count(L, E) * slots * sizeof(uint2) + 255) / 256 * 256);
+    return b;
+}
+
+// Keys of a batch: slot p holds keys 2p (real part) and 2p+1, if any (imaginary part), or, with
+// pack, key p's even and odd bits (a half-length transform). The transform input is key bits
+// koff .. koff+n-1 (koff = m for the modified Toeplitz hash).
+struct KeyBits {
+    const uint64_t *keys = nullptr;
+    uint32_t nkeys = 0, slots = 0;
+    uint64_t kstride = 0, n = 0, koff = 0;
+    bool pack = false;
+};
+
+// The first pass whose bits are transposed: length 2^lgLEN of a length-L transform, E values per
+// thread, cols columns per CTA.
+struct BitForm {
+    uint64_t L;
+    int lgLEN, E, cols;
+};
+template <typename T>
+BitForm bit_form(int lgLEN, uint64_t L) {
+    return BitForm{L, lgLEN, Shape<T>::E, strided_cols_of(std::is_same<T, float>::value, 1 << lgLEN)};
+}
+
+// Transpose input bits (layout: see "Input bits" in pa_kernels.cuh). The key forms also leave
+// partial popcounts (*nparts per slot) and zero the margins of their keys (blocks: margin_bits[id]).
+cudaError_t launch_key_bits(const KeyBits &k, const BitForm &f, BitScratch scratch, uint32_t *margin_bits,
+                            uint32_t *nparts, cudaStream_t st);
+// packed (or null): also for the half-length form, a length-packed->L transform whose element t holds
+// rotated positions 2t and 2t+1.
+cudaError_t launch_seed_bits(const uint64_t *seed, uint64_t n, uint64_t m, const BitForm &f, uint32_t *out,
+                             const BitForm *packed, uint32_t *packed_out, cudaStream_t st);
+cudaError_t launch_block_bits(const BlockDev *blocks, uint32_t nblocks, const BitForm &f, BitScratch scratch,
+                              uint32_t *margin_bits, uint32_t *nparts, cudaStream_t st);
 
 // Round x[0 .. count) in place to `bits` explicit significand bits (1 <= bits <= 22; other
 // values leave x as it is): the storage-precision study of pa_plan_set_storage_bits.
 cudaError_t launch_round_significand(float *x, uint64_t count, uint32_t bits, cudaStream_t st);
 
-// Level-1 forward pass of key pairs; also adds each key's popcount into popc[k]
-// (which must be zero beforehand: launch_zero_keys). The transform input is key
-// bits koff .. koff+n-1 (koff = m for the modified Toeplitz hash).
-// pack: one key per slot in a half-length transform (element t = key bits 2t, 2t+1).
+// What the level-1 forward pass transforms: slots of keys, a seed, or the blocks of a class. The pass
+// also adds up the partial popcounts of its slots: popc[slot * ppk] (+1 for the imaginary part's
+// key; ppk = 1: both parts are one key's), or popc[id] of a block.
+enum class In { KEYS, SEED, BLOCKS };
+struct FwdArgs {
+    const uint32_t *bits;   // L / E words per slot
+    const uint2 *parts;     // popcounts (real, imaginary part): nparts per slot
+    uint32_t nparts, ppk, nkeys;
+    uint32_t *popc;
+    SeedRange re, im;       // SEED
+    const BlockDev *blocks; // BLOCKS
+};
 template <typename T>
-cudaError_t launch_fwd_keys(int lgLEN, const uint64_t *keys, uint32_t nkeys, uint64_t kstride, uint64_t n,
-                            cx<T> *W, uint64_t L, uint32_t pairs, TwTab<T> tw, uint32_t *popc, cudaStream_t st,
-                            uint64_t koff = 0, bool pack = false);
-// pack: the seed of a length-2L convolution in a length-L transform (positions 2t, 2t+1).
+cudaError_t launch_fwd(int lgLEN, In kind, const FwdArgs &in, uint32_t slots, cx<T> *W, uint64_t L, TwTab<T> tw,
+                       cudaStream_t st);
+
+// Transpose the bits of keys or blocks for launch_fwd, which takes *in.
 template <typename T>
-cudaError_t launch_fwd_seed(int lgLEN, const uint64_t *seed, uint64_t n, uint64_t m, cx<T> *W, uint64_t L,
-                            TwTab<T> tw, cudaStream_t st, bool pack = false);
+cudaError_t prepare_keys(int lgLEN, const KeyBits &k, uint64_t L, BitScratch scratch, uint32_t *popc,
+                         uint32_t *margin_bits, cudaStream_t st, FwdArgs *in) {
+    *in = FwdArgs();
+    in->bits = scratch.bits;
+    in->parts = scratch.parts;
+    in->ppk = k.pack ? 1 : 2;
+    in->nkeys = k.nkeys;
+    in->popc = popc;
+    return launch_key_bits(k, bit_form<T>(lgLEN, L), scratch, margin_bits, &in->nparts, st);
+}
+template <typename T>
+cudaError_t prepare_blocks(int lgLEN, const BlockDev *blocks, uint32_t nblocks, uint64_t L, BitScratch scratch,
+                           uint32_t *popc, uint32_t *margin_bits, cudaStream_t st, FwdArgs *in) {
+    *in = FwdArgs();
+    in->bits = scratch.bits;
+    in->parts = scratch.parts;
+    in->popc = popc;
+    in->blocks = blocks;
+    return launch_block_bits(blocks, nblocks, bit_form<T>(lgLEN, L), scratch, margin_bits, &in->nparts, st);
+}
+// The first pass's input from transposed seed bits. Rotated position t holds seed bit t + n - 1 (mod
+// the cyclic length): a seed value for t < m or t > length - n.
+template <typename T>
+FwdArgs seed_args(const uint32_t *bits, uint64_t n, uint64_t m, bool pack, uint64_t L) {
+    FwdArgs in{};
+    in.bits = bits;
+    const uint64_t D = L / Shape<T>::E;
+    if (pack) {
+        in.re = SeedRange((m + 1) / 2, (2 * L - n + 2) / 2, D);
+        in.im = SeedRange(m / 2, (2 * L - n + 1) / 2, D);
+    } else {
+        in.re = SeedRange(m, L - n + 1, D);
+        in.im = SeedRange(0, L, D);
+    }
+    return in;
+}
 // S: innermost length (the stride of the middle strided pass).
 template <typename T>
 cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S, uint32_t pairs, TwTab<T> tw,
@@ -120,17 +237,10 @@ bool encode_tile_map(CUtensorMap *map, const void *base, uint64_t cols, uint64_t
                      uint32_t box_rows);
 
 // ---- uneven batch (complex arithmetic only: the Eq. 5-10 split needs conjugation) ----
-struct BlockDev;
 template <typename T> struct MaxLgSplit;
 template <> struct MaxLgSplit<float> { static constexpr int v = 13; };
 template <> struct MaxLgSplit<double> { static constexpr int v = 12; };
 
-// Zero popc[id] and margin_bits[id] of every block (launch_fwd_keyseed accumulates the popcounts).
-cudaError_t launch_zero_blocks(const BlockDev *blocks, uint32_t nblocks, uint32_t *popc, uint32_t *margin_bits,
-                               cudaStream_t st);
-template <typename T>
-cudaError_t launch_fwd_keyseed(int lgLEN, const BlockDev *blocks, uint32_t nblocks, cx<T> *W, uint64_t L,
-                               TwTab<T> tw, uint32_t *popc, cudaStream_t st);
 template <typename T>
 cudaError_t launch_middle_split(int ro, int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks,
                                 uint32_t lgL1, uint32_t lgM, TwTab<T> tw, cudaStream_t st);

@@ -114,7 +114,10 @@ int launch_batch(pa_server_t *s, Slot &sl) {
     size_t off_cnt = 0;
     size_t off_desc = align256(2 * (size_t)nb * sizeof(uint32_t));
     size_t total = off_desc + align256((size_t)nb * sizeof(BlockDev));
-    std::vector<std::pair<size_t, size_t>> work_off;  // (Wf, Wi) offsets per class
+    struct WorkOff {
+        size_t wf, wi, bits;
+    };
+    std::vector<WorkOff> work_off;  // per class
     for (auto &kv : byL) {
         const size_t L = (size_t)kv.first;
         const size_t k = kv.second.size();
@@ -122,7 +125,9 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         total += align256(k * L * esz);
         const size_t wi = total;
         total += align256(((k + 1) / 2) * L * esz);
-        work_off.push_back({wf, wi});
+        const size_t bits = total;
+        total += align256(pa::blocks::class_bit_bytes(L, s->cfg.dtype, k));
+        work_off.push_back({wf, wi, bits});
     }
     unsigned char *mem = nullptr;
     cudaError_t e = cudaMallocFromPoolAsync((void **)&mem, total, s->pool, sl.st);
@@ -137,7 +142,7 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         class_first.push_back(pos);
         for (uint32_t i : kv.second) {
             const pa_block_desc_t &d = sl.reqs[i].d;
-            sl.h_desc[pos++] = BlockDev{d.n, d.m, d.key, d.seed, d.out, i, 0u};
+            sl.h_desc[pos++] = pa::blocks::block_dev(d, i, kv.first, s->cfg.dtype);
         }
     }
     int rc = PA_OK;
@@ -152,8 +157,9 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         if (rc != PA_OK) break;
         c.d_blocks = d_desc + class_first[ci];
         c.nb = (uint32_t)kv.second.size();
-        c.Wf = mem + work_off[ci].first;
-        c.Wi = mem + work_off[ci].second;
+        c.Wf = mem + work_off[ci].wf;
+        c.Wi = mem + work_off[ci].wi;
+        c.bits = mem + work_off[ci].bits;
         rc = pa::blocks::run_complex(s->cfg.dtype, c, popc, marg, sl.st);
         ++ci;
     }

@@ -9,7 +9,7 @@
 // those callers use this entry point instead. All of its scratch -- the
 // transform work slot, the seed spectrum, the twiddle tables and the per-key
 // counters -- lives in one file-scope __device__ array of kScratchBytes bytes
-// (65 MiB), which every GPU that loads the library holds until the process
+// (66.1 MiB), which every GPU that loads the library holds until the process
 // exits. Inputs and outputs stay caller-owned.
 //
 // The paper has no counterpart to this entry point; it is a deployment aid.
@@ -35,7 +35,8 @@ namespace {
 constexpr int kMaxLgL = 21;
 constexpr size_t kSlotBytes = ((size_t)1 << kMaxLgL) * 16;        // 32 MiB
 constexpr size_t kTableBytes = (size_t)960 << 10;                     // twiddle tables (at most 720 KiB are used)
-constexpr size_t kScratchBytes = 2 * kSlotBytes + ((size_t)1 << 20);  // + 1 MiB tables and counters
+constexpr size_t kBitBytes = ((size_t)1 << 20) + (64u << 10);         // transposed input bits and partial popcounts
+constexpr size_t kScratchBytes = 2 * kSlotBytes + ((size_t)1 << 20) + kBitBytes;  // 1 MiB: tables and counters
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -145,10 +146,15 @@ int run_static(unsigned char *base, int lgL, uint64_t n, uint64_t m, const uint6
     if (lay.total * sizeof(cx<T>) > kTableBytes) return PA_EUNSUPPORTED;
     STATIC_CUDA(tw_fill(lay, dtype, tail, st));
     const TwTab<T> tw = tw_tab<T>(lay, tail);
-    STATIC_CUDA(launch_fwd_seed<T>(lg1, seed, n, m, W, L, tw, st));
+    if (bit_scratch_bytes(L, Shape<T>::E, 1) > kBitBytes) return PA_EUNSUPPORTED;
+    const BitScratch bits = bit_scratch_at(tail + ((size_t)1 << 20), L, Shape<T>::E, 1);
+    FwdArgs in = seed_args<T>(bits.bits, n, m, false, L);
+    STATIC_CUDA(launch_seed_bits(seed, n, m, bit_form<T>(lg1, L), bits.bits, nullptr, nullptr, st));
+    STATIC_CUDA(launch_fwd<T>(lg1, In::SEED, in, 1, W, L, tw, st));
     STATIC_CUDA(launch_middle<T>(1, lg2, 1, W, spec, L, 1, tw, scale_of<T>(L), st));
-    STATIC_CUDA(launch_zero_keys(nkeys, popc, marg, st));  // the forward pass accumulates the popcounts
-    STATIC_CUDA(launch_fwd_keys<T>(lg1, keys, nkeys, kstride, n, W, L, 1, tw, popc, st));
+    const KeyBits kb{keys, nkeys, 1, kstride, n, 0, false};
+    STATIC_CUDA(prepare_keys<T>(lg1, kb, L, bits, popc, marg, st, &in));
+    STATIC_CUDA(launch_fwd<T>(lg1, In::KEYS, in, 1, W, L, tw, st));
     STATIC_CUDA(launch_middle<T>(1, lg2, 0, W, spec, L, 1, tw, unit<T>(), st));
     STATIC_CUDA(launch_inv_bits<T>(lg1, W, L, m, nkeys, popc, marg, out, ostride, 1, tw, st));
     return PA_OK;

@@ -39,6 +39,7 @@ struct UClass {
     std::vector<uint32_t> ids;       // caller indices of the blocks in this class
     BlockDev *d_blocks = nullptr;    // device descriptors
     void *Wf = nullptr, *Wi = nullptr;  // forward slots (one per block), inverse slots (one per pair)
+    void *bits = nullptr;               // bit scratch of the first pass
     void *spec = nullptr;            // NTT mode: one seed-spectrum slot, blocks run one after another
     TwSet tw;                        // twiddle tables of geo
     cudaStream_t st = nullptr;
@@ -50,6 +51,7 @@ struct UClass {
         r.nb = (uint32_t)ids.size();
         r.Wf = Wf;
         r.Wi = Wi;
+        r.bits = bits;
         r.spec = spec;
         r.tw = tw;
         return r;
@@ -118,8 +120,9 @@ int run_class_complex(const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStr
     const uint32_t nb = c.nb;
     const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
     cx<T> *Wf = static_cast<cx<T> *>(c.Wf), *Wi = static_cast<cx<T> *>(c.Wi);
-    U_CUDA(launch_zero_blocks(c.d_blocks, nb, popc, marg, st));
-    U_CUDA(launch_fwd_keyseed<T>(g.lg1, c.d_blocks, nb, Wf, g.L, tw, popc, st));
+    FwdArgs in;
+    U_CUDA(prepare_blocks<T>(g.lg1, c.d_blocks, nb, g.L, bit_scratch_at(c.bits, g.L, Shape<T>::E, nb), popc, marg, st, &in));
+    U_CUDA(launch_fwd<T>(g.lg1, In::BLOCKS, in, nb, Wf, g.L, tw, st));
     if (g.lgM) {
         int rc = mid_chunks<T>(c, false, Wf, nb, st);
         if (rc != PA_OK) return rc;
@@ -141,14 +144,18 @@ int run_class_ntt(const ClassRun &c, const pa_block_desc_t *hb, const uint32_t *
     const Geometry &g = c.geo;
     const uint64_t L = g.L;
     const cx<Zp> invL = zp_pow_host(L, kP - 2);
+    const BitScratch bs = bit_scratch_at(c.bits, L, Shape<Zp>::E, 1);
     for (uint32_t i = 0; i < c.nb; ++i) {
         const pa_block_desc_t &b = hb[ids[i]];
         const uint64_t kw = (b.n + 63) / 64;
-        U_CUDA(launch_fwd_seed<Zp>(g.lg1, b.seed, b.n, b.m, W, L, tw, st));
+        FwdArgs in = seed_args<Zp>(bs.bits, b.n, b.m, false, L);
+        U_CUDA(launch_seed_bits(b.seed, b.n, b.m, bit_form<Zp>(g.lg1, L), bs.bits, nullptr, nullptr, st));
+        U_CUDA(launch_fwd<Zp>(g.lg1, In::SEED, in, 1, W, L, tw, st));
         if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, false, W, L, g.inner(), 1, tw, st));
         U_CUDA(launch_middle<Zp>(g.ro, g.lgI, 1, W, spec, L, 1, tw, invL, st));
-        U_CUDA(launch_zero_keys(1, popc + ids[i], marg + ids[i], st));
-        U_CUDA(launch_fwd_keys<Zp>(g.lg1, b.key, 1, kw, b.n, W, L, 1, tw, popc + ids[i], st));
+        const KeyBits kb{b.key, 1, 1, kw, b.n, 0, false};
+        U_CUDA(prepare_keys<Zp>(g.lg1, kb, L, bs, popc + ids[i], marg + ids[i], st, &in));
+        U_CUDA(launch_fwd<Zp>(g.lg1, In::KEYS, in, 1, W, L, tw, st));
         if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, false, W, L, g.inner(), 1, tw, st));
         U_CUDA(launch_middle<Zp>(g.ro, g.lgI, 0, W, spec, L, 1, tw, (cx<Zp>)1, st));
         if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, true, W, L, g.inner(), 1, tw, st));
@@ -220,6 +227,7 @@ void free_uneven(pa_uneven_t *u) {
         cudaFree(c.d_blocks);
         cudaFree(c.Wf);
         cudaFree(c.Wi);
+        cudaFree(c.bits);
         cudaFree(c.spec);
         pa_internal_free_twiddles(&c.tw);
         if (c.st) cudaStreamDestroy(c.st);
@@ -249,7 +257,7 @@ std::vector<BlockDev> class_descs(const pa_uneven_t *u, const UClass &c) {
     std::vector<BlockDev> v(c.ids.size());
     for (size_t i = 0; i < c.ids.size(); ++i) {
         const pa_block_desc_t &b = u->blocks[c.ids[i]];
-        v[i] = BlockDev{b.n, b.m, b.key, b.seed, b.out, c.ids[i], 0u};
+        v[i] = pa::blocks::block_dev(b, c.ids[i], c.geo.L, u->dtype);
     }
     return v;
 }
@@ -295,10 +303,21 @@ uint64_t class_length(uint64_t n, uint64_t m, pa_dtype_t dtype) {
     return choose_geometry(n + m - 1, dtype, dtype != PA_NTT64).L;
 }
 
+BlockDev block_dev(const pa_block_desc_t &b, uint32_t id, uint64_t L, pa_dtype_t dtype) {
+    const int E = dtype == PA_FP32_GUARD ? Shape<float>::E : Shape<double>::E;
+    return BlockDev{b.n, b.m, b.key, b.seed, b.out, id, 0u, SeedRange(b.m, L - b.n + 1, L / E)};
+}
+
+size_t class_bit_bytes(uint64_t L, pa_dtype_t dtype, uint64_t slots) {
+    const int E = dtype == PA_FP32_GUARD ? Shape<float>::E : dtype == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
+    return bit_scratch_bytes(L, E, slots);
+}
+
 size_t scratch_per_block(uint64_t L, pa_dtype_t dtype) {
     if (dtype == PA_NTT64) return 2 * L * 8;
     const size_t e = dtype == PA_FP32_GUARD ? sizeof(float2) : sizeof(double2);
-    return L * e + (L * e + 1) / 2 + sizeof(BlockDev) + 8;  // forward slot, half an inverse slot, descriptor, counters
+    // forward slot, half an inverse slot, bit scratch, descriptor, counters
+    return L * e + (L * e + 1) / 2 + class_bit_bytes(L, dtype, 1) + sizeof(BlockDev) + 8;
 }
 
 int run_complex(pa_dtype_t dtype, const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStream_t st) {
@@ -397,6 +416,7 @@ int pa_uneven_create(const pa_block_desc_t *blocks, uint32_t nblocks, pa_dtype_t
             U_TRY(cudaMalloc(&c.Wf, (size_t)nb * L * esz));
             U_TRY(cudaMalloc(&c.Wi, (size_t)((nb + 1) / 2) * L * esz));
         }
+        U_TRY(cudaMalloc(&c.bits, pa::blocks::class_bit_bytes(L, dtype, dtype == PA_NTT64 ? 1 : nb)));
         rc = tune_class(u, c);
         if (rc != PA_OK) return fail(rc);
     }
