@@ -355,22 +355,114 @@ __device__ __forceinline__ void load_pair(const unsigned long long *p, unsigned 
     a = q.x;
     b = q.y;
 }
-// The ROWS multipliers of butterfly k of a stage of span P.
+template <typename T>
+constexpr Rows kRows = std::is_same<T, Zp>::value ? Rows::EXACT : std::is_same<T, float>::value ? Rows::SINGLE : Rows::DOUBLE;
+// The ROWS multipliers at index k of a table of P butterflies.
 template <typename T, int ROWS, int P>
 __device__ __forceinline__ void load_rows(const cx<T> *tab, uint32_t k, cx<T> *w) {
-    const cx<T> *t = tab + 2 * k;
+    if constexpr (ROWS == 1) {
+        w[0] = __ldg(tab + k);
+    } else {
+        const cx<T> *t = tab + 2 * k;
 #pragma unroll
-    for (int r = 0; r < ROWS; r += 2) {
-        if (r + 1 < ROWS) {
-            load_pair(t + r * P, w[r], w[r + 1]);
-        } else {
-            w[r] = __ldg(t + r * P);
+        for (int r = 0; r < ROWS; r += 2) {
+            if (r + 1 < ROWS) {
+                load_pair(t + r * P, w[r], w[r + 1]);
+            } else {
+                w[r] = __ldg(t + r * P);
+            }
         }
     }
 }
 
-// DFT of v[r] * w^r, r < R, natural order in and out, with the multipliers of stage_list's
-// rows for this w: level l, sub-transform p needs (w w_R^p)^(R / 2^(l+1)), and the upper half
+// w^2 of a root of unity: (1 - 2 s^2, 2 s c).
+__device__ __forceinline__ float2 square_root_of_unity(float2 w) {
+    const float t = w.y + w.y;
+    return make_float2(fmaf(-t, w.y, 1.f), t * w.x);
+}
+// w * w_N^J for a compile-time turn.
+template <int N, int J>
+__device__ __forceinline__ float2 turn(float2 w) {
+    if constexpr (J % N == 0) {
+        return w;
+    } else {
+        constexpr float c = (float)cos_frac(J % N, N), s = -(float)sin_frac(J % N, N);
+        const float2 t = f2_mul(make_float2(c, c), w);
+        return make_float2(fmaf(-s, w.y, t.x), fmaf(s, w.x, t.y));
+    }
+}
+// m[] = the multipliers of the levels of a radix-R stage (dft_rows) for the root pw[l] * w_TURN_N^(TURN * R/2^(l+1))
+// of level l, where pw[l] = w^(R / 2^(l+1)): rows p of a level are further turns by w_{2^(l+1)}^p.
+template <int R, int N, int TURN, int LEVEL = 0, int P = 0>
+__device__ __forceinline__ void level_multipliers(const float2 *pw, float2 *m) {
+    if constexpr ((1 << LEVEL) < R) {
+        constexpr int half = LEVEL ? 1 << (LEVEL - 1) : 1, h = R >> (LEVEL + 1);
+        if constexpr (P < half) {
+            // exponent of w_M, M = N * 2^(LEVEL+1): TURN h / N + P / 2^(LEVEL+1)
+            constexpr int M = N << (LEVEL + 1);
+            m[LEVEL ? half + P : 0] = turn<M, (TURN * h << (LEVEL + 1)) + P * N>(pw[LEVEL]);
+            level_multipliers<R, N, TURN, LEVEL, P + 1>(pw, m);
+        } else {
+            level_multipliers<R, N, TURN, LEVEL + 1, 0>(pw, m);
+        }
+    }
+}
+// pw[l] = w^(R / 2^(l+1)), l = log2 R - 1 .. 0.
+template <int R>
+__device__ __forceinline__ void level_powers(float2 w, float2 *pw) {
+#pragma unroll
+    for (int l = ilog2(R) - 1; l >= 0; --l) {
+        pw[l] = w;
+        if (l) w = square_root_of_unity(w);
+    }
+}
+
+// The multipliers of a power-of-two stage at table index k.
+template <typename T, int R, int P>
+__device__ __forceinline__ void stage_multipliers(const cx<T> *tab, uint32_t k, cx<T> *m) {
+    if constexpr (kRows<T> == Rows::SINGLE) {
+        cx<T> w, pw[ilog2(R)];
+        load_rows<T, 1, P>(tab, k, &w);
+        level_powers<R>(w, pw);
+        level_multipliers<R, 1, 0>(pw, m);
+    } else {
+        load_rows<T, stage_rows(R, kRows<T>), P>(tab, k, m);
+    }
+}
+// The multipliers of the odd stage (odd_exponent) at table index k.
+template <int RO, int R0, int K1 = 0>
+__device__ __forceinline__ void odd_level_multipliers(const float2 *pw, float2 *w) {
+    if constexpr (K1 < RO) {
+        float2 m[R0 / 2];
+        level_multipliers<R0, RO * R0, K1>(pw, m);
+#pragma unroll
+        for (int r = 0; r < R0 / 2; ++r) w[RO - 1 + r * RO + K1] = m[r];
+        odd_level_multipliers<RO, R0, K1 + 1>(pw, w);
+    }
+}
+template <typename T, int RO, int R0, int P>
+__device__ __forceinline__ void odd_multipliers(const cx<T> *tab, uint32_t k, cx<T> *w) {
+    if constexpr (kRows<T> == Rows::SINGLE) {
+        cx<T> b;  // w, then w^R0
+        load_rows<T, 1, P>(tab, k, &b);
+        if constexpr (R0 > 1) {
+            cx<T> pw[ilog2(R0)];
+            level_powers<R0>(b, pw);
+            odd_level_multipliers<RO, R0>(pw, w);
+            b = square_root_of_unity(pw[0]);
+        }
+        // w[i] = b^(i + 1): even powers by squaring, odd ones by a product
+        w[0] = b;
+#pragma unroll
+        for (int n = 2; n < RO; ++n)
+            w[n - 1] = n % 2 == 0 ? square_root_of_unity(w[n / 2 - 1]) : Arith<T>::mul(w[n / 2 - 1], w[(n + 1) / 2 - 1]);
+    } else {
+        load_rows<T, odd_rows(RO, R0, kRows<T>), P>(tab, k, w);
+    }
+}
+
+// DFT of v[r] * w^r, r < R, natural order in and out, with the multipliers of
+// stage_multipliers for this w: level l, sub-transform p needs (w w_R^p)^(R / 2^(l+1)), and the upper half
 // of the p are a quarter turn away from the lower half, so R/2 multipliers do. Every
 // butterfly absorbs its multiplier (bfly): a radix-16 stage takes 192 multiply-add slots,
 // where twiddling first (15 products, and 14 more to form the powers) took 284.
@@ -471,9 +563,8 @@ __device__ __forceinline__ void dft_comp(cx<T> *x) {
 // multipliers carry w w_RC^{k1}.
 template <typename T, int RO, int R0, int P, bool INV>
 __device__ __forceinline__ void dft_comp_rows(cx<T> *x, const cx<T> *tab, uint32_t k) {
-    constexpr int ROWS = odd_rows(RO, R0);
-    cx<T> w[ROWS];
-    load_rows<T, ROWS, P>(tab, k, w);
+    cx<T> w[odd_level_rows(RO, R0)];
+    odd_multipliers<T, RO, R0, P>(tab, k, w);
     if constexpr (INV) {
 #pragma unroll
         for (int r = 0; r < RO - 1; ++r) w[r].y = -w[r].y;
@@ -561,7 +652,7 @@ constexpr uint32_t smem_elems() { return (uint32_t)LEN * COLS + ((uint32_t)LEN *
 
 // The stage plan at compile time.
 template <typename T, int LEN, int E> struct Plan {
-    static constexpr StagePlan p = stage_plan(LEN, E, !std::is_same<T, Zp>::value);
+    static constexpr StagePlan p = stage_plan(LEN, E, kRows<T>);
     static constexpr int RO = p.RO, TC = p.TC, r0 = p.r0, n = p.n;
     static_assert(RO == 1 || RO == 3 || RO == 5 || RO == 9, "odd factor must be 1, 3, 5 or 9");
     static_assert(n >= 2 && p.R[n - 1] == E, "at least two stages, the last of radix E");
@@ -661,8 +752,8 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
         if constexpr (row.rows == 0) {
             dft<T, M::R, INV>(v + g * M::R);
         } else {
-            cx<T> w[row.rows];
-            load_rows<T, row.rows, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
+            cx<T> w[kRows<T> == Rows::EXACT ? M::R - 1 : level_rows(M::R)];
+            stage_multipliers<T, M::R, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
             dft_rows<T, M::R, INV>(v + g * M::R, w);
         }
     }

@@ -16,13 +16,14 @@ uint64_t take(uint64_t *total, uint64_t n) {
 
 // Exponent (of w_L, not reduced) of element i of the block; inverse tables of the exact
 // transform come back with *neg set. Padding elements read as w^0.
-__device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, bool complex_, bool *neg) {
+__device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, Rows kind, bool *neg) {
+    const bool complex_ = kind != Rows::EXACT;
     *neg = false;
     if (i >= y.hi && i < y.hi + y.nhi) return (i - y.hi) << y.B;
     if (i >= y.lo && i < y.lo + y.nlo) return i - y.lo;
     for (int p = 0; p < 3; ++p) {
         if (y.len[p] == 0) continue;
-        const StagePlan l = stage_plan(y.len[p], y.E, complex_);
+        const StagePlan l = stage_plan(y.len[p], y.E, kind);
         if (i < y.st[p] || i >= y.st[p] + (uint64_t)l.total) continue;
         const int o = (int)(i - y.st[p]);
         for (int j = 0; j < 2 * l.n; ++j) {
@@ -30,13 +31,14 @@ __device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, bool complex_, bo
             const bool inv = j >= l.n;
             const StageRow r = inv ? l.inv[stage] : l.fwd[stage];
             const int count = inv ? l.s[stage] : l.P[stage];
-            if (r.rows == 0 || o < r.off || o >= r.off + (r.rows + 1) / 2 * 2 * count) continue;
-            const int q = (o - r.off) / 2, row = 2 * (q / count) + ((o - r.off) & 1);
+            if (r.rows == 0 || o < r.off || o >= r.off + row_entries(r.rows, count)) continue;
+            const int q = r.rows == 1 ? o - r.off : (o - r.off) / 2;
+            const int row = r.rows == 1 ? q / count : 2 * (q / count) + ((o - r.off) & 1);
             const uint32_t x = (uint32_t)(q % count);
             if (row >= r.rows) return 0;
             *neg = !complex_ && inv;
-            if (inv && stage == 0 && l.RO > 1) return odd_exponent(l.RO, l.R0C, count, row, x, y.L);
-            return stage_exponent(l.R[stage], count, row, inv ? x : block_freq(l, stage, x), y.L, complex_);
+            if (inv && stage == 0 && l.RO > 1) return odd_exponent(l.RO, l.R0C, count, row, x, y.L, kind);
+            return stage_exponent(l.R[stage], count, row, inv ? x : block_freq(l, stage, x), y.L, kind);
         }
         return 0;
     }
@@ -78,10 +80,9 @@ __device__ cx<Zp> root_power<Zp>(uint64_t e, uint64_t, uint64_t w) {
 
 template <typename T>
 __global__ void k_fill_tables(cx<T> *mem, TwLayout y, uint64_t root) {
-    constexpr bool kComplex = !std::is_same<T, Zp>::value;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < y.total; i += (uint64_t)gridDim.x * blockDim.x) {
         bool neg;
-        uint64_t e = exponent_at(y, i, kComplex, &neg) % y.L;
+        uint64_t e = exponent_at(y, i, kRows<T>, &neg) % y.L;
         if (neg && e) e = y.L - e;
         mem[i] = root_power<T>(e, y.L, root);
     }
@@ -117,7 +118,8 @@ uint64_t zp_pow_host(uint64_t a, uint64_t e) {
 }
 
 TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
-    const bool complex_ = dtype != PA_NTT64;
+    const Rows kind = dtype == PA_FP32_GUARD ? kRows<float> : dtype == PA_FP64 ? kRows<double> : kRows<Zp>;
+    const bool complex_ = kind != Rows::EXACT;
     TwLayout y;
     y.L = g.L;
     int lgL = 0;
@@ -132,7 +134,7 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
     y.hi = take(&y.total, y.nhi);
     y.lo = take(&y.total, y.nlo);
     for (int p = 0; p < 3; ++p)
-        if (y.len[p]) y.st[p] = take(&y.total, (uint64_t)stage_plan(y.len[p], y.E, complex_).total);
+        if (y.len[p]) y.st[p] = take(&y.total, (uint64_t)stage_plan(y.len[p], y.E, kind).total);
     for (int p = 0; p < 2; ++p) {
         if (!y.len[p]) continue;
         PassShape &t = y.pass[p];

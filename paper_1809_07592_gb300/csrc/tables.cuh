@@ -44,19 +44,35 @@ struct StagePlan {
     int R[kMaxStages], N[kMaxStages], s[kMaxStages], P[kMaxStages];
     // Twiddle tables: butterfly (block b, offset j) of forward stage i reads rows at index b < P[i],
     // of inverse stage i at index j < s[i]. Rows are stored in pairs, entry (row, x) at
-    // off + 2*((row/2)*count + x) + row%2, so that one 16-byte load of single-precision values
-    // brings two multipliers. rows = 0: no twiddles (forward stage 0, inverse stage n-1).
+    // off + 2*((row/2)*count + x) + row%2 (one row: off + x), so that a pair takes one wide
+    // load. rows = 0: no twiddles (forward stage 0, inverse stage n-1).
     StageRow fwd[kMaxStages], inv[kMaxStages];
     int total;  // entries
 };
 
-// Rows of a radix-R power-of-two stage. Complex arithmetic: the distinct multipliers of the
-// log2 R butterfly levels (dft_rows in fft_core.cuh); the exact transform: w^r, r = 1 .. R-1.
-__host__ __device__ constexpr int stage_rows(int R, bool complex_) { return complex_ ? R / 2 : R - 1; }
-// Rows of the odd stage of radix RO * R0: w^{R0 n1}, then the levels of a radix-R0 stage per k1 < RO.
-__host__ __device__ constexpr int odd_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
+// The three arithmetics' table rows. A complex stage needs the multipliers of its butterfly levels
+// (dft_rows in fft_core.cuh), R/2 of a radix-R power-of-two stage, RO-1 + RO*R0/2 of an odd one.
+// Double precision reads them all: its passes are bound by the FP64 pipe, the load path is idle. Single
+// precision reads w alone and forms the others (squarings and constant turns): its innermost
+// pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing four
+// wavefronts whatever the addresses) and has multiply-add slots to spare. The exact transform
+// reads w^r, r = 1 .. R-1.
+enum class Rows { SINGLE, DOUBLE, EXACT };
+__host__ __device__ constexpr int level_rows(int R) { return R / 2; }
+__host__ __device__ constexpr int odd_level_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
+__host__ __device__ constexpr int stage_rows(int R, Rows kind) {
+    return kind == Rows::SINGLE ? 1 : kind == Rows::DOUBLE ? level_rows(R) : R - 1;
+}
+__host__ __device__ constexpr int odd_rows(int RO, int R0, Rows kind) {
+    return kind == Rows::SINGLE ? 1 : odd_level_rows(RO, R0);
+}
 
-__host__ __device__ constexpr StagePlan stage_plan(int len, int E, bool complex_) {
+// Entries of a stage's rows (whole pairs, except a single row; even, so that every table starts on a pair).
+__host__ __device__ constexpr int row_entries(int rows, int count) {
+    return rows == 1 ? (count + 1) / 2 * 2 : (rows + 1) / 2 * 2 * count;
+}
+
+__host__ __device__ constexpr StagePlan stage_plan(int len, int E, Rows kind) {
     StagePlan l{};
     l.RO = odd_part(len);
     const int k = ilog2(len / l.RO), e = ilog2(E);
@@ -73,15 +89,15 @@ __host__ __device__ constexpr StagePlan stage_plan(int len, int E, bool complex_
         l.P[i] = P;
         l.N[i] = len / P;
         l.s[i] = l.N[i] / l.R[i];
-        const int rows = i == 0 ? 0 : stage_rows(l.R[i], complex_);
+        const int rows = i == 0 ? 0 : stage_rows(l.R[i], kind);
         l.fwd[i] = StageRow{rows, off};
-        off += (rows + 1) / 2 * 2 * P;
+        off += row_entries(rows, P);
         P *= l.R[i];
     }
     for (int i = 0; i < l.n; ++i) {
-        const int rows = i == l.n - 1 ? 0 : i == 0 && l.RO > 1 ? odd_rows(l.RO, l.R0C) : stage_rows(l.R[i], complex_);
+        const int rows = i == l.n - 1 ? 0 : i == 0 && l.RO > 1 ? odd_rows(l.RO, l.R0C, kind) : stage_rows(l.R[i], kind);
         l.inv[i] = StageRow{rows, off};
-        off += (rows + 1) / 2 * 2 * l.s[i];
+        off += row_entries(rows, l.s[i]);
     }
     l.total = off;
     return l;
@@ -103,14 +119,15 @@ __host__ __device__ constexpr int row_level(int row) { return row == 0 ? 0 : ilo
 __host__ __device__ constexpr int row_pos(int row) { return row == 0 ? 0 : row - (1 << ilog2(row)); }
 
 // Exponent e (of w_L) held by row `row` of a radix-R stage for the twiddle base w_{R P}^k.
-__host__ __device__ inline uint64_t stage_exponent(int R, uint64_t P, int row, uint64_t k, uint64_t L, bool complex_) {
+__host__ __device__ inline uint64_t stage_exponent(int R, uint64_t P, int row, uint64_t k, uint64_t L, Rows kind) {
     const uint64_t unit = L / ((uint64_t)R * P);  // w_{R P} = w_L^unit
-    if (!complex_) return (uint64_t)(row + 1) * k * unit;
+    if (kind != Rows::DOUBLE) return (uint64_t)(row + 1) * k * unit;
     const int l = row_level(row);
     return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)row_pos(row) * (L >> (l + 1));
 }
-__host__ __device__ inline uint64_t odd_exponent(int RO, int R0, uint64_t P, int row, uint64_t k, uint64_t L) {
+__host__ __device__ inline uint64_t odd_exponent(int RO, int R0, uint64_t P, int row, uint64_t k, uint64_t L, Rows kind) {
     const uint64_t RC = (uint64_t)RO * R0, unit = L / (RC * P);
+    if (kind == Rows::SINGLE) return k * unit;
     if (row < RO - 1) return (uint64_t)R0 * (row + 1) * k * unit;
     const int t = row - (RO - 1), k1 = t % RO, r = t / RO;  // level row r of the radix-R0 stage of k1
     const int l = row_level(r);
