@@ -26,6 +26,18 @@
 
 namespace pa {
 
+// First statement of every pass kernel (they are launched with launch_chained): lets the stream's next
+// kernel start once every CTA of this one has begun, then waits until the previous kernel has
+// finished and its writes are visible. A chain of small launches loses the launch latency between
+// its kernels, and a large one's first CTAs fill the SMs that the last wave of the kernel before
+// leaves empty.
+__device__ __forceinline__ void begin_after_previous() {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+#endif
+}
+
 // Element arithmetic of the transforms. Arith<float> / Arith<double> work on
 // complex numbers (x = real, y = imaginary); Arith<Zp> (zp.cuh) on residues
 // modulo the prime p = 2^64 - 2^32 + 1. The FFT engine below only uses add,

@@ -220,6 +220,7 @@ __device__ __forceinline__ uint32_t bits_at(const uint64_t *v, uint64_t nbits, u
 template <typename T, int LEN, int COLS, int E, In KIND>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_fwd(FwdArgs in, cx<T> *__restrict__ W, uint64_t L, TwTab<T> tw) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
@@ -274,6 +275,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 template <typename T, int LEN, int COLS, int E, bool INV>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_mid(cx<T> *__restrict__ W, uint64_t L, uint32_t S, TwTab<T> tw) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
@@ -302,6 +304,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T>)))
     k_middle(cx<T> *__restrict__ W, cx<T> *__restrict__ spec, uint64_t L, TwTab<T> tw, cx<T> scale) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t tq = threadIdx.x;
@@ -442,6 +445,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_inv_bits(const cx<T> *__restrict__ W, uint64_t L, uint64_t m, uint32_t nkeys,
                const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, uint64_t *__restrict__ out,
                uint64_t ostride, TwTab<T> tw, const uint64_t *__restrict__ xkeys, uint64_t xstride) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     using word_t = typename BitsWord<COLS>::type;
@@ -549,6 +553,7 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
                    const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, uint64_t *__restrict__ out,
                    uint64_t ostride, TwTab<float> tw, const uint64_t *__restrict__ xkeys, uint64_t xstride,
                    uint32_t *__restrict__ ctl, uint32_t expire_ns) {
+    begin_after_previous();
     using T = float;
     constexpr int E = 16, COLS = 16;
     static_assert(LEN <= 256 && LEN >= 64, "one tiled copy moves at most 256 rows");
@@ -673,6 +678,7 @@ template <typename T, int LEN, int E>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
     k_middle_split(const cx<T> *__restrict__ Wf, cx<T> *__restrict__ Wi, uint64_t L, uint32_t nblocks,
                    uint32_t lgL1, uint32_t lgM, TwTab<T> tw, T inv_L) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
@@ -752,6 +758,7 @@ template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
     k_middle_real(cx<T> *__restrict__ W, cx<T> *__restrict__ tabs, uint64_t N, uint32_t lgL1, uint32_t lgM,
                   TwTab<T> tw, T scale) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
@@ -825,6 +832,7 @@ template <typename T, int LEN, int COLS, int E>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_inv_bits_blocks(const cx<T> *__restrict__ W, uint64_t L, const BlockDev *__restrict__ blocks, uint32_t nblocks,
                       const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, TwTab<T> tw) {
+    begin_after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     using word_t = typename BitsWord<COLS>::type;

@@ -50,8 +50,7 @@ cudaError_t fwd_at(const FwdArgs &in, uint32_t slots, cx<T> *W, uint64_t L, TwTa
     cudaError_t e = set_smem(kern, sb);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((L / LEN) / COLS), slots);
-    kern<<<grid, COLS * LEN / E, sb, st>>>(in, W, L, tw);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, COLS * LEN / E, sb, st, in, W, L, tw);
 }
 
 template <typename T>
@@ -83,14 +82,13 @@ cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S
             auto kern = k_mid<T, LEN, COLS, E, true>;
             cudaError_t e = set_smem(kern, sb);
             if (e != cudaSuccess) return e;
-            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, tw);
+            return launch_chained(kern, grid, COLS * LEN / E, sb, st, W, L, S, tw);
         } else {
             auto kern = k_mid<T, LEN, COLS, E, false>;
             cudaError_t e = set_smem(kern, sb);
             if (e != cudaSuccess) return e;
-            kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, S, tw);
+            return launch_chained(kern, grid, COLS * LEN / E, sb, st, W, L, S, tw);
         }
-        return cudaGetLastError();
     });
 }
 
@@ -125,14 +123,13 @@ cudaError_t middle_at(int mode, cx<T> *W, cx<T> *spec, uint64_t L, uint32_t pair
         auto kern = k_middle<T, LEN, E, 0>;
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
-        kern<<<grid, LEN / E, sb, st>>>(W, spec, L, tw, scale);
+        return launch_chained(kern, grid, LEN / E, sb, st, W, spec, L, tw, scale);
     } else {
         auto kern = k_middle<T, LEN, E, 1>;
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
-        kern<<<grid, LEN / E, sb, st>>>(W, spec, L, tw, scale);
+        return launch_chained(kern, grid, LEN / E, sb, st, W, spec, L, tw, scale);
     }
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -201,10 +198,9 @@ cudaError_t inv_bits_tma_at(const float2 *W, uint64_t L, uint64_t m, uint32_t nk
     const uint64_t ntiles = (S / COLS) * pairs;
     if (ntiles > 0xFFFFFFFFull) return cudaErrorInvalidValue;
     const uint32_t grid = (uint32_t)(ntiles < ctas ? ntiles : ctas);
-    kern<<<grid, LEN, sb, st>>>(map, L, m, nkeys, pairs, popc, margin_bits, out, ostride, tw, xkeys, xstride, ctl,
-                                expire_ns);
     *done = true;
-    return cudaGetLastError();
+    return launch_chained(kern, grid, LEN, sb, st, map, L, m, nkeys, pairs, popc, margin_bits, out, ostride, tw, xkeys,
+                          xstride, ctl, expire_ns);
 }
 
 template <typename T, int LEN, bool PACK>
@@ -226,8 +222,7 @@ cudaError_t inv_bits_at(const cx<T> *W, uint64_t L, uint64_t m, uint32_t nkeys, 
     cudaError_t e = set_smem(kern, sb);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)((L / LEN) / COLS), pairs);
-    kern<<<grid, COLS * LEN / E, sb, st>>>(W, L, m, nkeys, popc, margin_bits, out, ostride, tw, xkeys, xstride);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, COLS * LEN / E, sb, st, W, L, m, nkeys, popc, margin_bits, out, ostride, tw, xkeys, xstride);
 }
 
 template <typename T>
@@ -270,9 +265,8 @@ cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, u
     if (e != cudaSuccess) return e;
     const uint32_t R = (uint32_t)(L / LEN);
     dim3 grid(R / 2 + 1, (nblocks + 1) / 2);
-    kern<<<grid, 2 * (LEN / E), sb, st>>>(Wf, Wi, L, nblocks, lgL1, lgM, tw,
+    return launch_chained(kern, grid, 2 * (LEN / E), sb, st, Wf, Wi, L, nblocks, lgL1, lgM, tw,
                                          (T)(kSpecScale / (double)L));
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -324,8 +318,7 @@ cudaError_t launch_inv_bits_blocks(int lgLEN, const cx<T> *Wi, uint64_t L, const
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
         dim3 grid((unsigned)((L / LEN) / COLS), (nblocks + 1) / 2);
-        kern<<<grid, COLS * LEN / E, sb, st>>>(Wi, L, blocks, nblocks, popc, margin_bits, tw);
-        return cudaGetLastError();
+        return launch_chained(kern, grid, COLS * LEN / E, sb, st, Wi, L, blocks, nblocks, popc, margin_bits, tw);
     });
 }
 
@@ -349,14 +342,13 @@ cudaError_t real_at(int mode, cx<T> *W, cx<T> *tabs, uint64_t N, uint32_t lgL1, 
         auto kern = k_middle_real<T, LEN, E, 0>;
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 2 * (LEN / E), sb, st>>>(W, tabs, N, lgL1, lgM, tw, scale);
+        return launch_chained(kern, grid, 2 * (LEN / E), sb, st, W, tabs, N, lgL1, lgM, tw, scale);
     } else {
         auto kern = k_middle_real<T, LEN, E, 1>;
         cudaError_t e = set_smem(kern, sb);
         if (e != cudaSuccess) return e;
-        kern<<<grid, 2 * (LEN / E), sb, st>>>(W, tabs, N, lgL1, lgM, tw, scale);
+        return launch_chained(kern, grid, 2 * (LEN / E), sb, st, W, tabs, N, lgL1, lgM, tw, scale);
     }
-    return cudaGetLastError();
 }
 
 template <typename T, int RO, int LG = kMinLgOdd>

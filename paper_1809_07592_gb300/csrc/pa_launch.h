@@ -16,6 +16,24 @@
 
 namespace pa {
 
+// Launches a kernel whose first instruction is begin_after_previous (fft_core.cuh): its CTAs may
+// start filling the SMs while the last CTAs of the stream's previous kernel still run.
+template <typename... Params, typename... Args>
+cudaError_t launch_chained(void (*kern)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                           Args... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 // Per-type kernel shape: E complex values per thread, COLS columns per CTA in
 // the strided passes. FP64 halves both to keep registers and shared memory
 // within one SM's budget.

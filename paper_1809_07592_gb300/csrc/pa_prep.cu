@@ -234,6 +234,7 @@ __device__ __forceinline__ void store_part(uint2 *parts, uint32_t ca, uint32_t c
 template <int E, bool PACK>
 __global__ void __launch_bounds__(kBitThreads) k_key_bits(KeyBits k, BitShape h, BitScratch out,
                                                           uint32_t *__restrict__ margin_bits) {
+    begin_after_previous();
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x, slot = blockIdx.y;
     uint32_t *bits = out.bits + (uint64_t)slot * h.S * h.TC;
     uint32_t ca = 0, cb = 0;
@@ -263,6 +264,7 @@ template <int E>
 __global__ void __launch_bounds__(kBitThreads) k_seed_bits(const uint64_t *__restrict__ seed, uint64_t n, uint64_t m,
                                                            BitShape h0, uint64_t len0, uint32_t *out0, BitShape h1,
                                                            uint64_t len1, uint32_t *out1) {
+    begin_after_previous();
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x;
     uint32_t ca, cb;
     if (blockIdx.y == 0) {
@@ -276,6 +278,7 @@ __global__ void __launch_bounds__(kBitThreads) k_seed_bits(const uint64_t *__res
 template <int E>
 __global__ void __launch_bounds__(kBitThreads) k_block_bits(const BlockDev *__restrict__ blocks, BitShape h, uint64_t L,
                                                             BitScratch out, uint32_t *__restrict__ margin_bits) {
+    begin_after_previous();
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x;
     const BlockDev &b = blocks[blockIdx.y];
     uint32_t ca = 0, cb = 0;
@@ -298,11 +301,12 @@ cudaError_t launch_key_bits(const KeyBits &k, const BitForm &f, BitScratch scrat
     const BitShape h = bit_shape(f);
     *nparts = (uint32_t)parts_count(f.L, f.E);
     const dim3 grid(*nparts, k.slots);
-    if (f.E == 16 && k.pack) k_key_bits<16, true><<<grid, kBitThreads, 0, st>>>(k, h, scratch, margin_bits);
-    else if (f.E == 16) k_key_bits<16, false><<<grid, kBitThreads, 0, st>>>(k, h, scratch, margin_bits);
-    else if (k.pack) k_key_bits<8, true><<<grid, kBitThreads, 0, st>>>(k, h, scratch, margin_bits);
-    else k_key_bits<8, false><<<grid, kBitThreads, 0, st>>>(k, h, scratch, margin_bits);
-    return cudaGetLastError();
+    cudaError_t e;
+    if (f.E == 16 && k.pack) e = launch_chained(k_key_bits<16, true>, grid, kBitThreads, 0, st, k, h, scratch, margin_bits);
+    else if (f.E == 16) e = launch_chained(k_key_bits<16, false>, grid, kBitThreads, 0, st, k, h, scratch, margin_bits);
+    else if (k.pack) e = launch_chained(k_key_bits<8, true>, grid, kBitThreads, 0, st, k, h, scratch, margin_bits);
+    else e = launch_chained(k_key_bits<8, false>, grid, kBitThreads, 0, st, k, h, scratch, margin_bits);
+    return e;
 }
 
 cudaError_t launch_seed_bits(const uint64_t *seed, uint64_t n, uint64_t m, const BitForm &f, uint32_t *out,
@@ -312,9 +316,10 @@ cudaError_t launch_seed_bits(const uint64_t *seed, uint64_t n, uint64_t m, const
     uint64_t x = parts_count(f.L, f.E);
     if (packed && parts_count(L1, f.E) > x) x = parts_count(L1, f.E);
     const dim3 grid((unsigned)x, packed ? 2 : 1);
-    if (f.E == 16) k_seed_bits<16><<<grid, kBitThreads, 0, st>>>(seed, n, m, h0, f.L, out, h1, L1, packed_out);
-    else k_seed_bits<8><<<grid, kBitThreads, 0, st>>>(seed, n, m, h0, f.L, out, h1, L1, packed_out);
-    return cudaGetLastError();
+    cudaError_t e;
+    if (f.E == 16) e = launch_chained(k_seed_bits<16>, grid, kBitThreads, 0, st, seed, n, m, h0, f.L, out, h1, L1, packed_out);
+    else e = launch_chained(k_seed_bits<8>, grid, kBitThreads, 0, st, seed, n, m, h0, f.L, out, h1, L1, packed_out);
+    return e;
 }
 
 cudaError_t launch_block_bits(const BlockDev *blocks, uint32_t nblocks, const BitForm &f, BitScratch scratch,
@@ -322,9 +327,10 @@ cudaError_t launch_block_bits(const BlockDev *blocks, uint32_t nblocks, const Bi
     const BitShape h = bit_shape(f);
     *nparts = (uint32_t)parts_count(f.L, f.E);
     const dim3 grid(*nparts, nblocks);
-    if (f.E == 16) k_block_bits<16><<<grid, kBitThreads, 0, st>>>(blocks, h, f.L, scratch, margin_bits);
-    else k_block_bits<8><<<grid, kBitThreads, 0, st>>>(blocks, h, f.L, scratch, margin_bits);
-    return cudaGetLastError();
+    cudaError_t e;
+    if (f.E == 16) e = launch_chained(k_block_bits<16>, grid, kBitThreads, 0, st, blocks, h, f.L, scratch, margin_bits);
+    else e = launch_chained(k_block_bits<8>, grid, kBitThreads, 0, st, blocks, h, f.L, scratch, margin_bits);
+    return e;
 }
 
 // Round every float of x[0 .. count) to `bits` explicit significand bits (round to
