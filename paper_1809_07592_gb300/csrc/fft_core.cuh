@@ -30,12 +30,15 @@ namespace pa {
 // kernel start once every CTA of this one has begun, then waits until the previous kernel has
 // finished and its writes are visible. A chain of small launches loses the launch latency between
 // its kernels, and a large one's first CTAs fill the SMs that the last wave of the kernel before
-// leaves empty.
-__device__ __forceinline__ void begin_after_previous() {
-#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
+// leaves empty. The arguments are the pointers to data that earlier kernels of the stream write: their
+// values pass through the wait, because a load the compiler takes for one of constant memory
+// (const __restrict__, __ldg) may otherwise move above it.
+template <typename... P>
+__device__ __forceinline__ void begin_after_previous(P &...p) {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-#endif
+    const auto behind = [](auto &q) { asm volatile("" : "+l"(q)::"memory"); };
+    (behind(p), ...);
 }
 
 // Element arithmetic of the transforms. Arith<float> / Arith<double> work on
@@ -185,7 +188,8 @@ template <typename T> struct TwTab {
     const cx<T> *lo;
     uint32_t B;              // w_L^e = hi[e >> B] * lo[e & (2^B - 1)]
     const cx<T> *st[3];      // stage tables: first pass, middle strided pass, innermost pass
-    PassTw<T> fw[2], iv[2];  // pass tables of the first and the middle strided pass
+    PassTw<T> fw[2], iv[2];  // pass tables of the first and the middle strided pass (iv: exact transform)
+    const cx<T> *col[2];     // their inverse column tables (complex arithmetic)
 };
 
 template <typename T> struct ComplexArith {
@@ -199,9 +203,12 @@ template <typename T> struct ComplexArith {
     static __device__ __forceinline__ E mulk(T k, E a) { return mk(k * a.x, k * a.y); }
     // (a, b) -> (a + w b, a - w b), w = c + i s: six fused multiply-adds, the difference
     // as 2a - (a + w b).
-    static __device__ __forceinline__ void bfly(E &a, E &b, T c, T s) {
+    static __device__ __forceinline__ E add_mul(E a, E b, T c, T s) {
         const E t = fmak(c, b, a);
-        const E p = mk(fma(-s, b.y, t.x), fma(s, b.x, t.y));
+        return mk(fma(-s, b.y, t.x), fma(s, b.x, t.y));
+    }
+    static __device__ __forceinline__ void bfly(E &a, E &b, T c, T s) {
+        const E p = add_mul(a, b, c, s);
         b = mk(fma((T)2, a.x, -p.x), fma((T)2, a.y, -p.y));
         a = p;
     }
@@ -266,9 +273,12 @@ template <> struct Arith<float> : ComplexArith<float> {
     static __device__ __forceinline__ E sub(E a, E b) { return f2_sub(a, b); }
     static __device__ __forceinline__ E fmak(float k, E a, E c) { return f2_fma(make_float2(k, k), a, c); }
     static __device__ __forceinline__ E mulk(float k, E a) { return f2_mul(make_float2(k, k), a); }
-    static __device__ __forceinline__ void bfly(E &a, E &b, float c, float s) {
+    static __device__ __forceinline__ E add_mul(E a, E b, float c, float s) {
         const E t = fmak(c, b, a);
-        const E p = mk(fmaf(-s, b.y, t.x), fmaf(s, b.x, t.y));
+        return mk(fmaf(-s, b.y, t.x), fmaf(s, b.x, t.y));
+    }
+    static __device__ __forceinline__ void bfly(E &a, E &b, float c, float s) {
+        const E p = add_mul(a, b, c, s);
         b = mk(fmaf(2.f, a.x, -p.x), fmaf(2.f, a.y, -p.y));
         a = p;
     }
@@ -388,44 +398,45 @@ __device__ __forceinline__ void load_rows(const cx<T> *tab, uint32_t k, cx<T> *w
 }
 
 // w^2 of a root of unity: (1 - 2 s^2, 2 s c).
-__device__ __forceinline__ float2 square_root_of_unity(float2 w) {
-    const float t = w.y + w.y;
-    return make_float2(fmaf(-t, w.y, 1.f), t * w.x);
+template <typename T>
+__device__ __forceinline__ cx<T> square_root_of_unity(cx<T> w) {
+    const T t = w.y + w.y;
+    return Arith<T>::mk(fma(-t, w.y, (T)1), t * w.x);
 }
 // w * w_N^J for a compile-time turn.
-template <int N, int J>
-__device__ __forceinline__ float2 turn(float2 w) {
+template <typename T, int N, int J>
+__device__ __forceinline__ cx<T> turn(cx<T> w) {
     if constexpr (J % N == 0) {
         return w;
     } else {
-        constexpr float c = (float)cos_frac(J % N, N), s = -(float)sin_frac(J % N, N);
-        const float2 t = f2_mul(make_float2(c, c), w);
-        return make_float2(fmaf(-s, w.y, t.x), fmaf(s, w.x, t.y));
+        constexpr T c = (T)cos_frac(J % N, N), s = -(T)sin_frac(J % N, N);
+        const cx<T> t = Arith<T>::mulk(c, w);
+        return Arith<T>::mk(fma(-s, w.y, t.x), fma(s, w.x, t.y));
     }
 }
 // m[] = the multipliers of the levels of a radix-R stage (dft_rows) for the root pw[l] * w_TURN_N^(TURN * R/2^(l+1))
 // of level l, where pw[l] = w^(R / 2^(l+1)): rows p of a level are further turns by w_{2^(l+1)}^p.
-template <int R, int N, int TURN, int LEVEL = 0, int P = 0>
-__device__ __forceinline__ void level_multipliers(const float2 *pw, float2 *m) {
+template <typename T, int R, int N, int TURN, int LEVEL = 0, int P = 0>
+__device__ __forceinline__ void level_multipliers(const cx<T> *pw, cx<T> *m) {
     if constexpr ((1 << LEVEL) < R) {
         constexpr int half = LEVEL ? 1 << (LEVEL - 1) : 1, h = R >> (LEVEL + 1);
         if constexpr (P < half) {
             // exponent of w_M, M = N * 2^(LEVEL+1): TURN h / N + P / 2^(LEVEL+1)
             constexpr int M = N << (LEVEL + 1);
-            m[LEVEL ? half + P : 0] = turn<M, (TURN * h << (LEVEL + 1)) + P * N>(pw[LEVEL]);
-            level_multipliers<R, N, TURN, LEVEL, P + 1>(pw, m);
+            m[LEVEL ? half + P : 0] = turn<T, M, (TURN * h << (LEVEL + 1)) + P * N>(pw[LEVEL]);
+            level_multipliers<T, R, N, TURN, LEVEL, P + 1>(pw, m);
         } else {
-            level_multipliers<R, N, TURN, LEVEL + 1, 0>(pw, m);
+            level_multipliers<T, R, N, TURN, LEVEL + 1, 0>(pw, m);
         }
     }
 }
 // pw[l] = w^(R / 2^(l+1)), l = log2 R - 1 .. 0.
-template <int R>
-__device__ __forceinline__ void level_powers(float2 w, float2 *pw) {
+template <typename T, int R>
+__device__ __forceinline__ void level_powers(cx<T> w, cx<T> *pw) {
 #pragma unroll
     for (int l = ilog2(R) - 1; l >= 0; --l) {
         pw[l] = w;
-        if (l) w = square_root_of_unity(w);
+        if (l) w = square_root_of_unity<T>(w);
     }
 }
 
@@ -435,21 +446,21 @@ __device__ __forceinline__ void stage_multipliers(const cx<T> *tab, uint32_t k, 
     if constexpr (kRows<T> == Rows::SINGLE) {
         cx<T> w, pw[ilog2(R)];
         load_rows<T, 1, P>(tab, k, &w);
-        level_powers<R>(w, pw);
-        level_multipliers<R, 1, 0>(pw, m);
+        level_powers<T, R>(w, pw);
+        level_multipliers<T, R, 1, 0>(pw, m);
     } else {
         load_rows<T, stage_rows(R, kRows<T>), P>(tab, k, m);
     }
 }
 // The multipliers of the odd stage (odd_exponent) at table index k.
-template <int RO, int R0, int K1 = 0>
-__device__ __forceinline__ void odd_level_multipliers(const float2 *pw, float2 *w) {
+template <typename T, int RO, int R0, int K1 = 0>
+__device__ __forceinline__ void odd_level_multipliers(const cx<T> *pw, cx<T> *w) {
     if constexpr (K1 < RO) {
-        float2 m[R0 / 2];
-        level_multipliers<R0, RO * R0, K1>(pw, m);
+        cx<T> m[R0 / 2];
+        level_multipliers<T, R0, RO * R0, K1>(pw, m);
 #pragma unroll
         for (int r = 0; r < R0 / 2; ++r) w[RO - 1 + r * RO + K1] = m[r];
-        odd_level_multipliers<RO, R0, K1 + 1>(pw, w);
+        odd_level_multipliers<T, RO, R0, K1 + 1>(pw, w);
     }
 }
 template <typename T, int RO, int R0, int P>
@@ -459,15 +470,15 @@ __device__ __forceinline__ void odd_multipliers(const cx<T> *tab, uint32_t k, cx
         load_rows<T, 1, P>(tab, k, &b);
         if constexpr (R0 > 1) {
             cx<T> pw[ilog2(R0)];
-            level_powers<R0>(b, pw);
-            odd_level_multipliers<RO, R0>(pw, w);
-            b = square_root_of_unity(pw[0]);
+            level_powers<T, R0>(b, pw);
+            odd_level_multipliers<T, RO, R0>(pw, w);
+            b = square_root_of_unity<T>(pw[0]);
         }
         // w[i] = b^(i + 1): even powers by squaring, odd ones by a product
         w[0] = b;
 #pragma unroll
         for (int n = 2; n < RO; ++n)
-            w[n - 1] = n % 2 == 0 ? square_root_of_unity(w[n / 2 - 1]) : Arith<T>::mul(w[n / 2 - 1], w[(n + 1) / 2 - 1]);
+            w[n - 1] = n % 2 == 0 ? square_root_of_unity<T>(w[n / 2 - 1]) : Arith<T>::mul(w[n / 2 - 1], w[(n + 1) / 2 - 1]);
     } else {
         load_rows<T, odd_rows(RO, R0, kRows<T>), P>(tab, k, w);
     }
@@ -478,7 +489,9 @@ __device__ __forceinline__ void odd_multipliers(const cx<T> *tab, uint32_t k, cx
 // of the p are a quarter turn away from the lower half, so R/2 multipliers do. Every
 // butterfly absorbs its multiplier (bfly): a radix-16 stage takes 192 multiply-add slots,
 // where twiddling first (15 products, and 14 more to form the powers) took 284.
-template <typename T, int R, bool INV>
+// With FULL < log2 R only outputs k < 2^FULL are formed: from level FULL on the differences, which
+// the other outputs need, are left out.
+template <typename T, int R, bool INV, int FULL = ilog2(R)>
 __device__ __forceinline__ void dft_rows(cx<T> *v, const cx<T> *w) {
     if constexpr (std::is_same<T, Zp>::value) {
 #pragma unroll
@@ -489,15 +502,20 @@ __device__ __forceinline__ void dft_rows(cx<T> *v, const cx<T> *w) {
         for (int l = 0; (1 << l) < R; ++l) {
             const int h = R >> (l + 1);
 #pragma unroll
-            for (int p = 0; p < (1 << l); ++p) {
+            for (int p = 0; p < (1 << l) && p < (1 << FULL); ++p) {
                 const int half = l ? (1 << (l - 1)) : 1;
                 const cx<T> m = w[l ? half + (p % half) : 0];
-                const bool turn = p >= half;  // a further factor -i (inverse: i)
-                const T c = turn ? m.y : m.x, s = turn ? -m.x : m.y;
+                const bool turned = p >= half;  // a further factor -i (inverse: i)
+                const T c = turned ? m.y : m.x, s = turned ? -m.x : m.y;
                 const int base = bitrev(p, l) * (R >> l);
 #pragma unroll
-                for (int r = 0; r < h; ++r)
-                    Arith<T>::bfly(v[base + r], v[base + r + h], c, INV ? -s : s);
+                for (int r = 0; r < h; ++r) {
+                    if (l < FULL) {
+                        Arith<T>::bfly(v[base + r], v[base + r + h], c, INV ? -s : s);
+                    } else {
+                        v[base + r] = Arith<T>::add_mul(v[base + r], v[base + r + h], c, INV ? -s : s);
+                    }
+                }
             }
         }
         bitrev_regs<T, R>(v);
@@ -813,6 +831,75 @@ __device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32
         fwd_stages<T, LEN, COLS, E, 0, true>(sm, v, tq, col, st);
     } else {
         inv_stages<T, LEN, COLS, E, PL::n - 1, 0, false>(sm, v, tq, col, st);
+    }
+}
+
+// Inverse transform of a strided pass's columns with the pass twiddle w^{-k u} (column u of stride S)
+// in the stages' multipliers: frequency k = k_0 + R_0 (k_1 + ...), and stage i, which sums over k_i with
+// w_{N_i}^{-j k_i}, takes w_{N_i S}^{-(S j + u) k_i} instead, the product of its table's entry and
+// h[i][u]. Twiddling the inputs first cost a product for every value, another to form its twiddle
+// (248 of a 256-point column thread's 866 instructions in single precision) and left the first stage's
+// butterflies without multipliers to absorb. Only outputs of butterfly slots below `need` (of stage 0's
+// radix) are wanted: with few of them stage 0 leaves out the butterflies of the others.
+template <typename T, int LEN, int E, int I>
+__device__ __forceinline__ void col_multipliers(uint32_t tq, int g, const cx<T> *st, cx<T> w, cx<T> *m) {
+    using M = StageMap<T, LEN, E, I>;
+    constexpr StagePlan p = Plan<T, LEN, E>::p;
+    if constexpr (I < p.n - 1) {
+        // the stage table's entry w itself: its only row, or (double precision) row R/4, at least 0
+        constexpr int row = kRows<T> == Rows::SINGLE ? 0 : M::R / 4;
+        const uint32_t j = M::offset(tq, g);
+        const cx<T> *t = st + p.inv[I].off + (p.inv[I].rows == 1 ? j : 2 * (row / 2 * (uint32_t)M::s + j) + row % 2);
+        w = Arith<T>::mul(w, __ldg(t));
+    }
+    cx<T> pw[ilog2(M::R)];
+    level_powers<T, M::R>(w, pw);
+    level_multipliers<T, M::R, 1, 0>(pw, m);
+}
+template <typename T, int LEN, int COLS, int E, int I>
+__device__ __forceinline__ void inv_col_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st,
+                                               const cx<T> *h, uint32_t S, uint32_t need) {
+    using PL = Plan<T, LEN, E>;
+    using M = StageMap<T, LEN, E, I>;
+    const cx<T> hu = __ldg(h + (uint32_t)I * S);
+#pragma unroll
+    for (int g = 0; g < M::groups; ++g) {
+        cx<T> m[level_rows(M::R)];
+        col_multipliers<T, LEN, E, I>(tq, g, st, hu, m);
+        cx<T> *x = v + g * M::R;
+        if constexpr (I == 0 && M::R == 16) {
+            if (need <= 2) dft_rows<T, 16, true, 1>(x, m);
+            else if (need <= 4) dft_rows<T, 16, true, 2>(x, m);
+            else dft_rows<T, 16, true>(x, m);
+        } else if constexpr (I == 0 && M::R == 8 && M::groups == 1) {
+            if (need <= 1) dft_rows<T, 8, true, 0>(x, m);
+            else if (need <= 2) dft_rows<T, 8, true, 1>(x, m);
+            else dft_rows<T, 8, true>(x, m);
+        } else {
+            dft_rows<T, M::R, true>(x, m);
+        }
+    }
+    if constexpr (I > 0) {
+        store_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
+        exchange_barrier<COLS * PL::p.N[I - 1], E>();
+        load_stage<T, LEN, COLS, E, I - 1>(sm, v, tq, col);
+        inv_col_stages<T, LEN, COLS, E, I - 1>(sm, v, tq, col, st, h, S, need);
+    }
+}
+// The inverse transform of column u of a strided pass (pass 0 or 1 of tw; column block blk of nblk,
+// stride S), pass twiddle included: v holds frequencies freq_of(tq) + s*TC on entry, elements
+// elem_of(tq, s) on exit, of which the rows below nrow are wanted.
+template <typename T, int LEN, int COLS, int E, int PASS>
+__device__ __forceinline__ void inverse_columns(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw,
+                                                uint32_t nblk, uint32_t blk, uint32_t S, uint32_t nrow) {
+    using PL = Plan<T, LEN, E>;
+    if constexpr (std::is_same<T, Zp>::value) {
+        pass_twiddles<T, true, E, COLS>(v, tw.iv[PASS], nblk, freq_of<T, LEN, E>(tq), blk, col);
+        cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[PASS]);
+    } else {
+        constexpr uint32_t K = LEN / PL::r0;  // rows of one butterfly slot of stage 0
+        inv_col_stages<T, LEN, COLS, E, PL::n - 1>(sm, v, tq, col, tw.st[PASS], tw.col[PASS] + blk * COLS + col, S,
+                                                   (nrow + K - 1) / K);
     }
 }
 

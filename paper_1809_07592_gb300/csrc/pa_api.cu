@@ -69,6 +69,8 @@ struct RealMode {
     bool seeded = false;
 };
 
+constexpr uint32_t kCtlWords = 4;  // control words in front of a plan's per-key words
+
 // The arguments of an issued batch, kept for its guard step.
 struct PendingBatch {
     bool active = false;
@@ -104,7 +106,7 @@ struct pa_plan {
     uint32_t store_bits = 0;       // storage-precision study: significand bits kept between passes (0: all)
     uint32_t expire_launches = 0;  // test hook: staged launches left whose first wait is made to run out
     uint32_t key_cap = 0;
-    float *h_marg = nullptr;     // pinned: h_cap margins, then the error word
+    uint32_t *h_ctl = nullptr;   // pinned: the control words, then h_cap margins (float bits)
     uint32_t h_cap = 0;
     uint64_t *seed_copy = nullptr;  // the seed bits, kept for an escalation plan
     bool seeded = false;
@@ -236,24 +238,39 @@ int ensure_work(pa_plan_t *p, uint32_t pairs) {
     return PA_OK;
 }
 
+// Per-key words of up to nkeys keys behind the control words (which a larger block takes over). One
+// block, so that one copy brings the error word and the margins back.
 int ensure_keys(pa_plan_t *p, uint32_t nkeys) {
     if (nkeys <= p->key_cap) return PA_OK;
-    if (p->popc) cudaFree(p->popc);
-    if (p->marg) cudaFree(p->marg);
-    p->popc = p->marg = nullptr;
-    p->key_cap = 0;
-    PA_CUDA(cudaMalloc(&p->popc, (size_t)nkeys * sizeof(uint32_t)));
-    PA_CUDA(cudaMalloc(&p->marg, (size_t)nkeys * sizeof(uint32_t)));
+    uint32_t *block = nullptr;
+    cudaError_t e = cudaMalloc(&block, (kCtlWords + 2 * (size_t)nkeys) * sizeof(uint32_t));
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return PA_ENOMEM;
+    }
+    if (e == cudaSuccess && p->err) e = cudaDeviceSynchronize();  // nothing in flight still writes the old control words
+    if (e == cudaSuccess)
+        e = p->err ? cudaMemcpy(block, p->err, kCtlWords * sizeof(uint32_t), cudaMemcpyDeviceToDevice)
+                   : cudaMemset(block, 0, kCtlWords * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // before any stream of the plan uses them
+    if (e != cudaSuccess) {
+        cudaFree(block);
+        return cuda_fail(e, "control words");
+    }
+    cudaFree(p->err);
+    p->err = block;
+    p->marg = block + kCtlWords;
+    p->popc = p->marg + nkeys;
     p->key_cap = nkeys;
     return PA_OK;
 }
 
 int ensure_host(pa_plan_t *p, uint32_t nkeys) {
     if (nkeys <= p->h_cap) return PA_OK;
-    if (p->h_marg) cudaFreeHost(p->h_marg);
-    p->h_marg = nullptr;
+    if (p->h_ctl) cudaFreeHost(p->h_ctl);
+    p->h_ctl = nullptr;
     p->h_cap = 0;
-    PA_CUDA(cudaMallocHost(&p->h_marg, ((size_t)nkeys + 1) * sizeof(float)));
+    PA_CUDA(cudaMallocHost(&p->h_ctl, (kCtlWords + (size_t)nkeys) * sizeof(uint32_t)));
     p->h_cap = nkeys;
     return PA_OK;
 }
@@ -419,11 +436,9 @@ void free_plan(pa_plan_t *p) {
     pa_internal_free_twiddles(&p->tw);
     cudaFree(p->spec);
     cudaFree(p->work);
-    cudaFree(p->popc);
-    cudaFree(p->marg);
-    cudaFree(p->err);
+    cudaFree(p->err);  // with the margins and popcounts behind it
     cudaFree(p->seed_copy);
-    if (p->h_marg) cudaFreeHost(p->h_marg);
+    if (p->h_ctl) cudaFreeHost(p->h_ctl);
     if (p->done) cudaEventDestroy(p->done);
     free_real_mode(p);
     cudaFree(p->stage_keys);
@@ -690,9 +705,6 @@ int plan_create(uint64_t n, uint64_t m, pa_dtype_t dtype, const Geometry *force,
     p->L = geo.L;
     p->geo = geo;
     cudaError_t e = cudaMalloc(&p->spec, (size_t)p->L * elem_bytes(dtype));
-    if (e == cudaSuccess) e = cudaMalloc(&p->err, 4 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemset(p->err, 0, 4 * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);  // zero before any stream of the plan uses them
     if (e != cudaSuccess) {
         free_plan(p);
         if (e == cudaErrorMemoryAllocation) {
@@ -702,8 +714,8 @@ int plan_create(uint64_t n, uint64_t m, pa_dtype_t dtype, const Geometry *force,
         return cuda_fail(e, "cudaMalloc(spec)");
     }
     p->max_chunk_pairs = chunk_pairs_limit(p);
-    int rc = PA_OK;
-    if (!force && tuning_enabled()) {
+    int rc = ensure_keys(p, 64);
+    if (rc == PA_OK && !force && tuning_enabled()) {
         const std::vector<Geometry> cand = geometry_candidates(p->L, dtype, false);
         if (cand.size() > 1) rc = tune_split(p, cand);
     }
@@ -769,9 +781,8 @@ int issue_batch(pa_plan_t *p, const uint64_t *keys_dev, uint32_t nkeys, uint64_t
     else
         rc = run_keys<Zp>(p, keys_dev, nkeys, kstride, out_dev, ostride, p->popc, p->marg, st);
     if (rc != PA_OK) return rc;
-    // the margins and the error word travel back behind the kernels; pa_batch_finish waits for them
-    PA_CUDA(cudaMemcpyAsync(p->h_marg, p->marg, (size_t)nkeys * sizeof(float), cudaMemcpyDeviceToHost, st));
-    PA_CUDA(cudaMemcpyAsync(p->h_marg + nkeys, p->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    // the error word and the margins travel back behind the kernels; pa_batch_finish waits for them
+    PA_CUDA(cudaMemcpyAsync(p->h_ctl, p->err, (kCtlWords + (size_t)nkeys) * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     return PA_OK;
 }
 
@@ -1070,8 +1081,7 @@ int pa_batch_finish(pa_plan_t *p, pa_batch_info_t *info) {
     DeviceGuard g(p->device);
     if (!g.ok) return cuda_fail(cudaGetLastError(), "cudaSetDevice");
     PA_CUDA(cudaEventSynchronize(p->done));
-    uint32_t err_word = 0;
-    std::memcpy(&err_word, p->h_marg + b.nkeys, sizeof(uint32_t));
+    const uint32_t err_word = p->h_ctl[0];
     if (err_word != 0) {
         PA_CUDA(cudaMemset(p->err, 0, sizeof(uint32_t)));
         // this batch's outputs are not valid: bit 0, a bounded device wait ran out; bit 1, a
@@ -1083,7 +1093,8 @@ int pa_batch_finish(pa_plan_t *p, pa_batch_info_t *info) {
     if (info) info->escalated = 0;
     uint32_t escalated = 0;
     for (uint32_t k = 0; k < b.nkeys; ++k) {
-        float mk_ = p->h_marg[k];
+        float mk_;
+        std::memcpy(&mk_, p->h_ctl + kCtlWords + k, sizeof(float));
         int32_t mode = (int32_t)p->dtype;
         if (p->dtype == PA_FP32_GUARD && !(mk_ <= p->guard)) {
             // Recompute this key one mode wider (the guard's escalation): FP32 -> FP64 (-> exact NTT

@@ -220,12 +220,15 @@ __device__ __forceinline__ uint32_t bits_at(const uint64_t *v, uint64_t nbits, u
 template <typename T, int LEN, int COLS, int E, In KIND>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_fwd(FwdArgs in, cx<T> *__restrict__ W, uint64_t L, TwTab<T> tw) {
-    begin_after_previous();
+    const uint32_t *bits = in.bits;
+    const uint2 *parts = in.parts;
+    const BlockDev *blocks = in.blocks;
+    begin_after_previous(bits, parts, blocks, W);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
     const uint32_t S = (uint32_t)(L >> ilog2(LEN)), u = blockIdx.x * COLS + col;
-    const uint32_t x = __ldg(in.bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
+    const uint32_t x = __ldg(bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
     cx<T> v[E];
     if constexpr (KIND == In::KEYS) {
 #pragma unroll
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = Enc<T>::seed(x, re, im, slot_pos<T, LEN, E>(s));
     } else {
-        const uint32_t inside = in.blocks[blockIdx.y].in.mask(tq * S + u);
+        const uint32_t inside = blocks[blockIdx.y].in.mask(tq * S + u);
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, inside, slot_pos<T, LEN, E>(s));
     }
@@ -249,7 +252,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         if (blockIdx.x == 0 && threadIdx.x < 32) {
             uint32_t ca = 0, cb = 0;
             for (uint32_t i = threadIdx.x; i < in.nparts; i += 32) {
-                const uint2 c = in.parts[(uint64_t)blockIdx.y * in.nparts + i];
+                const uint2 c = parts[(uint64_t)blockIdx.y * in.nparts + i];
                 ca += c.x;
                 cb += c.y;
             }
@@ -257,7 +260,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
             cb = __reduce_add_sync(0xffffffffu, cb);
             if (threadIdx.x == 0) {
                 if constexpr (KIND == In::BLOCKS) {
-                    in.popc[in.blocks[blockIdx.y].id] = ca;
+                    in.popc[blocks[blockIdx.y].id] = ca;
                 } else if (in.ppk == 1) {
                     in.popc[blockIdx.y] = ca + cb;
                 } else {
@@ -275,7 +278,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 template <typename T, int LEN, int COLS, int E, bool INV>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_mid(cx<T> *__restrict__ W, uint64_t L, uint32_t S, TwTab<T> tw) {
-    begin_after_previous();
+    begin_after_previous(W);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
@@ -288,9 +291,12 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     cx<T> v[E];
 #pragma unroll
     for (int s = 0; s < E; ++s) v[s] = w[(INV ? f + s * (LEN / E) : elem_of<T, LEN, E>(tq, s)) * S];
-    if (INV) pass_twiddles<T, true, E, COLS>(v, tw.iv[1], gridDim.x, f, blockIdx.x, col);
-    cta_fft<T, LEN, COLS, E, INV>(sm, v, tq, col, tw.st[1]);
-    if (!INV) pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
+    if constexpr (INV) {
+        inverse_columns<T, LEN, COLS, E, 1>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, S, LEN);
+    } else {
+        cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[1]);
+        pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
+    }
     // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
     // addresses in registers through the transform (80 bytes of spills)
     asm volatile("" : "+r"(S));
@@ -304,7 +310,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T>)))
     k_middle(cx<T> *__restrict__ W, cx<T> *__restrict__ spec, uint64_t L, TwTab<T> tw, cx<T> scale) {
-    begin_after_previous();
+    begin_after_previous(W, spec);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t tq = threadIdx.x;
@@ -345,6 +351,12 @@ template <> struct BitsWord<32> { using type = uint32_t; };
 __device__ __forceinline__ float margin_to_float(float x) { return x; }
 __device__ __forceinline__ float margin_to_float(double x) { return __double2float_ru(x); }
 
+// Output bits up to the end of the last word, and the rows t1 of the column block at u0 with t1*S + u0 < end.
+__device__ __forceinline__ uint32_t words_end(uint64_t m) { return (uint32_t)(((m + 63) >> 6) << 6); }
+__device__ __forceinline__ uint32_t output_rows(uint32_t end, uint32_t u0, uint32_t S) {
+    return end > u0 ? (end - u0 + S - 1u) / S : 0u;
+}
+
 // Round, mod 2 and pack the outputs of the level-1 inverse transform of one column
 // (pair form): v holds rows t1 = elem_of(tq, s) of column u = u0 + col, the real part
 // belonging to key ka with ma_bits outputs, the imaginary part to key kb (if has_b) with
@@ -371,10 +383,10 @@ __device__ __forceinline__ void pack_pair_bits(const cx<T> *v, uint32_t tq, uint
     // slot past it.
     const uint32_t S32 = (uint32_t)S, u032 = (uint32_t)u0;
     const uint32_t ma32 = (uint32_t)ma_bits, mb32 = has_b ? (uint32_t)mb_bits : 0u;
-    const uint32_t mwa = (uint32_t)(((ma_bits + 63) >> 6) << 6), mwb = has_b ? (uint32_t)(((mb_bits + 63) >> 6) << 6) : 0u;
+    const uint32_t mwa = words_end(ma_bits), mwb = has_b ? words_end(mb_bits) : 0u;
     const uint32_t mw = mwa > mwb ? mwa : mwb;
     const uint32_t tq0 = (threadIdx.x & ~31u) / COLS;  // the warp's first tq
-    const uint32_t nrow = mw > u032 ? (mw - u032 + S32 - 1u) / S32 : 0u;  // rows t1 with t1*S + u0 < mw
+    const uint32_t nrow = output_rows(mw, u032, S32);
     typename Enc<T>::M ma = 0, mb = 0;
     [[maybe_unused]] float wa_max = 0.f, wb_max = 0.f;  // single precision: largest |w| of each key
     [[maybe_unused]] const float2 half_p = make_float2(0.5f * (float)(popa & 3u), 0.5f * (float)(popb & 3u));
@@ -445,7 +457,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_inv_bits(const cx<T> *__restrict__ W, uint64_t L, uint64_t m, uint32_t nkeys,
                const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, uint64_t *__restrict__ out,
                uint64_t ostride, TwTab<T> tw, const uint64_t *__restrict__ xkeys, uint64_t xstride) {
-    begin_after_previous();
+    begin_after_previous(W, popc, margin_bits, out, xkeys);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     using word_t = typename BitsWord<COLS>::type;
@@ -461,9 +473,9 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)(f + s * (LEN / E)) * S + u];
-    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, f, blockIdx.x, col);
-    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
+    for (int s = 0; s < E; ++s) v[s] = w[(f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u];
+    const uint32_t nrow = output_rows(PACK ? (words_end(m) >> 1) : words_end(m), (uint32_t)u0, (uint32_t)S);
+    inverse_columns<T, LEN, COLS, E, 0>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, (uint32_t)S, nrow);
 
     const uint32_t popa = popc[ka];
     const uint32_t popb = PACK ? popa : (has_b ? popc[kb] : 0u);
@@ -478,10 +490,8 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         using word2_t = typename BitsWord<2 * COLS>::type;
         word2_t *o2 = reinterpret_cast<word2_t *>(out + (uint64_t)ka * ostride);
         const uint32_t S32 = (uint32_t)S, u032 = (uint32_t)u0, m32 = (uint32_t)m;
-        const uint32_t mw = (uint32_t)(((m + 63) >> 6) << 6);  // output bits up to the end of the last word
+        const uint32_t mw = words_end(m);
         const uint32_t tq0 = (threadIdx.x & ~31u) / COLS;
-        const uint32_t half = mw >> 1;  // rows t1 with 2*(t1*S + u0) < mw: t1 < nrow
-        const uint32_t nrow = half > u032 ? (half - u032 + S32 - 1u) / S32 : 0u;
 #pragma unroll
         for (int s = 0; s < E; ++s) {
             const uint32_t t1 = elem_of<T, LEN, E>(tq, s);
@@ -553,7 +563,6 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
                    const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, uint64_t *__restrict__ out,
                    uint64_t ostride, TwTab<float> tw, const uint64_t *__restrict__ xkeys, uint64_t xstride,
                    uint32_t *__restrict__ ctl, uint32_t expire_ns) {
-    begin_after_previous();
     using T = float;
     constexpr int E = 16, COLS = 16;
     static_assert(LEN <= 256 && LEN >= 64, "one tiled copy moves at most 256 rows");
@@ -617,8 +626,8 @@ __global__ void __launch_bounds__(LEN, 768 / LEN)
         const uint64_t u0 = (uint64_t)(t % ncolt) * COLS;
         const uint32_t ka = 2 * pair, kb = ka + 1;
         const bool has_b = kb < nkeys;
-        pass_twiddles<T, true, E, COLS>(v, tw.iv[0], ncolt, freq_of<T, LEN, E>(tq), t % ncolt, col);
-        cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
+        inverse_columns<T, LEN, COLS, E, 0>(sm, v, tq, col, tw, ncolt, t % ncolt, (uint32_t)S,
+                                            output_rows(words_end(m), (uint32_t)u0, (uint32_t)S));
         const uint32_t popa = popc[ka], popb = has_b ? popc[kb] : 0u;
         word_t *oa = reinterpret_cast<word_t *>(out + (uint64_t)ka * ostride);
         word_t *ob = reinterpret_cast<word_t *>(out + (uint64_t)kb * ostride);
@@ -678,7 +687,7 @@ template <typename T, int LEN, int E>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
     k_middle_split(const cx<T> *__restrict__ Wf, cx<T> *__restrict__ Wi, uint64_t L, uint32_t nblocks,
                    uint32_t lgL1, uint32_t lgM, TwTab<T> tw, T inv_L) {
-    begin_after_previous();
+    begin_after_previous(Wf, Wi);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
@@ -758,7 +767,7 @@ template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
     k_middle_real(cx<T> *__restrict__ W, cx<T> *__restrict__ tabs, uint64_t N, uint32_t lgL1, uint32_t lgM,
                   TwTab<T> tw, T scale) {
-    begin_after_previous();
+    begin_after_previous(W, tabs);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
     constexpr uint32_t TC = LEN / E;
@@ -832,7 +841,7 @@ template <typename T, int LEN, int COLS, int E>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_inv_bits_blocks(const cx<T> *__restrict__ W, uint64_t L, const BlockDev *__restrict__ blocks, uint32_t nblocks,
                       const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, TwTab<T> tw) {
-    begin_after_previous();
+    begin_after_previous(W, blocks, popc, margin_bits);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     using word_t = typename BitsWord<COLS>::type;
@@ -848,9 +857,10 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(uint64_t)(f + s * (LEN / E)) * S + u];
-    pass_twiddles<T, true, E, COLS>(v, tw.iv[0], gridDim.x, f, blockIdx.x, col);
-    cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[0]);
+    for (int s = 0; s < E; ++s) v[s] = w[(f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u];
+    const uint32_t mw = words_end(ba_.m > bb_.m ? ba_.m : bb_.m);
+    inverse_columns<T, LEN, COLS, E, 0>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, (uint32_t)S,
+                                        output_rows(mw, (uint32_t)u0, (uint32_t)S));
     const uint32_t popa = popc[ba_.id];
     const uint32_t popb = has_b ? popc[bb_.id] : 0u;
     word_t *oa = reinterpret_cast<word_t *>(ba_.out);

@@ -199,8 +199,10 @@ cudaError_t inv_bits_tma_at(const float2 *W, uint64_t L, uint64_t m, uint32_t nk
     if (ntiles > 0xFFFFFFFFull) return cudaErrorInvalidValue;
     const uint32_t grid = (uint32_t)(ntiles < ctas ? ntiles : ctas);
     *done = true;
-    return launch_chained(kern, grid, LEN, sb, st, map, L, m, nkeys, pairs, popc, margin_bits, out, ostride, tw, xkeys,
-                          xstride, ctl, expire_ns);
+    // an ordinary launch: its tiled copies read what the previous kernel has written
+    kern<<<grid, LEN, sb, st>>>(map, L, m, nkeys, pairs, popc, margin_bits, out, ostride, tw, xkeys, xstride, ctl,
+                                expire_ns);
+    return cudaGetLastError();
 }
 
 template <typename T, int LEN, bool PACK>

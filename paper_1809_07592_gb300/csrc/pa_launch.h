@@ -62,6 +62,7 @@ TwTab<T> tw_tab(const TwLayout &y, const void *mem) {
     for (int p = 0; p < 2; ++p) {
         t.fw[p] = PassTw<T>{m + y.pass[p].a, m + y.pass[p].c, m + y.pass[p].g};
         t.iv[p] = PassTw<T>{m + y.pass[p].ai, m + y.pass[p].ci, m + y.pass[p].gi};
+        t.col[p] = m + y.pass[p].h;
     }
     return t;
 }

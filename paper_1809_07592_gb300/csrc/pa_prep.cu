@@ -234,7 +234,7 @@ __device__ __forceinline__ void store_part(uint2 *parts, uint32_t ca, uint32_t c
 template <int E, bool PACK>
 __global__ void __launch_bounds__(kBitThreads) k_key_bits(KeyBits k, BitShape h, BitScratch out,
                                                           uint32_t *__restrict__ margin_bits) {
-    begin_after_previous();
+    begin_after_previous(k.keys, out.bits, out.parts, margin_bits);
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x, slot = blockIdx.y;
     uint32_t *bits = out.bits + (uint64_t)slot * h.S * h.TC;
     uint32_t ca = 0, cb = 0;
@@ -264,7 +264,7 @@ template <int E>
 __global__ void __launch_bounds__(kBitThreads) k_seed_bits(const uint64_t *__restrict__ seed, uint64_t n, uint64_t m,
                                                            BitShape h0, uint64_t len0, uint32_t *out0, BitShape h1,
                                                            uint64_t len1, uint32_t *out1) {
-    begin_after_previous();
+    begin_after_previous(seed, out0, out1);
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x;
     uint32_t ca, cb;
     if (blockIdx.y == 0) {
@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(kBitThreads) k_seed_bits(const uint64_t *__res
 template <int E>
 __global__ void __launch_bounds__(kBitThreads) k_block_bits(const BlockDev *__restrict__ blocks, BitShape h, uint64_t L,
                                                             BitScratch out, uint32_t *__restrict__ margin_bits) {
-    begin_after_previous();
+    begin_after_previous(blocks, out.bits, out.parts, margin_bits);
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x;
     const BlockDev &b = blocks[blockIdx.y];
     uint32_t ca = 0, cb = 0;
@@ -316,10 +316,10 @@ cudaError_t launch_seed_bits(const uint64_t *seed, uint64_t n, uint64_t m, const
     uint64_t x = parts_count(f.L, f.E);
     if (packed && parts_count(L1, f.E) > x) x = parts_count(L1, f.E);
     const dim3 grid((unsigned)x, packed ? 2 : 1);
-    cudaError_t e;
-    if (f.E == 16) e = launch_chained(k_seed_bits<16>, grid, kBitThreads, 0, st, seed, n, m, h0, f.L, out, h1, L1, packed_out);
-    else e = launch_chained(k_seed_bits<8>, grid, kBitThreads, 0, st, seed, n, m, h0, f.L, out, h1, L1, packed_out);
-    return e;
+    // an ordinary launch: the tables that the passes behind it read may be the kernel's before it
+    if (f.E == 16) k_seed_bits<16><<<grid, kBitThreads, 0, st>>>(seed, n, m, h0, f.L, out, h1, L1, packed_out);
+    else k_seed_bits<8><<<grid, kBitThreads, 0, st>>>(seed, n, m, h0, f.L, out, h1, L1, packed_out);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_block_bits(const BlockDev *blocks, uint32_t nblocks, const BitForm &f, BitScratch scratch,

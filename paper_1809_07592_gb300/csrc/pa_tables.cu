@@ -53,6 +53,12 @@ __device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, Rows kind, bool *
             if (i >= c && i < c + (uint64_t)t.tc * t.cols) return (i - c) / t.cols * ((i - c) % t.cols) * mult;
             if (i >= g && i < g + t.stride) return t.tc * (i - g) * mult;
         }
+        if (complex_) {
+            *neg = false;
+            const StagePlan l = stage_plan(y.len[p], y.E, kind);
+            if (i >= t.h && i < t.h + (uint64_t)l.n * t.stride)
+                return (uint64_t)l.P[(i - t.h) / t.stride] * ((i - t.h) % t.stride) * mult;
+        }
     }
     *neg = false;
     return 0;
@@ -141,10 +147,12 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
         t.tc = (uint32_t)(y.len[p] / y.E);
         t.cols = (uint32_t)strided_cols_of(dtype == PA_FP32_GUARD, y.len[p]);
         t.stride = p == 0 ? g.L >> g.lg1 : (uint64_t)g.inner();
-        t.a = t.ai = take(&y.total, t.tc * (t.stride / t.cols));
-        t.c = t.ci = take(&y.total, (uint64_t)t.tc * t.cols);
-        t.g = t.gi = take(&y.total, t.stride);
-        if (!complex_) {  // residues have no conjugate: the inverse passes read tables of their own
+        t.a = take(&y.total, t.tc * (t.stride / t.cols));
+        t.c = take(&y.total, (uint64_t)t.tc * t.cols);
+        t.g = take(&y.total, t.stride);
+        if (complex_) {
+            t.h = take(&y.total, (uint64_t)stage_plan(y.len[p], y.E, kind).n * t.stride);
+        } else {  // residues have no conjugate: the inverse passes read tables of their own
             t.ai = take(&y.total, t.tc * (t.stride / t.cols));
             t.ci = take(&y.total, (uint64_t)t.tc * t.cols);
             t.gi = take(&y.total, t.stride);

@@ -9,8 +9,10 @@
 //   hi, lo       w_L^e = hi[e >> B] * lo[e mod 2^B], for single powers at any e;
 //   stage tables (one per pass length): the multipliers of every in-CTA butterfly stage
 //                (stage_plan gives the stages, stage_exponent what each row holds);
-//   pass tables  (one set per strided pass): w^{k u} for output k = tq + s*TC of column
-//                u = blk*COLS + col as a[tq][blk] * c[tq][col] * g[u]^s.
+//   pass tables  (one set per strided pass): the pass twiddle w^{k u} of frequency k = f + s*TC in
+//                column u = blk*COLS + col. Forward: a[f][blk] * c[f][col] * g[u]^s. Inverse, complex
+//                arithmetic: it goes into the stages' multipliers (inv_col_stages in fft_core.cuh),
+//                stage i needing h[i][u] = w^{P_i u} beside its stage table.
 #pragma once
 
 #include <cstdint>
@@ -139,7 +141,8 @@ struct PassShape {
     uint32_t tc = 0, cols = 0;  // threads per column, columns per CTA
     uint64_t stride = 0;        // S: distance of a column's elements
     uint64_t a = 0, c = 0, g = 0;      // forward pass tables
-    uint64_t ai = 0, ci = 0, gi = 0;   // inverse ones (the exact transform; else the same)
+    uint64_t ai = 0, ci = 0, gi = 0;   // inverse ones (the exact transform)
+    uint64_t h = 0;                    // complex arithmetic: n tables of `stride` entries for the inverse stages
 };
 struct TwLayout {
     uint64_t L = 0;
