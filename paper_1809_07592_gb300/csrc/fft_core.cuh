@@ -26,20 +26,23 @@
 
 namespace pa {
 
-// First statement of every pass kernel (they are launched with launch_chained): lets the stream's next
-// kernel start once every CTA of this one has begun, then waits until the previous kernel has
-// finished and its writes are visible. A chain of small launches loses the launch latency between
-// its kernels, and a large one's first CTAs fill the SMs that the last wave of the kernel before
-// leaves empty. The arguments are the pointers to data that earlier kernels of the stream write: their
-// values pass through the wait, because a load the compiler takes for one of constant memory
-// (const __restrict__, __ldg) may otherwise move above it.
+// First statement of every pass kernel (they are launched with launch_chained): waits until the stream's
+// previous kernel has finished and its writes are visible, then lets the next kernel start once
+// every CTA of this one has got here. A chain of small launches loses the launch latency between its
+// kernels, and a large one's first CTAs fill the SMs that the last wave of the kernel before leaves
+// empty. What earlier kernels of the stream write is read with fresh() or plain loads, never as
+// constant memory (__ldg, const __restrict__): the compiler and the assembler move constant loads
+// above the wait (then a key read another launch's popcount, and escalated without need), and the
+// pointers pass through the wait for the same reason.
 template <typename... P>
 __device__ __forceinline__ void begin_after_previous(P &...p) {
-    asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const auto behind = [](auto &q) { asm volatile("" : "+l"(q)::"memory"); };
     (behind(p), ...);
 }
+// A load from L2, past L1.
+template <typename V> __device__ __forceinline__ V fresh(const V *p) { return __ldcg(p); }
 
 // Element arithmetic of the transforms. Arith<float> / Arith<double> work on
 // complex numbers (x = real, y = imaginary); Arith<Zp> (zp.cuh) on residues

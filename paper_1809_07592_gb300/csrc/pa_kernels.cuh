@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
     const uint32_t S = (uint32_t)(L >> ilog2(LEN)), u = blockIdx.x * COLS + col;
-    const uint32_t x = __ldg(bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
+    const uint32_t x = fresh(bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
     cx<T> v[E];
     if constexpr (KIND == In::KEYS) {
 #pragma unroll
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         if (blockIdx.x == 0 && threadIdx.x < 32) {
             uint32_t ca = 0, cb = 0;
             for (uint32_t i = threadIdx.x; i < in.nparts; i += 32) {
-                const uint2 c = parts[(uint64_t)blockIdx.y * in.nparts + i];
+                const uint2 c = fresh(parts + (uint64_t)blockIdx.y * in.nparts + i);
                 ca += c.x;
                 cb += c.y;
             }
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(INV ? f + s * (LEN / E) : elem_of<T, LEN, E>(tq, s)) * S];
+    for (int s = 0; s < E; ++s) v[s] = fresh(w + (INV ? f + s * (LEN / E) : elem_of<T, LEN, E>(tq, s)) * S);
     if constexpr (INV) {
         inverse_columns<T, LEN, COLS, E, 1>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, S, LEN);
     } else {
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
 // only, scaled by 1/L, written as the seed spectrum.
 template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T>)))
-    k_middle(cx<T> *__restrict__ W, cx<T> *__restrict__ spec, uint64_t L, TwTab<T> tw, cx<T> scale) {
+    k_middle(cx<T> *__restrict__ W, cx<T> *spec, uint64_t L, TwTab<T> tw, cx<T> scale) {
     begin_after_previous(W, spec);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *sm = reinterpret_cast<cx<T> *>(smem_raw);
@@ -321,10 +321,10 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
     cx<T> v[E];
     if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
+        for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
         cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
+        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
     }
     if constexpr (MODE == 1) {
 #pragma unroll
@@ -473,12 +473,12 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u];
+    for (int s = 0; s < E; ++s) v[s] = fresh(w + (f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u);
     const uint32_t nrow = output_rows(PACK ? (words_end(m) >> 1) : words_end(m), (uint32_t)u0, (uint32_t)S);
     inverse_columns<T, LEN, COLS, E, 0>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, (uint32_t)S, nrow);
 
-    const uint32_t popa = popc[ka];
-    const uint32_t popb = PACK ? popa : (has_b ? popc[kb] : 0u);
+    const uint32_t popa = fresh(popc + ka);
+    const uint32_t popb = PACK ? popa : (has_b ? fresh(popc + kb) : 0u);
     word_t *oa = reinterpret_cast<word_t *>(out + (uint64_t)ka * ostride);
     word_t *ob = reinterpret_cast<word_t *>(out + (uint64_t)kb * ostride);
     if constexpr (PACK) {
@@ -713,10 +713,10 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
         __syncthreads();  // previous use of the scratch is finished
         if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-            for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
+            for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
             cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
         } else {
-            cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
+            cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
         }
         store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
         __syncthreads();
@@ -765,7 +765,7 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
 // MODE 1 builds the tables from the seed slot instead (forward transform and split only).
 template <typename T, int LEN, int E, int MODE>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
-    k_middle_real(cx<T> *__restrict__ W, cx<T> *__restrict__ tabs, uint64_t N, uint32_t lgL1, uint32_t lgM,
+    k_middle_real(cx<T> *__restrict__ W, cx<T> *tabs, uint64_t N, uint32_t lgL1, uint32_t lgM,
                   TwTab<T> tw, T scale) {
     begin_after_previous(W, tabs);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -785,10 +785,10 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     cx<T> v[E];
     if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = wt[elem_of<T, LEN, E>(0, s)];
+        for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
         cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return wt[o]; });
+        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
     }
     store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
     __syncthreads();
@@ -839,7 +839,7 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
 // 2p, imaginary part: block 2p+1), each with its own m and output pointer.
 template <typename T, int LEN, int COLS, int E>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
-    k_inv_bits_blocks(const cx<T> *__restrict__ W, uint64_t L, const BlockDev *__restrict__ blocks, uint32_t nblocks,
+    k_inv_bits_blocks(const cx<T> *__restrict__ W, uint64_t L, const BlockDev *blocks, uint32_t nblocks,
                       const uint32_t *__restrict__ popc, uint32_t *__restrict__ margin_bits, TwTab<T> tw) {
     begin_after_previous(W, blocks, popc, margin_bits);
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -857,12 +857,12 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t f = freq_of<T, LEN, E>(tq);
     cx<T> v[E];
 #pragma unroll
-    for (int s = 0; s < E; ++s) v[s] = w[(f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u];
+    for (int s = 0; s < E; ++s) v[s] = fresh(w + (f + s * (LEN / E)) * (uint32_t)S + (uint32_t)u);
     const uint32_t mw = words_end(ba_.m > bb_.m ? ba_.m : bb_.m);
     inverse_columns<T, LEN, COLS, E, 0>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, (uint32_t)S,
                                         output_rows(mw, (uint32_t)u0, (uint32_t)S));
-    const uint32_t popa = popc[ba_.id];
-    const uint32_t popb = has_b ? popc[bb_.id] : 0u;
+    const uint32_t popa = fresh(popc + ba_.id);
+    const uint32_t popb = has_b ? fresh(popc + bb_.id) : 0u;
     word_t *oa = reinterpret_cast<word_t *>(ba_.out);
     word_t *ob = reinterpret_cast<word_t *>(bb_.out);
     // each block decoded with its own m: the real part is block 2p, the imaginary part block 2p+1

@@ -60,11 +60,11 @@ template <int E, class At>
 __device__ __forceinline__ void bits_rows(const uint32_t *__restrict__ p, uint32_t nbits, At at, uint32_t *w) {
     const uint32_t last = (nbits - 1) >> 5, r = at(0) & 31u;
 #pragma unroll
-    for (int j = 0; j < E; ++j) w[j] = __ldg(p + min(at(j) >> 5, last));
+    for (int j = 0; j < E; ++j) w[j] = fresh(p + min(at(j) >> 5, last));
     if (r) {
         uint32_t hi[E];
 #pragma unroll
-        for (int j = 0; j < E; ++j) hi[j] = __ldg(p + min((at(j) >> 5) + 1, last));
+        for (int j = 0; j < E; ++j) hi[j] = fresh(p + min((at(j) >> 5) + 1, last));
 #pragma unroll
         for (int j = 0; j < E; ++j) w[j] = __funnelshift_r(w[j], hi[j], r);
     }
@@ -131,7 +131,7 @@ struct Rotated {
         };
         bits_rows<E>(p, nbits, at, w);
         const uint32_t r = rot & 31u;
-        const uint32_t first = r ? __ldg(p) & __funnelshift_lc(0xffffffffu, 0u, nbits) : 0u;  // the seed's first 32 bits
+        const uint32_t first = r ? fresh(p) & __funnelshift_lc(0xffffffffu, 0u, nbits) : 0u;  // the seed's first 32 bits
 #pragma unroll
         for (int j = 0; j < E; ++j)  // the 32 positions may wrap to the seed's start
             if (at(j) + 32 > len) w[j] |= first << (len - at(j));
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kBitThreads) k_seed_bits(const uint64_t *__res
 }
 
 template <int E>
-__global__ void __launch_bounds__(kBitThreads) k_block_bits(const BlockDev *__restrict__ blocks, BitShape h, uint64_t L,
+__global__ void __launch_bounds__(kBitThreads) k_block_bits(const BlockDev *blocks, BitShape h, uint64_t L,
                                                             BitScratch out, uint32_t *__restrict__ margin_bits) {
     begin_after_previous(blocks, out.bits, out.parts, margin_bits);
     const uint32_t idx = blockIdx.x * kBitThreads + threadIdx.x;

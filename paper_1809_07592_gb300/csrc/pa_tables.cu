@@ -14,16 +14,21 @@ uint64_t take(uint64_t *total, uint64_t n) {
     return at;
 }
 
+// The stage plans of a layout's passes (worked out once on the host: they are loops over divisions).
+struct StagePlans {
+    StagePlan pass[3];
+};
+
 // Exponent (of w_L, not reduced) of element i of the block; inverse tables of the exact
 // transform come back with *neg set. Padding elements read as w^0.
-__device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, Rows kind, bool *neg) {
+__device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint64_t i, Rows kind, bool *neg) {
     const bool complex_ = kind != Rows::EXACT;
     *neg = false;
     if (i >= y.hi && i < y.hi + y.nhi) return (i - y.hi) << y.B;
     if (i >= y.lo && i < y.lo + y.nlo) return i - y.lo;
     for (int p = 0; p < 3; ++p) {
         if (y.len[p] == 0) continue;
-        const StagePlan l = stage_plan(y.len[p], y.E, kind);
+        const StagePlan &l = plans[p];
         if (i < y.st[p] || i >= y.st[p] + (uint64_t)l.total) continue;
         const int o = (int)(i - y.st[p]);
         for (int j = 0; j < 2 * l.n; ++j) {
@@ -55,7 +60,7 @@ __device__ uint64_t exponent_at(const TwLayout &y, uint64_t i, Rows kind, bool *
         }
         if (complex_) {
             *neg = false;
-            const StagePlan l = stage_plan(y.len[p], y.E, kind);
+            const StagePlan &l = plans[p];
             if (i >= t.h && i < t.h + (uint64_t)l.n * t.stride)
                 return (uint64_t)l.P[(i - t.h) / t.stride] * ((i - t.h) % t.stride) * mult;
         }
@@ -85,10 +90,11 @@ __device__ cx<Zp> root_power<Zp>(uint64_t e, uint64_t, uint64_t w) {
 }
 
 template <typename T>
-__global__ void k_fill_tables(cx<T> *mem, TwLayout y, uint64_t root) {
+__global__ void k_fill_tables(cx<T> *mem, const __grid_constant__ TwLayout y, const __grid_constant__ StagePlans plans,
+                              uint64_t root) {
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < y.total; i += (uint64_t)gridDim.x * blockDim.x) {
         bool neg;
-        uint64_t e = exponent_at(y, i, kRows<T>, &neg) % y.L;
+        uint64_t e = exponent_at(y, plans.pass, i, kRows<T>, &neg) % y.L;
         if (neg && e) e = y.L - e;
         mem[i] = root_power<T>(e, y.L, root);
     }
@@ -162,16 +168,20 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
 }
 
 cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t st) {
+    const Rows kind = dtype == PA_FP32_GUARD ? kRows<float> : dtype == PA_FP64 ? kRows<double> : kRows<Zp>;
+    StagePlans plans{};
+    for (int p = 0; p < 3; ++p)
+        if (y.len[p]) plans.pass[p] = stage_plan(y.len[p], y.E, kind);
     const uint64_t want = (y.total + 255) / 256;
     const unsigned grid = (unsigned)(want < 1216 ? want : 1216);
     if (dtype == PA_FP32_GUARD) {
-        k_fill_tables<float><<<grid, 256, 0, st>>>(static_cast<float2 *>(mem), y, 0);
+        k_fill_tables<float><<<grid, 256, 0, st>>>(static_cast<float2 *>(mem), y, plans, 0);
     } else if (dtype == PA_FP64) {
-        k_fill_tables<double><<<grid, 256, 0, st>>>(static_cast<double2 *>(mem), y, 0);
+        k_fill_tables<double><<<grid, 256, 0, st>>>(static_cast<double2 *>(mem), y, plans, 0);
     } else {
         const uint64_t w = (y.L & (y.L - 1)) ? 0 : zp_root(y.L);  // the exact transform keeps power-of-two lengths
         if (!w) return cudaErrorInvalidValue;
-        k_fill_tables<Zp><<<grid, 256, 0, st>>>(static_cast<unsigned long long *>(mem), y, w);
+        k_fill_tables<Zp><<<grid, 256, 0, st>>>(static_cast<unsigned long long *>(mem), y, plans, w);
     }
     return cudaGetLastError();
 }
