@@ -67,7 +67,9 @@ typedef struct CUstream_st *pa_stream_t;
  *   PA_FP32_GUARD  single-precision complex FFTs; every key's rounding margin
  *                  max_i |v_i - rint(v_i)| is checked, and a key whose margin
  *                  exceeds 0.25 is recomputed in FP64.
- *   PA_NTT64       exact number-theoretic transform modulo p = 2^64 - 2^32 + 1.
+ *   PA_NTT64       exact number-theoretic transform: modulo the prime 7 * 2^26 + 1 for
+ *                  transform lengths up to 2^26 (it exceeds every count the hash can form,
+ *                  n <= 2^27, so the counts come out exactly), modulo 2^64 - 2^32 + 1 beyond.
  * The output bits are the same in every mode.
  */
 typedef enum { PA_FP64 = 0, PA_FP32_GUARD = 1, PA_NTT64 = 2 } pa_dtype_t;

@@ -291,6 +291,7 @@ template <> struct Arith<double> : ComplexArith<double> {};
 }  // namespace pa
 
 #include "zp.cuh"
+#include "zq.cuh"
 
 namespace pa {
 
@@ -298,7 +299,14 @@ namespace pa {
 // the whole and quarter turns without multiplications.
 template <typename T, int J, bool INV>
 __device__ __forceinline__ void bfly32(cx<T> &a, cx<T> &b) {
-    if constexpr (J == 0) {
+    if constexpr (std::is_same<T, Zq>::value) {
+        constexpr uint32_t w = zq_root32(INV ? (32 - J) % 32 : J), wq = zq_quotient(w);
+        if constexpr (J == 0) {
+            Arith<Zq>::bfly1(a, b);
+        } else {
+            Arith<Zq>::bfly(a, b, make_uint2(w, wq));
+        }
+    } else if constexpr (J == 0) {
         const cx<T> p = Arith<T>::add(a, b);
         b = Arith<T>::sub(a, b);
         a = p;
@@ -381,7 +389,18 @@ __device__ __forceinline__ void load_pair(const unsigned long long *p, unsigned 
     b = q.y;
 }
 template <typename T>
-constexpr Rows kRows = std::is_same<T, Zp>::value ? Rows::EXACT : std::is_same<T, float>::value ? Rows::SINGLE : Rows::DOUBLE;
+constexpr Rows kRows = std::is_same<T, Zp>::value      ? Rows::EXACT
+                       : std::is_same<T, Zq>::value    ? Rows::LEVELS
+                       : std::is_same<T, float>::value ? Rows::SINGLE
+                                                       : Rows::DOUBLE;
+// Multipliers a thread holds for a radix-R stage.
+template <typename T>
+constexpr int multipliers(int R) { return is_complex(kRows<T>) ? level_rows(R) : R - 1; }
+__device__ __forceinline__ void load_pair(const uint2 *p, uint2 &a, uint2 &b) {
+    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(p));
+    a = make_uint2(q.x, q.y);
+    b = make_uint2(q.z, q.w);
+}
 // The ROWS multipliers at index k of a table of P butterflies.
 template <typename T, int ROWS, int P>
 __device__ __forceinline__ void load_rows(const cx<T> *tab, uint32_t k, cx<T> *w) {
@@ -500,6 +519,17 @@ __device__ __forceinline__ void dft_rows(cx<T> *v, const cx<T> *w) {
 #pragma unroll
         for (int r = 1; r < R; ++r) v[r] = Arith<T>::mul(v[r], w[r - 1]);
         dft<T, R, INV>(v);
+    } else if constexpr (std::is_same<T, Zq>::value) {
+#pragma unroll
+        for (int l = 0; (1 << l) < R; ++l) {
+#pragma unroll
+            for (int p = 0; p < (1 << l); ++p) {
+                const int h = R >> (l + 1), base = bitrev(p, l) * (R >> l);
+#pragma unroll
+                for (int r = 0; r < h; ++r) Arith<Zq>::bfly(v[base + r], v[base + r + h], w[(1 << l) - 1 + p]);
+            }
+        }
+        bitrev_regs<T, R>(v);
     } else {
 #pragma unroll
         for (int l = 0; (1 << l) < R; ++l) {
@@ -639,6 +669,15 @@ __device__ __forceinline__ void dft_comp_rows(cx<T> *x, const cx<T> *tab, uint32
 template <typename T, bool INV, int N, int COLS>
 __device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint32_t nblk, uint32_t tq, uint32_t blk,
                                               uint32_t col) {
+    if constexpr (std::is_same<T, Zq>::value) {  // multipliers do not multiply: one product per table
+        const uint32_t S = nblk * COLS, u = blk * COLS + col;
+        const cx<T> p = __ldg(t.a + (uint64_t)tq * S + u);
+#pragma unroll
+        for (int s = 0; s < N; ++s) {
+            if (s) v[s] = Arith<T>::mul(v[s], __ldg(t.g + (uint64_t)s * S + u));
+            v[s] = Arith<T>::mul(v[s], p);
+        }
+    } else {
     cx<T> w = Arith<T>::mul(__ldg(t.a + (uint64_t)tq * nblk + blk), __ldg(t.c + tq * COLS + col));
     cx<T> g = __ldg(t.g + blk * COLS + col);
     if constexpr (INV && !std::is_same<T, Zp>::value) {
@@ -649,6 +688,7 @@ __device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint
     for (int r = 0; r < N; ++r) {
         v[r] = Arith<T>::mul(v[r], w);
         if (r + 1 < N) w = Arith<T>::mul(w, g);
+    }
     }
 }
 
@@ -785,7 +825,7 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
         if constexpr (row.rows == 0) {
             dft<T, M::R, INV>(v + g * M::R);
         } else {
-            cx<T> w[kRows<T> == Rows::EXACT ? M::R - 1 : level_rows(M::R)];
+            cx<T> w[multipliers<T>(M::R)];
             stage_multipliers<T, M::R, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
             dft_rows<T, M::R, INV>(v + g * M::R, w);
         }
@@ -896,7 +936,7 @@ template <typename T, int LEN, int COLS, int E, int PASS>
 __device__ __forceinline__ void inverse_columns(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const TwTab<T> &tw,
                                                 uint32_t nblk, uint32_t blk, uint32_t S, uint32_t nrow) {
     using PL = Plan<T, LEN, E>;
-    if constexpr (std::is_same<T, Zp>::value) {
+    if constexpr (!is_complex(kRows<T>)) {
         pass_twiddles<T, true, E, COLS>(v, tw.iv[PASS], nblk, freq_of<T, LEN, E>(tq), blk, col);
         cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[PASS]);
     } else {

@@ -184,6 +184,10 @@ template <typename T> cx<T> spec_scale(uint64_t L) {
     return s;
 }
 template <> cx<Zp> spec_scale<Zp>(uint64_t L) { return zp_pow_host(L, kP - 2); }
+template <> cx<Zq> spec_scale<Zq>(uint64_t L) {
+    const uint32_t w = zq_pow((uint32_t)L, kQ - 2);
+    return make_uint2(w, zq_quotient(w));
+}
 template <typename T> cx<T> one() {
     cx<T> s;
     s.x = 1;
@@ -191,9 +195,14 @@ template <typename T> cx<T> one() {
     return s;
 }
 template <> cx<Zp> one<Zp>() { return 1; }
+template <> cx<Zq> one<Zq>() { return make_uint2(1u, 0u); }
 
-int elems_per_thread(pa_dtype_t d) {
-    return d == PA_FP32_GUARD ? Shape<float>::E : d == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
+// Calls f(T()) for the arithmetic a plan's kernels run in.
+template <typename F> auto with_type(const pa_plan_t *p, F &&f) {
+    if (p->dtype == PA_FP32_GUARD) return f(float());
+    if (p->dtype == PA_FP64) return f(double());
+    if (narrow_exact(p->dtype, p->L)) return f(Zq());
+    return f(Zp());
 }
 
 // Values of `pairs` slots; the transposed input bits and partial popcounts of the first pass follow them.
@@ -207,7 +216,7 @@ uint64_t real_slots(const pa_plan_t *p, const RealMode *r) {
 
 BitScratch bit_scratch(const pa_plan_t *p, uint64_t L, uint64_t slots) {
     return bit_scratch_at(static_cast<unsigned char *>(p->work) + work_bytes(p, p->work_pairs), L,
-                          elems_per_thread(p->dtype), slots);
+                          values_per_thread(p->dtype, p->L), slots);
 }
 
 int ensure_work(pa_plan_t *p, uint32_t pairs) {
@@ -218,7 +227,7 @@ int ensure_work(pa_plan_t *p, uint32_t pairs) {
         p->work_pairs = 0;
         if (e != cudaSuccess) return cuda_fail(e, "cudaFree(work)");
     }
-    const int E = elems_per_thread(p->dtype);
+    const int E = values_per_thread(p->dtype, p->L);
     size_t scratch = bit_scratch_bytes(p->L, E, pairs);
     if (p->real) {
         uint64_t slots = (uint64_t)pairs * p->L / p->real->geo.L;
@@ -322,7 +331,7 @@ int run_seed(pa_plan_t *p, const uint64_t *seed, cudaStream_t st) {
     }
     { Timed t_(p, K_MIDDLE_SPEC, st); PA_CUDA(launch_middle<T>(g.ro, g.lgI, 1, W, spec, p->L, 1, tw, spec_scale<T>(p->L), st)); }
     PA_CUDA(round_stored<T>(p, spec, 1, st));
-    if constexpr (!std::is_same<T, Zp>::value) {
+    if constexpr (!kExact<T>) {
         if (RealMode *r = p->real) {  // seed tables: packed seed transform, then the bin-pair split
             const TwTab<T> twr = tw_tab<T>(r->tw.lay, r->tw.mem);
             const Geometry &h = r->geo;
@@ -377,7 +386,7 @@ uint32_t take_expire(pa_plan_t *p) {
 template <typename T>
 int run_keys(pa_plan_t *p, const uint64_t *keys, uint32_t nkeys, uint64_t kstride, uint64_t *out,
              uint64_t ostride, uint32_t *popc, uint32_t *marg, cudaStream_t st) {
-    if constexpr (!std::is_same<T, Zp>::value) {
+    if constexpr (!kExact<T>) {
         // A lone key (alone, or the last of an odd batch) takes the half-length form; key
         // pairs stay in the pair form (measured 28 % faster per key than the half-length form).
         if (p->real && p->real->seeded && (nkeys & 1) && p->store_bits == 0) {
@@ -553,9 +562,7 @@ int tune_split(pa_plan_t *p, const std::vector<Geometry> &cand) {
         p->geo = cand[i];
         if ((rc = pa_internal_twiddles(p->geo, p->dtype, &p->tw)) != PA_OK) return fail(rc);
         float ms = 0.f;
-        rc = (p->dtype == PA_FP32_GUARD) ? time_split<float>(p, nkeys, keys, kw, out, ow, st, a, b, &ms)
-             : (p->dtype == PA_FP64)     ? time_split<double>(p, nkeys, keys, kw, out, ow, st, a, b, &ms)
-                                         : time_split<Zp>(p, nkeys, keys, kw, out, ow, st, a, b, &ms);
+        rc = with_type(p, [&](auto t) { return time_split<decltype(t)>(p, nkeys, keys, kw, out, ow, st, a, b, &ms); });
         pa_internal_free_twiddles(&p->tw);
         if (rc != PA_OK) return fail(rc);
         if (i == 0 || ms < best) {
@@ -774,12 +781,9 @@ int issue_batch(pa_plan_t *p, const uint64_t *keys_dev, uint32_t nkeys, uint64_t
     // The plan's work buffers are shared by its batches: a batch issued on another stream
     // than the previous one waits for it (a no-op on the same stream).
     PA_CUDA(cudaStreamWaitEvent(st, p->done, 0));
-    if (p->dtype == PA_FP32_GUARD)
-        rc = run_keys<float>(p, keys_dev, nkeys, kstride, out_dev, ostride, p->popc, p->marg, st);
-    else if (p->dtype == PA_FP64)
-        rc = run_keys<double>(p, keys_dev, nkeys, kstride, out_dev, ostride, p->popc, p->marg, st);
-    else
-        rc = run_keys<Zp>(p, keys_dev, nkeys, kstride, out_dev, ostride, p->popc, p->marg, st);
+    rc = with_type(p, [&](auto t) {
+        return run_keys<decltype(t)>(p, keys_dev, nkeys, kstride, out_dev, ostride, p->popc, p->marg, st);
+    });
     if (rc != PA_OK) return rc;
     // the error word and the margins travel back behind the kernels; pa_batch_finish waits for them
     PA_CUDA(cudaMemcpyAsync(p->h_ctl, p->err, (kCtlWords + (size_t)nkeys) * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
@@ -986,9 +990,7 @@ int pa_set_seed(pa_plan_t *p, const uint64_t *seed_dev, uint64_t seed_bits, pa_s
     if (!p->seed_copy) PA_CUDA(cudaMalloc(&p->seed_copy, sw * sizeof(uint64_t)));
     PA_CUDA(cudaMemcpyAsync(p->seed_copy, seed_dev, sw * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st));
     if (p->real) p->real->seeded = false;
-    rc = (p->dtype == PA_FP32_GUARD) ? run_seed<float>(p, p->seed_copy, st)
-         : (p->dtype == PA_FP64)     ? run_seed<double>(p, p->seed_copy, st)
-                                     : run_seed<Zp>(p, p->seed_copy, st);
+    rc = with_type(p, [&](auto t) { return run_seed<decltype(t)>(p, p->seed_copy, st); });
     if (rc != PA_OK) return rc;
     if (p->real) p->real->seeded = true;
     PA_CUDA(cudaEventRecord(p->done, st));

@@ -31,6 +31,11 @@ struct Geometry {
     }
 };
 
+// Whether the exact transform of length L runs modulo the word-sized prime of zq.cuh (lengths up to
+// 2^26, where it has roots of unity) instead of the 64-bit one, and the values a thread holds.
+inline bool narrow_exact(pa_dtype_t dtype, uint64_t L) { return dtype == PA_NTT64 && L <= (1ull << 26); }
+inline int values_per_thread(pa_dtype_t dtype, uint64_t L) { return dtype == PA_FP32_GUARD || narrow_exact(dtype, L) ? 16 : 8; }
+
 // Every valid split of length L for the arithmetic `dtype` (split = the
 // innermost pass is the two-row Eq. 5-10 kernel of the uneven batch).
 std::vector<Geometry> geometry_candidates(uint64_t L, pa_dtype_t dtype, bool split);

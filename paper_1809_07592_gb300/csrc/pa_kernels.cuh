@@ -138,6 +138,27 @@ template <> struct Enc<Zp> {
 };
 
 // ---------------------------------------------------------------------------
+template <> struct Enc<Zq> {
+    using E = cx<Zq>;
+    using M = float;
+    static __device__ __forceinline__ E keys(uint32_t x, int j) { return make_uint2((x >> j) & 1u, (x >> (16 + j)) & 1u); }
+    static __device__ __forceinline__ E seed(uint32_t x, uint32_t, uint32_t, int j) { return make_uint2((x >> j) & 1u, 0u); }
+    static __device__ __forceinline__ void decode2(E v, uint32_t, uint32_t, bool valid_a, bool valid_b, bool &bit_a,
+                                                   bool &bit_b, M &, M &) {
+        bit_a = valid_a && (Arith<Zq>::canonical(v.x) & 1u);
+        bit_b = valid_b && (Arith<Zq>::canonical(v.y) & 1u);
+    }
+};
+// A value of the seed's spectrum as the product takes it.
+template <typename T>
+__device__ __forceinline__ cx<T> spectrum_value(cx<T> v) {
+    if constexpr (std::is_same<T, Zq>::value) {
+        return Arith<Zq>::multiplier(v);
+    } else {
+        return v;
+    }
+}
+
 // Input bits of the level-1 forward passes. Thread (tq, col) of column block blk transforms the
 // rows tq + j*TC, j < E, of column blk*COLS + col, whose bits lie E/32 of a row apart in memory:
 // a CTA would touch LEN lines for LEN words of 16 bits each (32 wavefronts per load and warp). The
@@ -328,7 +349,7 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
     }
     if constexpr (MODE == 1) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) spt[s * (LEN / E)] = Arith<T>::mul(v[s], scale);
+        for (int s = 0; s < E; ++s) spt[s * (LEN / E)] = spectrum_value<T>(Arith<T>::mul(v[s], scale));
     } else {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = Arith<T>::mul(v[s], spt[s * (LEN / E)]);

@@ -60,7 +60,7 @@ cudaError_t launch_fwd(int lgLEN, In kind, const FwdArgs &in, uint32_t slots, cx
         constexpr int LEN = decltype(c)::value;
         if (kind == In::KEYS) return fwd_at<T, LEN, In::KEYS>(in, slots, W, L, tw, st);
         if (kind == In::SEED) return fwd_at<T, LEN, In::SEED>(in, slots, W, L, tw, st);
-        if constexpr (!std::is_same<T, Zp>::value) {  // residues have no key+seed form
+        if constexpr (!kExact<T>) {  // residues have no key+seed form
             return fwd_at<T, LEN, In::BLOCKS>(in, slots, W, L, tw, st);
         } else {
             return cudaErrorInvalidValue;
@@ -140,7 +140,7 @@ cudaError_t launch_middle(int ro, int lg, int mode, cx<T> *W, cx<T> *spec, uint6
             return middle_at<T, decltype(c)::value>(mode, W, spec, L, pairs, tw, scale, st);
         });
     }
-    if constexpr (std::is_same<T, Zp>::value) {
+    if constexpr (kExact<T>) {
         return cudaErrorInvalidValue;  // the exact transform keeps power-of-two lengths
     } else {
         if (ro == 3) return launch_middle_odd<T, 3>(lg, mode, W, spec, L, pairs, tw, scale, st);
@@ -234,7 +234,7 @@ cudaError_t launch_inv_bits(int lgLEN, const cx<T> *W, uint64_t L, uint64_t m, u
                             uint64_t xstride, bool pack, uint32_t *ctl, uint32_t expire_ns) {
     return by_len<kMinLgStrided, kMaxLgStrided>(lgLEN, [&](auto c) {
         constexpr int LEN = decltype(c)::value;
-        if constexpr (!std::is_same<T, Zp>::value) {
+        if constexpr (!kExact<T>) {
             if (pack)
                 return inv_bits_at<T, LEN, true>(W, L, m, nkeys, popc, margin_bits, out, ostride, pairs, tw, st,
                                                  xkeys, xstride, nullptr, 0u);

@@ -41,13 +41,15 @@ template <typename T> struct Shape;
 template <> struct Shape<float> { static constexpr int E = 16, COLS = 16; };
 template <> struct Shape<double> { static constexpr int E = 8, COLS = 8; };
 template <> struct Shape<Zp> { static constexpr int E = 8, COLS = 8; };
-// Columns per CTA of a strided pass of length LEN: single precision takes 8 instead of 16 at
+template <> struct Shape<Zq> { static constexpr int E = 16, COLS = 16; };
+template <typename T> constexpr bool kExact = std::is_same<T, Zp>::value || std::is_same<T, Zq>::value;
+// Columns per CTA of a strided pass of length LEN: the types with 16 values per thread take 8 instead of 16 at
 // LEN = 1024 (512 threads, two CTAs per SM instead of one).
-constexpr int strided_cols_of(bool single, int len) { return single ? (len >= 1024 ? 8 : Shape<float>::COLS) : 8; }
+constexpr int strided_cols_of(bool wide, int len) { return wide ? (len >= 1024 ? 8 : 16) : 8; }
 template <typename T, int LEN>
 constexpr int strided_cols() {
-    static_assert(Shape<double>::COLS == 8 && Shape<Zp>::COLS == 8, "one width for the 64-bit types");
-    return strided_cols_of(std::is_same<T, float>::value, LEN);
+    static_assert(Shape<T>::COLS == (Shape<T>::E == 16 ? 16 : 8), "the width goes with the values per thread");
+    return strided_cols_of(Shape<T>::E == 16, LEN);
 }
 
 // The kernels' view of a transform's tables at mem (layout y).
@@ -76,6 +78,7 @@ template <typename T> struct MaxLgMiddle;
 template <> struct MaxLgMiddle<float> { static constexpr int v = 14; };
 template <> struct MaxLgMiddle<double> { static constexpr int v = 13; };
 template <> struct MaxLgMiddle<Zp> { static constexpr int v = 13; };
+template <> struct MaxLgMiddle<Zq> { static constexpr int v = 13; };
 constexpr int kMinLgMiddle = 6;
 
 // Which elements of a rotated seed are inside the seed: element t holds a seed value iff t < M or
@@ -142,7 +145,7 @@ struct BitForm {
 };
 template <typename T>
 BitForm bit_form(int lgLEN, uint64_t L) {
-    return BitForm{L, lgLEN, Shape<T>::E, strided_cols_of(std::is_same<T, float>::value, 1 << lgLEN)};
+    return BitForm{L, lgLEN, Shape<T>::E, strided_cols_of(Shape<T>::E == 16, 1 << lgLEN)};
 }
 
 // Transpose input bits (layout: see "Input bits" in pa_kernels.cuh). The key forms also leave

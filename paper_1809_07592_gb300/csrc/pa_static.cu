@@ -34,7 +34,7 @@ namespace {
 // plus twiddle tables and per-key counters.
 constexpr int kMaxLgL = 21;
 constexpr size_t kSlotBytes = ((size_t)1 << kMaxLgL) * 16;        // 32 MiB
-constexpr size_t kTableBytes = (size_t)960 << 10;                     // twiddle tables (at most 720 KiB are used)
+constexpr size_t kTableBytes = (size_t)960 << 10;                     // FP64 twiddle tables (at most 860 KiB are used)
 constexpr size_t kBitBytes = ((size_t)1 << 20) + (64u << 10);         // transposed input bits and partial popcounts
 constexpr size_t kScratchBytes = 2 * kSlotBytes + ((size_t)1 << 20) + kBitBytes;  // 1 MiB: tables and counters
 
@@ -110,11 +110,14 @@ float static_guard() {
 template <typename T> cx<T> scale_of(uint64_t L);
 template <> cx<float> scale_of<float>(uint64_t L) { return make_float2((float)(kSpecScale / (double)L), 0.f); }
 template <> cx<double> scale_of<double>(uint64_t L) { return make_double2(kSpecScale / (double)L, 0.0); }
-template <> cx<Zp> scale_of<Zp>(uint64_t L) { return zp_pow_host(L, kP - 2); }
+template <> cx<Zq> scale_of<Zq>(uint64_t L) {
+    const uint32_t w = zq_pow((uint32_t)L, kQ - 2);
+    return make_uint2(w, zq_quotient(w));
+}
 template <typename T> cx<T> unit();
 template <> cx<float> unit<float>() { return make_float2(1.f, 0.f); }
 template <> cx<double> unit<double>() { return make_double2(1.0, 0.0); }
-template <> cx<Zp> unit<Zp>() { return 1ull; }
+template <> cx<Zq> unit<Zq>() { return make_uint2(0u, 0u); }
 
 #define STATIC_CUDA(x)                               \
     do {                                             \
@@ -143,9 +146,12 @@ int run_static(unsigned char *base, int lgL, uint64_t n, uint64_t m, const uint6
     geo.lg1 = lg1;
     geo.lgI = lg2;
     const TwLayout lay = tw_layout(geo, dtype);
-    if (lay.total * sizeof(cx<T>) > kTableBytes) return PA_EUNSUPPORTED;
-    STATIC_CUDA(tw_fill(lay, dtype, tail, st));
-    const TwTab<T> tw = tw_tab<T>(lay, tail);
+    // 8-byte elements use half of each slot: their tables take the upper half of the spectrum's
+    constexpr bool half = sizeof(cx<T>) == 8;
+    unsigned char *tables = half ? base + kSlotBytes + kSlotBytes / 2 : tail;
+    if (lay.total * sizeof(cx<T>) > (half ? kSlotBytes / 2 : kTableBytes)) return PA_EUNSUPPORTED;
+    STATIC_CUDA(tw_fill(lay, dtype, tables, st));
+    const TwTab<T> tw = tw_tab<T>(lay, tables);
     if (bit_scratch_bytes(L, Shape<T>::E, 1) > kBitBytes) return PA_EUNSUPPORTED;
     const BitScratch bits = bit_scratch_at(tail + ((size_t)1 << 20), L, Shape<T>::E, 1);
     FwdArgs in = seed_args<T>(bits.bits, n, m, false, L);
@@ -184,7 +190,7 @@ extern "C" int pa_hash_static(uint64_t n, uint64_t m, pa_dtype_t dtype, const ui
     uint32_t *marg = reinterpret_cast<uint32_t *>(base + 2 * kSlotBytes + kTableBytes) + 2;
 
     if (dtype == PA_NTT64) {
-        rc = run_static<Zp>(base, lgL, n, m, seed_dev, keys_dev, nkeys, key_stride_words, out_dev,
+        rc = run_static<Zq>(base, lgL, n, m, seed_dev, keys_dev, nkeys, key_stride_words, out_dev,
                             out_stride_words, st);
         if (rc == PA_OK && margin) margin[0] = 0.f;
         return rc;
@@ -212,7 +218,7 @@ extern "C" int pa_hash_static(uint64_t n, uint64_t m, pa_dtype_t dtype, const ui
             return PA_OK;
         }
         if (mode == PA_FP64) {  // FP64 failed its guard: recompute exactly
-            rc = run_static<Zp>(base, lgL, n, m, seed_dev, keys_dev, nkeys, key_stride_words, out_dev,
+            rc = run_static<Zq>(base, lgL, n, m, seed_dev, keys_dev, nkeys, key_stride_words, out_dev,
                                 out_stride_words, st);
             if (rc == PA_OK && margin) margin[0] = 0.f;
             return rc;

@@ -22,7 +22,7 @@ struct StagePlans {
 // Exponent (of w_L, not reduced) of element i of the block; inverse tables of the exact
 // transform come back with *neg set. Padding elements read as w^0.
 __device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint64_t i, Rows kind, bool *neg) {
-    const bool complex_ = kind != Rows::EXACT;
+    const bool complex_ = is_complex(kind);
     *neg = false;
     if (i >= y.hi && i < y.hi + y.nhi) return (i - y.hi) << y.B;
     if (i >= y.lo && i < y.lo + y.nlo) return i - y.lo;
@@ -54,6 +54,12 @@ __device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint6
         for (int inv = 0; inv < (complex_ ? 1 : 2); ++inv) {
             const uint64_t a = inv ? t.ai : t.a, c = inv ? t.ci : t.c, g = inv ? t.gi : t.g;
             *neg = inv != 0;
+            if (kind == Rows::LEVELS) {
+                if (i >= a && i < a + t.tc * t.stride) return (i - a) / t.stride * ((i - a) % t.stride) * mult;
+                if (i >= g && i < g + (uint64_t)y.E * t.stride)
+                    return t.tc * ((i - g) / t.stride) * ((i - g) % t.stride) * mult;
+                continue;
+            }
             if (i >= a && i < a + t.tc * nblk) return (i - a) / nblk * ((i - a) % nblk) * t.cols * mult;
             if (i >= c && i < c + (uint64_t)t.tc * t.cols) return (i - c) / t.cols * ((i - c) % t.cols) * mult;
             if (i >= g && i < g + t.stride) return t.tc * (i - g) * mult;
@@ -87,6 +93,12 @@ __device__ cx<Zp> root_power<Zp>(uint64_t e, uint64_t, uint64_t w) {
         b = zp_mul(b, b);
     }
     return r;
+}
+
+template <>
+__device__ cx<Zq> root_power<Zq>(uint64_t e, uint64_t, uint64_t w) {
+    const uint32_t r = zq_pow((uint32_t)w, e);
+    return make_uint2(r, zq_quotient(r));
 }
 
 template <typename T>
@@ -129,9 +141,16 @@ uint64_t zp_pow_host(uint64_t a, uint64_t e) {
     return r;
 }
 
+static Rows rows_of(pa_dtype_t dtype, uint64_t L) {
+    return dtype == PA_FP32_GUARD       ? kRows<float>
+           : dtype == PA_FP64           ? kRows<double>
+           : narrow_exact(dtype, L) ? kRows<Zq>
+                                        : kRows<Zp>;
+}
+
 TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
-    const Rows kind = dtype == PA_FP32_GUARD ? kRows<float> : dtype == PA_FP64 ? kRows<double> : kRows<Zp>;
-    const bool complex_ = kind != Rows::EXACT;
+    const Rows kind = rows_of(dtype, g.L);
+    const bool complex_ = is_complex(kind);
     TwLayout y;
     y.L = g.L;
     int lgL = 0;
@@ -139,7 +158,7 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
     y.B = (uint32_t)(lgL + 1) / 2;
     y.nlo = 1ull << y.B;
     y.nhi = (g.L + y.nlo - 1) >> y.B;
-    y.E = dtype == PA_FP32_GUARD ? Shape<float>::E : dtype == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
+    y.E = values_per_thread(dtype, g.L);
     y.len[0] = 1 << g.lg1;
     y.len[1] = g.lgM ? 1 << g.lgM : 0;
     y.len[2] = (int)g.inner();
@@ -151,8 +170,15 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
         if (!y.len[p]) continue;
         PassShape &t = y.pass[p];
         t.tc = (uint32_t)(y.len[p] / y.E);
-        t.cols = (uint32_t)strided_cols_of(dtype == PA_FP32_GUARD, y.len[p]);
+        t.cols = (uint32_t)strided_cols_of(y.E == 16, y.len[p]);
         t.stride = p == 0 ? g.L >> g.lg1 : (uint64_t)g.inner();
+        if (kind == Rows::LEVELS) {
+            t.a = take(&y.total, t.tc * t.stride);
+            t.g = take(&y.total, (uint64_t)y.E * t.stride);
+            t.ai = take(&y.total, t.tc * t.stride);
+            t.gi = take(&y.total, (uint64_t)y.E * t.stride);
+            continue;
+        }
         t.a = take(&y.total, t.tc * (t.stride / t.cols));
         t.c = take(&y.total, (uint64_t)t.tc * t.cols);
         t.g = take(&y.total, t.stride);
@@ -168,7 +194,7 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
 }
 
 cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t st) {
-    const Rows kind = dtype == PA_FP32_GUARD ? kRows<float> : dtype == PA_FP64 ? kRows<double> : kRows<Zp>;
+    const Rows kind = rows_of(dtype, y.L);
     StagePlans plans{};
     for (int p = 0; p < 3; ++p)
         if (y.len[p]) plans.pass[p] = stage_plan(y.len[p], y.E, kind);
@@ -178,6 +204,9 @@ cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t
         k_fill_tables<float><<<grid, 256, 0, st>>>(static_cast<float2 *>(mem), y, plans, 0);
     } else if (dtype == PA_FP64) {
         k_fill_tables<double><<<grid, 256, 0, st>>>(static_cast<double2 *>(mem), y, plans, 0);
+    } else if (narrow_exact(dtype, y.L)) {
+        if (y.L & (y.L - 1)) return cudaErrorInvalidValue;  // the exact transforms keep power-of-two lengths
+        k_fill_tables<Zq><<<grid, 256, 0, st>>>(static_cast<uint2 *>(mem), y, plans, zq_pow(3u, (kQ - 1) / y.L));
     } else {
         const uint64_t w = (y.L & (y.L - 1)) ? 0 : zp_root(y.L);  // the exact transform keeps power-of-two lengths
         if (!w) return cudaErrorInvalidValue;

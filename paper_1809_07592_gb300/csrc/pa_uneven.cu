@@ -137,32 +137,45 @@ int run_class_complex(const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStr
 }
 
 // NTT mode: per block, seed transform into the class's spectrum slot, then the key.
-int run_class_ntt(const ClassRun &c, const pa_block_desc_t *hb, const uint32_t *ids, uint32_t *popc,
+template <typename T>
+int run_class_exact(const ClassRun &c, const pa_block_desc_t *hb, const uint32_t *ids, uint32_t *popc,
                   uint32_t *marg, cudaStream_t st) {
-    const TwTab<Zp> tw = tw_tab<Zp>(c.tw.lay, c.tw.mem);
-    cx<Zp> *W = static_cast<cx<Zp> *>(c.Wf), *spec = static_cast<cx<Zp> *>(c.spec);
+    const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
+    cx<T> *W = static_cast<cx<T> *>(c.Wf), *spec = static_cast<cx<T> *>(c.spec);
     const Geometry &g = c.geo;
     const uint64_t L = g.L;
-    const cx<Zp> invL = zp_pow_host(L, kP - 2);
-    const BitScratch bs = bit_scratch_at(c.bits, L, Shape<Zp>::E, 1);
+    cx<T> invL;  // the spectrum's scale, as a multiplier
+    if constexpr (std::is_same<T, Zq>::value) {
+        const uint32_t w = zq_pow((uint32_t)L, kQ - 2);
+        invL = make_uint2(w, zq_quotient(w));
+    } else {
+        invL = zp_pow_host(L, kP - 2);
+    }
+    const BitScratch bs = bit_scratch_at(c.bits, L, Shape<T>::E, 1);
     for (uint32_t i = 0; i < c.nb; ++i) {
         const pa_block_desc_t &b = hb[ids[i]];
         const uint64_t kw = (b.n + 63) / 64;
-        FwdArgs in = seed_args<Zp>(bs.bits, b.n, b.m, false, L);
-        U_CUDA(launch_seed_bits(b.seed, b.n, b.m, bit_form<Zp>(g.lg1, L), bs.bits, nullptr, nullptr, st));
-        U_CUDA(launch_fwd<Zp>(g.lg1, In::SEED, in, 1, W, L, tw, st));
-        if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, false, W, L, g.inner(), 1, tw, st));
-        U_CUDA(launch_middle<Zp>(g.ro, g.lgI, 1, W, spec, L, 1, tw, invL, st));
+        FwdArgs in = seed_args<T>(bs.bits, b.n, b.m, false, L);
+        U_CUDA(launch_seed_bits(b.seed, b.n, b.m, bit_form<T>(g.lg1, L), bs.bits, nullptr, nullptr, st));
+        U_CUDA(launch_fwd<T>(g.lg1, In::SEED, in, 1, W, L, tw, st));
+        if (g.lgM) U_CUDA(launch_mid<T>(g.lgM, false, W, L, g.inner(), 1, tw, st));
+        U_CUDA(launch_middle<T>(g.ro, g.lgI, 1, W, spec, L, 1, tw, invL, st));
         const KeyBits kb{b.key, 1, 1, kw, b.n, 0, false};
-        U_CUDA(prepare_keys<Zp>(g.lg1, kb, L, bs, popc + ids[i], marg + ids[i], st, &in));
-        U_CUDA(launch_fwd<Zp>(g.lg1, In::KEYS, in, 1, W, L, tw, st));
-        if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, false, W, L, g.inner(), 1, tw, st));
-        U_CUDA(launch_middle<Zp>(g.ro, g.lgI, 0, W, spec, L, 1, tw, (cx<Zp>)1, st));
-        if (g.lgM) U_CUDA(launch_mid<Zp>(g.lgM, true, W, L, g.inner(), 1, tw, st));
-        U_CUDA(launch_inv_bits<Zp>(g.lg1, W, L, b.m, 1, popc + ids[i], marg + ids[i], b.out, (b.m + 63) / 64, 1, tw,
+        U_CUDA(prepare_keys<T>(g.lg1, kb, L, bs, popc + ids[i], marg + ids[i], st, &in));
+        U_CUDA(launch_fwd<T>(g.lg1, In::KEYS, in, 1, W, L, tw, st));
+        if (g.lgM) U_CUDA(launch_mid<T>(g.lgM, false, W, L, g.inner(), 1, tw, st));
+        U_CUDA(launch_middle<T>(g.ro, g.lgI, 0, W, spec, L, 1, tw, invL, st));
+        if (g.lgM) U_CUDA(launch_mid<T>(g.lgM, true, W, L, g.inner(), 1, tw, st));
+        U_CUDA(launch_inv_bits<T>(g.lg1, W, L, b.m, 1, popc + ids[i], marg + ids[i], b.out, (b.m + 63) / 64, 1, tw,
                                    st));
     }
     return PA_OK;
+}
+
+int run_class_ntt(const ClassRun &c, const pa_block_desc_t *hb, const uint32_t *ids, uint32_t *popc, uint32_t *marg,
+                  cudaStream_t st) {
+    return narrow_exact(PA_NTT64, c.geo.L) ? run_class_exact<Zq>(c, hb, ids, popc, marg, st)
+                                           : run_class_exact<Zp>(c, hb, ids, popc, marg, st);
 }
 
 int run_class(pa_uneven_t *u, const UClass &c, cudaStream_t st) {
@@ -309,8 +322,7 @@ BlockDev block_dev(const pa_block_desc_t &b, uint32_t id, uint64_t L, pa_dtype_t
 }
 
 size_t class_bit_bytes(uint64_t L, pa_dtype_t dtype, uint64_t slots) {
-    const int E = dtype == PA_FP32_GUARD ? Shape<float>::E : dtype == PA_FP64 ? Shape<double>::E : Shape<Zp>::E;
-    return bit_scratch_bytes(L, E, slots);
+    return bit_scratch_bytes(L, values_per_thread(dtype, L), slots);
 }
 
 size_t scratch_per_block(uint64_t L, pa_dtype_t dtype) {

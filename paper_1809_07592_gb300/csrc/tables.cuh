@@ -12,7 +12,8 @@
 //   pass tables  (one set per strided pass): the pass twiddle w^{k u} of frequency k = f + s*TC in
 //                column u = blk*COLS + col. Forward: a[f][blk] * c[f][col] * g[u]^s. Inverse, complex
 //                arithmetic: it goes into the stages' multipliers (inv_col_stages in fft_core.cuh),
-//                stage i needing h[i][u] = w^{P_i u} beside its stage table.
+//                stage i needing h[i][u] = w^{P_i u} beside its stage table. The exact transform of
+//                zq.cuh, whose multipliers cannot be multiplied with each other: a[f][u] and g[s][u].
 #pragma once
 
 #include <cstdint>
@@ -57,9 +58,10 @@ struct StagePlan {
 // Double precision reads them all: its passes are bound by the FP64 pipe, the load path is idle. Single
 // precision reads w alone and forms the others (squarings and constant turns): its innermost
 // pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing four
-// wavefronts whatever the addresses) and has multiply-add slots to spare. The exact transform
-// reads w^r, r = 1 .. R-1.
-enum class Rows { SINGLE, DOUBLE, EXACT };
+// wavefronts whatever the addresses) and has multiply-add slots to spare. The exact transforms read w^r, r = 1 .. R-1 (EXACT), or every level's
+// multipliers, R-1 as well, no two of which are a free quarter turn apart (LEVELS).
+enum class Rows { SINGLE, DOUBLE, EXACT, LEVELS };
+__host__ __device__ constexpr bool is_complex(Rows kind) { return kind == Rows::SINGLE || kind == Rows::DOUBLE; }
 __host__ __device__ constexpr int level_rows(int R) { return R / 2; }
 __host__ __device__ constexpr int odd_level_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
 __host__ __device__ constexpr int stage_rows(int R, Rows kind) {
@@ -123,6 +125,10 @@ __host__ __device__ constexpr int row_pos(int row) { return row == 0 ? 0 : row -
 // Exponent e (of w_L) held by row `row` of a radix-R stage for the twiddle base w_{R P}^k.
 __host__ __device__ inline uint64_t stage_exponent(int R, uint64_t P, int row, uint64_t k, uint64_t L, Rows kind) {
     const uint64_t unit = L / ((uint64_t)R * P);  // w_{R P} = w_L^unit
+    if (kind == Rows::LEVELS) {  // level l: rows 2^l - 1 .., one per sub-transform p
+        const int l = ilog2(row + 1), p = row + 1 - (1 << l);
+        return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)p * (L >> (l + 1));
+    }
     if (kind != Rows::DOUBLE) return (uint64_t)(row + 1) * k * unit;
     const int l = row_level(row);
     return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)row_pos(row) * (L >> (l + 1));
@@ -141,7 +147,7 @@ struct PassShape {
     uint32_t tc = 0, cols = 0;  // threads per column, columns per CTA
     uint64_t stride = 0;        // S: distance of a column's elements
     uint64_t a = 0, c = 0, g = 0;      // forward pass tables
-    uint64_t ai = 0, ci = 0, gi = 0;   // inverse ones (the exact transform)
+    uint64_t ai = 0, ci = 0, gi = 0;   // inverse ones (the exact transforms)
     uint64_t h = 0;                    // complex arithmetic: n tables of `stride` entries for the inverse stages
 };
 struct TwLayout {
