@@ -295,6 +295,15 @@ template <> struct Arith<double> : ComplexArith<double> {};
 
 namespace pa {
 
+// f(0), ..., f(N-1) with compile-time arguments.
+template <int N, int I = 0, class F>
+__device__ __forceinline__ void static_for(F &&f) {
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        static_for<N, I + 1>(f);
+    }
+}
+
 // (a, b) -> (a + w b, a - w b) for w = w_32^J (forward root; the inverse uses the conjugate),
 // the whole and quarter turns without multiplications.
 template <typename T, int J, bool INV>

@@ -65,7 +65,7 @@ inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 struct RealMode {
     Geometry geo;  // the length-N transform, N = geo.L
     TwSet tw;      // its twiddle tables
-    void *tabs = nullptr;  // 3N values: E_s, O_s, w_N^k O_s (times 1/N), digit-reversed bin order
+    void *tabs = nullptr;  // seed tables E_s, O_s (, w_N^k O_s), times 1/N, digit-reversed bin order
     bool seeded = false;
 };
 
@@ -203,6 +203,11 @@ template <typename F> auto with_type(const pa_plan_t *p, F &&f) {
     if (p->dtype == PA_FP64) return f(double());
     if (narrow_exact(p->dtype, p->L)) return f(Zq());
     return f(Zp());
+}
+
+// Bytes of the half-length form's seed tables.
+size_t real_table_bytes(const pa_plan_t *p, uint64_t N) {
+    return (size_t)(p->dtype == PA_FP32_GUARD ? kRealTables<float> : kRealTables<double>) * N * elem_bytes(p->dtype);
 }
 
 // Values of `pairs` slots; the transposed input bits and partial popcounts of the first pass follow them.
@@ -632,7 +637,7 @@ int tune_real(pa_plan_t *p, RealMode *r) {
     cudaError_t e = cudaMalloc(&key, kw * 8);
     if (e == cudaSuccess) e = cudaMalloc(&out, ow * 8);
     if (e == cudaSuccess) e = cudaMemset(key, 0, kw * 8);
-    if (e == cudaSuccess) e = cudaMemset(r->tabs, 0, (size_t)3 * r->geo.L * elem_bytes(p->dtype));
+    if (e == cudaSuccess) e = cudaMemset(r->tabs, 0, real_table_bytes(p, r->geo.L));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
@@ -675,7 +680,7 @@ int build_real_mode(pa_plan_t *p) {
     RealMode *r = new RealMode();
     r->geo = g;
     p->real = r;  // released with the plan, also on failure
-    cudaError_t e = cudaMalloc(&r->tabs, (size_t)3 * g.L * elem_bytes(p->dtype));
+    cudaError_t e = cudaMalloc(&r->tabs, real_table_bytes(p, g.L));
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         return PA_ENOMEM;

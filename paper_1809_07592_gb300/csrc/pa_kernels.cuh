@@ -45,14 +45,24 @@ __host__ __device__ constexpr int min_blocks(int threads) { return threads >= 10
 // and rows of 4608 (288 threads) for four (1152 threads, at most 56), both without
 // spills: the pass ran 8.8 % faster on the DV-QKD batches with three CTAs than with
 // two, and 0.6 % faster again with the fourth for 4608; four CTAs of 320 threads
-// and three of 384 (6144 values) spill and were slower. The two-row split kernel
-// keeps 512 (it spills above).
+// and three of 384 (6144 values) spill and were slower.
 __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes = 16) {
     return elem_bytes > 8 ? (threads >= 512 ? 1 : (512 / threads > 16 ? 16 : 512 / threads))
                           : (threads >= 768 ? 1
                                             : threads == 288 ? 4
                                             : threads == 320 ? 3
                                                              : (768 / threads > 8 ? 8 : 768 / threads));
+}
+
+// The two-row kernels in single precision (double precision keeps the 512 threads of the rule above). The
+// split kernel asks for 1024 threads: the 256-block uneven batch took 9.99 ms, with 768, 640 and 512
+// threads 10.06, 10.25 and 10.47. The half-length kernel asks for 640: the 2^27-bit block took 1.179 ms, with
+// 512 and 768 threads 1.210 and 1.190.
+__host__ __device__ constexpr int min_blocks_split(int threads, int elem_bytes) {
+    return elem_bytes > 8 ? min_blocks_inner(threads) : min_blocks(threads);
+}
+__host__ __device__ constexpr int min_blocks_real(int threads, int elem_bytes) {
+    return elem_bytes > 8 ? min_blocks_inner(threads) : threads >= 640 ? 1 : 640 / threads > 16 ? 16 : 640 / threads;
 }
 
 // Rounding to the nearest integer (ties to even) by adding and subtracting
@@ -703,11 +713,13 @@ template <typename T, int LEN, int E> struct Mirror {
 // Fused innermost pass of the uneven batch. CTA (rho, pair): rows rho and
 // -rho of blocks 2*pair and 2*pair+1 (if present), one thread group per row.
 // Forward transform, Eq. 5-10 split with the mirror bin, X*V/L, then the
-// inverse transform of Y1 + i*Y2 written to the pair's slot in Wi.
+// inverse transform of Y1 + i*Y2 written to the pair's slot in Wi. The first block's product waits in
+// the row it came from, which the transform has consumed, while the second block is transformed: in
+// registers it took 32 of a thread's, so that one CTA of 512 threads filled an SM and long rows spilled.
 template <typename T, int LEN, int E>
-__global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
-    k_middle_split(const cx<T> *__restrict__ Wf, cx<T> *__restrict__ Wi, uint64_t L, uint32_t nblocks,
-                   uint32_t lgL1, uint32_t lgM, TwTab<T> tw, T inv_L) {
+__global__ void __launch_bounds__(2 * (LEN / E), min_blocks_split(2 * (LEN / E), sizeof(cx<T>)))
+    k_middle_split(cx<T> *Wf, cx<T> *__restrict__ Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1, uint32_t lgM,
+                   TwTab<T> tw, T inv_L) {
     begin_after_previous(Wf, Wi);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T> *smem = reinterpret_cast<cx<T> *>(smem_raw);
@@ -722,15 +734,12 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     const bool self_paired = rho == rho_m;
     cx<T> *sm = smem + g * SE;                          // this group's transform scratch
     const cx<T> *sm_other = smem + (self_paired ? g : 1u - g) * SE;  // where the mirror row's spectrum sits
-    const uint32_t b1 = 2 * blockIdx.y, b2 = b1 + 1;
-    const bool has2 = b2 < nblocks;
+    const uint32_t b1 = 2 * blockIdx.y, nb = b1 + 1 < nblocks ? 2u : 1u;
     const Mirror<T, LEN, E> mir(sm_other, tq, my_rho == 0);
-    cx<T> y[E];
-#pragma unroll
-    for (int s = 0; s < E; ++s) y[s] = Arith<T>::mk((T)0, (T)0);
-    for (int which = 0; which < (has2 ? 2 : 1); ++which) {
-        const cx<T> *wt = Wf + (uint64_t)(which ? b2 : b1) * L + (uint64_t)row * LEN + tq;
-        cx<T> v[E];
+    cx<T> *const w1 = Wf + (uint64_t)b1 * L + (uint64_t)row * LEN + tq;
+    cx<T> v[E];
+    for (uint32_t which = 0; which < nb; ++which) {
+        const cx<T> *wt = w1 + which * L;
         __syncthreads();  // previous use of the scratch is finished
         if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
@@ -747,27 +756,27 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
             // Eq. 7-10: X = (Z(k) + conj Z(-k)) / 2, V = (Z(k) - conj Z(-k)) / (2i)
             const cx<T> X = Arith<T>::mk((z.x + zm.x) * (T)0.5, (z.y - zm.y) * (T)0.5);
             const cx<T> V = Arith<T>::mk((z.y + zm.y) * (T)0.5, (zm.x - z.x) * (T)0.5);
-            cx<T> Y = Arith<T>::mul(X, V);
-            Y.x *= inv_L;
-            Y.y *= inv_L;
+            const cx<T> P = Arith<T>::mul(X, V);
+            cx<T> Y = Arith<T>::mk(P.x * inv_L, P.y * inv_L);
             if (which == 0) {
-                y[s] = Y;
-            } else {  // y += i * Y2
-                y[s].x -= Y.y;
-                y[s].y += Y.x;
+                if (nb == 2) w1[s * TC] = Y;  // a self-paired row's two groups write the same values
+            } else {  // Y1 + i * Y2
+                const cx<T> Y1 = w1[s * TC];
+                Y = Arith<T>::mk(Y1.x - Y.y, Y1.y + Y.x);
             }
+            v[s] = Y;
         }
     }
     __syncthreads();
     cx<T> *wot = Wi + (uint64_t)blockIdx.y * L + (uint64_t)row * LEN + tq;
     const bool store = !(self_paired && g == 1);  // a self-paired row is written once
     if constexpr (Plan<T, LEN, E>::RO == 1) {
-        cta_fft<T, LEN, 1, E, true>(sm, y, tq, 0, tw.st[2]);
+        cta_fft<T, LEN, 1, E, true>(sm, v, tq, 0, tw.st[2]);
         if (!store) return;
 #pragma unroll
-        for (int s = 0; s < E; ++s) wot[elem_of<T, LEN, E>(0, s)] = y[s];
+        for (int s = 0; s < E; ++s) wot[elem_of<T, LEN, E>(0, s)] = v[s];
     } else {
-        cta_fft_inv_odd<T, LEN, E>(sm, y, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
+        cta_fft_inv_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o, cx<T> x) {
             if (store) wot[o] = x;
         });
     }
@@ -778,14 +787,14 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
 // a seed). The slot holds Z = FFT_N(z), z[t] = x[2t] + i x[2t+1], N = L/2. With the
 // mirror bin Z' = Z[N-k]: E_x = (Z + conj Z')/2 and O_x = (Z - conj Z')/(2i) are the
 // spectra of the even and odd key bits, and with the seed tables (per bin, times 1/N)
-// Es = E_s, Os = O_s and Bp = w_N^k O_s of the seed's even/odd spectra, the product
-// Y = S X of the length-L transforms is, in even/odd form,
-//     E_y = Es E_x + Bp O_x,   O_y = Es O_x + Os E_x,
+// Es = E_s and Os = O_s of the seed's even/odd spectra, the product Y = S X of the length-L
+// transforms is, in even/odd form (kRealTables: double precision also keeps w_N^k O_s),
+//     E_y = Es E_x + Os (w_N^k O_x),   O_y = Es O_x + Os E_x,
 // and the inverse transform of E_y + i O_y returns y[2t] + i y[2t+1].
 // CTA (rho, slot): rows rho and -rho (one thread group each), as in k_middle_split.
 // MODE 1 builds the tables from the seed slot instead (forward transform and split only).
 template <typename T, int LEN, int E, int MODE>
-__global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E)))
+__global__ void __launch_bounds__(2 * (LEN / E), min_blocks_real(2 * (LEN / E), sizeof(cx<T>)))
     k_middle_real(cx<T> *__restrict__ W, cx<T> *tabs, uint64_t N, uint32_t lgL1, uint32_t lgM,
                   TwTab<T> tw, T scale) {
     begin_after_previous(W, tabs);
@@ -814,11 +823,14 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
     store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
     __syncthreads();
     const Mirror<T, LEN, E> mir(sm_other, tq, my_rho == 0);
-    [[maybe_unused]] const uint32_t f = freq_of<T, LEN, E>(tq);
-    const cx<T> *Es = tabs, *Os = tabs + N, *Bp = tabs + 2 * N;
+    constexpr bool THREE = kRealTables<T> == 3;
+    const cx<T> *Es = tabs, *Os = tabs + N;
+    [[maybe_unused]] const uint32_t k0 = my_rho + R * freq_of<T, LEN, E>(tq);  // frequency of bin s: k0 + R s TC
+    [[maybe_unused]] cx<T> w0;
+    if constexpr (MODE == 0 && !THREE) w0 = Arith<T>::template omega<false>(tw, k0);
     const bool write_tab = !(self_paired && g == 1);
-#pragma unroll
-    for (int s = 0; s < E; ++s) {
+    static_for<E>([&](auto slot) {
+        constexpr int s = decltype(slot)::value;
         const cx<T> z = v[s], zm = mir.at(s);
         const cx<T> ex = Arith<T>::mk((z.x + zm.x) * (T)0.5, (z.y - zm.y) * (T)0.5);
         const cx<T> ox = Arith<T>::mk((z.y + zm.y) * (T)0.5, (zm.x - z.x) * (T)0.5);
@@ -827,19 +839,23 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_inner(2 * (LEN / E))
             if (write_tab) {
                 const cx<T> es = Arith<T>::mk(ex.x * scale, ex.y * scale);
                 const cx<T> os = Arith<T>::mk(ox.x * scale, ox.y * scale);
-                // frequency of this bin: low part from the strided passes, high part from the row
-                const uint32_t k = my_rho + R * (f + s * TC);
                 tabs[e] = es;
                 tabs[N + e] = os;
-                tabs[2 * N + e] = Arith<T>::mul(Arith<T>::template omega<false>(tw, k), os);
+                if constexpr (THREE) tabs[2 * N + e] = Arith<T>::mul(Arith<T>::template omega<false>(tw, k0 + R * (s * TC)), os);
             }
         } else {
-            const cx<T> es = Es[e], os = Os[e], bp = Bp[e];
-            const cx<T> ey = Arith<T>::add(Arith<T>::mul(es, ex), Arith<T>::mul(bp, ox));
+            const cx<T> es = Es[e], os = Os[e];
+            cx<T> t;  // w_N^k O_s O_x
+            if constexpr (THREE) {
+                t = Arith<T>::mul(tabs[2 * N + e], ox);
+            } else {  // w_N^{R s TC} = w_E^s
+                t = Arith<T>::mul(os, Arith<T>::mul(turn<T, E, s>(w0), ox));
+            }
+            const cx<T> ey = Arith<T>::add(Arith<T>::mul(es, ex), t);
             const cx<T> oy = Arith<T>::add(Arith<T>::mul(es, ox), Arith<T>::mul(os, ex));
             v[s] = Arith<T>::mk(ey.x - oy.y, ey.y + oy.x);  // E_y + i O_y
         }
-    }
+    });
     if constexpr (MODE == 0) {
         __syncthreads();  // the mirror reads of both groups are done
         const bool store = !(self_paired && g == 1);  // a self-paired row is written once

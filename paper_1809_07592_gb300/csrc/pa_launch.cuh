@@ -258,7 +258,7 @@ cudaError_t launch_inv_bits(int lgLEN, const cx<T> *W, uint64_t L, uint64_t m, u
                                             const uint64_t *, uint64_t, bool, uint32_t *, uint32_t);
 
 template <typename T, int LEN>
-cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1, uint32_t lgM,
+cudaError_t split_at(cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1, uint32_t lgM,
                      TwTab<T> tw, cudaStream_t st) {
     constexpr int E = Shape<T>::E;
     auto kern = k_middle_split<T, LEN, E>;
@@ -272,7 +272,7 @@ cudaError_t split_at(const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, u
 }
 
 template <typename T>
-cudaError_t launch_middle_split(int ro, int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks,
+cudaError_t launch_middle_split(int ro, int lg, cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks,
                                 uint32_t lgL1, uint32_t lgM, TwTab<T> tw, cudaStream_t st) {
     if (ro == 1) {
         return by_len<kMinLgMiddle, MaxLgSplit<T>::v>(lg, [&](auto c) {
@@ -286,7 +286,7 @@ cudaError_t launch_middle_split(int ro, int lg, const cx<T> *Wf, cx<T> *Wi, uint
 }
 
 template <typename T, int RO, int LG = kMinLgOdd>
-cudaError_t odd_split_dispatch(int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
+cudaError_t odd_split_dispatch(int lg, cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
                                uint32_t lgM, TwTab<T> tw, cudaStream_t st) {
     if constexpr (LG > kMaxLgOdd) {
         return cudaErrorInvalidValue;
@@ -303,7 +303,7 @@ cudaError_t odd_split_dispatch(int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, u
 }
 
 template <typename T, int RO>
-cudaError_t launch_middle_split_odd(int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
+cudaError_t launch_middle_split_odd(int lg, cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
                                     uint32_t lgM, TwTab<T> tw, cudaStream_t st) {
     return odd_split_dispatch<T, RO>(lg, Wf, Wi, L, nblocks, lgL1, lgM, tw, st);
 }
@@ -325,7 +325,7 @@ cudaError_t launch_inv_bits_blocks(int lgLEN, const cx<T> *Wi, uint64_t L, const
 }
 
 #define PA_INSTANTIATE_UNEVEN(T)                                                                                 \
-    template cudaError_t launch_middle_split<T>(int, int, const cx<T> *, cx<T> *, uint64_t, uint32_t, uint32_t,  \
+    template cudaError_t launch_middle_split<T>(int, int, cx<T> *, cx<T> *, uint64_t, uint32_t, uint32_t,  \
                                                 uint32_t, TwTab<T>, cudaStream_t);                               \
     template cudaError_t launch_inv_bits_blocks<T>(int, const cx<T> *, uint64_t, const BlockDev *, uint32_t,     \
                                                    const uint32_t *, uint32_t *, TwTab<T>, cudaStream_t);        \
@@ -394,7 +394,7 @@ cudaError_t launch_middle_real(int ro, int lg, int mode, cx<T> *W, cx<T> *tabs, 
 #define PA_INSTANTIATE_ODD(T, RO)                                                                               \
     template cudaError_t launch_middle_odd<T, RO>(int, int, cx<T> *, cx<T> *, uint64_t, uint32_t, TwTab<T>,     \
                                                   cx<T>, cudaStream_t);                                         \
-    template cudaError_t launch_middle_split_odd<T, RO>(int, const cx<T> *, cx<T> *, uint64_t, uint32_t,        \
+    template cudaError_t launch_middle_split_odd<T, RO>(int, cx<T> *, cx<T> *, uint64_t, uint32_t,        \
                                                         uint32_t, uint32_t, TwTab<T>, cudaStream_t);            \
     template cudaError_t launch_middle_real_odd<T, RO>(int, int, cx<T> *, cx<T> *, uint64_t, uint32_t, uint32_t, \
                                                        TwTab<T>, T, uint32_t, cudaStream_t);

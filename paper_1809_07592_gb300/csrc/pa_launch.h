@@ -42,6 +42,10 @@ template <> struct Shape<float> { static constexpr int E = 16, COLS = 16; };
 template <> struct Shape<double> { static constexpr int E = 8, COLS = 8; };
 template <> struct Shape<Zp> { static constexpr int E = 8, COLS = 8; };
 template <> struct Shape<Zq> { static constexpr int E = 16, COLS = 16; };
+// Seed tables of the half-length form. Single precision forms w_N^k (a third table would be a fifth of the
+// innermost pass's memory traffic, and that pass runs at 0.8 of the HBM rate on the 2^27-bit block);
+// double precision, bound by the FP64 pipe, reads w_N^k O_s.
+template <typename T> constexpr int kRealTables = std::is_same<T, float>::value ? 2 : 3;
 template <typename T> constexpr bool kExact = std::is_same<T, Zp>::value || std::is_same<T, Zq>::value;
 // Columns per CTA of a strided pass of length LEN: the types with 16 values per thread take 8 instead of 16 at
 // LEN = 1024 (512 threads, two CTAs per SM instead of one).
@@ -264,10 +268,10 @@ template <> struct MaxLgSplit<float> { static constexpr int v = 13; };
 template <> struct MaxLgSplit<double> { static constexpr int v = 12; };
 
 template <typename T>
-cudaError_t launch_middle_split(int ro, int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks,
+cudaError_t launch_middle_split(int ro, int lg, cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks,
                                 uint32_t lgL1, uint32_t lgM, TwTab<T> tw, cudaStream_t st);
 template <typename T, int RO>
-cudaError_t launch_middle_split_odd(int lg, const cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
+cudaError_t launch_middle_split_odd(int lg, cx<T> *Wf, cx<T> *Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1,
                                     uint32_t lgM, TwTab<T> tw, cudaStream_t st);
 template <typename T>
 cudaError_t launch_inv_bits_blocks(int lgLEN, const cx<T> *Wi, uint64_t L, const BlockDev *blocks, uint32_t nblocks,
@@ -275,7 +279,7 @@ cudaError_t launch_inv_bits_blocks(int lgLEN, const cx<T> *Wi, uint64_t L, const
 
 // ---- single keys in half-length transforms (complex arithmetic only) ----
 // Innermost pass of length ro * 2^lg over a length-N slot (slots of N elements from W):
-// mode 0 multiplies with the seed tables (3N values: E_s, O_s, w_N^k O_s, times 1/N) and
+// mode 0 multiplies with the seed tables (kRealTables * N values: E_s, O_s, w_N^k O_s, times 1/N) and
 // transforms back; mode 1 builds those tables from the packed seed's transform (scale 1/N).
 template <typename T>
 cudaError_t launch_middle_real(int ro, int lg, int mode, cx<T> *W, cx<T> *tabs, uint64_t N, uint32_t lgL1,
