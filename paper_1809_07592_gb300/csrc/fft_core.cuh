@@ -358,7 +358,8 @@ __device__ __forceinline__ void bitrev_regs(cx<T> *v) {
 // decimation in time; level l combines the halves of the 2^l sub-transforms p (outputs
 // k = p mod 2^l) with the root w_{2^(l+1)}^p, which the butterfly's multiply-adds absorb.
 // Exact transform: decimation in frequency with the shift roots.
-template <typename T, int R, bool INV>
+// FROM > 0: the values are those of the first FROM levels already (complex).
+template <typename T, int R, bool INV, int FROM = 0>
 __device__ __forceinline__ void dft(cx<T> *v) {
     static_assert(R >= 1 && R <= 32 && (R & (R - 1)) == 0, "radix must be a power of two <= 32");
     if constexpr (R > 1) {
@@ -376,7 +377,7 @@ __device__ __forceinline__ void dft(cx<T> *v) {
                 }
             }
         } else {
-            dft_const<T, R, INV, 0>(v);
+            dft_const<T, R, INV, FROM>(v);
         }
         bitrev_regs<T, R>(v);
     }
@@ -823,7 +824,7 @@ __device__ __forceinline__ void store_stage(cx<T> *sm, const cx<T> *v, uint32_t 
     }
 }
 // The butterflies of stage I on the thread's registers.
-template <typename T, int LEN, int E, int I, bool INV>
+template <typename T, int LEN, int E, int I, bool INV, int FROM = 0>
 __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *st) {
     using M = StageMap<T, LEN, E, I>;
     constexpr StagePlan p = Plan<T, LEN, E>::p;
@@ -832,7 +833,7 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
 #pragma unroll
     for (int g = 0; g < M::groups; ++g) {
         if constexpr (row.rows == 0) {
-            dft<T, M::R, INV>(v + g * M::R);
+            dft<T, M::R, INV, FROM>(v + g * M::R);
         } else {
             cx<T> w[multipliers<T>(M::R)];
             stage_multipliers<T, M::R, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
@@ -843,14 +844,14 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
 
 // Forward stages I .. n-1, stage I's inputs in shared memory (a barrier away) unless FROM_REGS;
 // the outputs end in registers (frequencies freq_of(tq) + s*TC).
-template <typename T, int LEN, int COLS, int E, int I, bool FROM_REGS>
+template <typename T, int LEN, int COLS, int E, int I, bool FROM_REGS, int FROM = 0>
 __device__ __forceinline__ void fwd_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     using PL = Plan<T, LEN, E>;
     if constexpr (!FROM_REGS) {
         exchange_barrier<COLS * PL::p.N[I - 1], E>();
         load_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
     }
-    stage_regs<T, LEN, E, I, false>(v, tq, st);
+    stage_regs<T, LEN, E, I, false, FROM>(v, tq, st);
     if constexpr (I < PL::n - 1) {
         store_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
         fwd_stages<T, LEN, COLS, E, I + 1, false>(sm, v, tq, col, st);

@@ -37,15 +37,12 @@ namespace pa {
 // threads, so the register allocation stays <= 64 per thread and at least two
 // CTAs overlap their load, transform and store phases.
 __host__ __device__ constexpr int min_blocks(int threads) { return threads >= 1024 ? 1 : (1024 / threads > 16 ? 16 : 1024 / threads); }
-// The fused innermost passes ask for 512 resident threads per SM (<= 128
-// registers each; at most 16 CTAs). In single precision (8-byte elements) they ask for 768, at
-// most 8 CTAs: measured on the DV-QKD lengths, 17-31 % faster than 512 (more CTAs
-// overlap their barrier and load phases) with no spills. Rows of 5120 values
-// (CTAs of 320 threads) ask for three CTAs (960 threads, at most 68 registers)
-// and rows of 4608 (288 threads) for four (1152 threads, at most 56), both without
-// spills: the pass ran 8.8 % faster on the DV-QKD batches with three CTAs than with
-// two, and 0.6 % faster again with the fourth for 4608; four CTAs of 320 threads
-// and three of 384 (6144 values) spill and were slower.
+// The fused innermost passes ask for 512 resident threads per SM (<= 128 registers each; at most 16 CTAs).
+// In single precision they ask for 768, at most 8 CTAs: 17-31 % faster than 512 on the lengths around 2^20
+// (more CTAs overlap their barrier and load phases) with no spills. Rows of 5120 values (CTAs of 320 threads)
+// ask for three CTAs and rows of 4608 (288 threads) for four: 8.8 % and 0.6 % faster than with one less
+// (all with self-sorting stages). On the in-place stages a fourth CTA for 5120 took the pass over 32 pairs
+// from 156 to 213 us.
 __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes = 16) {
     return elem_bytes > 8 ? (threads >= 512 ? 1 : (512 / threads > 16 ? 16 : 512 / threads))
                           : (threads >= 768 ? 1
@@ -242,6 +239,24 @@ __device__ __forceinline__ uint32_t bits_at(const uint64_t *v, uint64_t nbits, u
     return w;
 }
 
+// The first stage's first two butterfly levels on input bits, in double precision: their values are
+// integers up to 8 in magnitude (sums of four inputs 0 or +-2), so single precision is exact, and the
+// encoding of such a float becomes the double's with integer instructions. The pass is bound by the
+// FP64 pipe (90 % busy), which these levels occupied for 4 of its 32 operations per value: a batch of 64 keys
+// of 10^6 bits took 10.09 ms instead of 10.41.
+template <int R> constexpr int kExactLevels = R >= 4 ? 2 : 1;
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t b = __float_as_uint(x), mag = b & 0x7fffffffu;
+    return __hiloint2double((int)((mag ? (mag >> 3) + 0x38000000u : 0u) | (b & 0x80000000u)), 0);
+}
+template <int R, int LEVEL = 0>
+__device__ __forceinline__ void exact_levels(float2 *u) {
+    if constexpr (LEVEL < kExactLevels<R>) {
+        dft_const_sub<float, R, false, LEVEL, 0>(u);
+        exact_levels<R, LEVEL + 1>(u);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Level-1 forward pass from transposed bits. Grid (S/COLS, slots). KEYS: slot p holds keys 2p
 // and 2p+1 (or, one key per slot, its even and odd bits); SEED: the rotated, +-1 encoded seed in
@@ -260,20 +275,34 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     const uint32_t col = threadIdx.x % COLS, tq = threadIdx.x / COLS;
     const uint32_t S = (uint32_t)(L >> ilog2(LEN)), u = blockIdx.x * COLS + col;
     const uint32_t x = fresh(bits + (uint64_t)blockIdx.y * (L / E) + blockIdx.x * (COLS * LEN / E) + threadIdx.x);
-    cx<T> v[E];
+    // double precision: the inputs and the first levels in single (exact)
+    using I = typename std::conditional<std::is_same<T, double>::value, float, T>::type;
+    cx<I> b[E];
     if constexpr (KIND == In::KEYS) {
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = Enc<T>::keys(x, slot_pos<T, LEN, E>(s));
+        for (int s = 0; s < E; ++s) b[s] = Enc<I>::keys(x, slot_pos<T, LEN, E>(s));
     } else if constexpr (KIND == In::SEED) {
         const uint32_t re = in.re.mask(tq * S + u), im = in.im.mask(tq * S + u);
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = Enc<T>::seed(x, re, im, slot_pos<T, LEN, E>(s));
+        for (int s = 0; s < E; ++s) b[s] = Enc<I>::seed(x, re, im, slot_pos<T, LEN, E>(s));
     } else {
         const uint32_t inside = blocks[blockIdx.y].in.mask(tq * S + u);
 #pragma unroll
-        for (int s = 0; s < E; ++s) v[s] = Enc<T>::key_seed(x, inside, slot_pos<T, LEN, E>(s));
+        for (int s = 0; s < E; ++s) b[s] = Enc<I>::key_seed(x, inside, slot_pos<T, LEN, E>(s));
     }
-    cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+    cx<T> v[E];
+    if constexpr (std::is_same<T, double>::value) {
+        constexpr int R = Plan<T, LEN, E>::r0;
+#pragma unroll
+        for (int g = 0; g < E / R; ++g) exact_levels<R>(b + g * R);
+#pragma unroll
+        for (int s = 0; s < E; ++s) v[s] = make_double2(widen(b[s].x), widen(b[s].y));
+        fwd_stages<T, LEN, COLS, E, 0, true, kExactLevels<R>>(sm, v, tq, col, tw.st[0]);
+    } else {
+#pragma unroll
+        for (int s = 0; s < E; ++s) v[s] = b[s];
+        cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+    }
     const uint32_t f = freq_of<T, LEN, E>(tq);
     pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
     cx<T> *w = W + (uint64_t)blockIdx.y * L + u;
