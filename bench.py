@@ -109,7 +109,7 @@ class ClockSampler:
 
 # The files that define the pass kernels, their launch shapes and the transform splits;
 # an ncu summary's DRAM figures hold while these are unchanged.
-KERNEL_SOURCES = ("fft_core.cuh", "pa_kernels.cuh", "bulk.cuh", "zp.cuh", "pa_launch.h", "pa_launch.cuh",
+KERNEL_SOURCES = ("tables.cuh", "fft_core.cuh", "pa_kernels.cuh", "bulk.cuh", "zp.cuh", "zq.cuh", "pa_launch.h", "pa_launch.cuh",
                   "pa_geometry.cu", "pa_f32.cu", "pa_f32_r3.cu", "pa_f32_r5.cu", "pa_f32_r9.cu")
 
 
@@ -159,7 +159,7 @@ def algorithmic_bytes(kind: str, n: int, m: int, L: int, pairs: int, nkeys: int,
     if kind in ("mid_fwd", "mid_inv"):
         return 2 * pairs * slot
     if kind == "prep":
-        return nkeys * 8  # popcount and margin words reset
+        return nkeys * 8  # popcount and margin words (the transposed bits are no compulsory traffic)
     return 0.0
 
 
@@ -434,20 +434,21 @@ def long_block_work(mode: str, L: int) -> tuple:
     return 2 * (N / 2) * math.log2(N) + N, "modmul"
 
 
-def long_block_pass_bytes(L: int, n: int, m: int) -> dict:
-    """Bytes each pass of a single-key (half-length, N = L/2, W = 8 N bytes) FP32 block must move."""
+def long_block_pass_bytes(L: int, n: int, m: int, tables: int = 3) -> dict:
+    """Bytes each pass of a single-key (half-length, N = L/2, W = 8 N bytes) FP32 block must move,
+    with `tables` seed tables read by the innermost pass (single precision reads two)."""
     W = 8 * (L // 2)
-    return {"fwd_keys": W + n / 8, "mid_fwd": 2 * W, "middle_conv": 5 * W, "mid_inv": 2 * W, "inv_bits": W + m / 8}
+    return {"fwd_keys": W + n / 8, "mid_fwd": 2 * W, "middle_conv": (2 + tables) * W, "mid_inv": 2 * W, "inv_bits": W + m / 8}
 
 
 def long_block_passes(pa, plan, kd, out, stream, torch, n, m, block_ms, reps=5):
     """Per-pass roofline of the FP32 long block (one key, half-length form, N = L/2 complex values,
     W = 8 N bytes): each pass's live CUDA-event time (the library's per-launch events, in runs kept
     apart from the timed ones) against the bytes that pass must move -- first pass W + n/8, each
-    middle strided pass 2 W, the fused innermost pass W in, the three seed tables (3 W) and W out,
+    middle strided pass 2 W, the fused innermost pass W in, the two seed tables (2 W) and W out,
     the last pass W + m/8 -- and the block against the FP32 path's floor of 20 L + (n+m)/8 bytes."""
     L = plan.shape()[0]
-    need = long_block_pass_bytes(L, n, m)
+    need = long_block_pass_bytes(L, n, m, tables=2)
     peak, kind = measured_peaks()
     pa.pa_profile_enable(plan.handle, True)
     pa.pa_profile_read(plan.handle, reset=True)
