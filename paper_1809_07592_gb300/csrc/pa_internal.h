@@ -24,11 +24,6 @@ struct Geometry {
     uint64_t L = 0;
     int lg1 = 0, lgM = 0, ro = 1, lgI = 0;
     uint32_t inner() const { return (uint32_t)ro << lgI; }
-    uint32_t F() const {
-        int m = lg1 > lgM ? lg1 : lgM;
-        if (lgI > m) m = lgI;
-        return (uint32_t)ro << m;
-    }
 };
 
 // Whether the exact transform of length L runs modulo the word-sized prime of zq.cuh (lengths up to

@@ -8,6 +8,7 @@
 // them, and sends two blocks' products through one inverse as Y1 + i*Y2. The
 // whole schedule can be captured once into a CUDA graph whose branches (one per
 // class) run concurrently; replaying it costs one graph launch.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -353,7 +354,15 @@ bool cached_split(uint64_t L, pa_dtype_t dtype, Geometry *out) {
     tune_load_locked();
     auto it = g_tune.find({L, (int)dtype});
     if (it == g_tune.end()) return false;
-    *out = it->second;
+    // A split from a file counts only if the planner offers it: tables are laid out for the split before a
+    // launch could refuse it.
+    const Geometry &k = it->second;
+    const auto same = [&](const Geometry &g) {
+        return g.lg1 == k.lg1 && g.lgM == k.lgM && g.ro == k.ro && g.lgI == k.lgI;
+    };
+    const std::vector<Geometry> cand = candidates(L, dtype);
+    if (!same(default_split(L, dtype)) && std::none_of(cand.begin(), cand.end(), same)) return false;
+    *out = k;
     return true;
 }
 
