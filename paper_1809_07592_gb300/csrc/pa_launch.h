@@ -35,9 +35,11 @@ cudaError_t launch_chained(void (*kern)(Params...), dim3 grid, unsigned threads,
     cfg.stream = st;
     cfg.attrs = &attr;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(st, &capture);
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
     cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here: the next <<<>>> launch must not find it again
+    return e;
 }
 
 // Per-type kernel shape: E complex values per thread, COLS columns per CTA in
