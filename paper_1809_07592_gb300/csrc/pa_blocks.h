@@ -21,8 +21,8 @@ struct ClassRun {
     const BlockDev *d_blocks = nullptr;  // nb descriptors
     uint32_t nb = 0;
     void *Wf = nullptr;    // complex: nb slots of L values; NTT: one slot
-    void *bits = nullptr;  // bit scratch of as many slots (bit_scratch_bytes)
     void *Wi = nullptr;    // complex: ceil(nb/2) slots
+    void *bits = nullptr;  // NTT: bit scratch of one slot (bit_scratch_bytes)
     void *spec = nullptr;  // NTT: one seed-spectrum slot
     TwSet tw;              // twiddle tables of geo (not owned)
 };
@@ -32,9 +32,6 @@ uint64_t class_length(uint64_t n, uint64_t m, pa_dtype_t dtype);
 
 // Device descriptor of a block in a class of transform length L.
 BlockDev block_dev(const pa_block_desc_t &b, uint32_t id, uint64_t L, pa_dtype_t dtype);
-
-// Bytes of bit scratch of `slots` blocks of a class.
-size_t class_bit_bytes(uint64_t L, pa_dtype_t dtype, uint64_t slots);
 
 // Bytes of device scratch one block of transform length L needs in a class run.
 size_t scratch_per_block(uint64_t L, pa_dtype_t dtype);

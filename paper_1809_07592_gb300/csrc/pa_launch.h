@@ -97,10 +97,11 @@ constexpr int kMinLgMiddle = 6;
 // t >= Z. For a thread's elements x + j*D (D = L / E, x < D), j < E, that is j < M/D + (x < M%D) or
 // j >= Z/D + (x < Z%D).
 struct SeedRange {
-    uint32_t mq, mr, zq, zr;
-    __host__ __device__ SeedRange() : mq(0), mr(0), zq(0), zr(0) {}
+    uint32_t mr, zr;
+    uint16_t mq, zq;  // at most E
+    __host__ __device__ SeedRange() : mr(0), zr(0), mq(0), zq(0) {}
     __host__ __device__ SeedRange(uint64_t M, uint64_t Z, uint64_t D)
-        : mq((uint32_t)(M / D)), mr((uint32_t)(M % D)), zq((uint32_t)(Z / D)), zr((uint32_t)(Z % D)) {}
+        : mr((uint32_t)(M % D)), zr((uint32_t)(Z % D)), mq((uint16_t)(M / D)), zq((uint16_t)(Z / D)) {}
     __device__ __forceinline__ uint32_t mask(uint32_t x) const {
         const uint32_t below = (1u << (mq + (x < mr))) - 1u, from = (1u << (zq + (x < zr))) - 1u;  // both counts <= 16
         return below | ~from;
@@ -109,14 +110,14 @@ struct SeedRange {
 
 // Device-side block descriptor of the uneven batch.
 struct BlockDev {
-    uint64_t n, m;
     const uint64_t *key;   // ceil(n/64) words
     const uint64_t *seed;  // ceil((n+m-1)/64) words
     uint64_t *out;         // ceil(m/64) words
+    uint32_t n, m;         // at most 2^27
     uint32_t id;           // index of the block in the caller's list (popcount / margin slot)
-    uint32_t pad;
     SeedRange in;          // seed window of the block in its class's transform
 };
+static_assert(sizeof(BlockDev) == 48, "counted into a served block's scratch, which callers cap to the byte");
 
 // Scratch of the level-1 forward passes: transposed input bits (bits_words per slot) and partial
 // popcounts (parts_count per slot).

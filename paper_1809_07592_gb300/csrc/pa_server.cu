@@ -114,10 +114,7 @@ int launch_batch(pa_server_t *s, Slot &sl) {
     size_t off_cnt = 0;
     size_t off_desc = align256(2 * (size_t)nb * sizeof(uint32_t));
     size_t total = off_desc + align256((size_t)nb * sizeof(BlockDev));
-    struct WorkOff {
-        size_t wf, wi, bits;
-    };
-    std::vector<WorkOff> work_off;  // per class
+    std::vector<std::pair<size_t, size_t>> work_off;  // (Wf, Wi) offsets per class
     for (auto &kv : byL) {
         const size_t L = (size_t)kv.first;
         const size_t k = kv.second.size();
@@ -125,9 +122,7 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         total += align256(k * L * esz);
         const size_t wi = total;
         total += align256(((k + 1) / 2) * L * esz);
-        const size_t bits = total;
-        total += align256(pa::blocks::class_bit_bytes(L, s->cfg.dtype, k));
-        work_off.push_back({wf, wi, bits});
+        work_off.push_back({wf, wi});
     }
     unsigned char *mem = nullptr;
     cudaError_t e = cudaMallocFromPoolAsync((void **)&mem, total, s->pool, sl.st);
@@ -157,9 +152,8 @@ int launch_batch(pa_server_t *s, Slot &sl) {
         if (rc != PA_OK) break;
         c.d_blocks = d_desc + class_first[ci];
         c.nb = (uint32_t)kv.second.size();
-        c.Wf = mem + work_off[ci].wf;
-        c.Wi = mem + work_off[ci].wi;
-        c.bits = mem + work_off[ci].bits;
+        c.Wf = mem + work_off[ci].first;
+        c.Wi = mem + work_off[ci].second;
         rc = pa::blocks::run_complex(s->cfg.dtype, c, popc, marg, sl.st);
         ++ci;
     }

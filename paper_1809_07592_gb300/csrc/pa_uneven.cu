@@ -40,7 +40,7 @@ struct UClass {
     std::vector<uint32_t> ids;       // caller indices of the blocks in this class
     BlockDev *d_blocks = nullptr;    // device descriptors
     void *Wf = nullptr, *Wi = nullptr;  // forward slots (one per block), inverse slots (one per pair)
-    void *bits = nullptr;               // bit scratch of the first pass
+    void *bits = nullptr;            // NTT mode: bit scratch of one slot
     void *spec = nullptr;            // NTT mode: one seed-spectrum slot, blocks run one after another
     TwSet tw;                        // twiddle tables of geo
     cudaStream_t st = nullptr;
@@ -121,8 +121,11 @@ int run_class_complex(const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStr
     const uint32_t nb = c.nb;
     const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
     cx<T> *Wf = static_cast<cx<T> *>(c.Wf), *Wi = static_cast<cx<T> *>(c.Wi);
+    // The bits lie in the inverse slots, which nothing else uses before the split pass: at least 4 or 8 bytes
+    // a value of each block, of which the bits and popcounts take 4 / E and little more.
+    const BitScratch bits = bit_scratch_at(c.Wi, g.L, Shape<T>::E, nb);
     FwdArgs in;
-    U_CUDA(prepare_blocks<T>(g.lg1, c.d_blocks, nb, g.L, bit_scratch_at(c.bits, g.L, Shape<T>::E, nb), popc, marg, st, &in));
+    U_CUDA(prepare_blocks<T>(g.lg1, c.d_blocks, nb, g.L, bits, popc, marg, st, &in));
     U_CUDA(launch_fwd<T>(g.lg1, In::BLOCKS, in, nb, Wf, g.L, tw, st));
     if (g.lgM) {
         int rc = mid_chunks<T>(c, false, Wf, nb, st);
@@ -319,18 +322,13 @@ uint64_t class_length(uint64_t n, uint64_t m, pa_dtype_t dtype) {
 
 BlockDev block_dev(const pa_block_desc_t &b, uint32_t id, uint64_t L, pa_dtype_t dtype) {
     const int E = dtype == PA_FP32_GUARD ? Shape<float>::E : Shape<double>::E;
-    return BlockDev{b.n, b.m, b.key, b.seed, b.out, id, 0u, SeedRange(b.m, L - b.n + 1, L / E)};
-}
-
-size_t class_bit_bytes(uint64_t L, pa_dtype_t dtype, uint64_t slots) {
-    return bit_scratch_bytes(L, values_per_thread(dtype, L), slots);
+    return BlockDev{b.key, b.seed, b.out, (uint32_t)b.n, (uint32_t)b.m, id, SeedRange(b.m, L - b.n + 1, L / E)};
 }
 
 size_t scratch_per_block(uint64_t L, pa_dtype_t dtype) {
     if (dtype == PA_NTT64) return 2 * L * 8;
     const size_t e = dtype == PA_FP32_GUARD ? sizeof(float2) : sizeof(double2);
-    // forward slot, half an inverse slot, bit scratch, descriptor, counters
-    return L * e + (L * e + 1) / 2 + class_bit_bytes(L, dtype, 1) + sizeof(BlockDev) + 8;
+    return L * e + (L * e + 1) / 2 + sizeof(BlockDev) + 8;  // forward slot, half an inverse slot, descriptor, counters
 }
 
 int run_complex(pa_dtype_t dtype, const ClassRun &c, uint32_t *popc, uint32_t *marg, cudaStream_t st) {
@@ -433,11 +431,11 @@ int pa_uneven_create(const pa_block_desc_t *blocks, uint32_t nblocks, pa_dtype_t
         if (dtype == PA_NTT64) {
             U_TRY(cudaMalloc(&c.Wf, L * esz));
             U_TRY(cudaMalloc(&c.spec, L * esz));
+            U_TRY(cudaMalloc(&c.bits, bit_scratch_bytes(L, values_per_thread(dtype, L), 1)));
         } else {
             U_TRY(cudaMalloc(&c.Wf, (size_t)nb * L * esz));
             U_TRY(cudaMalloc(&c.Wi, (size_t)((nb + 1) / 2) * L * esz));
         }
-        U_TRY(cudaMalloc(&c.bits, pa::blocks::class_bit_bytes(L, dtype, dtype == PA_NTT64 ? 1 : nb)));
         rc = tune_class(u, c);
         if (rc != PA_OK) return fail(rc);
     }
