@@ -890,31 +890,46 @@ __device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32
 // Inverse transform of a strided pass's columns with the pass twiddle w^{-k u} (column u of stride S)
 // in the stages' multipliers: frequency k = k_0 + R_0 (k_1 + ...), and stage i, which sums over k_i with
 // w_{N_i}^{-j k_i}, takes w_{N_i S}^{-(S j + u) k_i} instead, the product of its table's entry and
-// h[i][u]. Twiddling the inputs first cost a product for every value, another to form its twiddle
+// an entry of the column tables. Twiddling the inputs first cost a product for every value, another to form its twiddle
 // (248 of a 256-point column thread's 866 instructions in single precision) and left the first stage's
 // butterflies without multipliers to absorb. Only outputs of butterfly slots below `need` (of stage 0's
 // radix) are wanted: with few of them stage 0 leaves out the butterflies of the others.
+// Single precision reads one column table per stage, w^{P_i u}, and forms the stage's multipliers by squarings, as it
+// does elsewhere. Double precision reads one per butterfly level: every multiplier is then the product of two
+// rounded roots, off by 4.25 units of 2^-53 at most (2.1 seen). Formed by squarings they were off by up to 18: the
+// rounding margins of a 2^23-bit key (512 * 64 * 384) were 8.2e-12 in the mean, now 4.3e-12 (with twiddled
+// inputs 6.5e-12), and a batch of 64 keys of 10^6 bits takes 10.05 ms instead of 10.11.
+// hu[l] = the entry of level l of stage I (SINGLE: hu[0], the last level's) in column u, h its entry in table 0.
 template <typename T, int LEN, int E, int I>
-__device__ __forceinline__ void col_multipliers(uint32_t tq, int g, const cx<T> *st, cx<T> w, cx<T> *m) {
+__device__ __forceinline__ void load_col(const cx<T> *h, uint32_t S, cx<T> *hu) {
+    constexpr StagePlan p = Plan<T, LEN, E>::p;
+#pragma unroll
+    for (int l = 0; l < stage_col_tables(p.R[I], kRows<T>); ++l) hu[l] = __ldg(h + (uint32_t)(first_col_table(p, I, kRows<T>) + l) * S);
+}
+template <typename T, int LEN, int E, int I>
+__device__ __forceinline__ void col_multipliers(uint32_t tq, int g, const cx<T> *st, const cx<T> *hu, cx<T> *m) {
     using M = StageMap<T, LEN, E, I>;
     constexpr StagePlan p = Plan<T, LEN, E>::p;
-    if constexpr (I < p.n - 1) {
-        // the stage table's entry w itself: its only row, or (double precision) row R/4, at least 0
-        constexpr int row = kRows<T> == Rows::SINGLE ? 0 : M::R / 4;
-        const uint32_t j = M::offset(tq, g);
-        const cx<T> *t = st + p.inv[I].off + (p.inv[I].rows == 1 ? j : 2 * (row / 2 * (uint32_t)M::s + j) + row % 2);
-        w = Arith<T>::mul(w, __ldg(t));
+    if constexpr (kRows<T> == Rows::SINGLE) {
+        cx<T> w = hu[0], pw[ilog2(M::R)];
+        if constexpr (I < p.n - 1) w = Arith<T>::mul(w, __ldg(st + p.inv[I].off + M::offset(tq, g)));
+        level_powers<T, M::R>(w, pw);
+        level_multipliers<T, M::R, 1, 0>(pw, m);
+    } else if constexpr (I < p.n - 1) {
+        load_rows<T, level_rows(M::R), M::s>(st + p.inv[I].off, M::offset(tq, g), m);
+#pragma unroll
+        for (int r = 0; r < level_rows(M::R); ++r) m[r] = Arith<T>::mul(m[r], hu[row_level(r)]);
+    } else {
+        level_multipliers<T, M::R, 1, 0>(hu, m);
     }
-    cx<T> pw[ilog2(M::R)];
-    level_powers<T, M::R>(w, pw);
-    level_multipliers<T, M::R, 1, 0>(pw, m);
 }
 template <typename T, int LEN, int COLS, int E, int I>
 __device__ __forceinline__ void inv_col_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st,
                                                const cx<T> *h, uint32_t S, uint32_t need) {
     using PL = Plan<T, LEN, E>;
     using M = StageMap<T, LEN, E, I>;
-    const cx<T> hu = __ldg(h + (uint32_t)I * S);
+    cx<T> hu[stage_col_tables(M::R, kRows<T>)];
+    load_col<T, LEN, E, I>(h, S, hu);
 #pragma unroll
     for (int g = 0; g < M::groups; ++g) {
         cx<T> m[level_rows(M::R)];

@@ -9,7 +9,7 @@
 // those callers use this entry point instead. All of its scratch -- the
 // transform work slot, the seed spectrum, the twiddle tables and the per-key
 // counters -- lives in one file-scope __device__ array of kScratchBytes bytes
-// (66.1 MiB), which every GPU that loads the library holds until the process
+// (66.4 MiB), which every GPU that loads the library holds until the process
 // exits. Inputs and outputs stay caller-owned.
 //
 // The paper has no counterpart to this entry point; it is a deployment aid.
@@ -34,9 +34,10 @@ namespace {
 // plus twiddle tables and per-key counters.
 constexpr int kMaxLgL = 21;
 constexpr size_t kSlotBytes = ((size_t)1 << kMaxLgL) * 16;        // 32 MiB
-constexpr size_t kTableBytes = (size_t)960 << 10;                     // FP64 twiddle tables (at most 860 KiB are used)
+constexpr size_t kTableBytes = (size_t)1344 << 10;                    // FP64 twiddle tables (at most 1290 KiB are used)
 constexpr size_t kBitBytes = ((size_t)1 << 20) + (64u << 10);         // transposed input bits and partial popcounts
-constexpr size_t kScratchBytes = 2 * kSlotBytes + ((size_t)1 << 20) + kBitBytes;  // 1 MiB: tables and counters
+constexpr size_t kTailBytes = kTableBytes + (4u << 10);               // tables, then counters
+constexpr size_t kScratchBytes = 2 * kSlotBytes + kTailBytes + kBitBytes;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -153,7 +154,7 @@ int run_static(unsigned char *base, int lgL, uint64_t n, uint64_t m, const uint6
     STATIC_CUDA(tw_fill(lay, dtype, tables, st));
     const TwTab<T> tw = tw_tab<T>(lay, tables);
     if (bit_scratch_bytes(L, Shape<T>::E, 1) > kBitBytes) return PA_EUNSUPPORTED;
-    const BitScratch bits = bit_scratch_at(tail + ((size_t)1 << 20), L, Shape<T>::E, 1);
+    const BitScratch bits = bit_scratch_at(tail + kTailBytes, L, Shape<T>::E, 1);
     FwdArgs in = seed_args<T>(bits.bits, n, m, false, L);
     STATIC_CUDA(launch_seed_bits(seed, n, m, bit_form<T>(lg1, L), bits.bits, nullptr, nullptr, st));
     STATIC_CUDA(launch_fwd<T>(lg1, In::SEED, in, 1, W, L, tw, st));

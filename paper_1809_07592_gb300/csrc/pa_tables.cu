@@ -65,10 +65,10 @@ __device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint6
             if (i >= g && i < g + t.stride) return t.tc * (i - g) * mult;
         }
         if (complex_) {
-            *neg = false;
             const StagePlan &l = plans[p];
-            if (i >= t.h && i < t.h + (uint64_t)l.n * t.stride)
-                return (uint64_t)l.P[(i - t.h) / t.stride] * ((i - t.h) % t.stride) * mult;
+            *neg = false;
+            if (i >= t.h && i < t.h + (uint64_t)col_tables(l, kind) * t.stride)
+                return col_exponent(l, (int)((i - t.h) / t.stride), kind) * ((i - t.h) % t.stride) * mult;
         }
     }
     *neg = false;
@@ -183,7 +183,7 @@ TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
         t.c = take(&y.total, (uint64_t)t.tc * t.cols);
         t.g = take(&y.total, t.stride);
         if (complex_) {
-            t.h = take(&y.total, (uint64_t)stage_plan(y.len[p], y.E, kind).n * t.stride);
+            t.h = take(&y.total, (uint64_t)col_tables(stage_plan(y.len[p], y.E, kind), kind) * t.stride);
         } else {  // residues have no conjugate: the inverse passes read tables of their own
             t.ai = take(&y.total, t.tc * (t.stride / t.cols));
             t.ci = take(&y.total, (uint64_t)t.tc * t.cols);

@@ -12,7 +12,8 @@
 //   pass tables  (one set per strided pass): the pass twiddle w^{k u} of frequency k = f + s*TC in
 //                column u = blk*COLS + col. Forward: a[f][blk] * c[f][col] * g[u]^s. Inverse, complex
 //                arithmetic: it goes into the stages' multipliers (inv_col_stages in fft_core.cuh),
-//                stage i needing h[i][u] = w^{P_i u} beside its stage table. The exact transform of
+//                stage i needing w^{P_i u} (single precision) or its powers for every butterfly level
+//                (double) beside its stage table: the column tables. The exact transform of
 //                zq.cuh, whose multipliers cannot be multiplied with each other: a[f][u] and g[s][u].
 #pragma once
 
@@ -142,13 +143,28 @@ __host__ __device__ inline uint64_t odd_exponent(int RO, int R0, uint64_t P, int
     return (uint64_t)(R0 >> (l + 1)) * (k * unit + (uint64_t)k1 * (L / RC)) + (uint64_t)row_pos(r) * (L >> (l + 1));
 }
 
+// Column tables (complex arithmetic): stage i has one (SINGLE, w^{P_i u}) or one per level l of its butterflies
+// (DOUBLE, w^{(R_i / 2^(l+1)) P_i u}), stage after stage. The factor of u in table t's exponent is col_exponent.
+__host__ __device__ constexpr int stage_col_tables(int R, Rows kind) { return kind == Rows::SINGLE ? 1 : ilog2(R); }
+__host__ __device__ constexpr int first_col_table(const StagePlan &l, int i, Rows kind) {
+    int t = 0;
+    for (int s = 0; s < i; ++s) t += stage_col_tables(l.R[s], kind);
+    return t;
+}
+__host__ __device__ constexpr int col_tables(const StagePlan &l, Rows kind) { return first_col_table(l, l.n, kind); }
+__host__ __device__ constexpr uint64_t col_exponent(const StagePlan &l, int t, Rows kind) {
+    int i = 0;
+    while (t >= stage_col_tables(l.R[i], kind)) t -= stage_col_tables(l.R[i++], kind);
+    return (uint64_t)l.P[i] * (kind == Rows::SINGLE ? 1u : (uint32_t)l.R[i] >> (t + 1));
+}
+
 // Where every table of one transform sits in its block of memory (offsets in elements).
 struct PassShape {
     uint32_t tc = 0, cols = 0;  // threads per column, columns per CTA
     uint64_t stride = 0;        // S: distance of a column's elements
     uint64_t a = 0, c = 0, g = 0;      // forward pass tables
     uint64_t ai = 0, ci = 0, gi = 0;   // inverse ones (the exact transforms)
-    uint64_t h = 0;                    // complex arithmetic: n tables of `stride` entries for the inverse stages
+    uint64_t h = 0;                    // complex arithmetic: column tables of `stride` entries for the inverse stages
 };
 struct TwLayout {
     uint64_t L = 0;
