@@ -16,12 +16,27 @@
 
 namespace pa {
 
+// Whether this thread's launch_chained makes ordinary launches: under stream capture. A graph launches its next kernel
+// without delay, and CTAs that start early there crowd onto the SMs the running kernel leaves free instead of
+// spreading over all of them. Two FP64 blocks of a class of length 262144 replayed in 244 us with such
+// edges and in 133 with ordinary ones (launched one by one: 150); 256 uneven blocks take the same time either way
+// (9.96 and 9.99 ms). The calls that can be captured set it for their duration: asking the stream at every launch
+// cost a call of eight launches 1.2 us.
+inline thread_local bool t_ordinary_launches = false;
+struct LaunchesFor {
+    bool before = t_ordinary_launches;
+    explicit LaunchesFor(cudaStream_t st) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+        t_ordinary_launches = capture != cudaStreamCaptureStatusNone;
+    }
+    ~LaunchesFor() { t_ordinary_launches = before; }
+    LaunchesFor(const LaunchesFor &) = delete;
+    LaunchesFor &operator=(const LaunchesFor &) = delete;
+};
+
 // Launches a kernel whose first instruction is begin_after_previous (fft_core.cuh): its CTAs may
-// start filling the SMs while the last CTAs of the stream's previous kernel still run. Not under stream
-// capture: a graph launches its next kernel without delay, and CTAs that start early there crowd onto the
-// SMs the running kernel leaves free instead of spreading over all of them. Two FP64 blocks of a class of length 262144
-// replayed in 244 us with such edges and in 133 with ordinary ones (launched one by one: 150); 256 uneven
-// blocks take the same time either way (9.96 and 9.99 ms).
+// start filling the SMs while the last CTAs of the stream's previous kernel still run.
 template <typename... Params, typename... Args>
 cudaError_t launch_chained(void (*kern)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
                            Args... args) {
@@ -34,9 +49,7 @@ cudaError_t launch_chained(void (*kern)(Params...), dim3 grid, unsigned threads,
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &attr;
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = t_ordinary_launches ? 0 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
     if (e != cudaSuccess) cudaGetLastError();  // reported here: the next <<<>>> launch must not find it again
     return e;

@@ -188,6 +188,7 @@ extern "C" int pa_hash_static(uint64_t n, uint64_t m, pa_dtype_t dtype, const ui
     int rc = scratch_address(&base);
     if (rc != PA_OK) return rc;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const LaunchesFor scope(st);  // a caller may capture the call
     uint32_t *marg = reinterpret_cast<uint32_t *>(base + 2 * kSlotBytes + kTableBytes) + 2;
 
     if (dtype == PA_NTT64) {

@@ -280,6 +280,7 @@ std::vector<BlockDev> class_descs(const pa_uneven_t *u, const UClass &c) {
 }
 
 int record_all(pa_uneven_t *u, cudaStream_t st) {
+    const LaunchesFor scope(st);  // a caller may capture a batch without a graph of its own
     for (const UClass &c : u->classes) {
         int rc = run_class(u, c, st);
         if (rc != PA_OK) return rc;
@@ -293,7 +294,8 @@ int capture_graph(pa_uneven_t *u) {
     cudaError_t e = cudaEventRecord(u->fork, u->cap);
     for (UClass &c : u->classes) {
         if (e != cudaSuccess || rc != PA_OK) break;
-        e = cudaStreamWaitEvent(c.st, u->fork, 0);
+        e = cudaStreamWaitEvent(c.st, u->fork, 0);  // c.st joins the capture
+        const LaunchesFor scope(c.st);
         if (e == cudaSuccess) rc = run_class(u, c, c.st);
         if (e == cudaSuccess && rc == PA_OK) e = cudaEventRecord(c.done, c.st);
         if (e == cudaSuccess && rc == PA_OK) e = cudaStreamWaitEvent(u->cap, c.done, 0);
