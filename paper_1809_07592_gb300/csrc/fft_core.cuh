@@ -471,14 +471,27 @@ __device__ __forceinline__ void level_powers(cx<T> w, cx<T> *pw) {
         if (l) w = square_root_of_unity<T>(w);
     }
 }
+// The same from a stage's table entries in single precision: w and, for R >= 8, w^4. At most one squaring away from a
+// rounded root, a power is off by 3.2 units of 2^-24 at most; from w alone w^8 was off by up to 10.
+// The uneven batch separates a block's key and seed spectra, which carries an error of the key's large low
+// frequencies into the seed's: margins there fell to 0.5 of what they were in the geometric mean over 33 splits of eight lengths
+// (two blocks of 2^24 bits to 2^23, 256 * 128 * 768: 7.8e-2, now 3.5e-2).
+template <typename T, int R>
+__device__ __forceinline__ void entry_powers(const cx<T> *w, cx<T> *pw) {
+    level_powers<T, R>(w[0], pw);
+    if constexpr (R >= 8) {
+        pw[ilog2(R) - 3] = w[1];
+        if constexpr (R == 16) pw[0] = square_root_of_unity<T>(w[1]);
+    }
+}
 
 // The multipliers of a power-of-two stage at table index k.
 template <typename T, int R, int P>
 __device__ __forceinline__ void stage_multipliers(const cx<T> *tab, uint32_t k, cx<T> *m) {
     if constexpr (kRows<T> == Rows::SINGLE) {
-        cx<T> w, pw[ilog2(R)];
-        load_rows<T, 1, P>(tab, k, &w);
-        level_powers<T, R>(w, pw);
+        cx<T> w[stage_rows(R, Rows::SINGLE)], pw[ilog2(R)];
+        load_rows<T, stage_rows(R, Rows::SINGLE), P>(tab, k, w);
+        entry_powers<T, R>(w, pw);
         level_multipliers<T, R, 1, 0>(pw, m);
     } else {
         load_rows<T, stage_rows(R, kRows<T>), P>(tab, k, m);
@@ -912,7 +925,7 @@ __device__ __forceinline__ void col_multipliers(uint32_t tq, int g, const cx<T> 
     constexpr StagePlan p = Plan<T, LEN, E>::p;
     if constexpr (kRows<T> == Rows::SINGLE) {
         cx<T> w = hu[0], pw[ilog2(M::R)];
-        if constexpr (I < p.n - 1) w = Arith<T>::mul(w, __ldg(st + p.inv[I].off + M::offset(tq, g)));
+        if constexpr (I < p.n - 1) w = Arith<T>::mul(w, __ldg(st + p.inv[I].off + (p.inv[I].rows == 1 ? 1 : 2) * M::offset(tq, g)));
         level_powers<T, M::R>(w, pw);
         level_multipliers<T, M::R, 1, 0>(pw, m);
     } else if constexpr (I < p.n - 1) {

@@ -57,16 +57,18 @@ struct StagePlan {
 // The three arithmetics' table rows. A complex stage needs the multipliers of its butterfly levels
 // (dft_rows in fft_core.cuh), R/2 of a radix-R power-of-two stage, RO-1 + RO*R0/2 of an odd one.
 // Double precision reads them all: its passes are bound by the FP64 pipe, the load path is idle. Single
-// precision reads w alone and forms the others (squarings and constant turns): its innermost
-// pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing four
-// wavefronts whatever the addresses) and has multiply-add slots to spare. The exact transforms read w^r, r = 1 .. R-1 (EXACT), or every level's
-// multipliers, R-1 as well, no two of which are a free quarter turn apart (LEVELS).
+// precision reads w, and w^4 for R >= 8, in one load and forms the others (at most one squaring, and constant turns):
+// its innermost pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing
+// four wavefronts whatever the addresses) and has multiply-add slots to spare. w alone would do, but w^8 is
+// then three squarings off (entry_powers in fft_core.cuh); the second row costs a batch of 64 keys of 10^6 bits 0.4 %
+// (292.3 -> 293.4 us) and saves the 2^27-bit block 1.8 % (1177 -> 1156 us). The exact transforms read w^r,
+// r = 1 .. R-1 (EXACT), or every level's multipliers, R-1 as well, no two of which are a free quarter turn apart (LEVELS).
 enum class Rows { SINGLE, DOUBLE, EXACT, LEVELS };
 __host__ __device__ constexpr bool is_complex(Rows kind) { return kind == Rows::SINGLE || kind == Rows::DOUBLE; }
 __host__ __device__ constexpr int level_rows(int R) { return R / 2; }
 __host__ __device__ constexpr int odd_level_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
 __host__ __device__ constexpr int stage_rows(int R, Rows kind) {
-    return kind == Rows::SINGLE ? 1 : kind == Rows::DOUBLE ? level_rows(R) : R - 1;
+    return kind == Rows::SINGLE ? (R >= 8 ? 2 : 1) : kind == Rows::DOUBLE ? level_rows(R) : R - 1;
 }
 __host__ __device__ constexpr int odd_rows(int RO, int R0, Rows kind) {
     return kind == Rows::SINGLE ? 1 : odd_level_rows(RO, R0);
@@ -130,6 +132,7 @@ __host__ __device__ inline uint64_t stage_exponent(int R, uint64_t P, int row, u
         const int l = ilog2(row + 1), p = row + 1 - (1 << l);
         return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)p * (L >> (l + 1));
     }
+    if (kind == Rows::SINGLE) return (row ? 4 : 1) * k * unit;
     if (kind != Rows::DOUBLE) return (uint64_t)(row + 1) * k * unit;
     const int l = row_level(row);
     return (uint64_t)(R >> (l + 1)) * k * unit + (uint64_t)row_pos(row) * (L >> (l + 1));

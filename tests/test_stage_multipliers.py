@@ -19,3 +19,11 @@ def test_double_precision_column_multipliers(tmp_path):
     so by 2 sqrt(2) u. Together 3 sqrt(2) u, and terms of order u^2."""
     worst = max(float(v) for v in compiled("multipliers", tmp_path).split())
     assert 0 < worst <= 3 * 2 ** 0.5 * (1 + 1e-9)
+
+
+def test_single_precision_stage_powers(tmp_path):
+    """A power is a rounded root or one squaring (1 - 2 s^2, 2 s c) away from one. In units u = 2^-24: s and c are off by
+    at most u/2, which moves the parts by at most 4 |s| u/2 and 2 (|s| + |c|) u/2, 2 u and sqrt(2) u; each is
+    rounded once more, by u/2. Together hypot(2.5, 1.92) u = 3.16 u, and terms of order u^2."""
+    worst = float(compiled("powers", tmp_path))
+    assert 0 < worst <= (2.5 ** 2 + (2 ** 0.5 + 0.5) ** 2) ** 0.5 * (1 + 1e-6)
