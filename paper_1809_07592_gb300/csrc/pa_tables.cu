@@ -78,11 +78,13 @@ __device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint6
 // exp(-2 pi i e / L), each part rounded once from double precision.
 template <typename T>
 __device__ cx<T> root_power(uint64_t e, uint64_t L, uint64_t) {
+    uint32_t q;
     double s, c;
-    sincospi(2.0 * ((double)e / (double)L), &s, &c);
+    sincospi(0.5 * quarter_turns((uint32_t)e, (uint32_t)L, &q), &s, &c);
+    const double x = q & 1 ? -s : c, y = q & 1 ? -c : -s;  // the first quarter turn: times -i
     cx<T> w;
-    w.x = (T)c;
-    w.y = (T)-s;
+    w.x = (T)(q & 2 ? -x : x);
+    w.y = (T)(q & 2 ? -y : y);
     return w;
 }
 template <>

@@ -146,6 +146,14 @@ __host__ __device__ inline uint64_t odd_exponent(int RO, int R0, uint64_t P, int
     return (uint64_t)(R0 >> (l + 1)) * (k * unit + (uint64_t)k1 * (L / RC)) + (uint64_t)row_pos(r) * (L >> (l + 1));
 }
 
+// e of L parts of a turn (e < L <= 2^28, 4 | L) as (q + x) quarter turns with |x| <= 1/2: integers reduce the angle, so that
+// x, the only rounded number, is off by 2^-55 of a quarter turn at most. (e / L, near 1, was off by eight times that in angle
+// for lengths with an odd factor.)
+__host__ __device__ inline double quarter_turns(uint32_t e, uint32_t L, uint32_t *q) {
+    *q = (4u * e + L / 2u) / L;
+    return (double)((int32_t)(4u * e) - (int32_t)(*q * L)) / (double)L;
+}
+
 // Column tables (complex arithmetic): stage i has one (SINGLE, w^{P_i u}) or one per level l of its butterflies
 // (DOUBLE, w^{(R_i / 2^(l+1)) P_i u}), stage after stage. The factor of u in table t's exponent is col_exponent.
 __host__ __device__ constexpr int stage_col_tables(int R, Rows kind) { return kind == Rows::SINGLE ? 1 : ilog2(R); }

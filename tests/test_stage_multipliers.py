@@ -27,3 +27,8 @@ def test_single_precision_stage_powers(tmp_path):
     rounded once more, by u/2. Together hypot(2.5, 1.92) u = 3.16 u, and terms of order u^2."""
     worst = float(compiled("powers", tmp_path))
     assert 0 < worst <= (2.5 ** 2 + (2 ** 0.5 + 0.5) ** 2) ** 0.5 * (1 + 1e-6)
+
+
+def test_table_angles_are_reduced_exactly(tmp_path):
+    """The angle of a table root is a quotient below one half of a quarter turn, rounded once: by 2^-55 of it at most."""
+    assert 0 < float(compiled("turns", tmp_path)) <= 1
