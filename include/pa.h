@@ -92,7 +92,8 @@ typedef struct {
  * {1, 3, 5, 9} (ro = 1 only for PA_NTT64), factors it into two or three passes,
  * builds twiddle tables, and allocates the seed-spectrum slot (L complex values)
  * on the current CUDA device. Where L has several valid pass splits, the first
- * plan of each (L, dtype) in a process times every split on a batch of zero keys
+ * plan of each (L, dtype) and, in the complex modes, share m / L (up to an eighth, up to
+ * a quarter, above) in a process times every split on a batch of zero keys
  * (stream-ordered on a private stream, up to 32 key pairs; set the environment
  * variable PA_PLAN_TUNE=0 to skip this and take the default split) and later
  * plans reuse the winner. Work buffers are allocated by the first pa_hash_batch
@@ -304,7 +305,8 @@ typedef struct pa_uneven pa_uneven_t;
  * powers of two only), as pa_plan chooses it; every class gets its own work buffers, twiddle
  * tables and a device copy of its block descriptors, and its pass split is chosen by the
  * built-in autotuner (timed on the class's own buffers, cached per (L, dtype) for the process
- * and, if the environment variable PA_TUNE_CACHE names a file, across processes).
+ * and, if the environment variable PA_TUNE_CACHE names a file, across processes: the first
+ * batch with blocks of a length decides for later ones, whatever their compression).
  * In PA_FP32_GUARD and PA_FP64 mode each block's key and seed share one complex transform,
  * z = x + i*sigma, and are separated after the forward transform with the paper's real-valued
  * FFT identities (Eq. 5-10); two blocks share each inverse transform. PA_NTT64 blocks run one

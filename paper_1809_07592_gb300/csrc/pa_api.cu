@@ -14,6 +14,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "pa.h"
@@ -502,11 +503,22 @@ void split_lengths(const Geometry &g, uint32_t *L1, uint32_t *L2, uint32_t *L3) 
 // ---- split autotuner ---------------------------------------------------------------------------
 // Every valid split of a transform length runs the same arithmetic in a different
 // pass structure; which one is fastest depends on the kernel instances and is
-// measured, not modelled: once per (L, dtype) and process, each candidate hashes a
+// measured, not modelled: once per SplitKey and process, each candidate hashes a
 // batch of all-zero keys (the kernels' cost does not depend on the bit values)
 // and the fastest is kept. PA_PLAN_TUNE=0 turns it off (the default split is used).
+//
+// The last pass of the complex transforms leaves out butterflies where at most an eighth or a quarter of the
+// outputs are kept (inv_col_stages), for some first-pass lengths only, so the fastest split depends on that share:
+// 64 FP64 keys of length 1310720 take 10.1 ms with the split that suits m = 0.45 L where m = 0.05 L, 9.8 with its own.
+struct SplitKey {
+    uint64_t L;
+    int dtype, kept;  // kept: 0, 1 or 2 for shares up to an eighth, up to a quarter and above
+    SplitKey(uint64_t length, pa_dtype_t d, uint64_t outputs)
+        : L(length), dtype((int)d), kept(d == PA_NTT64 || 4 * outputs > length ? 2 : 8 * outputs > length ? 1 : 0) {}
+    bool operator<(const SplitKey &o) const { return std::tie(L, dtype, kept) < std::tie(o.L, o.dtype, o.kept); }
+};
 std::mutex g_split_mu;
-std::map<std::pair<uint64_t, int>, Geometry> g_split;
+std::map<SplitKey, Geometry> g_split;
 
 bool tuning_enabled() {
     const char *s = std::getenv("PA_PLAN_TUNE");
@@ -531,10 +543,10 @@ int time_split(pa_plan_t *p, uint32_t nkeys, const uint64_t *keys, uint64_t kw, 
     return PA_OK;
 }
 
-// Chooses p->geo among the candidates of p->L (cached per process). The plan's spectrum
+// Chooses p->geo among the candidates of p->L (cached per SplitKey and process). The plan's spectrum
 // slot must exist; twiddles and work buffers made for the trials are released again.
 int tune_split(pa_plan_t *p, const std::vector<Geometry> &cand) {
-    const std::pair<uint64_t, int> key{p->L, (int)p->dtype};
+    const SplitKey key(p->L, p->dtype, p->m);
     {
         std::lock_guard<std::mutex> lk(g_split_mu);
         auto it = g_split.find(key);
@@ -602,8 +614,8 @@ int tune_split(pa_plan_t *p, const std::vector<Geometry> &cand) {
 // The half-length form of a plan: the smallest supported N with 2N >= n+m-1 whose
 // innermost pass fits the two-row kernel; left out (nullptr) if there is none.
 // Split autotuner of the half-length form (as tune_split, on one zero key, cached per
-// (N, dtype)). r->tabs must exist; the chosen split's twiddles are built by the caller.
-std::map<std::pair<uint64_t, int>, Geometry> g_real_split;
+// SplitKey of N and the output pairs). r->tabs must exist; the chosen split's twiddles are built by the caller.
+std::map<SplitKey, Geometry> g_real_split;
 
 template <typename T>
 int time_real(pa_plan_t *p, const uint64_t *key, uint64_t kw, uint64_t *out, uint64_t ow, cudaStream_t st,
@@ -623,7 +635,7 @@ int time_real(pa_plan_t *p, const uint64_t *key, uint64_t kw, uint64_t *out, uin
 }
 
 int tune_real(pa_plan_t *p, RealMode *r) {
-    const std::pair<uint64_t, int> cache_key{r->geo.L, (int)p->dtype};
+    const SplitKey cache_key(r->geo.L, p->dtype, (p->m + 1) / 2);
     {
         std::lock_guard<std::mutex> lk(g_split_mu);
         auto it = g_real_split.find(cache_key);
