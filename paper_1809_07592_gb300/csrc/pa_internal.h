@@ -6,7 +6,7 @@
 
 #include <cuda_runtime.h>
 
-#include "tables.cuh"
+#include "fft_core.cuh"
 
 // Records "what: cuda error string" as the calling thread's last CUDA error and returns PA_ECUDA.
 int pa_internal_cuda_fail(cudaError_t e, const char *what);
@@ -27,8 +27,8 @@ struct Geometry {
 };
 
 // Whether the exact transform of length L runs modulo the word-sized prime of zq.cuh (lengths up to
-// 2^26, where it has roots of unity) instead of the 64-bit one, and the values a thread holds.
-inline bool narrow_exact(pa_dtype_t dtype, uint64_t L) { return dtype == PA_NTT64 && L <= (1ull << 26); }
+// 2^kMaxLgZq, where it has roots of unity) instead of the 64-bit one, and the values a thread holds.
+inline bool narrow_exact(pa_dtype_t dtype, uint64_t L) { return dtype == PA_NTT64 && L <= (1ull << kMaxLgZq); }
 inline int values_per_thread(pa_dtype_t dtype, uint64_t L) { return dtype == PA_FP32_GUARD || narrow_exact(dtype, L) ? 16 : 8; }
 
 // Every valid split of length L for the arithmetic `dtype` (split = the

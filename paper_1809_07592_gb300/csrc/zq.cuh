@@ -19,6 +19,9 @@ struct Zq {};  // tag type: two residues modulo q per element
 
 constexpr uint32_t kQ = 469762049u;  // 7 * 2^26 + 1, prime; 3 generates the multiplicative group
 constexpr int kMaxLgZq = 26;
+static_assert(kQ > (1u << 27), "above every count of a key of up to 2^27 bits");
+static_assert((kQ - 1) % (1u << kMaxLgZq) == 0, "roots of unity of order 2^kMaxLgZq");
+static_assert(4ull * kQ <= 1ull << 32, "lazy residues below 4q fit a word");
 
 __host__ __device__ constexpr uint32_t zq_mul(uint32_t a, uint32_t b) { return (uint32_t)((uint64_t)a * b % kQ); }
 __host__ __device__ constexpr uint32_t zq_pow(uint32_t a, uint64_t e) {
