@@ -449,7 +449,7 @@ int pa_alu_peaks(double *fp64_gflops, double *zp_gmul_s, pa_stream_t stream);
  * allocation after start-up.
  *
  * All scratch (work slot, seed spectrum, twiddle tables, per-key counters) sits
- * in one static device array of 66.4 MiB inside libpa.so, which every GPU that
+ * in one static device array of 66.3 MiB inside libpa.so, which every GPU that
  * loads the library holds until the process exits. Limits: n + m - 1 <= 2^21
  * (larger sizes return PA_EUNSUPPORTED), nkeys is 1 or 2. Arguments are those of
  * pa_plan + pa_set_seed + pa_hash_batch for one call (seed_dev holds n+m-1 bits);

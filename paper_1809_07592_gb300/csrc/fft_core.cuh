@@ -689,7 +689,7 @@ __device__ __forceinline__ void dft_comp_rows(cx<T> *x, const cx<T> *tab, uint32
 
 // The pass twiddles: v[s] *= w^{(tq + s*TC) u} for s = 0 .. N-1 and column u = blk*COLS + col
 // (nblk column blocks): one product for s = 0, then a chain of products with g = w^{TC u}.
-template <typename T, bool INV, int N, int COLS>
+template <typename T, int N, int COLS>
 __device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint32_t nblk, uint32_t tq, uint32_t blk,
                                               uint32_t col) {
     if constexpr (std::is_same<T, Zq>::value) {  // multipliers do not multiply: one product per table
@@ -701,17 +701,13 @@ __device__ __forceinline__ void pass_twiddles(cx<T> *v, const PassTw<T> &t, uint
             v[s] = Arith<T>::mul(v[s], p);
         }
     } else {
-    cx<T> w = Arith<T>::mul(__ldg(t.a + (uint64_t)tq * nblk + blk), __ldg(t.c + tq * COLS + col));
-    cx<T> g = __ldg(t.g + blk * COLS + col);
-    if constexpr (INV && !std::is_same<T, Zp>::value) {
-        w.y = -w.y;
-        g.y = -g.y;
-    }
+        cx<T> w = Arith<T>::mul(__ldg(t.a + (uint64_t)tq * nblk + blk), __ldg(t.c + tq * COLS + col));
+        const cx<T> g = __ldg(t.g + blk * COLS + col);
 #pragma unroll
-    for (int r = 0; r < N; ++r) {
-        v[r] = Arith<T>::mul(v[r], w);
-        if (r + 1 < N) w = Arith<T>::mul(w, g);
-    }
+        for (int r = 0; r < N; ++r) {
+            v[r] = Arith<T>::mul(v[r], w);
+            if (r + 1 < N) w = Arith<T>::mul(w, g);
+        }
     }
 }
 
@@ -975,7 +971,7 @@ __device__ __forceinline__ void inverse_columns(cx<T> *sm, cx<T> *v, uint32_t tq
                                                 uint32_t nblk, uint32_t blk, uint32_t S, uint32_t nrow) {
     using PL = Plan<T, LEN, E>;
     if constexpr (!is_complex(kRows<T>)) {
-        pass_twiddles<T, true, E, COLS>(v, tw.iv[PASS], nblk, freq_of<T, LEN, E>(tq), blk, col);
+        pass_twiddles<T, E, COLS>(v, tw.iv[PASS], nblk, freq_of<T, LEN, E>(tq), blk, col);
         cta_fft<T, LEN, COLS, E, true>(sm, v, tq, col, tw.st[PASS]);
     } else {
         constexpr uint32_t K = LEN / PL::r0;  // rows of one butterfly slot of stage 0

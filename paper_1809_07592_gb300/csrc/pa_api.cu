@@ -197,7 +197,7 @@ template <typename T> cx<T> one() {
     return s;
 }
 template <> cx<Zp> one<Zp>() { return 1; }
-template <> cx<Zq> one<Zq>() { return make_uint2(1u, 0u); }
+template <> cx<Zq> one<Zq>() { return make_uint2(1u, zq_quotient(1u)); }
 
 // Calls f(T()) for the arithmetic a plan's kernels run in.
 template <typename F> auto with_type(const pa_plan_t *p, F &&f) {
@@ -677,7 +677,7 @@ int tune_real(pa_plan_t *p, RealMode *r) {
     Geometry bestg = r->geo;
     for (size_t i = 0; i < cand.size(); ++i) {
         r->geo = cand[i];
-        rc = pa_internal_twiddles(r->geo, p->dtype, &r->tw);
+        rc = pa_internal_twiddles(r->geo, p->dtype, &r->tw, true);
         float ms = 0.f;
         if (rc == PA_OK)
             rc = (p->dtype == PA_FP32_GUARD) ? time_real<float>(p, key, kw, out, ow, st, a, b, &ms)
@@ -712,7 +712,7 @@ int build_real_mode(pa_plan_t *p) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(real tables)");
     int rc = tune_real(p, r);
     if (rc != PA_OK) return rc;
-    return pa_internal_twiddles(r->geo, p->dtype, &r->tw);
+    return pa_internal_twiddles(r->geo, p->dtype, &r->tw, true);
 }
 
 // pa_plan (or pa_plan_modified), with the split forced when `force` is given. For the

@@ -15,11 +15,9 @@ int pa_internal_cuda_fail(cudaError_t e, const char *what);
 
 namespace pa {
 
-// Transform geometry: length L = lgL-free description
-//   L = 2^lg1 * 2^lgM * (ro * 2^lgI)
+// Transform geometry: length L = 2^lg1 * 2^lgM * (ro * 2^lgI),
 // strided level-1 pass 2^lg1, optional middle strided pass 2^lgM (lgM = 0: none),
-// innermost pass ro * 2^lgI (ro in {1, 3, 5, 9}). F = lcm of the pass lengths is
-// the length of the stage-twiddle table.
+// innermost pass ro * 2^lgI (ro in {1, 3, 5, 9}).
 struct Geometry {
     uint64_t L = 0;
     int lg1 = 0, lgM = 0, ro = 1, lgI = 0;
@@ -41,8 +39,9 @@ Geometry default_geometry(uint64_t L, pa_dtype_t dtype, bool split);
 Geometry choose_geometry(uint64_t need, pa_dtype_t dtype, bool split);
 
 // Twiddle tables of a transform: where they sit in one block of memory, and filling that
-// block on `st` (cudaErrorInvalidValue if the arithmetic has no root of order L).
-TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype);
+// block on `st` (cudaErrorInvalidValue if the arithmetic has no root of order L). powers: with the tables of
+// single powers (TwTab hi, lo), which only the half-length form's innermost pass reads.
+TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype, bool powers = false);
 cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t st);
 
 // The tables of one transform in device memory of their own.
@@ -56,5 +55,5 @@ uint64_t zp_pow_host(uint64_t a, uint64_t e);  // a^e mod p (the exact transform
 }  // namespace pa
 
 // Allocate and fill the tables (waits for the fill) / release them.
-int pa_internal_twiddles(const pa::Geometry &g, pa_dtype_t dtype, pa::TwSet *out);
+int pa_internal_twiddles(const pa::Geometry &g, pa_dtype_t dtype, pa::TwSet *out, bool powers = false);
 void pa_internal_free_twiddles(pa::TwSet *t);

@@ -108,10 +108,6 @@ template <typename T> struct Enc {
         return Arith<T>::mk(pm_two(x, j, in_re, j), pm_two(x, 16 + j, in_im, j));
     }
     // bits and margins of the two values carried by v (valid_b: the imaginary part's own range)
-    static __device__ __forceinline__ void decode(E v, uint32_t popa, uint32_t popb, bool valid, bool &bit_a,
-                                                  bool &bit_b, M &ma, M &mb) {
-        decode2(v, popa, popb, valid, valid, bit_a, bit_b, ma, mb);
-    }
     static __device__ __forceinline__ void decode2(E v, uint32_t popa, uint32_t popb, bool valid_a, bool valid_b,
                                                    bool &bit_a, bool &bit_b, M &ma, M &mb) {
         const T wa = ((T)(popa & 3u) - v.x) * (T)0.5, wb = ((T)(popb & 3u) - v.y) * (T)0.5;
@@ -131,12 +127,6 @@ template <> struct Enc<Zp> {
     }
     // (the exact transform has no half-length packing and no key+seed form: its values are not complex)
     static __device__ __forceinline__ E seed(uint32_t x, uint32_t, uint32_t, int j) { return (E)((x >> j) & 1u); }
-    static __device__ __forceinline__ E key_seed(uint32_t, uint32_t, int) { return 0ull; }
-    static __device__ __forceinline__ void decode(E v, uint32_t, uint32_t, bool valid, bool &bit_a, bool &bit_b, M &,
-                                                  M &) {
-        bit_a = valid && (v & 1ull);
-        bit_b = valid && ((v >> 32) & 1ull);
-    }
     static __device__ __forceinline__ void decode2(E v, uint32_t, uint32_t, bool valid_a, bool valid_b, bool &bit_a,
                                                    bool &bit_b, M &, M &) {
         bit_a = valid_a && (v & 1ull);
@@ -144,7 +134,6 @@ template <> struct Enc<Zp> {
     }
 };
 
-// ---------------------------------------------------------------------------
 template <> struct Enc<Zq> {
     using E = cx<Zq>;
     using M = float;
@@ -156,6 +145,7 @@ template <> struct Enc<Zq> {
         bit_b = valid_b && (Arith<Zq>::canonical(v.y) & 1u);
     }
 };
+
 // A value of the seed's spectrum as the product takes it.
 template <typename T>
 __device__ __forceinline__ cx<T> spectrum_value(cx<T> v) {
@@ -304,7 +294,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
     }
     const uint32_t f = freq_of<T, LEN, E>(tq);
-    pass_twiddles<T, false, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
+    pass_twiddles<T, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
     cx<T> *w = W + (uint64_t)blockIdx.y * L + u;
 #pragma unroll
     for (int s = 0; s < E; ++s) w[(f + s * (LEN / E)) * S] = v[s];
@@ -355,7 +345,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         inverse_columns<T, LEN, COLS, E, 1>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, S, LEN);
     } else {
         cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[1]);
-        pass_twiddles<T, false, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
+        pass_twiddles<T, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
     }
     // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
     // addresses in registers through the transform (80 bytes of spills)

@@ -9,7 +9,7 @@
 // those callers use this entry point instead. All of its scratch -- the
 // transform work slot, the seed spectrum, the twiddle tables and the per-key
 // counters -- lives in one file-scope __device__ array of kScratchBytes bytes
-// (66.4 MiB), which every GPU that loads the library holds until the process
+// (66.3 MiB), which every GPU that loads the library holds until the process
 // exits. Inputs and outputs stay caller-owned.
 //
 // The paper has no counterpart to this entry point; it is a deployment aid.
@@ -34,7 +34,7 @@ namespace {
 // plus twiddle tables and per-key counters.
 constexpr int kMaxLgL = 21;
 constexpr size_t kSlotBytes = ((size_t)1 << kMaxLgL) * 16;        // 32 MiB
-constexpr size_t kTableBytes = (size_t)1344 << 10;                    // FP64 twiddle tables (at most 1290 KiB are used)
+constexpr size_t kTableBytes = (size_t)1280 << 10;                    // FP64 twiddle tables (at most 1242 KiB are used)
 constexpr size_t kBitBytes = ((size_t)1 << 20) + (64u << 10);         // transposed input bits and partial popcounts
 constexpr size_t kTailBytes = kTableBytes + (4u << 10);               // tables, then counters
 constexpr size_t kScratchBytes = 2 * kSlotBytes + kTailBytes + kBitBytes;
@@ -118,7 +118,7 @@ template <> cx<Zq> scale_of<Zq>(uint64_t L) {
 template <typename T> cx<T> unit();
 template <> cx<float> unit<float>() { return make_float2(1.f, 0.f); }
 template <> cx<double> unit<double>() { return make_double2(1.0, 0.0); }
-template <> cx<Zq> unit<Zq>() { return make_uint2(0u, 0u); }
+template <> cx<Zq> unit<Zq>() { return make_uint2(1u, zq_quotient(1u)); }
 
 #define STATIC_CUDA(x)                               \
     do {                                             \

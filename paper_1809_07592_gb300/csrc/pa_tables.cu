@@ -150,16 +150,18 @@ static Rows rows_of(pa_dtype_t dtype, uint64_t L) {
                                         : kRows<Zp>;
 }
 
-TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype) {
+TwLayout tw_layout(const Geometry &g, pa_dtype_t dtype, bool powers) {
     const Rows kind = rows_of(dtype, g.L);
     const bool complex_ = is_complex(kind);
     TwLayout y;
     y.L = g.L;
-    int lgL = 0;
-    while ((1ull << lgL) < g.L) ++lgL;
-    y.B = (uint32_t)(lgL + 1) / 2;
-    y.nlo = 1ull << y.B;
-    y.nhi = (g.L + y.nlo - 1) >> y.B;
+    if (powers) {
+        int lgL = 0;
+        while ((1ull << lgL) < g.L) ++lgL;
+        y.B = (uint32_t)(lgL + 1) / 2;
+        y.nlo = 1ull << y.B;
+        y.nhi = (g.L + y.nlo - 1) >> y.B;
+    }
     y.E = values_per_thread(dtype, g.L);
     y.len[0] = 1 << g.lg1;
     y.len[1] = g.lgM ? 1 << g.lgM : 0;
@@ -219,8 +221,8 @@ cudaError_t tw_fill(const TwLayout &y, pa_dtype_t dtype, void *mem, cudaStream_t
 
 }  // namespace pa
 
-int pa_internal_twiddles(const Geometry &g, pa_dtype_t dtype, TwSet *out) {
-    out->lay = tw_layout(g, dtype);
+int pa_internal_twiddles(const Geometry &g, pa_dtype_t dtype, TwSet *out, bool powers) {
+    out->lay = tw_layout(g, dtype, powers);
     const size_t esz = dtype == PA_FP32_GUARD ? sizeof(float2) : dtype == PA_FP64 ? sizeof(double2) : sizeof(uint64_t);
     cudaError_t e = cudaMalloc(&out->mem, out->lay.total * esz);
     if (e == cudaErrorMemoryAllocation) {

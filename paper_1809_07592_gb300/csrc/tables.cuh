@@ -6,7 +6,7 @@
 // lookups are whole 128-byte lines. (The passes used to gather from one table of powers:
 // on rows of 256 values those gathers were 150 of the 271 shared-memory/L1 wavefronts a
 // warp of the first pass needs.) Three kinds:
-//   hi, lo       w_L^e = hi[e >> B] * lo[e mod 2^B], for single powers at any e;
+//   hi, lo       w_L^e = hi[e >> B] * lo[e mod 2^B], for single powers at any e (the half-length form only);
 //   stage tables (one per pass length): the multipliers of every in-CTA butterfly stage
 //                (stage_plan gives the stages, stage_exponent what each row holds);
 //   pass tables  (one set per strided pass): the pass twiddle w^{k u} of frequency k = f + s*TC in
