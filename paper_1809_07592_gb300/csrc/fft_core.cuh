@@ -471,30 +471,35 @@ __device__ __forceinline__ void level_powers(cx<T> w, cx<T> *pw) {
         if (l) w = square_root_of_unity<T>(w);
     }
 }
-// The same from a stage's table entries in single precision: w and, for R >= 8, w^4. At most one squaring away from a
-// rounded root, a power is off by 3.2 units of 2^-24 at most; from w alone w^8 was off by up to 10.
-// The uneven batch separates a block's key and seed spectra, which carries an error of the key's large low
-// frequencies into the seed's: margins there fell to 0.5 of what they were in the geometric mean over 33 splits of eight lengths
-// (two blocks of 2^24 bits to 2^23, 256 * 128 * 768: 7.8e-2, now 3.5e-2).
-template <typename T, int R>
+// The same from a stage's table entries in single precision: w and, NEAR, w^4 (R >= 8). At most one squaring away from a
+// rounded root, a power is off by 3.2 units of 2^-24 at most; from w alone w^8 is off by up to 10.
+// NEAR is for the uneven batch's forward stages, which separate a block's key and seed spectra afterwards: that carries an
+// error of the key's large low frequencies into the seed's. Margins there fell to 0.5 of what they were in the geometric
+// mean over 33 splits of eight lengths (four blocks of 2^24 bits to 2^23, 256 * 128 * 768: 7.8e-2, now 3.5e-2).
+// It costs the split pass 5 and 8 % on rows of 3072 and 6144 values (registers) and saves it up to 6 % on others; 256
+// uneven blocks take the same 10.0 ms. The half-length form's two-row pass and the middle strided pass take it too (a
+// 2^27-bit block 1177 -> 1156 us). The plain passes of key pairs, whose margins are far below (0.54-0.83 of those with twiddled
+// inputs), read w alone: a second row made the innermost pass 1-3.5 % slower on most row lengths (4096: 118.2 -> 122.5 us).
+template <typename T, int R, bool NEAR>
 __device__ __forceinline__ void entry_powers(const cx<T> *w, cx<T> *pw) {
     level_powers<T, R>(w[0], pw);
-    if constexpr (R >= 8) {
+    if constexpr (NEAR && R >= 8) {
         pw[ilog2(R) - 3] = w[1];
         if constexpr (R == 16) pw[0] = square_root_of_unity<T>(w[1]);
     }
 }
 
 // The multipliers of a power-of-two stage at table index k.
-template <typename T, int R, int P>
+template <typename T, int R, int P, bool NEAR>
 __device__ __forceinline__ void stage_multipliers(const cx<T> *tab, uint32_t k, cx<T> *m) {
     if constexpr (kRows<T> == Rows::SINGLE) {
-        cx<T> w[stage_rows(R, Rows::SINGLE)], pw[ilog2(R)];
-        load_rows<T, stage_rows(R, Rows::SINGLE), P>(tab, k, w);
-        entry_powers<T, R>(w, pw);
+        cx<T> w[2], pw[ilog2(R)];
+        w[0] = __ldg(tab + k);
+        if constexpr (NEAR && R >= 8) w[1] = __ldg(tab + P + k);
+        entry_powers<T, R, NEAR>(w, pw);
         level_multipliers<T, R, 1, 0>(pw, m);
     } else {
-        load_rows<T, stage_rows(R, kRows<T>), P>(tab, k, m);
+        load_rows<T, stage_rows(R, kRows<T>, false), P>(tab, k, m);
     }
 }
 // The multipliers of the odd stage (odd_exponent) at table index k.
@@ -832,8 +837,8 @@ __device__ __forceinline__ void store_stage(cx<T> *sm, const cx<T> *v, uint32_t 
         for (int r = 0; r < M::R; ++r) sm[s0 + slot_of<T, COLS>((uint32_t)(r * M::s), 0)] = v[g * M::R + r];
     }
 }
-// The butterflies of stage I on the thread's registers.
-template <typename T, int LEN, int E, int I, bool INV, int FROM = 0>
+// The butterflies of stage I on the thread's registers (NEAR: entry_powers).
+template <typename T, int LEN, int E, int I, bool INV, int FROM = 0, bool NEAR = false>
 __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *st) {
     using M = StageMap<T, LEN, E, I>;
     constexpr StagePlan p = Plan<T, LEN, E>::p;
@@ -845,7 +850,7 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
             dft<T, M::R, INV, FROM>(v + g * M::R);
         } else {
             cx<T> w[multipliers<T>(M::R)];
-            stage_multipliers<T, M::R, COUNT>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
+            stage_multipliers<T, M::R, COUNT, NEAR && !INV>(st + row.off, INV ? M::offset(tq, g) : M::block(tq), w);
             dft_rows<T, M::R, INV>(v + g * M::R, w);
         }
     }
@@ -853,17 +858,17 @@ __device__ __forceinline__ void stage_regs(cx<T> *v, uint32_t tq, const cx<T> *s
 
 // Forward stages I .. n-1, stage I's inputs in shared memory (a barrier away) unless FROM_REGS;
 // the outputs end in registers (frequencies freq_of(tq) + s*TC).
-template <typename T, int LEN, int COLS, int E, int I, bool FROM_REGS, int FROM = 0>
+template <typename T, int LEN, int COLS, int E, int I, bool FROM_REGS, int FROM = 0, bool NEAR = false>
 __device__ __forceinline__ void fwd_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     using PL = Plan<T, LEN, E>;
     if constexpr (!FROM_REGS) {
         exchange_barrier<COLS * PL::p.N[I - 1], E>();
         load_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
     }
-    stage_regs<T, LEN, E, I, false, FROM>(v, tq, st);
+    stage_regs<T, LEN, E, I, false, FROM, NEAR>(v, tq, st);
     if constexpr (I < PL::n - 1) {
         store_stage<T, LEN, COLS, E, I>(sm, v, tq, col);
-        fwd_stages<T, LEN, COLS, E, I + 1, false>(sm, v, tq, col, st);
+        fwd_stages<T, LEN, COLS, E, I + 1, false, 0, NEAR>(sm, v, tq, col, st);
     }
 }
 // Inverse stages I .. LAST (counting down), stage I's inputs in registers; the outputs of stage LAST
@@ -885,12 +890,12 @@ __device__ __forceinline__ void inv_stages(cx<T> *sm, cx<T> *v, uint32_t tq, uin
 // other way round. A forward transform writes shared memory that other threads may still be
 // reading (from an earlier one): the caller puts a barrier before it. An inverse transform
 // first writes the slots the same thread read last in the forward one.
-template <typename T, int LEN, int COLS, int E, bool INV>
+template <typename T, int LEN, int COLS, int E, bool INV, bool NEAR = false>
 __device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32_t col, const cx<T> *st) {
     using PL = Plan<T, LEN, E>;
     static_assert(PL::RO == 1, "odd lengths use cta_fft_fwd_odd / cta_fft_inv_odd");
     if constexpr (!INV) {
-        fwd_stages<T, LEN, COLS, E, 0, true>(sm, v, tq, col, st);
+        fwd_stages<T, LEN, COLS, E, 0, true, 0, NEAR>(sm, v, tq, col, st);
     } else {
         inv_stages<T, LEN, COLS, E, PL::n - 1, 0, false>(sm, v, tq, col, st);
     }
@@ -921,7 +926,7 @@ __device__ __forceinline__ void col_multipliers(uint32_t tq, int g, const cx<T> 
     constexpr StagePlan p = Plan<T, LEN, E>::p;
     if constexpr (kRows<T> == Rows::SINGLE) {
         cx<T> w = hu[0], pw[ilog2(M::R)];
-        if constexpr (I < p.n - 1) w = Arith<T>::mul(w, __ldg(st + p.inv[I].off + (p.inv[I].rows == 1 ? 1 : 2) * M::offset(tq, g)));
+        if constexpr (I < p.n - 1) w = Arith<T>::mul(w, __ldg(st + p.inv[I].off + M::offset(tq, g)));
         level_powers<T, M::R>(w, pw);
         level_multipliers<T, M::R, 1, 0>(pw, m);
     } else if constexpr (I < p.n - 1) {
@@ -984,7 +989,7 @@ __device__ __forceinline__ void inverse_columns(cx<T> *sm, cx<T> *v, uint32_t tq
 // Stage 0 has the odd (or composite) radix RC: group b = tq + g TC < K = LEN / RC reads elements
 // b + r K through ld(offset), the offset g TC + r K counted from element tq (a compile-time
 // constant, so the caller's base pointer for thread tq takes immediate offsets).
-template <typename T, int LEN, int E, class Ld>
+template <typename T, int LEN, int E, bool NEAR, class Ld>
 __device__ __forceinline__ void cta_fft_fwd_odd(cx<T> *sm, cx<T> *v, uint32_t tq, const cx<T> *st, Ld ld) {
     constexpr StagePlan p = Plan<T, LEN, E>::p;
     constexpr int RC = p.RC, K = LEN / RC, TC = p.TC;
@@ -1002,7 +1007,7 @@ __device__ __forceinline__ void cta_fft_fwd_odd(cx<T> *sm, cx<T> *v, uint32_t tq
             for (int r = 0; r < RC; ++r) sm[s0 + slot_of<T, 1>((uint32_t)(r * K), 0)] = u[r];
         }
     }
-    fwd_stages<T, LEN, 1, E, 1, false>(sm, v, tq, 0, st);
+    fwd_stages<T, LEN, 1, E, 1, false, 0, NEAR>(sm, v, tq, 0, st);
 }
 
 // Inverse transform of a row (RO > 1): the power-of-two stages from registers into shared memory,

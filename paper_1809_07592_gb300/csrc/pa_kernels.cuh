@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     } else {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = b[s];
-        cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[0]);
+        cta_fft<T, LEN, COLS, E, false, KIND == In::BLOCKS>(sm, v, tq, col, tw.st[0]);
     }
     const uint32_t f = freq_of<T, LEN, E>(tq);
     pass_twiddles<T, E, COLS>(v, tw.fw[0], gridDim.x, f, blockIdx.x, col);
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     if constexpr (INV) {
         inverse_columns<T, LEN, COLS, E, 1>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, S, LEN);
     } else {
-        cta_fft<T, LEN, COLS, E, false>(sm, v, tq, col, tw.st[1]);
+        cta_fft<T, LEN, COLS, E, false, true>(sm, v, tq, col, tw.st[1]);
         pass_twiddles<T, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
     }
     // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(LEN / E, min_blocks_inner(LEN / E, sizeof(cx<T
         for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
         cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
+        cta_fft_fwd_odd<T, LEN, E, false>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
     }
     if constexpr (MODE == 1) {
 #pragma unroll
@@ -792,9 +792,9 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_split(2 * (LEN / E),
         if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
             for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
-            cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
+            cta_fft<T, LEN, 1, E, false, true>(sm, v, tq, 0, tw.st[2]);
         } else {
-            cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
+            cta_fft_fwd_odd<T, LEN, E, true>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
         }
         store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
         __syncthreads();
@@ -864,9 +864,9 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_real(2 * (LEN / E), 
     if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
-        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
+        cta_fft<T, LEN, 1, E, false, true>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
+        cta_fft_fwd_odd<T, LEN, E, true>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
     }
     store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
     __syncthreads();

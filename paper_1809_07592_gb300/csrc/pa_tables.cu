@@ -37,8 +37,9 @@ __device__ uint64_t exponent_at(const TwLayout &y, const StagePlan *plans, uint6
             const StageRow r = inv ? l.inv[stage] : l.fwd[stage];
             const int count = inv ? l.s[stage] : l.P[stage];
             if (r.rows == 0 || o < r.off || o >= r.off + row_entries(r.rows, count)) continue;
-            const int q = r.rows == 1 ? o - r.off : (o - r.off) / 2;
-            const int row = r.rows == 1 ? q / count : 2 * (q / count) + ((o - r.off) & 1);
+            const bool pairs = r.rows > 1 && kind != Rows::SINGLE;
+            const int q = pairs ? (o - r.off) / 2 : o - r.off;
+            const int row = pairs ? 2 * (q / count) + ((o - r.off) & 1) : q / count;
             const uint32_t x = (uint32_t)(q % count);
             if (row >= r.rows) return 0;
             *neg = !complex_ && inv;

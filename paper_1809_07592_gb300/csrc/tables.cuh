@@ -49,7 +49,8 @@ struct StagePlan {
     // Twiddle tables: butterfly (block b, offset j) of forward stage i reads rows at index b < P[i],
     // of inverse stage i at index j < s[i]. Rows are stored in pairs, entry (row, x) at
     // off + 2*((row/2)*count + x) + row%2 (one row: off + x), so that a pair takes one wide
-    // load. rows = 0: no twiddles (forward stage 0, inverse stage n-1).
+    // load; single precision's at off + row*count + x, most readers taking the first alone. rows = 0: no twiddles
+    // (forward stage 0, inverse stage n-1).
     StageRow fwd[kMaxStages], inv[kMaxStages];
     int total;  // entries
 };
@@ -57,18 +58,18 @@ struct StagePlan {
 // The three arithmetics' table rows. A complex stage needs the multipliers of its butterfly levels
 // (dft_rows in fft_core.cuh), R/2 of a radix-R power-of-two stage, RO-1 + RO*R0/2 of an odd one.
 // Double precision reads them all: its passes are bound by the FP64 pipe, the load path is idle. Single
-// precision reads w, and w^4 for R >= 8, in one load and forms the others (at most one squaring, and constant turns):
-// its innermost pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing
-// four wavefronts whatever the addresses) and has multiply-add slots to spare. w alone would do, but w^8 is
-// then three squarings off (entry_powers in fft_core.cuh); the second row costs a batch of 64 keys of 10^6 bits 0.4 %
-// (292.3 -> 293.4 us) and saves the 2^27-bit block 1.8 % (1177 -> 1156 us). The exact transforms read w^r,
-// r = 1 .. R-1 (EXACT), or every level's multipliers, R-1 as well, no two of which are a free quarter turn apart (LEVELS).
+// precision reads w alone and forms the others (squarings and constant turns): its innermost
+// pass is bound by the load/store data path (78 % busy with all rows read, a 16-byte load costing four
+// wavefronts whatever the addresses) and has multiply-add slots to spare. Its forward stages with R >= 8 also have a row of
+// w^4, for the passes that need the powers closer to their roots (entry_powers in fft_core.cuh). The exact transforms
+// read w^r, r = 1 .. R-1 (EXACT), or every level's multipliers, R-1 as well, no two of which are a free quarter
+// turn apart (LEVELS).
 enum class Rows { SINGLE, DOUBLE, EXACT, LEVELS };
 __host__ __device__ constexpr bool is_complex(Rows kind) { return kind == Rows::SINGLE || kind == Rows::DOUBLE; }
 __host__ __device__ constexpr int level_rows(int R) { return R / 2; }
 __host__ __device__ constexpr int odd_level_rows(int RO, int R0) { return RO - 1 + RO * (R0 / 2); }
-__host__ __device__ constexpr int stage_rows(int R, Rows kind) {
-    return kind == Rows::SINGLE ? (R >= 8 ? 2 : 1) : kind == Rows::DOUBLE ? level_rows(R) : R - 1;
+__host__ __device__ constexpr int stage_rows(int R, Rows kind, bool inverse) {
+    return kind == Rows::SINGLE ? (R >= 8 && !inverse ? 2 : 1) : kind == Rows::DOUBLE ? level_rows(R) : R - 1;
 }
 __host__ __device__ constexpr int odd_rows(int RO, int R0, Rows kind) {
     return kind == Rows::SINGLE ? 1 : odd_level_rows(RO, R0);
@@ -96,13 +97,13 @@ __host__ __device__ constexpr StagePlan stage_plan(int len, int E, Rows kind) {
         l.P[i] = P;
         l.N[i] = len / P;
         l.s[i] = l.N[i] / l.R[i];
-        const int rows = i == 0 ? 0 : stage_rows(l.R[i], kind);
+        const int rows = i == 0 ? 0 : stage_rows(l.R[i], kind, false);
         l.fwd[i] = StageRow{rows, off};
         off += row_entries(rows, P);
         P *= l.R[i];
     }
     for (int i = 0; i < l.n; ++i) {
-        const int rows = i == l.n - 1 ? 0 : i == 0 && l.RO > 1 ? odd_rows(l.RO, l.R0C, kind) : stage_rows(l.R[i], kind);
+        const int rows = i == l.n - 1 ? 0 : i == 0 && l.RO > 1 ? odd_rows(l.RO, l.R0C, kind) : stage_rows(l.R[i], kind, true);
         l.inv[i] = StageRow{rows, off};
         off += row_entries(rows, l.s[i]);
     }

@@ -1,5 +1,5 @@
 // The powers that single precision stages form from their table entries, against the exact roots of unity: prints the
-// largest distance over every stage of every pass and row length, in units of 2^-24.
+// largest distance over every forward stage of every pass and row length, in units of 2^-24.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -21,11 +21,11 @@ template <int R> void stage(int P) {
     for (int k = 0; k < P; ++k) {
         float2 w[2], pw[4];
         double c, s;
-        for (int r = 0; r < stage_rows(R, Rows::SINGLE); ++r) {
+        for (int r = 0; r < stage_rows(R, Rows::SINGLE, false); ++r) {
             exact(stage_exponent(R, P, r, k, n, Rows::SINGLE), n, &c, &s);
             w[r] = {(float)c, (float)s};
         }
-        entry_powers<float, R>(w, pw);
+        entry_powers<float, R, true>(w, pw);
         for (int l = 0; l < ilog2(R); ++l) {
             exact((uint64_t)(R >> (l + 1)) * k, n, &c, &s);
             worst = std::max(worst, hypot(pw[l].x - c, pw[l].y - s));
@@ -45,7 +45,6 @@ int main() {
             const StagePlan p = stage_plan(ro << lg, 16, Rows::SINGLE);
             for (int i = ro > 1 ? 1 : 0; i < p.n; ++i) {
                 any(p.R[i], p.P[i]);
-                any(p.R[i], p.s[i]);
             }
         }
     }
