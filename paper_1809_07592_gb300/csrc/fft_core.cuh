@@ -26,7 +26,7 @@
 
 namespace pa {
 
-// First statement of every pass kernel (they are launched with launch_chained): waits until the stream's
+// First statement of every pass kernel but the staged last pass (they are launched with launch_chained): waits until the stream's
 // previous kernel has finished and its writes are visible, then lets the next kernel start once
 // every CTA of this one has got here. A chain of small launches loses the launch latency between its
 // kernels, and a large one's first CTAs fill the SMs that the last wave of the kernel before leaves
@@ -911,7 +911,7 @@ __device__ __forceinline__ void cta_fft(cx<T> *sm, cx<T> *v, uint32_t tq, uint32
 // Single precision reads one column table per stage, w^{P_i u}, and forms the stage's multipliers by squarings, as it
 // does elsewhere. Double precision reads one per butterfly level: every multiplier is then the product of two
 // rounded roots, off by 4.25 units of 2^-53 at most (2.1 seen). Formed by squarings they were off by up to 18: the
-// rounding margins of a 2^23-bit key (512 * 64 * 384) were 8.2e-12 in the mean, now 4.3e-12 (with twiddled
+// rounding margins of a 2^23-bit key (512 * 64 * 384) were 8.2e-12 in the mean, now 4.0e-12 (with twiddled
 // inputs 6.5e-12), and a batch of 64 keys of 10^6 bits takes 10.05 ms instead of 10.11.
 // hu[l] = the entry of level l of stage I (SINGLE: hu[0], the last level's) in column u, h its entry in table 0.
 template <typename T, int LEN, int E, int I>

@@ -38,11 +38,12 @@ namespace pa {
 // CTAs overlap their load, transform and store phases.
 __host__ __device__ constexpr int min_blocks(int threads) { return threads >= 1024 ? 1 : (1024 / threads > 16 ? 16 : 1024 / threads); }
 // The fused innermost passes ask for 512 resident threads per SM (<= 128 registers each; at most 16 CTAs).
-// In single precision they ask for 768, at most 8 CTAs: 17-31 % faster than 512 on the lengths around 2^20
-// (more CTAs overlap their barrier and load phases) with no spills. Rows of 5120 values (CTAs of 320 threads)
-// ask for three CTAs and rows of 4608 (288 threads) for four: 8.8 % and 0.6 % faster than with one less
-// (all with self-sorting stages). On the in-place stages a fourth CTA for 5120 took the pass over 32 pairs
-// from 156 to 213 us.
+// In single precision they ask for 768, at most 8 CTAs (more CTAs overlap their barrier and load phases), with at most 8
+// bytes of spills. Rows of 5120 values (CTAs of 320 threads) ask for three CTAs and rows of 4608 (288 threads)
+// for four. Over 2^25 values (us, k_middle alone): rows of 4096 122 (with 512 threads 139), 6144 133 (193), 2304 125 (135),
+// 3072 120 (133); 5120 with two, three CTAs 140, 124, four took 32 pairs from 156 to 213; 4608 with three, four 125, 121.
+// Asking for 1024 threads is faster on 2304, 2560, 3072 and 4096 (117, 114, 114, 114; 2560 takes 126 with 768) and on
+// 8192 (176, 209 with 768), and the same on the shorter rows: not taken yet.
 __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes = 16) {
     return elem_bytes > 8 ? (threads >= 512 ? 1 : (512 / threads > 16 ? 16 : 512 / threads))
                           : (threads >= 768 ? 1
@@ -53,8 +54,10 @@ __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes =
 
 // The two-row kernels in single precision (double precision keeps the 512 threads of the rule above). The
 // split kernel asks for 1024 threads: the 256-block uneven batch took 9.99 ms, with 768, 640 and 512
-// threads 10.06, 10.25 and 10.47. The half-length kernel asks for 640: the 2^27-bit block took 1.179 ms, with
-// 512 and 768 threads 1.210 and 1.190.
+// threads 10.06, 10.25 and 10.47. By row length (2^25 values, us with 1024 and 768): 1280 117 and 131, 1536 115 and 121,
+// 2304 125 and 158, 2560 123 and 150, 4096 128 and 158; 512 54 and 51, 640 82 and 79, 768 85 and 80, 1024 103 and 98, 2048
+// 115 and 112, others alike. Rows of 384 to 2048 and 8192 values spill 24-112 bytes for it. The half-length kernel asks
+// for 640: the 2^27-bit block took 1.179 ms, with 512 and 768 threads 1.210 and 1.190 (before its second table row).
 __host__ __device__ constexpr int min_blocks_split(int threads, int elem_bytes) {
     return elem_bytes > 8 ? min_blocks_inner(threads) : min_blocks(threads);
 }
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
         pass_twiddles<T, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
     }
     // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
-    // addresses in registers through the transform (80 bytes of spills)
+    // addresses in registers through the transform (80 bytes of spills; length 256 still has 60 to 70)
     asm volatile("" : "+r"(S));
 #pragma unroll
     for (int s = 0; s < E; ++s) w[(INV ? elem_of<T, LEN, E>(tq, s) : f + s * (LEN / E)) * S] = v[s];
@@ -763,7 +766,7 @@ template <typename T, int LEN, int E> struct Mirror {
 // Forward transform, Eq. 5-10 split with the mirror bin, X*V/L, then the
 // inverse transform of Y1 + i*Y2 written to the pair's slot in Wi. The first block's product waits in
 // the row it came from, which the transform has consumed, while the second block is transformed: in
-// registers it took 32 of a thread's, so that one CTA of 512 threads filled an SM and long rows spilled.
+// registers it took 32 of a thread's, so that one CTA of 512 threads filled an SM.
 template <typename T, int LEN, int E>
 __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_split(2 * (LEN / E), sizeof(cx<T>)))
     k_middle_split(cx<T> *Wf, cx<T> *__restrict__ Wi, uint64_t L, uint32_t nblocks, uint32_t lgL1, uint32_t lgM,

@@ -18,10 +18,12 @@ namespace pa {
 
 // Whether this thread's launch_chained makes ordinary launches: under stream capture. A graph launches its next kernel
 // without delay, and CTAs that start early there crowd onto the SMs the running kernel leaves free instead of
-// spreading over all of them. Two FP64 blocks of a class of length 262144 replayed in 244 us with such
-// edges and in 133 with ordinary ones (launched one by one: 150); 256 uneven blocks take the same time either way
-// (9.96 and 9.99 ms). The calls that can be captured set it for their duration: asking the stream at every launch
-// cost a call of eight launches 1.2 us.
+// spreading over all of them. Two FP64 blocks of a class of length 262144 replay in 126 us with ordinary edges and in 236
+// with overlapped ones (launched one by one: 150), eight of length 65536 in 114 and 189; batches from 2^21 values
+// on take the same time either way (256 uneven blocks 9.99 and 9.96 ms), the smallest replay 2 us more (one FP32 block of
+// 65536: 35.5 and 33.2). Overlapping only grids of at most 16, 32 or 64 CTAs gained nothing (one FP64 block of 65536
+// 62.6, 79.1 and 79.1 us; with ordinary edges 62.6). The calls that can be captured set this for their duration: asking
+// the stream at every launch cost a call of eight launches 1.2 us.
 inline thread_local bool t_ordinary_launches = false;
 struct LaunchesFor {
     bool before = t_ordinary_launches;
