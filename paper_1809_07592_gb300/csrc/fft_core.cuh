@@ -477,9 +477,9 @@ __device__ __forceinline__ void level_powers(cx<T> w, cx<T> *pw) {
 // error of the key's large low frequencies into the seed's. Margins there fell to 0.5 of what they were in the geometric
 // mean over 33 splits of eight lengths (four blocks of 2^24 bits to 2^23, 256 * 128 * 768: 7.8e-2, now 3.5e-2).
 // It costs the split pass 5 and 8 % on rows of 3072 and 6144 values (registers) and saves it up to 6 % on others; 256
-// uneven blocks take the same 10.0 ms. The half-length form's two-row pass and the middle strided pass take it too (a
-// 2^27-bit block 1177 -> 1156 us). The plain passes of key pairs, whose margins are far below (0.54-0.83 of those with twiddled
-// inputs), read w alone: a second row made the innermost pass 1-3.5 % slower on most row lengths (4096: 118.2 -> 122.5 us).
+// uneven blocks take the same 10.0 ms. The passes of plans, whose margins are far below (0.42-0.83 of those with twiddled
+// inputs), read w alone: a second row made the innermost pass 1-3.5 % slower on most row lengths (4096: 118.2 -> 122.5 us)
+// and the middle strided pass of the 2^27-bit block 3 % (202.5 -> 209.0 us).
 template <typename T, int R, bool NEAR>
 __device__ __forceinline__ void entry_powers(const cx<T> *w, cx<T> *pw) {
     level_powers<T, R>(w[0], pw);

@@ -57,7 +57,7 @@ __host__ __device__ constexpr int min_blocks_inner(int threads, int elem_bytes =
 // threads 10.06, 10.25 and 10.47. By row length (2^25 values, us with 1024 and 768): 1280 117 and 131, 1536 115 and 121,
 // 2304 125 and 158, 2560 123 and 150, 4096 128 and 158; 512 54 and 51, 640 82 and 79, 768 85 and 80, 1024 103 and 98, 2048
 // 115 and 112, others alike. Rows of 384 to 2048 and 8192 values spill 24-112 bytes for it. The half-length kernel asks
-// for 640: the 2^27-bit block took 1.179 ms, with 512 and 768 threads 1.210 and 1.190 (before its second table row).
+// for 640: the 2^27-bit block took 1.179 ms, with 512 and 768 threads 1.210 and 1.190.
 __host__ __device__ constexpr int min_blocks_split(int threads, int elem_bytes) {
     return elem_bytes > 8 ? min_blocks_inner(threads) : min_blocks(threads);
 }
@@ -325,10 +325,10 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     }
 }
 
-// Middle-level strided pass (three-level plans only), forward or inverse.
+// Middle-level strided pass (three-level plans only), forward or inverse (NEAR: entry_powers).
 // S is the innermost length (the stride of this pass); blocks of LEN*S elements.
 // Grid (S/COLS, blocks * pairs).
-template <typename T, int LEN, int COLS, int E, bool INV>
+template <typename T, int LEN, int COLS, int E, bool INV, bool NEAR = false>
 __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     k_mid(cx<T> *__restrict__ W, uint64_t L, uint32_t S, TwTab<T> tw) {
     begin_after_previous(W);
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(COLS * LEN / E, min_blocks(COLS * LEN / E))
     if constexpr (INV) {
         inverse_columns<T, LEN, COLS, E, 1>(sm, v, tq, col, tw, gridDim.x, blockIdx.x, S, LEN);
     } else {
-        cta_fft<T, LEN, COLS, E, false, true>(sm, v, tq, col, tw.st[1]);
+        cta_fft<T, LEN, COLS, E, false, NEAR>(sm, v, tq, col, tw.st[1]);
         pass_twiddles<T, E, COLS>(v, tw.fw[1], gridDim.x, f, blockIdx.x, col);
     }
     // the stride anew: where loads and stores go to the same rows, the compiler would keep 16
@@ -867,9 +867,9 @@ __global__ void __launch_bounds__(2 * (LEN / E), min_blocks_real(2 * (LEN / E), 
     if constexpr (Plan<T, LEN, E>::RO == 1) {
 #pragma unroll
         for (int s = 0; s < E; ++s) v[s] = fresh(wt + elem_of<T, LEN, E>(0, s));
-        cta_fft<T, LEN, 1, E, false, true>(sm, v, tq, 0, tw.st[2]);
+        cta_fft<T, LEN, 1, E, false>(sm, v, tq, 0, tw.st[2]);
     } else {
-        cta_fft_fwd_odd<T, LEN, E, true>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
+        cta_fft_fwd_odd<T, LEN, E, false>(sm, v, tq, tw.st[2], [&](uint32_t o) { return fresh(wt + o); });
     }
     store_stage<T, LEN, 1, E, Plan<T, LEN, E>::n - 1>(sm, v, tq, 0);  // the slots this thread read last
     __syncthreads();

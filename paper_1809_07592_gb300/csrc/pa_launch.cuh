@@ -70,7 +70,7 @@ cudaError_t launch_fwd(int lgLEN, In kind, const FwdArgs &in, uint32_t slots, cx
 
 template <typename T>
 cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S, uint32_t pairs, TwTab<T> tw,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool near_roots) {
     constexpr int E = Shape<T>::E;
     return by_len<kMinLgStrided, kMaxLgStrided>(lgLEN, [&](auto c) {
         constexpr int LEN = decltype(c)::value;
@@ -85,6 +85,9 @@ cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S
             return launch_chained(kern, grid, COLS * LEN / E, sb, st, W, L, S, tw);
         } else {
             auto kern = k_mid<T, LEN, COLS, E, false>;
+            if constexpr (kRows<T> == Rows::SINGLE) {
+                if (near_roots) kern = k_mid<T, LEN, COLS, E, false, true>;
+            }
             cudaError_t e = set_smem(kern, sb);
             if (e != cudaSuccess) return e;
             return launch_chained(kern, grid, COLS * LEN / E, sb, st, W, L, S, tw);
@@ -250,7 +253,7 @@ cudaError_t launch_inv_bits(int lgLEN, const cx<T> *W, uint64_t L, uint64_t m, u
     template cudaError_t launch_fwd<T>(int, In, const FwdArgs &, uint32_t, cx<T> *, uint64_t, TwTab<T>,          \
                                        cudaStream_t);                                                            \
     template cudaError_t launch_mid<T>(int, bool, cx<T> *, uint64_t, uint32_t, uint32_t, TwTab<T>,               \
-                                       cudaStream_t);                                                           \
+                                       cudaStream_t, bool);                                                     \
     template cudaError_t launch_middle<T>(int, int, int, cx<T> *, cx<T> *, uint64_t, uint32_t, TwTab<T>, cx<T>,  \
                                           cudaStream_t);                                                        \
     template cudaError_t launch_inv_bits<T>(int, const cx<T> *, uint64_t, uint64_t, uint32_t, const uint32_t *,  \

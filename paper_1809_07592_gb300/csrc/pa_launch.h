@@ -245,10 +245,10 @@ FwdArgs seed_args(const uint32_t *bits, uint64_t n, uint64_t m, bool pack, uint6
     }
     return in;
 }
-// S: innermost length (the stride of the middle strided pass).
+// S: innermost length (the stride of the middle strided pass). near_roots: the forward pass's stages read w^4 (entry_powers).
 template <typename T>
 cudaError_t launch_mid(int lgLEN, bool inverse, cx<T> *W, uint64_t L, uint32_t S, uint32_t pairs, TwTab<T> tw,
-                       cudaStream_t st);
+                       cudaStream_t st, bool near_roots = false);
 // Innermost pass of length ro * 2^lg. mode 0: the fused convolution step; mode 1:
 // the seed spectrum.
 template <typename T>

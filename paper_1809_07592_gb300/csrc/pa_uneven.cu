@@ -109,7 +109,7 @@ int mid_chunks(const ClassRun &c, bool inverse, cx<T> *W, uint32_t slots, cudaSt
     const TwTab<T> tw = tw_tab<T>(c.tw.lay, c.tw.mem);
     for (uint32_t s0 = 0; s0 < slots; s0 += per) {
         const uint32_t k = (slots - s0 < per) ? slots - s0 : per;
-        U_CUDA(launch_mid<T>(c.geo.lgM, inverse, W + (uint64_t)s0 * c.geo.L, c.geo.L, c.geo.inner(), k, tw, st));
+        U_CUDA(launch_mid<T>(c.geo.lgM, inverse, W + (uint64_t)s0 * c.geo.L, c.geo.L, c.geo.inner(), k, tw, st, true));
     }
     return PA_OK;
 }
