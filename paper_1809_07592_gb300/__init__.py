@@ -239,7 +239,7 @@ def pa_plan_set_storage_bits(plan: int, bits: int) -> None:
 
 
 def pa_plan_expire_waits(plan: int, launches: int = 1) -> None:
-    """Test hook: the next `launches` pipelined convolution launches let their bounded wait run out."""
+    """Test hook: the next `launches` staged last-pass launches let their bounded wait run out."""
     _check(lib().pa_plan_expire_waits(plan, launches), "pa_plan_expire_waits")
 
 
